@@ -1,43 +1,43 @@
 // Block-sparse attention with online softmax on the sm_100a tensor cores.
 //
-// One CTA owns one 128-row query tile of one head: one query block of 128 tokens, or two query
-// blocks of 64 whose lists are merged into an ascending union (one flag bit per query block; rows of
-// the half that does not list a key block see -inf there).  Keys are processed 64 at a time: a "key
-// step" is one 64-token block, or one half of a 128-token block.
+// A query tile is 128 rows of one head: one query block of 128 tokens, or two query blocks of 64 whose
+// lists are merged (two flag bits per key block; rows of the half that does not list a key block get
+// weight 0 there).  Keys are processed 128 at a time: a "key step" is one 128-token block or two listed
+// 64-token blocks.
 //
-// Two CTAs share an SM (256 threads, 105 KB of shared memory and 256 of the 512 tensor-memory
-// columns each).  They work on different query tiles and drift out of phase, so while the softmax
-// warps of one compute exponentials -- the special-function unit is the scarcest resource of this
-// kernel -- those of the other wait, load scores or take maxima, and the set-up and the epilogue of
-// one tile hide behind the key steps of the other.  Inside a CTA the scores are double-buffered in
-// tensor memory: S of step h+1 is complete before the softmax of step h ends, so the serial chain
-// softmax -> P V -> Q K^T -> softmax is off the critical path.
+// What bounds it: for a 128 x 128 tile the tensor pipe needs 1024 clocks (512 for Q K^T, 512 for P V)
+// and the special-function units 1024 as well (ex2 issues every 8 clocks per sub-partition), and within
+// a tile the products and the softmax of a step are serial.  So one persistent CTA per SM runs two
+// independent streams on different query tiles, each with its own warps, barriers, buffers and half of
+// the tensor memory: while one stream takes exponentials the other has its products running.  A stream
+// draws its tiles from a counter; the loads and the first scores of its next tile overlap the end of
+// the present one.
 //
 // Warp roles (registers are moved from the helper warps to the softmax warps at start):
-//   warps 0-3   softmax, one thread per query row (lane quarter = warp).  Per key step a thread reads
-//               its row of S (64 columns), takes the max, rescales its row of O only when the max
-//               grew by more than 2^8, writes P = 2^(s*scale*log2e - m) as bf16 over the first half
-//               of the S buffer and adds the row sum; at the end it writes O / l (and lse).
-//   warps 4-7   one helper role each, rotated with the CTA index so that the two CTAs of an SM
-//               rarely put the same role on the same sub-partition:
-//               K producer  TMA loads of Q (once) and of the listed K blocks into a two-stage ring
-//                           (cp.async.bulk.tensor, 128-byte swizzle, completion on mbarriers);
-//               V producer  the same for V (its own ring: V_h is needed two key steps after K_h);
-//               QK issuer   S_h = Q K_h^T (tcgen05.mma, operands in shared memory), one elected lane;
-//               PV issuer   O += P_h V_h with P_h read from tensor memory.
-// Tensor memory (256 columns per CTA): O | S[2]  =  128 + 2 x 64; key step h uses S[h & 1] and
-// shared-memory stage h & 1; P_h aliases S[h & 1].
+//   warps 0-3, 4-7  softmax of stream 0, 1: one thread per query row (lane quarter = warp & 3).  Per key
+//               step a thread reads its row of S (128 columns), takes the max, rescales its row of O only
+//               when the max grew by more than 2^8, writes P = 2^(s*scale*log2e - m) as bf16 over the
+//               first half of the S columns and adds the row sum; at the end it writes O / l (and lse).
+//   warps 8, 9  MMA issuers: S_0 = Q K_0^T, then per step O += P_h V_h followed by S_{h+1} = Q K_{h+1}^T.
+//               The tensor pipe executes a stream's products in issue order, so S_{h+1} may overwrite the
+//               columns of P_h without a wait in between.  P V starts when 96 of the 128 keys of P_h are
+//               written, while the softmax still works on the others.  A step has ONE commit (a commit
+//               costs the issuing warp ~100 clocks): S_{h+1} complete, which also says that P_h V_h has
+//               released its half of V and Q K_{h+1}^T its K.
+//   warps 10, 11  producers: draw the tile, then TMA loads (cp.async.bulk.tensor, 128-byte swizzle,
+//               completion on mbarriers) of Q and of the steps' K (one 32 KB buffer: S_h complete frees it a
+//               whole softmax before the next product wants it) and V (first 64 keys double-buffered, last
+//               64 single).
+// Tensor memory (256 columns per stream): O (128) | S (128), P_h in the first 64 columns of S.
 //
-// CTAs run head-major (the K/V of one or two heads stay in L2).  Within a head the tiles are taken in
-// an order that tile_order_kernel writes just before the launch: by the first key block of their
-// lists, so that the ~300 tiles in flight together read neighbouring key blocks (a head's K and V no
-// longer fit one die's half of the L2 at 75 000 tokens and more), except for the last two heads of the
-// launch, whose tiles go longest-list-first so that the launch does not end on a long tile that
-// started late.  The K tile of the first listed key block is requested during set-up, before the step
-// list is complete, and that block is put first.
+// The step lists come from attn_plan_kernel (one warp per tile), which runs just before; the tiles are
+// taken head-major (the K/V of one or two heads stay in L2), within a head in the order of
+// tile_order_kernel: by the first key block of their lists once a head's K and V no longer fit one die's
+// half of the L2, except for the last two heads of the launch, whose tiles go longest-list-first so that
+// the launch does not end on a long tile that started late.
 //
-// Every wait is bounded; a wait that runs out raises a CTA-wide abort flag and the status word, the
-// roles drain, tensor memory is freed and the CTA exits.
+// Every wait is bounded; a wait that runs out raises the stream's abort flag and the status word, the
+// stream's roles drain and stop, the other streams take the remaining tiles.
 #include <cuda.h>
 
 #include "common.cuh"
@@ -46,72 +46,50 @@
 namespace heart {
 using namespace tc;
 
-constexpr int kAttnThreads = 256;
-// warp roles: 0-3 softmax (lane quarter = warp), then one helper per SM sub-partition
-constexpr int kRoleKProd = 0, kRoleVProd = 1, kRolePV = 2, kRoleQK = 3;  // helper warp 4 + ((role + CTA index) & 3)
-constexpr int kRegsSoftmax = 176, kRegsHelper = 80;  // (176 + 80) * 128 threads = the CTA's 256 x 128
-constexpr int kStep = 64;   // keys per key step
-constexpr int kStages = 2;  // K / V ring depth = number of S buffers
-constexpr int kTmemCols = 256;  // O (128) + S[2] (2 x 64): two CTAs share the 512 columns of an SM
-constexpr int kMaxNb = HEART_MAX_BLOCKS;
+constexpr int kStreams = 2;
+constexpr int kAttnThreads = 384;
+constexpr int kWarpMma = 8, kWarpProd = 10;  // + stream
+constexpr int kRegsSoftmax = 216, kRegsHelper = 72;  // 216 * 256 + 72 * 128 = the CTA's 384 x 168
+constexpr int kHalfBytes = 16384;  // 64 dims of 128 keys of K, or 64 keys of V
+constexpr int kQBytes = 2 * kHalfBytes;
 
-// Shared-memory plan.
-template <int B>
-struct AttnSmem {
-  static constexpr int HPB = B / kStep;         // key steps per key block (1 or 2)
-  static constexpr int QBT = 128 / B;           // query blocks per CTA (1 or 2)
-  static constexpr int Q_BYTES = 128 * 256;     // [2 dim halves][128 rows][64] bf16, 128-byte swizzle
-  static constexpr int KV_BYTES = kStep * 256;  // [2 dim halves][64 rows][64] bf16, 128-byte swizzle
-  static constexpr int OFF_Q = 0;
-  static constexpr int OFF_K = OFF_Q + Q_BYTES;
-  static constexpr int OFF_V = OFF_K + kStages * KV_BYTES;
-  static constexpr int OFF_UNI = OFF_V + kStages * KV_BYTES;  // int32[kMaxNb]: J | flags << 16
-  static constexpr int OFF_TBL = OFF_UNI + 4 * kMaxNb;        // uint32[kMaxNb]: flags per key block
-  static constexpr int OFF_BAR = OFF_TBL + 4 * kMaxNb;        // mbarriers and scalars
-  static constexpr int TOTAL = OFF_BAR + 512;
-};
+// Shared-memory plan (the dynamic allocation itself is 1024-byte aligned), per stream.
+constexpr int kOffQ = 0;                         // [2 dim halves][128 rows][64] bf16, 128-byte swizzle
+constexpr int kOffK = kOffQ + kQBytes;           // [2 dim halves][128 keys][64]
+constexpr int kOffVa = kOffK + 2 * kHalfBytes;   // two buffers [2 dim halves][64 keys][64]: keys 0-63 of a step
+constexpr int kOffVb = kOffVa + 2 * kHalfBytes;  // keys 64-127
+constexpr int kStreamBytes = kOffVb + kHalfBytes;
+constexpr int kOffBar = kStreams * kStreamBytes;
 
 struct AttnBars {
-  uint64_t q_full;
-  uint64_t k_full[kStages], v_full[kStages];  // TMA -> MMA issuer
-  uint64_t qk_done[kStages];                  // S_h complete: softmax may read it, K stage is free
-  uint64_t pv_done[kStages];                  // P_h V_h complete: V stage and S/P buffer are free
-  uint64_t p_full[kStages];                   // P_h written (one arrival per warp of the stream)
-  uint64_t drain[2];                          // abort path: the issuers' products in flight have landed
-  uint32_t tmem_base;
-  int chunk_cnt[32];  // flagged key blocks per 32-block chunk (set-up)
-  int n_union;
+  uint64_t q_full, k_full, va_full[2], vb_full;  // TMA -> issuer
+  uint64_t s_full;           // S_h complete, and with it every product issued before it
+  uint64_t p_full[2];        // keys 0-95 / 96-127 of P_h written (one arrival per softmax warp)
+  uint64_t o_done;           // the last product of a tile is complete
+  uint64_t tile_full[2], tile_empty[2];  // the producer's announcements of tiles
+  uint64_t drain;            // abort path: the issuer's products in flight have landed
+  int4 tile[2];              // query tile of its head, listed key blocks, head of the launch, 1 (0: no tile left)
   int abort;
-  int bad;
-  int first_j;  // key block whose K tile was requested before the step list existed (-1: none)
 };
+constexpr int kBarBytes = (sizeof(AttnBars) + 127) / 128 * 128;
+constexpr int kAttnSmem = kOffBar + kStreams * kBarBytes + 128;
 
+// A key step as the plan kernel writes it.  128-token blocks: the key block.  64-token blocks: two
+// halves of 16 bits, key block | (flag of query block 0, flag of query block 1) << 10 | ragged block << 12; no
+// flag: the keys do not count (the second half of the last step when the number of blocks is odd).
 struct AttnParams {
-  const int32_t *kv_idx, *kv_cnt;
+  const uint32_t *steps;  // [B*H][tiles of a head][step_pitch]
+  const uint32_t *tiles;  // [tiles of the launch] tile of the head | listed key blocks << 16, in launch order
+  int32_t *counter;       // tiles drawn beyond the first one of every stream (zeroed by the plan kernel)
   uint16_t *O;
   float *lse;
   int32_t *status;
   long long sb, sh, sn;
-  int H, N, nb, idx_stride, n_ctas_per_head, dense;
-  int h0, hcount, R_all;  // this launch covers heads [h0, h0 + hcount) of every batch entry; R_all = B*H
-  const int32_t *order;   // [heads of the launch][n_ctas_per_head]: tile of the head that CTA i takes (NULL: i)
+  int H, N, nb, n_tiles, n_tiles_per_head, step_pitch, dense;
+  int h0, hcount;  // this launch covers heads [h0, h0 + hcount) of every batch entry
   float scale_log2;
-  int test_skip_v;  // test-hook builds only: CTA 0 leaves out the V copy of its second key step
+  int test_skip_v;  // test-hook builds only: stream 0 of CTA 0 leaves out one V copy of its first tile
 };
-
-// Clock-stamp trace (compile with -DHEART_TRACE; the caller's lse buffer must then have one extra
-// row of N >= 4096 floats behind its R*N entries): CTA 0 records clock64() at the marked points of
-// its first 64 key steps.  Slots: 0-7 softmax warp 2, 16-23 softmax warp 6, 8-15 the MMA issuer.
-#ifdef HEART_TRACE
-#define HEART_TR(h, slot)                                                             \
-  do {                                                                                \
-    if (trace_base != nullptr && (h) < 64) trace_base[(h) * 32 + (slot)] = clock64(); \
-  } while (0)
-#else
-#define HEART_TR(h, slot) \
-  do {                    \
-  } while (0)
-#endif
 
 __device__ __forceinline__ float fmax3(float a, float b, float c) {
   float r;
@@ -119,197 +97,98 @@ __device__ __forceinline__ float fmax3(float a, float b, float c) {
   return r;
 }
 
-template <int B>
-__global__ void __launch_bounds__(kAttnThreads, 2)
-    attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_kv,
-                   const __grid_constant__ CUtensorMap map_v, const AttnParams p) {
-  using L = AttnSmem<B>;
-  constexpr int HPB = L::HPB;
-  extern __shared__ unsigned char smem_dyn[];
-  unsigned char *smem = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) &
-                                                          ~static_cast<uintptr_t>(1023));
-  unsigned char *Qs = smem + L::OFF_Q, *Ks = smem + L::OFF_K, *Vs = smem + L::OFF_V;
-  int32_t *uni = reinterpret_cast<int32_t *>(smem + L::OFF_UNI);
-  uint32_t *tbl = reinterpret_cast<uint32_t *>(smem + L::OFF_TBL);
-  AttnBars *bars = reinterpret_cast<AttnBars *>(smem + L::OFF_BAR);
-  volatile int *abort = &bars->abort;
+struct Sums {
+  float a, b, c, d;
+};
+// Weights 2^(s*c - m) of 32 scores of a row, packed to bf16, and their sums.  The row sum is taken over the
+// rounded weights, the ones the P V product really uses, so numerator and denominator carry the same
+// rounding: O stays a weighted mean.
+__device__ __forceinline__ void exp32(const uint32_t *s, uint64_t c2, uint64_t neg_m2, uint32_t *pk, Sums &sums) {
+#pragma unroll
+  for (int i = 0; i < 32; i += 4) {
+    float x0, x1, x2, x3;
+    unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(s[i]), __uint_as_float(s[i + 1])), c2, neg_m2), x0, x1);
+    unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(s[i + 2]), __uint_as_float(s[i + 3])), c2, neg_m2), x2, x3);
+    pk[i >> 1] = pack_bf16x2(ex2(x0), ex2(x1));
+    pk[(i >> 1) + 1] = pack_bf16x2(ex2(x2), ex2(x3));
+    add_bf16x2_to_f32(sums.a, sums.b, pk[i >> 1]);
+    add_bf16x2_to_f32(sums.c, sums.d, pk[(i >> 1) + 1]);
+  }
+}
+__device__ __forceinline__ float max64(const uint32_t *s) {
+  float m[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+  for (int i = 0; i < 64; i += 8)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) m[j] = fmax3(m[j], __uint_as_float(s[i + 2 * j]), __uint_as_float(s[i + 2 * j + 1]));
+  return fmaxf(fmaxf(m[0], m[1]), fmaxf(m[2], m[3]));
+}
 
+template <int B>
+__global__ void __launch_bounds__(kAttnThreads, 1)
+    attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
+                   const __grid_constant__ CUtensorMap map_v, const AttnParams p) {
+  extern __shared__ __align__(1024) unsigned char smem[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  // The helper roles rotate with the CTA index: the two CTAs that share an SM then rarely have the
-  // same role (above all the issuer of the score products) on the same sub-partition.
-  const int kWarpKProd = 4 + ((kRoleKProd + blockIdx.x) & 3), kWarpVProd = 4 + ((kRoleVProd + blockIdx.x) & 3),
-            kWarpPV = 4 + ((kRolePV + blockIdx.x) & 3), kWarpQK = 4 + ((kRoleQK + blockIdx.x) & 3);
-  // Tiles run head-major, which keeps the K/V of one or two heads in L2; within a head in the order
-  // of the table (tiles whose lists start at the same key block together; the last two heads
-  // longest-first, so that the launch ends on short tiles).
-  const int rr = blockIdx.x / p.n_ctas_per_head;
-  const int cta_in_head = p.order ? __ldg(&p.order[blockIdx.x]) : (int)(blockIdx.x % p.n_ctas_per_head);
-  const int bidx = rr / p.hcount, hidx = p.h0 + rr % p.hcount;
-  const int r = bidx * p.H + hidx;
-  const int row0 = cta_in_head * 128;  // first query token of this CTA
-  const int nb = p.nb;
-#ifdef HEART_TRACE
-  long long *trace_base = (blockIdx.x == 0 && p.lse != nullptr)
-                              ? reinterpret_cast<long long *>(p.lse + (size_t)p.R_all * p.N)
-                              : nullptr;
-#endif
+  const int st = warp < 8 ? warp >> 2 : warp & 1;  // stream of this warp
+  AttnBars *bars = reinterpret_cast<AttnBars *>(smem + kOffBar + st * kBarBytes);
+  uint32_t *tmem_base = reinterpret_cast<uint32_t *>(smem + kOffBar + kStreams * kBarBytes);
+  volatile int *abort = &bars->abort;
+  unsigned char *mem = smem + st * kStreamBytes;
 
   // ------------------------------------------------------------------ set-up
-  // A kernel that follows on the stream under programmatic stream serialisation (the next layer-step's
-  // block-sum pass) may be scheduled once every tile of this launch has started: its CTAs then fill the
-  // SMs that the last tiles leave behind and wait there for this launch to complete.
-  pdl_launch_dependents();
-  if (tid == 0) HEART_TR(0, 28);
-  // The lists of this tile's query blocks come from global memory: their loads are issued first
-  // (speculatively, inside the row pitch) so that their latency overlaps the rest of the set-up.
-  constexpr int kPre = kMaxNb / kAttnThreads;  // entries per thread held in registers
-  int cnt_q[L::QBT];
-  int32_t ent[L::QBT][kPre];
-#pragma unroll
-  for (int qb = 0; qb < L::QBT; ++qb) {
-    const int I = cta_in_head * L::QBT + qb;
-    const size_t row = (size_t)r * nb + I;
-    cnt_q[qb] = (I < nb) ? (p.dense ? nb : p.kv_cnt[row]) : 0;
-#pragma unroll
-    for (int k = 0; k < kPre; ++k) {
-      const int t = tid + k * kAttnThreads;
-      ent[qb][k] = (I < nb && !p.dense && t < p.idx_stride) ? p.kv_idx[row * p.idx_stride + t] : t;
+  if (tid < kStreams) {
+    AttnBars *b = reinterpret_cast<AttnBars *>(smem + kOffBar + tid * kBarBytes);
+    mbar_init(&b->q_full, 1);
+    mbar_init(&b->k_full, 1);
+    mbar_init(&b->va_full[0], 1);
+    mbar_init(&b->va_full[1], 1);
+    mbar_init(&b->vb_full, 1);
+    mbar_init(&b->s_full, 1);
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&b->p_full[i], 4);      // one arrival per softmax warp
+      mbar_init(&b->tile_full[i], 1);
+      mbar_init(&b->tile_empty[i], 5);  // the softmax warps and the issuer
     }
-  }
-  if (tid == 0) {
-    mbar_init(&bars->q_full, 1);
-    for (int i = 0; i < kStages; ++i) {
-      mbar_init(&bars->k_full[i], 1);
-      mbar_init(&bars->v_full[i], 1);
-      mbar_init(&bars->qk_done[i], 1);
-      mbar_init(&bars->pv_done[i], 1);
-      mbar_init(&bars->p_full[i], 4);  // one arrival per softmax warp
-    }
-    mbar_init(&bars->drain[0], 1);
-    mbar_init(&bars->drain[1], 1);
-    bars->abort = 0;
-    bars->bad = 0;
-    bars->n_union = 0;
+    mbar_init(&b->o_done, 1);
+    mbar_init(&b->drain, 1);
+    b->abort = 0;
     mbar_fence_init();
   }
-  for (int j = tid; j < nb; j += kAttnThreads) tbl[j] = 0u;
-  __syncthreads();
-  if (tid == 0) HEART_TR(1, 28);
-  if (warp == kWarpKProd && lane == 0) {  // the Q tile does not depend on the lists: start it now
-    tma_prefetch_desc(&map_q);
-    tma_prefetch_desc(&map_kv);
-    tma_prefetch_desc(&map_v);
-    mbar_expect_tx(&bars->q_full, L::Q_BYTES);
-    tma_load_4d(Qs, &map_q, &bars->q_full, 0, row0, hidx, bidx);
-    tma_load_4d(Qs + 128 * 128, &map_q, &bars->q_full, 64, row0, hidx, bidx);
-  }
-  if (tid == 0) {
-    // Thread 0 holds the first entry of each list.  Whatever the union turns out to be, that key
-    // block is in it: its K tile is requested now, ~2000 clocks before the step list is ready, and
-    // the compaction below puts the block first (for ascending lists it is the first anyway).
-    int j0 = 0x7fffffff;
-#pragma unroll
-    for (int qb = 0; qb < L::QBT; ++qb)
-      if (cnt_q[qb] > 0 && p.idx_stride > 0) j0 = min(j0, ent[qb][0] < 0 ? 0x7fffffff : ent[qb][0]);
-    if (j0 < nb) {
-      mbar_expect_tx(&bars->k_full[0], L::KV_BYTES);
-      tma_load_4d(Ks, &map_kv, &bars->k_full[0], 0, j0 * B, hidx, bidx);
-      tma_load_4d(Ks + kStep * 128, &map_kv, &bars->k_full[0], 64, j0 * B, hidx, bidx);
-      bars->first_j = j0;
-    } else {
-      bars->first_j = -1;
-    }
-  }
-#pragma unroll
-  for (int qb = 0; qb < L::QBT; ++qb) {  // scatter: flag bit qb of every key block listed by query block qb
-    const int I = cta_in_head * L::QBT + qb;
-    int cnt = cnt_q[qb];
-    if (cnt < 0 || cnt > p.idx_stride) {
-      bars->bad = 1;
-      cnt = cnt < 0 ? 0 : p.idx_stride;
-    }
-#pragma unroll
-    for (int k = 0; k < kPre; ++k) {
-      const int t = tid + k * kAttnThreads;
-      if (t < cnt) {
-        const int J = ent[qb][k];
-        if (J < 0 || J >= nb)
-          bars->bad = 1;  // skipped, reported
-        else
-          atomicOr(&tbl[J], 1u << qb);
-      }
-    }
-    if (cnt > kPre * kAttnThreads) {  // longer than any list of distinct blocks: the slow way
-      const int32_t *list = p.kv_idx + ((size_t)r * nb + I) * p.idx_stride;
-      for (int t = kPre * kAttnThreads + tid; t < cnt; t += kAttnThreads) {
-        const int J = list[t];
-        if (J < 0 || J >= nb)
-          bars->bad = 1;
-        else
-          atomicOr(&tbl[J], 1u << qb);
-      }
-    }
-  }
-  if (tid == 0) HEART_TR(1, 29);
-  if (warp == kWarpQK) {
-    tmem_alloc(&bars->tmem_base, kTmemCols);
+  if (warp == kWarpMma) {
+    tmem_alloc(tmem_base, 512);
     tmem_relinquish();
   }
-  __syncthreads();
-  if (tid == 0) HEART_TR(1, 30);
-  {  // ascending compaction of the flagged key blocks: warp w takes the 32-block chunks w, w+16
-    constexpr int kChunksPerWarp = kMaxNb / 32 / (kAttnThreads / 32);
-    uint32_t f[kChunksPerWarp];
-    unsigned ballot[kChunksPerWarp];
-#pragma unroll
-    for (int i = 0; i < kChunksPerWarp; ++i) {
-      const int J = (warp + i * (kAttnThreads / 32)) * 32 + lane;
-      f[i] = (J < nb) ? tbl[J] : 0u;
-      ballot[i] = __ballot_sync(0xffffffffu, f[i] != 0u);
-      if (lane == 0) bars->chunk_cnt[warp + i * (kAttnThreads / 32)] = __popc(ballot[i]);
-    }
-    __syncthreads();
-    // exclusive prefix over the 32 chunk counts (every warp computes it: lane = chunk)
-    const int mine = bars->chunk_cnt[lane];
-    int incl = mine;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int v = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += v;
-    }
-    // the block whose K tile is already on its way goes first: p0 = its ascending rank
-    const int first_j = bars->first_j;
-    int p0 = 0;
-    if (first_j >= 0) {
-      const unsigned in_chunk = __ballot_sync(0xffffffffu, tbl[(first_j & ~31) + lane] != 0u);
-      p0 = __shfl_sync(0xffffffffu, incl - mine, first_j >> 5) + __popc(in_chunk & ((1u << (first_j & 31)) - 1u));
-    }
-#pragma unroll
-    for (int i = 0; i < kChunksPerWarp; ++i) {
-      const int chunk = warp + i * (kAttnThreads / 32);
-      const int base = __shfl_sync(0xffffffffu, incl - mine, chunk);
-      if (f[i] != 0u) {
-        const int J = chunk * 32 + lane, q = base + __popc(ballot[i] & ((1u << lane) - 1u));
-        uni[J == first_j ? 0 : (q < p0 ? q + 1 : q)] = J | (int)(f[i] << 16);
-      }
-    }
-    const int total = __shfl_sync(0xffffffffu, incl, 31);
-    if (tid == 0) {
-      bars->n_union = total;
-      if (bars->bad) atomicExch(p.status, HEART_ERR_DEVICE_CHECK);
-    }
+  if (warp == kWarpProd && lane == 0) {
+    tma_prefetch_desc(&map_q);
+    tma_prefetch_desc(&map_k);
+    tma_prefetch_desc(&map_v);
   }
+  // Launched with programmatic stream serialisation: everything above overlaps the end of the kernels
+  // before it.  A kernel that follows (the next layer-step's block-sum pass) may be scheduled once every
+  // CTA of this launch has started: its CTAs then fill the SMs that finish first.
+  pdl_wait();
+  pdl_launch_dependents();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if (tid == 0) HEART_TR(0, 29);
-  const uint32_t tmem = bars->tmem_base;
-  const int U = bars->n_union;
-  const int NH = U * HPB;  // key steps; step h uses S buffer and shared-memory stage h & 1
-  // first key token of step h
-  auto key0_of = [&](int h) -> int { return (uni[h / HPB] & 0xffff) * B + (h % HPB) * kStep; };
+  const uint32_t tmem = *tmem_base + st * 256;
 
-  // ------------------------------------------------------------------ roles
+  auto n_steps_of = [](int U) -> int { return B == 128 ? U : (U + 1) / 2; };
+  auto step_entry = [&](const uint32_t *steps, int h) -> uint32_t {
+    if (!p.dense) return __ldcg(&steps[h]);
+    if (B == 128) return h;
+    const uint32_t ragged = (p.N & 63) ? p.nb - 1 : 0x3ff + 1, a = 2 * h, b = 2 * h + 1;
+    return (a | 3u << 10 | (a == ragged ? 1u << 12 : 0u)) | (b < (uint32_t)p.nb ? b | 3u << 10 | (b == ragged ? 1u << 12 : 0u) : a) << 16;
+  };
+  // The next announced tile; false: none left (or abort).  Every lane of the warp gets the same answer.
+  auto next_tile = [&](int t, int4 &ti) -> bool {
+    if (!__all_sync(0xffffffffu, mbar_wait(&bars->tile_full[t & 1], (t >> 1) & 1, abort))) return false;
+    ti = bars->tile[t & 1];
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&bars->tile_empty[t & 1]);
+    return ti.w != 0;
+  };
   // Shared memory must not be released under a copy in flight: a producer that stops early (abort)
   // waits, bounded, for the copies it has issued.
   auto settle = [&](uint64_t *bar, uint32_t parity) {
@@ -317,426 +196,647 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
     while (!mbar_try_wait(bar, parity) && clock64() - t0 < 40000000LL) {
     }
   };
-  if (warp >= 4) setmaxnreg_dec<kRegsHelper>();
-  if (warp == kWarpKProd) {
-    if (lane == 0) {  // ===== TMA producer (Q was started during set-up): K_h into stage h & 1
-      int issued = 0;
-      for (int h = 0; h < NH; ++h) {
-        const int s = h % kStages, ph = (h / kStages) & 1;
-        if (h == 0 && bars->first_j >= 0) {  // requested during set-up
-          issued = 1;
-          continue;
+
+  // ------------------------------------------------------------------ roles
+  if (warp >= kWarpMma) setmaxnreg_dec<kRegsHelper>();
+  if (warp >= kWarpProd) {
+    if (lane == 0) {  // ===== producer
+      bool ok = true;
+      int t = 0, n_q = 0, n_k = 0, n_va = 0, n_vb = 0;  // tiles announced, loads issued
+      // the tile that is announced next, fetched ahead of time
+      int nx = blockIdx.x + st * gridDim.x;  // the first tile of every stream is fixed, the others are drawn
+      uint32_t nx_word = 0, nx_e = 0;
+      const uint32_t *nx_steps = nullptr;
+      auto fetch = [&]() {
+        if (nx >= p.n_tiles) return;
+        const int rr = nx / p.n_tiles_per_head;
+        nx_word = p.dense ? (uint32_t)(nx - rr * p.n_tiles_per_head) | (uint32_t)p.nb << 16 : __ldcg(&p.tiles[nx]);
+        const int r = rr / p.hcount * p.H + p.h0 + rr % p.hcount;
+        nx_steps = p.steps + ((size_t)r * p.n_tiles_per_head + (nx_word & 0xffff)) * p.step_pitch;
+        if (nx_word >> 16) nx_e = step_entry(nx_steps, 0);
+      };
+      auto draw = [&]() {
+        nx = kStreams * gridDim.x + atomicAdd(p.counter, 1);
+        fetch();
+      };
+      int tile = 0, n_steps = 0, bidx = 0, hidx = 0;
+      const uint32_t *steps = nullptr;
+      uint32_t e = 0;
+      // announces tiles up to the next one that has key steps; false: none left
+      auto next_with_steps = [&]() -> bool {
+        for (;; draw()) {
+          if (t >= 2) ok = mbar_wait(&bars->tile_empty[t & 1], ((t >> 1) - 1) & 1, abort);
+          if (!ok) return false;
+          const bool none = nx >= p.n_tiles;
+          const int rr = none ? 0 : nx / p.n_tiles_per_head, U = nx_word >> 16;  // U = listed key blocks
+          bars->tile[t & 1] = none ? make_int4(0, 0, 0, 0) : make_int4(nx_word & 0xffff, U, rr, 1);
+          mbar_arrive(&bars->tile_full[t & 1]);
+          ++t;
+          if (none) return false;
+          if (U == 0) continue;
+          tile = nx_word & 0xffff;
+          n_steps = n_steps_of(U);
+          bidx = rr / p.hcount;
+          hidx = p.h0 + rr % p.hcount;
+          steps = nx_steps;
+          e = nx_e;
+          return true;
         }
-        // the stage is free once S_{h-4} = Q K_{h-4}^T is complete
-        if (h >= kStages && !mbar_wait_relaxed(&bars->qk_done[s], ph ^ 1, abort)) break;
-        const int key0 = key0_of(h);
-        unsigned char *dst = Ks + s * L::KV_BYTES;
-        mbar_expect_tx(&bars->k_full[s], L::KV_BYTES);
-        tma_load_4d(dst, &map_kv, &bars->k_full[s], 0, key0, hidx, bidx);
-        tma_load_4d(dst + kStep * 128, &map_kv, &bars->k_full[s], 64, key0, hidx, bidx);
-        issued = h + 1;
-      }
-      settle(&bars->q_full, 0);  // nobody else waits for Q when the union is empty
-      if (*abort)
-        for (int h = (issued > kStages ? issued - kStages : 0); h < issued; ++h) settle(&bars->k_full[h % kStages], (h / kStages) & 1);
-    }
-  } else if (warp == kWarpVProd) {
-    if (lane == 0) {  // ===== TMA producer: V_h into stage h & 1
-      int issued = 0;
-      for (int h = 0; h < NH; ++h) {
-        const int s = h % kStages, ph = (h / kStages) & 1;
-        if (h >= kStages && !mbar_wait_relaxed(&bars->pv_done[s], ph ^ 1, abort)) break;
+      };
+      auto key_of = [&](int half) -> int { return B == 128 ? (int)e * 128 + half * 64 : (int)((e >> (16 * half)) & 0x3ff) * 64; };
+      auto load_q = [&]() {
+        mbar_expect_tx(&bars->q_full, kQBytes);
+        tma_load_5d(mem + kOffQ, &map_q, &bars->q_full, 0, tile * 128, 0, hidx, bidx);
+        ++n_q;
+      };
+      auto load_k = [&]() {
+        mbar_expect_tx(&bars->k_full, 2 * kHalfBytes);
+        if (B == 128) {
+          tma_load_5d(mem + kOffK, &map_k, &bars->k_full, 0, key_of(0), 0, hidx, bidx);
+        } else {
+#pragma unroll
+          for (int i = 0; i < 4; ++i)  // dim half i >> 1 of block i & 1
+            tma_load_5d(mem + kOffK + i * (kHalfBytes / 2), &map_k, &bars->k_full, 0, key_of(i & 1), i >> 1, hidx, bidx);
+        }
+        ++n_k;
+      };
+      auto load_va = [&]() {
+        const int i = n_va & 1;
+        ++n_va;
 #ifdef HEART_TEST_HOOKS
         // Test-only library: one V tile is never requested (neither the byte count nor the copy), so the
-        // waits that depend on it run out and the abort path below is taken.
-        if (p.test_skip_v && blockIdx.x == 0 && h == 1) continue;
+        // waits that depend on it run out and the abort path is taken.
+        if (p.test_skip_v && blockIdx.x == 0 && st == 0 && n_va == 2) return;
 #endif
-        const int key0 = key0_of(h);
-        unsigned char *dst = Vs + s * L::KV_BYTES;
-        mbar_expect_tx(&bars->v_full[s], L::KV_BYTES);
-        tma_load_4d(dst, &map_v, &bars->v_full[s], 0, key0, hidx, bidx);
-        tma_load_4d(dst + kStep * 128, &map_v, &bars->v_full[s], 64, key0, hidx, bidx);
-        issued = h + 1;
-      }
-      if (*abort)
-        for (int h = (issued > kStages ? issued - kStages : 0); h < issued; ++h) settle(&bars->v_full[h % kStages], (h / kStages) & 1);
-    }
-  } else if (warp == kWarpPV || warp == kWarpQK) {
-    // ===== MMA issuers: warp 7 issues S_h = Q K_h^T, warp 6 issues O += P_h V_h.  Two warps, so that
-    // the barrier round trips of one overlap the issue of the other.  The whole warp runs the loop
-    // (uniform control flow keeps the descriptors in uniform registers), one elected lane issues.
-    if (NH > 0) {
-      constexpr uint32_t idesc_qk = idesc_bf16_f32(128, kStep, false, false);
-      constexpr uint32_t idesc_pv = idesc_bf16_f32(128, 128, false, true);
-      // Descriptors of one key step differ only in the start-address field (low word, no carry out
-      // of it): base + a compile-time offset per 16-element k-step.
-      //   Q, K (K-major): 64 dims = one 128-byte row; dim halves Q: 128*128 B apart, K: 64*128 B.
-      //   V (MN-major):   64 dims = one 128-byte row; dim halves 64*128 B apart (the LBO);
-      //                   16 keys = 16 rows = 2048 B per k-step.
-      auto at = [](uint64_t desc, uint32_t off16) -> uint64_t {
-        return (desc & 0xffffffff00000000ull) | (uint32_t)((uint32_t)desc + off16);
+        mbar_expect_tx(&bars->va_full[i], kHalfBytes);
+        tma_load_5d(mem + kOffVa + i * kHalfBytes, &map_v, &bars->va_full[i], 0, key_of(0), 0, hidx, bidx);
       };
-      const bool leader = elect_one();  // the same lane every time: commits track its MMAs
-      bool ok = true;
-      if (warp == kWarpQK) {
-        const uint64_t q_desc = smem_desc_sw128(smem_u32(Qs), 16, 1024);
-        const uint64_t k_desc = smem_desc_sw128(smem_u32(Ks), 16, 1024);
-        auto issue_qk = [&](int s) {  // S[s] = Q K^T with the K tile that sits in stage s
-          const uint32_t d = tmem + 128 + s * kStep;
-          const uint64_t ks_desc = at(k_desc, s * (L::KV_BYTES >> 4));
-          if (leader) {
-#pragma unroll
-            for (int ks = 0; ks < 8; ++ks)
-              mma_ss(d, at(q_desc, (ks >> 2) * 1024 + (ks & 3) * 2), at(ks_desc, (ks >> 2) * 512 + (ks & 3) * 2),
-                     idesc_qk, ks > 0 ? 1u : 0u);
-            tc_commit(&bars->qk_done[s]);
-          }
-          __syncwarp();
-        };
-        ok = mbar_wait(&bars->q_full, 0, abort);
-        for (int h = 0; h < kStages && h < NH && ok; ++h) {
-          ok = mbar_wait(&bars->k_full[h], 0, abort);
-          if (ok) {
-            tc_fence_after();
-            issue_qk(h);
-          }
-        }
-        for (int h = 0; h + kStages < NH && ok; ++h) {
-          const int s = h % kStages, ph = (h / kStages) & 1;
-          // S[s] holds P_h until the product P_h V_h has read it
-          ok = mbar_wait(&bars->k_full[s], ph ^ 1, abort);
-          if (ok) ok = mbar_wait(&bars->pv_done[s], ph, abort);
+      auto load_vb = [&]() {
+        mbar_expect_tx(&bars->vb_full, kHalfBytes);
+        tma_load_5d(mem + kOffVb, &map_v, &bars->vb_full, 0, key_of(1), 0, hidx, bidx);
+        ++n_vb;
+      };
+      fetch();
+      if (next_with_steps()) {
+        load_q();
+        load_k();
+        load_va();
+        load_vb();
+        draw();
+        int h = 0;
+        for (uint32_t g = 0;; ++g) {  // g: key steps so far, over all tiles
+          const uint32_t e_next = h + 1 < n_steps ? step_entry(steps, h + 1) : 0u;
+          // S of step g complete: K is free, and the product of step g - 1 has released its V
+          ok = mbar_wait(&bars->s_full, g & 1, abort);
           if (!ok) break;
-          HEART_TR(h, 10);
-          tc_fence_after();
-          issue_qk(s);
-          HEART_TR(h, 11);
-        }
-      } else {
-        const uint64_t v_desc = smem_desc_sw128(smem_u32(Vs), kStep * 128, 1024);
-        for (int h = 0; h < NH && ok; ++h) {  // O (+)= P_h V_h; P_h sits over S[h & 1]
-          const int s = h % kStages, ph = (h / kStages) & 1;
-          ok = mbar_wait(&bars->v_full[s], ph, abort);
-          HEART_TR(h, 12);
-          if (ok) ok = mbar_wait(&bars->p_full[s], ph, abort);
-          if (!ok) break;
-          HEART_TR(h, 8);
-          tc_fence_after();
-          const uint32_t d = tmem, pa = tmem + 128 + s * kStep;
-          const uint64_t vs_desc = at(v_desc, s * (L::KV_BYTES >> 4));
-          if (leader) {
-#pragma unroll
-            for (int ks = 0; ks < 4; ++ks)
-              mma_ts(d, pa + ks * 8, at(vs_desc, ks * 128), idesc_pv, (h > 0 || ks > 0) ? 1u : 0u);
-            tc_commit(&bars->pv_done[s]);
+          if (g > 0) load_vb();
+          if (++h < n_steps) {
+            e = e_next;
+            load_k();
+            load_va();
+          } else {
+            if (!next_with_steps()) break;
+            h = 0;
+            load_k();
+            load_q();
+            load_va();
+            draw();
           }
-          __syncwarp();
-          HEART_TR(h, 9);
         }
       }
       if (*abort) {
-        // Tensor memory must not be released under a product in flight: a commit arrives once
-        // everything this lane has issued is complete; the wait for it is bounded like the others.
-        uint64_t *bar = &bars->drain[warp == kWarpQK ? 0 : 1];
-        if (leader) tc_commit(bar);
-        __syncwarp();
-        settle(bar, 0);
+        if (n_q > 0) settle(&bars->q_full, (n_q - 1) & 1);
+        if (n_k > 0) settle(&bars->k_full, (n_k - 1) & 1);
+        if (n_vb > 0) settle(&bars->vb_full, (n_vb - 1) & 1);
+        for (int i = n_va > 2 ? n_va - 2 : 0; i < n_va; ++i) settle(&bars->va_full[i & 1], (i >> 1) & 1);
       }
+    }
+  } else if (warp >= kWarpMma) {
+    // ===== MMA issuer.  The whole warp runs the loop (uniform control flow keeps the descriptors in
+    // uniform registers), one elected lane issues.
+    constexpr uint32_t idesc_qk = idesc_bf16_f32(128, 128, false, false);
+    constexpr uint32_t idesc_pv = idesc_bf16_f32(128, 128, false, true);
+    // Descriptors differ only in the start-address field (low word, no carry out of it): base + a
+    // compile-time offset per 16-element k-step, in 16-byte units.
+    //   Q, K (K-major): 64 dims = one 128-byte row; the dim halves are 128*128 B apart.
+    //   V (MN-major):   64 dims = one 128-byte row; dim halves 64*128 B apart (the LBO);
+    //                   16 keys = 16 rows = 2048 B per k-step.
+    auto at = [](uint64_t desc, uint32_t off16) -> uint64_t {
+      return (desc & 0xffffffff00000000ull) | (uint32_t)((uint32_t)desc + off16);
+    };
+    const bool leader = elect_one();  // the same lane every time: commits track its MMAs
+    const uint64_t q_desc = smem_desc_sw128(smem_u32(mem + kOffQ), 16, 1024);
+    const uint64_t k_desc = smem_desc_sw128(smem_u32(mem + kOffK), 16, 1024);
+    const uint64_t va_desc = smem_desc_sw128(smem_u32(mem + kOffVa), 64 * 128, 1024);
+    const uint64_t vb_desc = smem_desc_sw128(smem_u32(mem + kOffVb), 64 * 128, 1024);
+    const uint32_t t_o = tmem, t_s = tmem + 128;
+    uint32_t g = 0, nq = 0;  // key steps and tiles with key steps so far
+    bool ok = true;
+    auto issue_qk = [&]() {  // S_g = Q K^T
+      ok = mbar_wait(&bars->k_full, g & 1, abort);
+      if (!ok) return;
+      tc_fence_after();
+      if (leader) {
+#pragma unroll
+        for (int ks = 0; ks < 8; ++ks)
+          mma_ss(t_s, at(q_desc, (ks >> 2) * 1024 + (ks & 3) * 2), at(k_desc, (ks >> 2) * 1024 + (ks & 3) * 2), idesc_qk, ks > 0 ? 1u : 0u);
+        tc_commit(&bars->s_full);
+      }
+      __syncwarp();
+    };
+    int4 ti;
+    for (int t = 0; ok && next_tile(t, ti); ++t) {
+      const int n_steps = n_steps_of(ti.y);
+      if (n_steps == 0) continue;
+      ok = mbar_wait(&bars->q_full, nq & 1, abort);
+      ++nq;
+      if (ok) issue_qk();
+      for (int h = 0; h < n_steps && ok; ++h) {
+        // O (+)= P_h V_h: keys 0-95, then 96-127
+        const uint64_t va = at(va_desc, (g & 1) * (kHalfBytes >> 4));
+        ok = mbar_wait(&bars->va_full[g & 1], (g >> 1) & 1, abort);
+        if (ok) ok = mbar_wait(&bars->vb_full, g & 1, abort);
+        if (ok) ok = mbar_wait(&bars->p_full[0], g & 1, abort);
+        if (!ok) break;
+        tc_fence_after();
+        if (leader) {
+#pragma unroll
+          for (int ks = 0; ks < 4; ++ks) mma_ts(t_o, t_s + ks * 8, at(va, ks * 128), idesc_pv, (h > 0 || ks > 0) ? 1u : 0u);
+#pragma unroll
+          for (int ks = 0; ks < 2; ++ks) mma_ts(t_o, t_s + 32 + ks * 8, at(vb_desc, ks * 128), idesc_pv, 1u);
+        }
+        __syncwarp();
+        ok = mbar_wait(&bars->p_full[1], g & 1, abort);
+        if (!ok) break;
+        tc_fence_after();
+        if (leader) {
+#pragma unroll
+          for (int ks = 2; ks < 4; ++ks) mma_ts(t_o, t_s + 32 + ks * 8, at(vb_desc, ks * 128), idesc_pv, 1u);
+        }
+        __syncwarp();
+        ++g;
+        if (h + 1 < n_steps) {
+          issue_qk();
+        } else {
+          if (leader) tc_commit(&bars->o_done);
+          __syncwarp();
+        }
+      }
+    }
+    if (*abort) {
+      // Tensor memory must not be released under a product in flight: a commit arrives once
+      // everything this lane has issued is complete; the wait for it is bounded like the others.
+      if (leader) tc_commit(&bars->drain);
+      __syncwarp();
+      settle(&bars->drain, 0);
     }
   } else {
     // ===== softmax / correction / epilogue: thread = one query row
     setmaxnreg_inc<kRegsSoftmax>();
-    const int q = warp;             // TMEM lane quarter this warp may touch
-    const int row = q * 32 + lane;  // row inside the 128-row query tile
-    const uint32_t lane_addr = tmem + ((uint32_t)(q * 32) << 16);
-    const uint32_t o_addr = lane_addr;
+    const int row = (warp & 3) * 32 + lane;  // row inside the 128-row query tile
+    const uint32_t o_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16), s_addr = o_addr + 128;
     const float c = p.scale_log2;
-    float m_ref = -INFINITY, l_run = 0.f;
-    bool ok = true;
-    const uint32_t my_bit = 1u << (row / B);  // query block of this row (uniform within a warp)
-#ifdef HEART_TRACE
-    const int tr0 = 0;
-    const bool trw = warp == 0 && lane == 0;
-#define HEART_TRS(slot)                   \
-  do {                                    \
-    if (trw) HEART_TR(h, tr0 + (slot));   \
-  } while (0)
-#else
-#define HEART_TRS(slot) \
-  do {                  \
-  } while (0)
-#endif
-    for (int h = 0; h < NH && ok; ++h) {
-      const int s = h % kStages, ph = (h / kStages) & 1;
-      HEART_TRS(0);
-      // key columns of this step that are real keys this row attends to
-      int lim = 0;
-      {
-        const uint32_t e = (uint32_t)uni[h / HPB];
-        if ((e >> 16) & my_bit) lim = max(0, min(kStep, p.N - ((int)(e & 0xffff) * B + (h % HPB) * kStep)));
-      }
-      const int lim0 = min(lim, 32), lim1 = max(lim - 32, 0);
-      const uint32_t s_addr = lane_addr + 128 + s * kStep;
-      ok = __all_sync(0xffffffffu, mbar_wait(&bars->qk_done[s], ph, abort));
-      if (!ok) break;
-      HEART_TRS(1);
-      tc_fence_after();
-      uint32_t sreg[64];
-      if (lim0 > 0) tmem_ld32(s_addr, *reinterpret_cast<uint32_t(*)[32]>(&sreg[0]));
-      if (lim1 > 0) tmem_ld32(s_addr + 32, *reinterpret_cast<uint32_t(*)[32]>(&sreg[32]));
-      tmem_wait_ld();
-      HEART_TRS(2);
-      if (lim < kStep) {  // rare: ragged last block, or a block this row's query block does not list
-#pragma unroll
-        for (int i = 0; i < 32; ++i) {
-          if (i >= lim0) sreg[i] = 0xff800000u;  // -inf: ignored by the max, 2^-inf = 0
-          if (i >= lim1) sreg[32 + i] = 0xff800000u;
-        }
-      }
-      float mx0 = -INFINITY, mx1 = -INFINITY, mx2 = -INFINITY, mx3 = -INFINITY;
-#pragma unroll
-      for (int i = 0; i < 64; i += 8) {
-        mx0 = fmax3(mx0, __uint_as_float(sreg[i]), __uint_as_float(sreg[i + 1]));
-        mx1 = fmax3(mx1, __uint_as_float(sreg[i + 2]), __uint_as_float(sreg[i + 3]));
-        mx2 = fmax3(mx2, __uint_as_float(sreg[i + 4]), __uint_as_float(sreg[i + 5]));
-        mx3 = fmax3(mx3, __uint_as_float(sreg[i + 6]), __uint_as_float(sreg[i + 7]));
-      }
-      const float x_max = fmaxf(fmaxf(mx0, mx1), fmaxf(mx2, mx3)) * c;  // -inf stays -inf (c > 0)
-      HEART_TRS(3);
-      float alpha = 1.f;
-      bool grow = false;
-      if (m_ref == -INFINITY) {
-        m_ref = x_max;  // nothing accumulated for this row yet: no rescale needed
-      } else if (x_max > m_ref + 8.f) {
+    const uint64_t c2 = pack_f32x2(c, c);
+    float m_ref, l_run;
+    // Moves the reference of the rows whose maximum grew by more than 2^8 and rescales what they have
+    // accumulated.  O is quiescent: its last product was issued before the scores of this step.
+    auto move_reference = [&](float x_max, bool has_o, float &alpha) {
+      if (x_max > m_ref + 8.f) {
         alpha = ex2(m_ref - x_max);
         m_ref = x_max;
-        grow = true;
       }
-      if (__any_sync(0xffffffffu, grow) && h >= 1) {
-        // O must be quiescent: the previous product has to be complete
-        ok = __all_sync(0xffffffffu, mbar_wait(&bars->pv_done[(h - 1) % kStages], ((h - 1) / kStages) & 1, abort));
-        if (!ok) break;
-        tc_fence_after();
+      if (has_o) {
         const uint64_t alpha2 = pack_f32x2(alpha, alpha);
 #pragma unroll 1
-        for (int ch = 0; ch < 4; ++ch) {
-          uint32_t v[32];
-          tmem_ld32(o_addr + ch * 32, v);
+        for (int ch = 0; ch < 8; ++ch) {
+          uint32_t v[16];
+          tmem_ld16(o_addr + ch * 16, v);
           tmem_wait_ld();
 #pragma unroll
-          for (int i = 0; i < 32; i += 2) {
+          for (int i = 0; i < 16; i += 2) {
             float lo, hi;
             unpack_f32x2(mul_f32x2(pack_f32x2(__uint_as_float(v[i]), __uint_as_float(v[i + 1])), alpha2), lo, hi);
             v[i] = __float_as_uint(lo);
             v[i + 1] = __float_as_uint(hi);
           }
-          tmem_st32(o_addr + ch * 32, v);
+          tmem_st16(o_addr + ch * 16, v);
         }
-        tmem_wait_st();
       }
-      HEART_TRS(4);
-      const float neg_m = (m_ref == -INFINITY) ? 0.f : -m_ref;
-      const uint64_t c2 = pack_f32x2(c, c), neg_m2 = pack_f32x2(neg_m, neg_m);
-      // p = 2^(s*c - m), packed to bf16 over columns [0, 32) of S[h & 1]; the product reads all 64
-      // keys of the step, so every column is written (zeros where the row has no key)
-      float sum0 = 0.f, sum1 = 0.f, sum2 = 0.f, sum3 = 0.f;
-#pragma unroll
-      for (int ch = 0; ch < 2; ++ch) {
-        uint32_t pk[16];
-        if ((ch ? lim1 : lim0) == 0) {
-#pragma unroll
-          for (int i = 0; i < 16; ++i) pk[i] = 0u;
-        } else {
-#pragma unroll
-          for (int i = 0; i < 32; i += 4) {
-            float x0, x1, x2, x3;
-            unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(sreg[ch * 32 + i]), __uint_as_float(sreg[ch * 32 + i + 1])), c2, neg_m2), x0, x1);
-            unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(sreg[ch * 32 + i + 2]), __uint_as_float(sreg[ch * 32 + i + 3])), c2, neg_m2), x2, x3);
-            // the row sum is taken over the bf16-rounded weights, the ones the PV product really
-            // uses, so numerator and denominator carry the same rounding: O stays a weighted mean
-            const uint32_t w0 = pack_bf16x2(ex2(x0), ex2(x1));
-            const uint32_t w1 = pack_bf16x2(ex2(x2), ex2(x3));
-            pk[i >> 1] = w0;
-            pk[(i >> 1) + 1] = w1;
-            add_bf16x2_to_f32(sum0, sum1, w0);
-            add_bf16x2_to_f32(sum2, sum3, w1);
-          }
-        }
-        tmem_st16(s_addr + ch * 16, pk);
-      }
-      l_run = l_run * alpha + ((sum0 + sum1) + (sum2 + sum3));
-      HEART_TRS(5);
+    };
+    // part v of P_h is written: the product may read it
+    auto arrive = [&](int v) {
       tmem_wait_st();
-      HEART_TRS(6);
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(&bars->p_full[s]);
-      HEART_TRS(7);
-#ifdef HEART_TRACE
-      if (lane == 0) HEART_TR(h, 24 + q);  // arrival time of each warp of the warpgroup
-#endif
-    }
-    // epilogue: O / l, one row per thread
-    const int tok = row0 + row;
-    const bool valid_row = tok < p.N;
-    // the products complete in issue order: the last one covers them all
-    if (ok && NH > 0)
-      ok = __all_sync(0xffffffffu, mbar_wait(&bars->pv_done[(NH - 1) % kStages], ((NH - 1) / kStages) & 1, abort));
-    if (ok) {
-      tc_fence_after();
-      const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
-      uint16_t *orow = p.O + (long long)bidx * p.sb + (long long)hidx * p.sh + (long long)tok * p.sn;
-#pragma unroll 1
-      for (int ch = 0; ch < 4; ++ch) {  // 32 output dims at a time
-        uint32_t v[32];
-        if (NH > 0) {
-          tmem_ld32(o_addr + ch * 32, v);
+      if (lane == 0) mbar_arrive(&bars->p_full[v]);
+    };
+    auto arrive_both = [&]() {
+      arrive(0);
+      if (lane == 0) mbar_arrive(&bars->p_full[1]);
+    };
+    uint32_t g = 0, nq = 0;
+    bool ok = true;
+    int4 ti;
+    for (int t = 0; ok && next_tile(t, ti); ++t) {
+      const int n_steps = n_steps_of(ti.y);
+      const int bidx = ti.z / p.hcount, hidx = p.h0 + ti.z % p.hcount;
+      const int r = bidx * p.H + hidx;
+      const uint32_t *steps = p.steps + ((size_t)r * p.n_tiles_per_head + ti.x) * p.step_pitch;
+      // below every logit: the first step moves it (and rows without a key keep it)
+      m_ref = -3.0e38f;
+      l_run = 0.f;
+      uint32_t e_next = n_steps > 0 ? step_entry(steps, 0) : 0u;
+      for (int h = 0; h < n_steps; ++h, ++g) {
+        // whether all 128 keys of the step count for this row, or the 64 of one block (warp-uniform)
+        const uint32_t e = e_next;
+        if (h + 1 < n_steps) e_next = step_entry(steps, h + 1);
+        const uint32_t qb = (warp & 3) >> 1, flags = (e >> (10 + qb)) & 0x10001u;  // (64-token blocks)
+        const bool full = B == 128 ? (int)(e + 1) * 128 <= p.N : flags == 0x10001u && !(e & 0x10001000u);
+        ok = __all_sync(0xffffffffu, mbar_wait(&bars->s_full, g & 1, abort));
+        if (!ok) break;
+        tc_fence_after();
+        Sums sums = {0.f, 0.f, 0.f, 0.f};
+        float alpha = 1.f;
+        if (__builtin_expect(full, 1)) {
+          // All 128 keys count.  The exponentials of the first 32 keys are taken with the running reference
+          // as it stands while the row maximum is found, and once more in the rare step that moves it.
+          uint32_t s[128], pk[32];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) tmem_ld32(s_addr + q * 32, *reinterpret_cast<uint32_t(*)[32]>(&s[q * 32]));
           tmem_wait_ld();
+          uint64_t neg_m2 = pack_f32x2(-m_ref, -m_ref);
+          exp32(&s[0], c2, neg_m2, &pk[0], sums);
+          const float x_max = fmaxf(max64(&s[0]), max64(&s[64])) * c;
+          if (__any_sync(0xffffffffu, x_max > m_ref + 8.f)) {
+            move_reference(x_max, h > 0, alpha);
+            neg_m2 = pack_f32x2(-m_ref, -m_ref);
+            sums = {0.f, 0.f, 0.f, 0.f};
+            exp32(&s[0], c2, neg_m2, &pk[0], sums);
+          }
+          exp32(&s[32], c2, neg_m2, &pk[16], sums);
+          tmem_st32(s_addr, pk);
+          exp32(&s[64], c2, neg_m2, &pk[0], sums);
+          tmem_st16(s_addr + 32, *reinterpret_cast<uint32_t(*)[16]>(&pk[0]));
+          arrive(0);
+          exp32(&s[96], c2, neg_m2, &pk[16], sums);
+          tmem_st16(s_addr + 48, *reinterpret_cast<uint32_t(*)[16]>(&pk[16]));
+          arrive(1);
+        } else if (B == 64 && (flags == 1u || flags == 0x10000u) && !(e & 0x10001000u)) {
+          // This row's query block lists one of the step's two blocks.  The product reads all 128 keys of
+          // the step: zeros for the other one.
+          const uint32_t v = flags >> 16;
+          const uint32_t mine = s_addr + v * 64, p_mine = s_addr + v * 32, p_other = s_addr + (32 - v * 32);
+          uint32_t s[64], pk[32];
+          tmem_ld32(mine, *reinterpret_cast<uint32_t(*)[32]>(&s[0]));
+          tmem_ld32(mine + 32, *reinterpret_cast<uint32_t(*)[32]>(&s[32]));
+#pragma unroll
+          for (int i = 0; i < 32; ++i) pk[i] = 0u;
+          tmem_wait_ld();
+          tmem_st32(p_other, pk);
+          const float x_max = max64(s) * c;
+          if (__any_sync(0xffffffffu, x_max > m_ref + 8.f)) move_reference(x_max, h > 0, alpha);
+          const uint64_t neg_m2 = pack_f32x2(-m_ref, -m_ref);
+          exp32(&s[0], c2, neg_m2, &pk[0], sums);
+          exp32(&s[32], c2, neg_m2, &pk[16], sums);
+          tmem_st32(p_mine, pk);
+          arrive_both();
+        } else if (B == 64 && flags == 0u) {
+          // none of the step's blocks is listed by this row's query block
+          uint32_t pk[32];
+#pragma unroll
+          for (int i = 0; i < 32; ++i) pk[i] = 0u;
+          tmem_st32(s_addr, pk);
+          tmem_st32(s_addr + 32, pk);
+          arrive_both();
+        } else {
+          // The ragged last block: one half at a time, the scores read twice (the weights of the first half
+          // only overwrite its own scores).
+          int lim0, lim1;  // keys of each half that count
+          if (B == 128) {
+            const int rem = p.N - (int)e * 128;
+            lim0 = min(rem, 64);
+            lim1 = max(0, min(rem - 64, 64));
+          } else {
+            lim0 = (flags & 1u) ? min(64, p.N - (int)(e & 0x3ff) * 64) : 0;
+            lim1 = (flags >> 16) ? min(64, p.N - (int)((e >> 16) & 0x3ff) * 64) : 0;
+          }
+          float x_max = -INFINITY;
+#pragma unroll 1
+          for (int pass = 0; pass < 4; ++pass) {
+            const int v = pass & 1, n = v ? lim1 : lim0;
+            uint32_t s[64], pk[32];
+            tmem_ld32(s_addr + v * 64, *reinterpret_cast<uint32_t(*)[32]>(&s[0]));
+            tmem_ld32(s_addr + v * 64 + 32, *reinterpret_cast<uint32_t(*)[32]>(&s[32]));
+            tmem_wait_ld();
+#pragma unroll
+            for (int i = 0; i < 64; ++i)
+              if (i >= n) s[i] = 0xff800000u;  // -inf: ignored by the max, 2^-inf = 0
+            if (pass < 2) {
+              x_max = fmaxf(x_max, max64(s) * c);
+            } else {
+              if (pass == 2 && __any_sync(0xffffffffu, x_max > m_ref + 8.f)) move_reference(x_max, h > 0, alpha);
+              const uint64_t neg_m2 = pack_f32x2(-m_ref, -m_ref);
+              exp32(&s[0], c2, neg_m2, &pk[0], sums);
+              exp32(&s[32], c2, neg_m2, &pk[16], sums);
+              tmem_st32(s_addr + v * 32, pk);
+              tmem_wait_st();
+            }
+          }
+          arrive_both();
         }
-        if (valid_row) {
+        l_run = l_run * alpha + ((sums.a + sums.b) + (sums.c + sums.d));
+      }
+      // epilogue: O / l, one row per thread
+      const int tok = ti.x * 128 + row;
+      const bool valid_row = tok < p.N;
+      if (ok && n_steps > 0) {
+        ok = __all_sync(0xffffffffu, mbar_wait(&bars->o_done, nq & 1, abort));
+        ++nq;
+      }
+      if (ok) {
+        tc_fence_after();
+        const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
+        uint16_t *orow = p.O + (long long)bidx * p.sb + (long long)hidx * p.sh + (long long)tok * p.sn;
+#pragma unroll 1
+        for (int ch = 0; ch < 4; ++ch) {  // 32 output dims at a time
+          uint32_t v[32];
+          if (n_steps > 0) {
+            tmem_ld32(o_addr + ch * 32, v);
+            tmem_wait_ld();
+          }
+          if (valid_row) {
 #pragma unroll
-          for (int g4 = 0; g4 < 4; ++g4) {
-            float o[8];
+            for (int g4 = 0; g4 < 4; ++g4) {
+              float o[8];
 #pragma unroll
-            for (int i = 0; i < 8; ++i) o[i] = NH > 0 ? __uint_as_float(v[g4 * 8 + i]) * inv : 0.f;
-            uint4 w;
-            w.x = pack_bf16x2(o[0], o[1]);
-            w.y = pack_bf16x2(o[2], o[3]);
-            w.z = pack_bf16x2(o[4], o[5]);
-            w.w = pack_bf16x2(o[6], o[7]);
-            *reinterpret_cast<uint4 *>(orow + ch * 32 + g4 * 8) = w;
+              for (int i = 0; i < 8; ++i) o[i] = n_steps > 0 ? __uint_as_float(v[g4 * 8 + i]) * inv : 0.f;
+              uint4 w;
+              w.x = pack_bf16x2(o[0], o[1]);
+              w.y = pack_bf16x2(o[2], o[3]);
+              w.z = pack_bf16x2(o[4], o[5]);
+              w.w = pack_bf16x2(o[6], o[7]);
+              *reinterpret_cast<uint4 *>(orow + ch * 32 + g4 * 8) = w;
+            }
           }
         }
+        if (valid_row && p.lse != nullptr)
+          p.lse[(size_t)r * p.N + tok] = l_run > 0.f ? (m_ref + log2f(l_run)) * 0.6931471805599453f : -INFINITY;
+        // (the first product of the next tile writes O only after this warp's next arrival on p_full)
       }
-      if (valid_row && p.lse != nullptr)
-        p.lse[(size_t)r * p.N + tok] = l_run > 0.f ? (m_ref + log2f(l_run)) * 0.6931471805599453f : -INFINITY;
     }
   }
 
   // ------------------------------------------------------------------ tear-down
-  if (tid == 0) HEART_TR(0, 30);
   tc_fence_before();
   __syncthreads();
-  if (tid == 0) HEART_TR(0, 31);
-  if (warp == kWarpQK) {
+  if (warp == kWarpMma) {
     tc_fence_after();
-    tmem_dealloc(tmem, kTmemCols);
+    tmem_dealloc(*tmem_base, 512);
   }
-  if (tid == 0 && bars->abort) atomicExch(p.status, HEART_ERR_DEVICE_CHECK);
+  if (tid < kStreams && reinterpret_cast<AttnBars *>(smem + kOffBar + tid * kBarBytes)->abort)
+    atomicExch(p.status, HEART_ERR_DEVICE_CHECK);
 }
 
-// Order of the tiles of every head of a launch.  One CTA per head; rank by counting over at most 1024
-// keys, so the result is a permutation whatever the lists hold.  Heads before the last two: index order
-// while a head's K and V fit the L2 comfortably; beyond that ascending by the first key block that the
-// tile's lists name (ties by tile index) -- tiles that read the same region of K and V run together.
-// The last two heads: descending by the number of listed key blocks.
-__global__ void __launch_bounds__(256) tile_order_kernel(const int32_t *__restrict__ kv_idx,
-                                                         const int32_t *__restrict__ kv_cnt, int nb, int qbt, int ncph,
-                                                         int idx_stride, int H, int h0, int hcount, int n_heads,
-                                                         int by_first_key, int32_t *__restrict__ order) {
-  __shared__ int key[1024];
-  const int rr = blockIdx.x, r = (rr / hcount) * H + h0 + rr % hcount;
-  const bool by_length = rr >= n_heads - 2;
-  for (int t = threadIdx.x; t < ncph; t += blockDim.x) {
-    int len = 0, first = 0x3fffffff;
-    for (int qb = 0; qb < qbt; ++qb) {
-      const int I = t * qbt + qb;
-      if (I >= nb) break;
-      const int c = min(max(__ldg(&kv_cnt[(size_t)r * nb + I]), 0), idx_stride);
-      len += c;
-      if (c > 0) first = min(first, max(__ldg(&kv_idx[((size_t)r * nb + I) * idx_stride]), 0));
+// Step lists of the tiles of a launch: one warp per tile.  The lists of the tile's query blocks (any
+// order; entries out of range are skipped and reported, duplicates merged) become bit sets, and those the
+// list of key steps.  64-token blocks: key blocks that both query blocks list come first, then blocks of
+// query block 0 paired with blocks of query block 1, so that in such a step every row has 64 exponentials
+// to take instead of half of the rows 128; ascending within each group.
+constexpr int kPlanWarps = 8;
+
+template <int B>
+__global__ void __launch_bounds__(32 * kPlanWarps)
+    attn_plan_kernel(const int32_t *__restrict__ kv_idx, const int32_t *__restrict__ kv_cnt, int nb, int ncph, int idx_stride,
+                     int H, int h0, int hcount, int n_tiles, int step_pitch, int ragged, uint32_t *__restrict__ steps,
+                     uint32_t *__restrict__ tiles, uint32_t *__restrict__ firsts, int32_t *__restrict__ counter,
+                     int32_t *__restrict__ status) {
+  constexpr int QBT = 128 / B;  // query blocks per tile
+  __shared__ uint32_t sets[kPlanWarps][QBT][32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int n = blockIdx.x * kPlanWarps + warp;
+  pdl_wait();  // the lists come from the kernel before this one
+  pdl_launch_dependents();
+  if (blockIdx.x == 0 && threadIdx.x == 0) *counter = 0;
+  if (n >= n_tiles) return;
+  const int rr = n / ncph, t = n % ncph;
+  const int r = (rr / hcount) * H + h0 + rr % hcount;
+#pragma unroll
+  for (int q = 0; q < QBT; ++q) sets[warp][q][lane] = 0u;
+  __syncwarp();
+  bool bad = false;
+#pragma unroll
+  for (int q = 0; q < QBT; ++q) {
+    const int I = t * QBT + q;
+    if (I >= nb) break;
+    const size_t row = (size_t)r * nb + I;
+    int cnt = __ldcg(&kv_cnt[row]);
+    if (cnt < 0 || cnt > idx_stride) {
+      bad = true;
+      cnt = cnt < 0 ? 0 : idx_stride;
     }
-    key[t] = by_length ? -len : (by_first_key ? first : t);
+    const int32_t *list = kv_idx + row * idx_stride;
+#pragma unroll 4
+    for (int k = lane; k < cnt; k += 32) {
+      const int J = __ldcg(&list[k]);
+      if (J < 0 || J >= nb)
+        bad = true;  // skipped, reported
+      else
+        atomicOr(&sets[warp][q][J >> 5], 1u << (J & 31));
+    }
+  }
+  __syncwarp();
+  if (bad) atomicExch(status, HEART_ERR_DEVICE_CHECK);
+  // exclusive prefix over the lanes of a count per lane
+  auto prefix = [lane](int v) {
+    int s = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int u = __shfl_up_sync(0xffffffffu, s, o);
+      if (lane >= o) s += u;
+    }
+    return s - v;
+  };
+  auto sum = [](int v) { return (int)__reduce_add_sync(0xffffffffu, (unsigned)v); };
+  uint32_t *out = steps + ((size_t)r * ncph + t) * step_pitch;
+  const uint32_t a = sets[warp][0][lane], b = QBT == 2 ? sets[warp][QBT - 1][lane] : 0u;
+  const uint32_t any = a | b;
+  const int U = sum(__popc(any));
+  if (B == 128) {
+    int pos = prefix(__popc(a));
+    for (uint32_t m = a; m; m &= m - 1) out[pos++] = lane * 32 + __ffs(m) - 1;
+  } else {
+    uint16_t *out16 = reinterpret_cast<uint16_t *>(out);
+    // the word of key block J, listed by the query blocks in `flags`
+    auto word = [&](int J, int flags) { return (uint16_t)(J | flags << 10 | (ragged && J == nb - 1 ? 1 << 12 : 0)); };
+    int last = -1;  // the last listed block, in the lane that writes it
+    const int D = sum(__popc(a & b));
+    int pos = prefix(__popc(a & b));
+    for (uint32_t m = a & b; m; m &= m - 1) {
+      const int J = lane * 32 + __ffs(m) - 1;
+      last = pos == U - 1 ? J : last;
+      out16[pos++] = word(J, 3);
+    }
+    int S[2] = {sum(__popc(a & ~b)), sum(__popc(b & ~a))};
+    int start = D, skip[2] = {0, 0};
+    if ((D & 1) && S[0] + S[1] > 0) {  // one single next to the last shared block; pairs start on a step
+      const int x = S[0] >= S[1] ? 0 : 1;
+      skip[x] = 1;
+      --S[x];
+      ++start;
+    }
+    const int paired = min(S[0], S[1]);
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const uint32_t only = q ? b & ~a : a & ~b;
+      int k = prefix(__popc(only)) - skip[q];
+      for (uint32_t m = only; m; m &= m - 1, ++k) {
+        const int at = k < 0 ? D : k < paired ? start + 2 * k + q : start + paired + k;
+        const int J = lane * 32 + __ffs(m) - 1;
+        last = at == U - 1 ? J : last;
+        out16[at] = word(J, 1 << q);
+      }
+    }
+    if ((U & 1) && last >= 0) out16[U] = (uint16_t)last;  // second half of the last step: the same block, without flags
+  }
+  const unsigned has = __ballot_sync(0xffffffffu, any != 0u);
+  const int src = has ? __ffs(has) - 1 : 0;
+  const int first = __shfl_sync(0xffffffffu, lane * 32 + __ffs(any) - 1, src);
+  if (lane == 0) {
+    tiles[n] = (uint32_t)t | (uint32_t)U << 16;
+    firsts[n] = has ? first : 0x3ff;
+  }
+}
+
+// Order of the tiles of every head of a launch: rank by counting over at most 1024 distinct keys, 256
+// tiles per CTA.  Heads before the last two: index order while a head's K and V fit the L2 comfortably;
+// beyond that ascending by the first key block that the tile's lists name (ties by tile index) -- tiles
+// that read the same region of K and V run together.  The last two heads: descending by the number of
+// listed key blocks.
+__global__ void __launch_bounds__(256) tile_order_kernel(const uint32_t *__restrict__ tiles, const uint32_t *__restrict__ firsts,
+                                                         int ncph, int n_heads, int by_first_key, uint32_t *__restrict__ order) {
+  __shared__ __align__(16) uint32_t key[1024];
+  const int rr = blockIdx.y, t = blockIdx.x * 256 + threadIdx.x;
+  pdl_wait();
+  pdl_launch_dependents();
+  const bool by_length = rr >= n_heads - 2;
+  const size_t base = (size_t)rr * ncph;
+  if (!by_length && !by_first_key) {
+    if (t < ncph) order[base + t] = __ldcg(&tiles[base + t]);
+    return;
+  }
+  uint32_t my_word = 0u;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int u = threadIdx.x + k * 256;
+    uint32_t v = 0xffffffffu;
+    if (u < ncph) {
+      const uint32_t w = __ldcg(&tiles[base + u]);
+      if (u == t) my_word = w;
+      v = (by_length ? 0xffffu - (w >> 16) : __ldcg(&firsts[base + u])) << 10 | (uint32_t)u;
+    }
+    key[u] = v;
   }
   __syncthreads();
-  for (int t = threadIdx.x; t < ncph; t += blockDim.x) {
-    const int mine = key[t];
-    int rank = 0;
-    for (int u = 0; u < ncph; ++u) rank += (key[u] < mine || (key[u] == mine && u < t)) ? 1 : 0;
-    order[(size_t)rr * ncph + rank] = t;
+  if (t >= ncph) return;
+  const uint32_t mine = key[t];
+  int rank = 0;
+  const uint4 *k4 = reinterpret_cast<const uint4 *>(key);
+#pragma unroll 4
+  for (int u = 0; u < (ncph + 3) / 4; ++u) {
+    const uint4 w = k4[u];
+    rank += (w.x < mine ? 1 : 0) + (w.y < mine ? 1 : 0) + (w.z < mine ? 1 : 0) + (w.w < mine ? 1 : 0);
   }
+  order[base + rank] = my_word;
 }
 
 // ---------------------------------------------------------------------- host side
 namespace {
 
-// bf16 [B,H,N,128] with element strides (sb, sh, sn, 1): box = 64 dims x `rows` tokens, 128-byte swizzle,
-// out-of-range rows read as zero.
-bool make_map(CUtensorMap *m, const void *base, const Geom &g, int rows) {
+constexpr int kSms = 148;
+
+// bf16 [B,H,N,128] with element strides (sb, sh, sn, 1) as (64 dims, token, dim half, head, batch): box =
+// 64 dims x `rows` tokens x `halves` dim halves, 128-byte swizzle, out-of-range rows read as zero.
+bool make_map(CUtensorMap *m, const void *base, const Geom &g, int rows, int halves) {
   EncodeTiledFn fn = encode_tiled_fn();
   if (!fn) return false;
-  cuuint64_t dims[4] = {(cuuint64_t)kD, (cuuint64_t)g.N, (cuuint64_t)g.H, (cuuint64_t)g.B};
-  cuuint64_t strides[3] = {(cuuint64_t)g.sn * 2, (cuuint64_t)g.sh * 2, (cuuint64_t)g.sb * 2};
-  cuuint32_t box[4] = {64, (cuuint32_t)rows, 1, 1};
-  cuuint32_t estr[4] = {1, 1, 1, 1};
-  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void *>(base), dims, strides, box, estr,
+  cuuint64_t dims[5] = {64, (cuuint64_t)g.N, 2, (cuuint64_t)g.H, (cuuint64_t)g.B};
+  cuuint64_t strides[4] = {(cuuint64_t)g.sn * 2, 128, (cuuint64_t)g.sh * 2, (cuuint64_t)g.sb * 2};
+  cuuint32_t box[5] = {64, (cuuint32_t)rows, (cuuint32_t)halves, 1, 1};
+  cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void *>(base), dims, strides, box, estr,
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 template <int B>
-cudaError_t launch_bk(const Geom &g, const CUtensorMap &mq, const CUtensorMap &mk, const CUtensorMap &mv,
-                      const AttnParams &prm, cudaStream_t s) {
-  const int smem = AttnSmem<B>::TOTAL + 1024;
-  cudaError_t e = cudaFuncSetAttribute(attn_tc_kernel<B>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+cudaError_t launch_bk(const Geom &g, const Workspace &w, const CUtensorMap &mq, const CUtensorMap &mk, const CUtensorMap &mv,
+                      AttnParams prm, const int32_t *kv_idx, const int32_t *kv_cnt, cudaStream_t s, int *launches) {
+  cudaError_t e;
+  const int n_heads = g.B * prm.hcount;
+  prm.n_tiles = n_heads * prm.n_tiles_per_head;
+  // the plan lives where the pooled scores of the mask predictor were: [R][tiles][steps], then two words per tile
+  uint32_t *steps = reinterpret_cast<uint32_t *>(w.scores);
+  prm.step_pitch = B == 128 ? g.nb : (g.nb + 1) / 2;
+  uint32_t *tiles = steps + (size_t)g.R * prm.n_tiles_per_head * prm.step_pitch;
+  uint32_t *firsts = tiles + (size_t)g.R * prm.n_tiles_per_head;
+  prm.steps = steps;
+  prm.tiles = tiles;
+  const int planned = prm.dense ? 0 : prm.n_tiles;  // (dense: the kernel only zeroes the counter)
+  e = launch_pdl(attn_plan_kernel<B>, dim3(planned ? (planned + kPlanWarps - 1) / kPlanWarps : 1), dim3(32 * kPlanWarps), 0, s,
+                 kv_idx, kv_cnt, g.nb, prm.n_tiles_per_head, g.idx_stride, g.H, prm.h0, prm.hcount, planned, prm.step_pitch,
+                 (int)(g.N % g.block != 0), steps, tiles, firsts, prm.counter, prm.status);
   if (e != cudaSuccess) return e;
-  // two CTAs per SM: all of the configurable shared memory
-  e = cudaFuncSetAttribute(attn_tc_kernel<B>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+  ++*launches;
+  if (planned > kStreams * kSms) {  // up to there every tile starts at once: no order to choose
+    // K + V of one head beyond 32 MB (about half of one die's share of the L2): order by key locality
+    const int by_first_key = (size_t)g.N * kD * 2 * 2 > (size_t)(32u << 20) ? 1 : 0;
+    e = launch_pdl(tile_order_kernel, dim3((prm.n_tiles_per_head + 255) / 256, n_heads), dim3(256), 0, s,
+                   (const uint32_t *)tiles, (const uint32_t *)firsts, prm.n_tiles_per_head, n_heads, by_first_key,
+                   reinterpret_cast<uint32_t *>(w.order));
+    if (e != cudaSuccess) return e;
+    ++*launches;
+    prm.tiles = reinterpret_cast<const uint32_t *>(w.order);
+  }
+  e = cudaFuncSetAttribute(attn_tc_kernel<B>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttnSmem);
   if (e != cudaSuccess) return e;
-  attn_tc_kernel<B><<<g.B * prm.hcount * prm.n_ctas_per_head, kAttnThreads, smem, s>>>(mq, mk, mv, prm);
-  return cudaGetLastError();
+  ++*launches;
+  return launch_pdl(attn_tc_kernel<B>, dim3(prm.n_tiles < kSms ? prm.n_tiles : kSms), dim3(kAttnThreads), kAttnSmem, s, mq, mk,
+                    mv, prm);
 }
 
 }  // namespace
 
-cudaError_t launch_attention(const Geom &g, const void *Q, const void *K, const void *V,
-                             const int32_t *kv_idx, const int32_t *kv_cnt, bool dense, void *O,
-                             float *lse, int32_t *status, int32_t *order, cudaStream_t s, int *launches, int h0,
-                             int hcount) {
+cudaError_t launch_attention(const Geom &g, const Workspace &w, const void *Q, const void *K, const void *V,
+                             const int32_t *kv_idx, const int32_t *kv_cnt, bool dense, void *O, float *lse,
+                             cudaStream_t s, int *launches, int h0, int hcount) {
   if (hcount <= 0) {
     h0 = 0;
     hcount = g.H;
   }
   CUtensorMap mq, mk, mv;
-  if (!make_map(&mq, Q, g, 128) || !make_map(&mk, K, g, kStep) || !make_map(&mv, V, g, kStep))
+  if (!make_map(&mq, Q, g, 128, 2) || !make_map(&mk, K, g, g.block, g.block == 128 ? 2 : 1) || !make_map(&mv, V, g, 64, 2))
     return cudaErrorInvalidValue;
-  AttnParams prm;
-  prm.kv_idx = kv_idx;
-  prm.kv_cnt = kv_cnt;
+  AttnParams prm = {};
   prm.O = static_cast<uint16_t *>(O);
   prm.lse = lse;
-  prm.status = status;
+  prm.status = w.status;
+  prm.counter = w.status + kStatusTileWord;
   prm.sb = g.sb;
   prm.sh = g.sh;
   prm.sn = g.sn;
   prm.H = g.H;
   prm.N = g.N;
   prm.nb = g.nb;
-  prm.idx_stride = g.idx_stride;
-  prm.n_ctas_per_head = (g.N + 127) / 128;
+  prm.n_tiles_per_head = (g.N + 127) / 128;
   prm.dense = dense ? 1 : 0;
   prm.h0 = h0;
   prm.hcount = hcount;
-  prm.R_all = g.R;
   prm.scale_log2 = (float)(g.scale * 1.4426950408889634);
-  prm.test_skip_v = 0;
 #ifdef HEART_TEST_HOOKS
   prm.test_skip_v = (g.flags & 0x80000000u) ? 1 : 0;
 #endif
-  prm.order = nullptr;
-  if (!dense && order != nullptr && prm.n_ctas_per_head <= 1024) {
-    const int rows = g.B * hcount;
-    // K + V of one head beyond 32 MB (about half of one die's share of the L2): order by key locality
-    const int by_first_key = (size_t)g.N * kD * 2 * 2 > (size_t)(32u << 20) ? 1 : 0;
-    tile_order_kernel<<<rows, 256, 0, s>>>(kv_idx, kv_cnt, g.nb, 128 / g.block, prm.n_ctas_per_head, g.idx_stride, g.H,
-                                           h0, hcount, rows, by_first_key, order);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    prm.order = order;
-    ++*launches;
-  }
-  ++*launches;
-  return g.block == 64 ? launch_bk<64>(g, mq, mk, mv, prm, s) : launch_bk<128>(g, mq, mk, mv, prm, s);
+  return g.block == 64 ? launch_bk<64>(g, w, mq, mk, mv, prm, kv_idx, kv_cnt, s, launches)
+                       : launch_bk<128>(g, w, mq, mk, mv, prm, kv_idx, kv_cnt, s, launches);
 }
 
 }  // namespace heart

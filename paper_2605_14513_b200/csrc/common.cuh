@@ -37,7 +37,8 @@ __host__ inline void set_chunks(Geom &g) {
 struct Workspace {
   int32_t *status;    // [64]   word 0: sticky device-check code; word 1: detail; word 8: ticket counter
                       //        of the drift kernel (zero between launches); words 10-11: signature of
-                      //        the (Q, K, shape) whose block means the workspace holds (0: none)
+                      //        the (Q, K, shape) whose block means the workspace holds (0: none); word 12:
+                      //        tiles that the streams of an attention launch have drawn
   double *bmean;      // [2][R][nb][D]  per-block (pooled) means of Q (0) and K (1)
   double *psum;       // [2][R][nchunks][D]  per-CTA partial token sums
   double *mean;       // [2][R][D]      token means of the current step
@@ -45,7 +46,8 @@ struct Workspace {
   uint8_t *refresh;   // [R]            final decision of the current step
   double *drift;      // [R]
   int32_t *order;     // [R * ceil(N / 128)] order in which an attention launch takes the tiles of each head
-  double *scores;     // [R][nb][pitch] pooled scores of the refreshed heads, pitch = nb rounded up to 32
+  double *scores;     // [R][nb][pitch] pooled scores of the refreshed heads, pitch = nb rounded up to 32;
+                      //        afterwards the step lists of the attention launch (at most half of the area)
   void *pairs;        // strided antidiagonal estimator only (HEART_ESTIMATOR_ANTIDIAG in the flags):
                       // float2 [R][N/16][nb], a (max, sum) pair per (query group, key block)
   size_t bytes_drift;  // what heart_drift alone touches (everything above `scores`)
@@ -84,7 +86,7 @@ __host__ inline Workspace carve(const Geom &g, void *base) {
   return w;
 }
 
-constexpr int kStatusTicketWord = 8, kStatusSigWord = 10;
+constexpr int kStatusTicketWord = 8, kStatusSigWord = 10, kStatusTileWord = 12;
 
 #ifdef __CUDACC__
 // Programmatic dependent launch: a kernel launched with the stream-serialisation attribute may be
@@ -164,10 +166,9 @@ cudaError_t launch_top_p(const Geom &g, const Workspace &w, const double *tau, c
 cudaError_t launch_antidiag_scores(const Geom &g, const Workspace &w, const void *Q, const void *K,
                                    const uint8_t *refresh, cudaStream_t s, int *launches);
 // h0/hcount select the heads [h0, h0 + hcount) of every batch entry (hcount <= 0: all heads).
-cudaError_t launch_attention(const Geom &g, const void *Q, const void *K, const void *V,
-                             const int32_t *kv_idx, const int32_t *kv_cnt, bool dense, void *O,
-                             float *lse, int32_t *status, int32_t *order, cudaStream_t s, int *launches,
-                             int h0 = 0, int hcount = 0);
+cudaError_t launch_attention(const Geom &g, const Workspace &w, const void *Q, const void *K, const void *V,
+                             const int32_t *kv_idx, const int32_t *kv_cnt, bool dense, void *O, float *lse,
+                             cudaStream_t s, int *launches, int h0 = 0, int hcount = 0);
 
 cudaError_t launch_token_drift(const Geom &g, const void *Qa, const void *Ka, const void *Qb,
                                const void *Kb, double *partial, double *drift_out, cudaStream_t s,
