@@ -5,30 +5,32 @@
 // weight 0 there).  Keys are processed 128 at a time: a "key step" is one 128-token block or two listed
 // 64-token blocks.
 //
-// What bounds it: for a 128 x 128 tile the tensor pipe needs 1024 clocks (512 for Q K^T, 512 for P V)
-// and the special-function units 1024 as well (ex2 issues every 8 clocks per sub-partition), and within
-// a tile the products and the softmax of a step are serial.  So one persistent CTA per SM runs two
-// independent streams on different query tiles, each with its own warps, barriers, buffers and half of
-// the tensor memory: while one stream takes exponentials the other has its products running.  A stream
-// draws its tiles from a counter; the loads and the first scores of its next tile overlap the end of
-// the present one.
+// What bounds it: for a 128 x 128 tile the tensor pipe needs 1024 clocks (512 for Q K^T, 512 for P V), the
+// special-function units 1024 as well (ex2 issues every 8 clocks per sub-partition) and shared memory
+// 1280 (operands of the products and the TMA writes, 128 bytes a clock).  The chain softmax -> products
+// -> softmax of one step is about 3000 clocks long, hand-overs included, so it has to be off the critical
+// path: one persistent CTA per SM works on one query tile at a time and two softmax warpgroups take its
+// key steps in turn.  Scores are double-buffered in tensor memory, and because P has columns of its own,
+// S_{h+2} is computed as soon as the scores of step h sit in registers: a warpgroup finds its next
+// scores ready when it ends a step.  (Two streams on different tiles with P over the scores, one
+// warpgroup each, ran at 1870-2100 clocks per tile and step: each stream waited 1200-1500 of ~3900 clocks for
+// its next scores.)  Tiles are drawn from a counter; the loads and the first scores of the next tile
+// overlap the end of the present one.
 //
-// Warp roles (registers are moved from the helper warps to the softmax warps at start):
-//   warps 0-3, 4-7  softmax of stream 0, 1: one thread per query row (lane quarter = warp & 3).  Per key
-//               step a thread reads its row of S (128 columns), takes the max, rescales its row of O only
-//               when the max grew by more than 2^8, writes P = 2^(s*scale*log2e - m) as bf16 over the
-//               first half of the S columns and adds the row sum; at the end it writes O / l (and lse).
-//   warps 8, 9  MMA issuers: S_0 = Q K_0^T, then per step O += P_h V_h followed by S_{h+1} = Q K_{h+1}^T.
-//               The tensor pipe executes a stream's products in issue order, so S_{h+1} may overwrite the
-//               columns of P_h without a wait in between.  P V starts when 96 of the 128 keys of P_h are
-//               written, while the softmax still works on the others.  A step has ONE commit (a commit
-//               costs the issuing warp ~100 clocks): S_{h+1} complete, which also says that P_h V_h has
-//               released its half of V and Q K_{h+1}^T its K.
-//   warps 10, 11  producers: draw the tile, then TMA loads (cp.async.bulk.tensor, 128-byte swizzle,
-//               completion on mbarriers) of Q and of the steps' K (one 32 KB buffer: S_h complete frees it a
-//               whole softmax before the next product wants it) and V (first 64 keys double-buffered, last
-//               64 single).
-// Tensor memory (256 columns per stream): O (128) | S (128), P_h in the first 64 columns of S.
+// Warp roles (registers are moved from the helper warps to the softmax warps at start); g counts the key
+// steps of a CTA over all its tiles, buffers and barriers go by g & 1:
+//   warps 0-3, 4-7  softmax of the even / odd steps: one thread per query row (lane quarter = warp & 3).  A
+//               thread loads its row of S_g (128 columns), hands the buffer back, takes the max, agrees on the
+//               row's reference with its partner in the other warpgroup, writes P_g = 2^(s*scale*log2e - m)
+//               as bf16 and adds the row sum.  The warpgroup that has a tile's last step writes O / l (and lse).
+//   warp 8      issues S_g = Q K_g^T once step g - 2 has emptied the buffer, warp 11 O += P_g V_g.
+//   warp 9      V producer, warp 10 K and Q producer (draws the tiles and announces them): TMA loads
+//               (cp.async.bulk.tensor, 128-byte swizzle, completion on mbarriers), two 32 KB buffers each.
+// The reference: m_g = m_{g-1} unless the row's maximum of step g exceeds it by more than 2^32.  Each warp
+// publishes the references of its 32 rows after the maximum of every step and reads those of the step
+// before; a row whose reference moved gets its part of O rescaled by the warp that moved it, once the
+// products of the steps before are complete, and both partners rescale their own row sums.
+// Tensor memory: O (128 columns) | S[2] (2 x 128) | P[2] (2 x 64).
 //
 // The step lists come from attn_plan_kernel (one warp per tile), which runs just before; the tiles are
 // taken head-major (the K/V of one or two heads stay in L2), within a head in the order of
@@ -36,8 +38,8 @@
 // half of the L2, except for the last two heads of the launch, whose tiles go longest-list-first so that
 // the launch does not end on a long tile that started late.
 //
-// Every wait is bounded; a wait that runs out raises the stream's abort flag and the status word, the
-// stream's roles drain and stop, the other streams take the remaining tiles.
+// Every wait is bounded; a wait that runs out raises the CTA's abort flag and the status word, its roles
+// drain and stop, the other CTAs take the remaining tiles.
 #include <cuda.h>
 
 #include "common.cuh"
@@ -46,33 +48,38 @@
 namespace heart {
 using namespace tc;
 
-constexpr int kStreams = 2;
 constexpr int kAttnThreads = 384;
-constexpr int kWarpMma = 8, kWarpProd = 10;  // + stream
+constexpr int kWarpQK = 8, kWarpV = 9, kWarpK = 10, kWarpPV = 11;
 constexpr int kRegsSoftmax = 216, kRegsHelper = 72;  // 216 * 256 + 72 * 128 = the CTA's 384 x 168
-constexpr int kHalfBytes = 16384;  // 64 dims of 128 keys of K, or 64 keys of V
-constexpr int kQBytes = 2 * kHalfBytes;
+constexpr int kTileBytes = 32768;  // 128 rows x 128 dims: [2 dim halves][128 rows][64] bf16, 128-byte swizzle
+constexpr int kTileRing = 4;       // announced tiles
+constexpr int kTileReaders = 11;   // softmax warps, issuers, V producer
+constexpr float kNoReference = -3.0e38f;  // below every logit: the first step moves it
+// A row's reference moves when its maximum exceeds it by this much (log2).  Weights, sums and O are floating
+// point with 8 exponent bits throughout, so a scale of up to 2^32 costs no precision and leaves 2^95 of
+// range; a move costs a rescale of O behind the products in flight.
+constexpr float kMaxGrowth = 32.f;
 
-// Shared-memory plan (the dynamic allocation itself is 1024-byte aligned), per stream.
-constexpr int kOffQ = 0;                         // [2 dim halves][128 rows][64] bf16, 128-byte swizzle
-constexpr int kOffK = kOffQ + kQBytes;           // [2 dim halves][128 keys][64]
-constexpr int kOffVa = kOffK + 2 * kHalfBytes;   // two buffers [2 dim halves][64 keys][64]: keys 0-63 of a step
-constexpr int kOffVb = kOffVa + 2 * kHalfBytes;  // keys 64-127
-constexpr int kStreamBytes = kOffVb + kHalfBytes;
-constexpr int kOffBar = kStreams * kStreamBytes;
+// Shared-memory plan (the dynamic allocation itself is 1024-byte aligned).
+constexpr int kOffQ = 0, kOffK = 2 * kTileBytes, kOffV = 4 * kTileBytes, kOffBar = 6 * kTileBytes;
 
-struct AttnBars {
-  uint64_t q_full, k_full, va_full[2], vb_full;  // TMA -> issuer
-  uint64_t s_full;           // S_h complete, and with it every product issued before it
-  uint64_t p_full[2];        // keys 0-95 / 96-127 of P_h written (one arrival per softmax warp)
-  uint64_t o_done;           // the last product of a tile is complete
-  uint64_t tile_full[2], tile_empty[2];  // the producer's announcements of tiles
-  uint64_t drain;            // abort path: the issuer's products in flight have landed
-  int4 tile[2];              // query tile of its head, listed key blocks, head of the launch, 1 (0: no tile left)
+struct AttnShared {
+  uint64_t q_full[2], k_full[2], v_full[2];  // TMA -> issuer
+  uint64_t s_full[2];      // S_g complete (K_g is free)
+  uint64_t s_free[2];      // S_g is in registers (one arrival per softmax warp)
+  uint64_t p_full[2];      // P_g written (one arrival per softmax warp)
+  uint64_t pv_done[2];     // P_g V_g complete (V_g and P_g are free)
+  uint64_t m_ready[2][4];  // references after step g, per lane quarter
+  uint64_t o_free;         // O of a tile has been read
+  uint64_t tile_full[kTileRing], tile_empty[kTileRing];
+  uint64_t drain[2];       // abort path: the issuers' products in flight have landed
+  int4 tile[kTileRing];    // query tile of its head, listed key blocks, head of the launch, 1 (0: no tile left)
+  float m[2][128];         // references after step g
+  float2 l[2][128];        // row sum and its reference of the warpgroup without the last step, per tile & 1
+  uint32_t tmem_base;
   int abort;
 };
-constexpr int kBarBytes = (sizeof(AttnBars) + 127) / 128 * 128;
-constexpr int kAttnSmem = kOffBar + kStreams * kBarBytes + 128;
+constexpr int kAttnSmem = kOffBar + sizeof(AttnShared);
 
 // A key step as the plan kernel writes it.  128-token blocks: the key block.  64-token blocks: two
 // halves of 16 bits, key block | (flag of query block 0, flag of query block 1) << 10 | ragged block << 12; no
@@ -80,7 +87,7 @@ constexpr int kAttnSmem = kOffBar + kStreams * kBarBytes + 128;
 struct AttnParams {
   const uint32_t *steps;  // [B*H][tiles of a head][step_pitch]
   const uint32_t *tiles;  // [tiles of the launch] tile of the head | listed key blocks << 16, in launch order
-  int32_t *counter;       // tiles drawn beyond the first one of every stream (zeroed by the plan kernel)
+  int32_t *counter;       // tiles drawn beyond the first one of every CTA (zeroed by the plan kernel)
   uint16_t *O;
   float *lse;
   int32_t *status;
@@ -88,7 +95,7 @@ struct AttnParams {
   int H, N, nb, n_tiles, n_tiles_per_head, step_pitch, dense;
   int h0, hcount;  // this launch covers heads [h0, h0 + hcount) of every batch entry
   float scale_log2;
-  int test_skip_v;  // test-hook builds only: stream 0 of CTA 0 leaves out one V copy of its first tile
+  int test_skip_v;  // test-hook builds only: CTA 0 leaves out the V copy of its second key step
 };
 
 __device__ __forceinline__ float fmax3(float a, float b, float c) {
@@ -129,37 +136,37 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                    const __grid_constant__ CUtensorMap map_v, const AttnParams p) {
   extern __shared__ __align__(1024) unsigned char smem[];
+  AttnShared &sh = *reinterpret_cast<AttnShared *>(smem + kOffBar);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int st = warp < 8 ? warp >> 2 : warp & 1;  // stream of this warp
-  AttnBars *bars = reinterpret_cast<AttnBars *>(smem + kOffBar + st * kBarBytes);
-  uint32_t *tmem_base = reinterpret_cast<uint32_t *>(smem + kOffBar + kStreams * kBarBytes);
-  volatile int *abort = &bars->abort;
-  unsigned char *mem = smem + st * kStreamBytes;
+  volatile int *abort = &sh.abort;
 
   // ------------------------------------------------------------------ set-up
-  if (tid < kStreams) {
-    AttnBars *b = reinterpret_cast<AttnBars *>(smem + kOffBar + tid * kBarBytes);
-    mbar_init(&b->q_full, 1);
-    mbar_init(&b->k_full, 1);
-    mbar_init(&b->va_full[0], 1);
-    mbar_init(&b->va_full[1], 1);
-    mbar_init(&b->vb_full, 1);
-    mbar_init(&b->s_full, 1);
+  if (tid == 0) {
     for (int i = 0; i < 2; ++i) {
-      mbar_init(&b->p_full[i], 4);      // one arrival per softmax warp
-      mbar_init(&b->tile_full[i], 1);
-      mbar_init(&b->tile_empty[i], 5);  // the softmax warps and the issuer
+      mbar_init(&sh.q_full[i], 1);
+      mbar_init(&sh.k_full[i], 1);
+      mbar_init(&sh.v_full[i], 1);
+      mbar_init(&sh.s_full[i], 1);
+      mbar_init(&sh.s_free[i], 4);
+      mbar_init(&sh.p_full[i], 4);
+      mbar_init(&sh.pv_done[i], 1);
+      for (int q = 0; q < 4; ++q) mbar_init(&sh.m_ready[i][q], 1);
     }
-    mbar_init(&b->o_done, 1);
-    mbar_init(&b->drain, 1);
-    b->abort = 0;
+    for (int i = 0; i < kTileRing; ++i) {
+      mbar_init(&sh.tile_full[i], 1);
+      mbar_init(&sh.tile_empty[i], kTileReaders);
+    }
+    mbar_init(&sh.o_free, 4);
+    mbar_init(&sh.drain[0], 1);
+    mbar_init(&sh.drain[1], 1);
+    sh.abort = 0;
     mbar_fence_init();
   }
-  if (warp == kWarpMma) {
-    tmem_alloc(tmem_base, 512);
+  if (warp == kWarpQK) {
+    tmem_alloc(&sh.tmem_base, 512);
     tmem_relinquish();
   }
-  if (warp == kWarpProd && lane == 0) {
+  if (warp == kWarpK && lane == 0) {
     tma_prefetch_desc(&map_q);
     tma_prefetch_desc(&map_k);
     tma_prefetch_desc(&map_v);
@@ -172,22 +179,46 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *tmem_base + st * 256;
+  const uint32_t tmem = sh.tmem_base;
 
   auto n_steps_of = [](int U) -> int { return B == 128 ? U : (U + 1) / 2; };
+  auto steps_of = [&](int rr, int tile) -> const uint32_t * {
+    const int r = rr / p.hcount * p.H + p.h0 + rr % p.hcount;
+    return p.steps + ((size_t)r * p.n_tiles_per_head + tile) * p.step_pitch;
+  };
   auto step_entry = [&](const uint32_t *steps, int h) -> uint32_t {
     if (!p.dense) return __ldcg(&steps[h]);
     if (B == 128) return h;
     const uint32_t ragged = (p.N & 63) ? p.nb - 1 : 0x3ff + 1, a = 2 * h, b = 2 * h + 1;
     return (a | 3u << 10 | (a == ragged ? 1u << 12 : 0u)) | (b < (uint32_t)p.nb ? b | 3u << 10 | (b == ragged ? 1u << 12 : 0u) : a) << 16;
   };
-  // The next announced tile; false: none left (or abort).  Every lane of the warp gets the same answer.
+  // Waits of a whole warp; ok turns false when one runs out or the CTA aborts.  The usual case is a barrier
+  // that is complete already.
+  bool ok = true;
+  auto complete = [](uint64_t *bar, uint32_t parity) { return __all_sync(0xffffffffu, mbar_test_wait(bar, parity)) != 0; };
+  auto wait = [&](uint64_t *bar, uint32_t parity) {
+    if (__builtin_expect(!complete(bar, parity), 0)) ok = __all_sync(0xffffffffu, mbar_wait(bar, parity, abort)) && ok;
+    return ok;
+  };
+  // The announced tile t; false: none left (or abort).  Every lane of the warp gets the same answer.
   auto next_tile = [&](int t, int4 &ti) -> bool {
-    if (!__all_sync(0xffffffffu, mbar_wait(&bars->tile_full[t & 1], (t >> 1) & 1, abort))) return false;
-    ti = bars->tile[t & 1];
+    const int i = t % kTileRing;
+    if (!wait(&sh.tile_full[i], (t / kTileRing) & 1)) return false;
+    ti = sh.tile[i];
     __syncwarp();
-    if (lane == 0) mbar_arrive(&bars->tile_empty[t & 1]);
+    if (lane == 0) mbar_arrive(&sh.tile_empty[i]);
     return ti.w != 0;
+  };
+  // K or V of one key step into a 32 KB buffer
+  auto load_step = [&](unsigned char *dst, const CUtensorMap *map, uint64_t *bar, uint32_t e, int hidx, int bidx) {
+    mbar_expect_tx(bar, kTileBytes);
+    if (B == 128) {
+      tma_load_5d(dst, map, bar, 0, (int)e * 128, 0, hidx, bidx);
+    } else {
+#pragma unroll
+      for (int i = 0; i < 4; ++i)  // dim half i >> 1 of block i & 1
+        tma_load_5d(dst + i * (kTileBytes / 4), map, bar, 0, (int)((e >> (16 * (i & 1))) & 0x3ff) * 64, i >> 1, hidx, bidx);
+    }
   };
   // Shared memory must not be released under a copy in flight: a producer that stops early (abort)
   // waits, bounded, for the copies it has issued.
@@ -196,365 +227,314 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     while (!mbar_try_wait(bar, parity) && clock64() - t0 < 40000000LL) {
     }
   };
+  auto settle_pair = [&](uint64_t *bar, int issued) {  // the last two of `issued` copies on a pair of barriers
+    for (int i = issued > 2 ? issued - 2 : 0; i < issued; ++i) settle(&bar[i & 1], (i >> 1) & 1);
+  };
+
+  // Descriptors differ only in the start-address field (low word, no carry out of it): base + an offset in
+  // 16-byte units.
+  auto desc_at = [](uint64_t desc, uint32_t off16) -> uint64_t {
+    return (desc & 0xffffffff00000000ull) | (uint32_t)((uint32_t)desc + off16);
+  };
+  // Tensor memory must not be released under a product in flight either: after an abort a commit arrives
+  // once everything the issuing lane has issued is complete; the wait for it is bounded like the others.
+  auto drain_products = [&](bool leader, uint64_t *bar) {
+    if (!*abort) return;
+    if (leader) tc_commit(bar);
+    __syncwarp();
+    settle(bar, 0);
+  };
 
   // ------------------------------------------------------------------ roles
-  if (warp >= kWarpMma) setmaxnreg_dec<kRegsHelper>();
-  if (warp >= kWarpProd) {
-    if (lane == 0) {  // ===== producer
-      bool ok = true;
-      int t = 0, n_q = 0, n_k = 0, n_va = 0, n_vb = 0;  // tiles announced, loads issued
-      // the tile that is announced next, fetched ahead of time
-      int nx = blockIdx.x + st * gridDim.x;  // the first tile of every stream is fixed, the others are drawn
-      uint32_t nx_word = 0, nx_e = 0;
-      const uint32_t *nx_steps = nullptr;
+  if (warp >= kWarpQK) setmaxnreg_dec<kRegsHelper>();
+  if (warp == kWarpK) {
+    if (lane == 0) {  // ===== K and Q producer
+      int t = 0, g = 0, nq = 0;  // tiles announced, key steps loaded, tiles with key steps
+      int n = blockIdx.x;        // the first tile of every CTA is fixed, the others are drawn
+      uint32_t word = 0, e = 0;  // tile n of the launch and its first key step, fetched ahead of time
       auto fetch = [&]() {
-        if (nx >= p.n_tiles) return;
-        const int rr = nx / p.n_tiles_per_head;
-        nx_word = p.dense ? (uint32_t)(nx - rr * p.n_tiles_per_head) | (uint32_t)p.nb << 16 : __ldcg(&p.tiles[nx]);
-        const int r = rr / p.hcount * p.H + p.h0 + rr % p.hcount;
-        nx_steps = p.steps + ((size_t)r * p.n_tiles_per_head + (nx_word & 0xffff)) * p.step_pitch;
-        if (nx_word >> 16) nx_e = step_entry(nx_steps, 0);
-      };
-      auto draw = [&]() {
-        nx = kStreams * gridDim.x + atomicAdd(p.counter, 1);
-        fetch();
-      };
-      int tile = 0, n_steps = 0, bidx = 0, hidx = 0;
-      const uint32_t *steps = nullptr;
-      uint32_t e = 0;
-      // announces tiles up to the next one that has key steps; false: none left
-      auto next_with_steps = [&]() -> bool {
-        for (;; draw()) {
-          if (t >= 2) ok = mbar_wait(&bars->tile_empty[t & 1], ((t >> 1) - 1) & 1, abort);
-          if (!ok) return false;
-          const bool none = nx >= p.n_tiles;
-          const int rr = none ? 0 : nx / p.n_tiles_per_head, U = nx_word >> 16;  // U = listed key blocks
-          bars->tile[t & 1] = none ? make_int4(0, 0, 0, 0) : make_int4(nx_word & 0xffff, U, rr, 1);
-          mbar_arrive(&bars->tile_full[t & 1]);
-          ++t;
-          if (none) return false;
-          if (U == 0) continue;
-          tile = nx_word & 0xffff;
-          n_steps = n_steps_of(U);
-          bidx = rr / p.hcount;
-          hidx = p.h0 + rr % p.hcount;
-          steps = nx_steps;
-          e = nx_e;
-          return true;
-        }
-      };
-      auto key_of = [&](int half) -> int { return B == 128 ? (int)e * 128 + half * 64 : (int)((e >> (16 * half)) & 0x3ff) * 64; };
-      auto load_q = [&]() {
-        mbar_expect_tx(&bars->q_full, kQBytes);
-        tma_load_5d(mem + kOffQ, &map_q, &bars->q_full, 0, tile * 128, 0, hidx, bidx);
-        ++n_q;
-      };
-      auto load_k = [&]() {
-        mbar_expect_tx(&bars->k_full, 2 * kHalfBytes);
-        if (B == 128) {
-          tma_load_5d(mem + kOffK, &map_k, &bars->k_full, 0, key_of(0), 0, hidx, bidx);
-        } else {
-#pragma unroll
-          for (int i = 0; i < 4; ++i)  // dim half i >> 1 of block i & 1
-            tma_load_5d(mem + kOffK + i * (kHalfBytes / 2), &map_k, &bars->k_full, 0, key_of(i & 1), i >> 1, hidx, bidx);
-        }
-        ++n_k;
-      };
-      auto load_va = [&]() {
-        const int i = n_va & 1;
-        ++n_va;
-#ifdef HEART_TEST_HOOKS
-        // Test-only library: one V tile is never requested (neither the byte count nor the copy), so the
-        // waits that depend on it run out and the abort path is taken.
-        if (p.test_skip_v && blockIdx.x == 0 && st == 0 && n_va == 2) return;
-#endif
-        mbar_expect_tx(&bars->va_full[i], kHalfBytes);
-        tma_load_5d(mem + kOffVa + i * kHalfBytes, &map_v, &bars->va_full[i], 0, key_of(0), 0, hidx, bidx);
-      };
-      auto load_vb = [&]() {
-        mbar_expect_tx(&bars->vb_full, kHalfBytes);
-        tma_load_5d(mem + kOffVb, &map_v, &bars->vb_full, 0, key_of(1), 0, hidx, bidx);
-        ++n_vb;
+        if (n >= p.n_tiles) return;
+        const int rr = n / p.n_tiles_per_head;
+        word = p.dense ? (uint32_t)(n - rr * p.n_tiles_per_head) | (uint32_t)p.nb << 16 : __ldcg(&p.tiles[n]);
+        if (word >> 16) e = step_entry(steps_of(rr, word & 0xffff), 0);
       };
       fetch();
-      if (next_with_steps()) {
-        load_q();
-        load_k();
-        load_va();
-        load_vb();
-        draw();
-        int h = 0;
-        for (uint32_t g = 0;; ++g) {  // g: key steps so far, over all tiles
+      for (; ok; ++t) {
+        const int i = t % kTileRing;
+        if (t >= kTileRing) ok = mbar_wait(&sh.tile_empty[i], (t / kTileRing - 1) & 1, abort);
+        if (!ok) break;
+        const bool none = n >= p.n_tiles;
+        const int rr = none ? 0 : n / p.n_tiles_per_head, tile = word & 0xffff, U = word >> 16;  // U = listed key blocks
+        sh.tile[i] = none ? make_int4(0, 0, 0, 0) : make_int4(tile, U, rr, 1);
+        mbar_arrive(&sh.tile_full[i]);
+        if (none) break;
+        const int n_steps = n_steps_of(U), bidx = rr / p.hcount, hidx = p.h0 + rr % p.hcount;
+        const uint32_t *steps = steps_of(rr, tile);
+        uint32_t e_now = e;
+        for (int h = 0; h < n_steps; ++h, ++g) {
           const uint32_t e_next = h + 1 < n_steps ? step_entry(steps, h + 1) : 0u;
-          // S of step g complete: K is free, and the product of step g - 1 has released its V
-          ok = mbar_wait(&bars->s_full, g & 1, abort);
+          if (g >= 2) ok = mbar_wait(&sh.s_full[g & 1], ((g - 2) >> 1) & 1, abort);
           if (!ok) break;
-          if (g > 0) load_vb();
-          if (++h < n_steps) {
-            e = e_next;
-            load_k();
-            load_va();
-          } else {
-            if (!next_with_steps()) break;
-            h = 0;
-            load_k();
-            load_q();
-            load_va();
-            draw();
+          load_step(smem + kOffK + (g & 1) * kTileBytes, &map_k, &sh.k_full[g & 1], e_now, hidx, bidx);
+          if (h == 0) {
+            // its buffer is free: the last step of the tile before the previous one is complete
+            mbar_expect_tx(&sh.q_full[nq & 1], kTileBytes);
+            tma_load_5d(smem + kOffQ + (nq & 1) * kTileBytes, &map_q, &sh.q_full[nq & 1], 0, tile * 128, 0, hidx, bidx);
+            ++nq;
           }
+          e_now = e_next;
+          if (h == 0) {
+            n = gridDim.x + atomicAdd(p.counter, 1);
+            fetch();
+          }
+        }
+        if (U == 0) {
+          n = gridDim.x + atomicAdd(p.counter, 1);
+          fetch();
         }
       }
       if (*abort) {
-        if (n_q > 0) settle(&bars->q_full, (n_q - 1) & 1);
-        if (n_k > 0) settle(&bars->k_full, (n_k - 1) & 1);
-        if (n_vb > 0) settle(&bars->vb_full, (n_vb - 1) & 1);
-        for (int i = n_va > 2 ? n_va - 2 : 0; i < n_va; ++i) settle(&bars->va_full[i & 1], (i >> 1) & 1);
+        settle_pair(sh.q_full, nq);
+        settle_pair(sh.k_full, g);
       }
     }
-  } else if (warp >= kWarpMma) {
-    // ===== MMA issuer.  The whole warp runs the loop (uniform control flow keeps the descriptors in
-    // uniform registers), one elected lane issues.
-    constexpr uint32_t idesc_qk = idesc_bf16_f32(128, 128, false, false);
-    constexpr uint32_t idesc_pv = idesc_bf16_f32(128, 128, false, true);
-    // Descriptors differ only in the start-address field (low word, no carry out of it): base + a
-    // compile-time offset per 16-element k-step, in 16-byte units.
-    //   Q, K (K-major): 64 dims = one 128-byte row; the dim halves are 128*128 B apart.
-    //   V (MN-major):   64 dims = one 128-byte row; dim halves 64*128 B apart (the LBO);
-    //                   16 keys = 16 rows = 2048 B per k-step.
-    auto at = [](uint64_t desc, uint32_t off16) -> uint64_t {
-      return (desc & 0xffffffff00000000ull) | (uint32_t)((uint32_t)desc + off16);
-    };
-    const bool leader = elect_one();  // the same lane every time: commits track its MMAs
-    const uint64_t q_desc = smem_desc_sw128(smem_u32(mem + kOffQ), 16, 1024);
-    const uint64_t k_desc = smem_desc_sw128(smem_u32(mem + kOffK), 16, 1024);
-    const uint64_t va_desc = smem_desc_sw128(smem_u32(mem + kOffVa), 64 * 128, 1024);
-    const uint64_t vb_desc = smem_desc_sw128(smem_u32(mem + kOffVb), 64 * 128, 1024);
-    const uint32_t t_o = tmem, t_s = tmem + 128;
-    uint32_t g = 0, nq = 0;  // key steps and tiles with key steps so far
-    bool ok = true;
-    auto issue_qk = [&]() {  // S_g = Q K^T
-      ok = mbar_wait(&bars->k_full, g & 1, abort);
-      if (!ok) return;
-      tc_fence_after();
-      if (leader) {
-#pragma unroll
-        for (int ks = 0; ks < 8; ++ks)
-          mma_ss(t_s, at(q_desc, (ks >> 2) * 1024 + (ks & 3) * 2), at(k_desc, (ks >> 2) * 1024 + (ks & 3) * 2), idesc_qk, ks > 0 ? 1u : 0u);
-        tc_commit(&bars->s_full);
+  } else if (warp == kWarpV) {
+    // ===== V producer
+    int g = 0;
+    int4 ti;
+    for (int t = 0; ok && next_tile(t, ti); ++t) {
+      const int n_steps = n_steps_of(ti.y), bidx = ti.z / p.hcount, hidx = p.h0 + ti.z % p.hcount;
+      const uint32_t *steps = steps_of(ti.z, ti.x);
+      uint32_t e_next = n_steps > 0 ? step_entry(steps, 0) : 0u;
+      for (int h = 0; h < n_steps; ++h, ++g) {
+        const uint32_t e = e_next;
+        if (h + 1 < n_steps) e_next = step_entry(steps, h + 1);
+        if (g >= 2 && !wait(&sh.pv_done[g & 1], ((g - 2) >> 1) & 1)) break;
+#ifdef HEART_TEST_HOOKS
+        // Test-only library: one V tile is never requested (neither the byte count nor the copy), so the
+        // waits that depend on it run out and the abort path is taken.
+        if (p.test_skip_v && blockIdx.x == 0 && g == 1) continue;
+#endif
+        if (lane == 0) load_step(smem + kOffV + (g & 1) * kTileBytes, &map_v, &sh.v_full[g & 1], e, hidx, bidx);
       }
-      __syncwarp();
-    };
+    }
+    if (*abort && lane == 0) settle_pair(sh.v_full, g);
+  } else if (warp == kWarpQK) {
+    // ===== issuer of the score products.  The whole warp runs the loop (uniform control flow keeps the
+    // descriptors in uniform registers), one elected lane issues.  The two kinds of products have a warp
+    // each: a step costs an issuing warp some 400 clocks of waits and hand-overs besides the products.
+    constexpr uint32_t idesc = idesc_bf16_f32(128, 128, false, false);
+    // Q, K (K-major): 64 dims = one 128-byte row; the dim halves are 128*128 B apart.
+    const uint64_t q_desc = smem_desc_sw128(smem_u32(smem + kOffQ), 16, 1024);
+    const uint64_t k_desc = smem_desc_sw128(smem_u32(smem + kOffK), 16, 1024);
+    const bool leader = elect_one();  // the same lane every time: commits track its MMAs
+    uint32_t g = 0, nq = 0;           // key steps and tiles with key steps so far
     int4 ti;
     for (int t = 0; ok && next_tile(t, ti); ++t) {
       const int n_steps = n_steps_of(ti.y);
       if (n_steps == 0) continue;
-      ok = mbar_wait(&bars->q_full, nq & 1, abort);
+      wait(&sh.q_full[nq & 1], (nq >> 1) & 1);
+      const uint64_t qd = desc_at(q_desc, (nq & 1) * (kTileBytes >> 4));
       ++nq;
-      if (ok) issue_qk();
-      for (int h = 0; h < n_steps && ok; ++h) {
-        // O (+)= P_h V_h: keys 0-95, then 96-127
-        const uint64_t va = at(va_desc, (g & 1) * (kHalfBytes >> 4));
-        ok = mbar_wait(&bars->va_full[g & 1], (g >> 1) & 1, abort);
-        if (ok) ok = mbar_wait(&bars->vb_full, g & 1, abort);
-        if (ok) ok = mbar_wait(&bars->p_full[0], g & 1, abort);
-        if (!ok) break;
+      for (int h = 0; h < n_steps; ++h, ++g) {  // S_g = Q K_g^T
+        const uint32_t b = g & 1;
+        if (g >= 2) wait(&sh.s_free[b], ((g - 2) >> 1) & 1);
+        if (!wait(&sh.k_full[b], (g >> 1) & 1)) break;
         tc_fence_after();
         if (leader) {
+          const uint64_t kd = desc_at(k_desc, b * (kTileBytes >> 4));
 #pragma unroll
-          for (int ks = 0; ks < 4; ++ks) mma_ts(t_o, t_s + ks * 8, at(va, ks * 128), idesc_pv, (h > 0 || ks > 0) ? 1u : 0u);
-#pragma unroll
-          for (int ks = 0; ks < 2; ++ks) mma_ts(t_o, t_s + 32 + ks * 8, at(vb_desc, ks * 128), idesc_pv, 1u);
+          for (int ks = 0; ks < 8; ++ks)
+            mma_ss(tmem + 128 + b * 128, desc_at(qd, (ks >> 2) * 1024 + (ks & 3) * 2), desc_at(kd, (ks >> 2) * 1024 + (ks & 3) * 2), idesc, ks > 0 ? 1u : 0u);
+          tc_commit(&sh.s_full[b]);
         }
         __syncwarp();
-        ok = mbar_wait(&bars->p_full[1], g & 1, abort);
-        if (!ok) break;
-        tc_fence_after();
-        if (leader) {
-#pragma unroll
-          for (int ks = 2; ks < 4; ++ks) mma_ts(t_o, t_s + 32 + ks * 8, at(vb_desc, ks * 128), idesc_pv, 1u);
-        }
-        __syncwarp();
-        ++g;
-        if (h + 1 < n_steps) {
-          issue_qk();
-        } else {
-          if (leader) tc_commit(&bars->o_done);
-          __syncwarp();
-        }
       }
     }
-    if (*abort) {
-      // Tensor memory must not be released under a product in flight: a commit arrives once
-      // everything this lane has issued is complete; the wait for it is bounded like the others.
-      if (leader) tc_commit(&bars->drain);
-      __syncwarp();
-      settle(&bars->drain, 0);
+    drain_products(leader, &sh.drain[0]);
+  } else if (warp == kWarpPV) {
+    // ===== issuer of the value products
+    constexpr uint32_t idesc = idesc_bf16_f32(128, 128, false, true);
+    // V (MN-major): 64 dims = one 128-byte row; dim halves 128*128 B apart (the LBO); 16 keys = 16 rows =
+    // 2048 B per k-step.
+    const uint64_t v_desc = smem_desc_sw128(smem_u32(smem + kOffV), kTileBytes / 2, 1024);
+    const bool leader = elect_one();
+    uint32_t g = 0, nt = 0;  // key steps and tiles with key steps so far
+    int4 ti;
+    for (int t = 0; ok && next_tile(t, ti); ++t) {
+      const int n_steps = n_steps_of(ti.y);
+      if (n_steps == 0) continue;
+      if (nt > 0) wait(&sh.o_free, (nt - 1) & 1);
+      ++nt;
+      for (int h = 0; h < n_steps; ++h, ++g) {  // O (+)= P_g V_g
+        const uint32_t b = g & 1;
+        wait(&sh.v_full[b], (g >> 1) & 1);
+        if (!wait(&sh.p_full[b], (g >> 1) & 1)) break;
+        tc_fence_after();
+        if (leader) {
+          const uint64_t vd = desc_at(v_desc, b * (kTileBytes >> 4));
+#pragma unroll
+          for (int ks = 0; ks < 8; ++ks)
+            mma_ts(tmem, tmem + 384 + b * 64 + ks * 8, desc_at(vd, ks * 128), idesc, (h > 0 || ks > 0) ? 1u : 0u);
+          tc_commit(&sh.pv_done[b]);
+        }
+        __syncwarp();
+      }
     }
-  } else {
-    // ===== softmax / correction / epilogue: thread = one query row
+    drain_products(leader, &sh.drain[1]);
+  } else if (warp < 8) {
+    // ===== softmax / correction / epilogue: thread = one query row, steps g with g & 1 == w
     setmaxnreg_inc<kRegsSoftmax>();
-    const int row = (warp & 3) * 32 + lane;  // row inside the 128-row query tile
-    const uint32_t o_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16), s_addr = o_addr + 128;
+    const uint32_t w = warp >> 2, quarter = warp & 3;
+    const int row = quarter * 32 + lane;  // row inside the 128-row query tile
+    const uint32_t o_addr = tmem + (quarter << 21), s_addr = o_addr + 128 + w * 128, p_addr = o_addr + 384 + w * 64;
     const float c = p.scale_log2;
     const uint64_t c2 = pack_f32x2(c, c);
-    float m_ref, l_run;
-    // Moves the reference of the rows whose maximum grew by more than 2^8 and rescales what they have
-    // accumulated.  O is quiescent: its last product was issued before the scores of this step.
-    auto move_reference = [&](float x_max, bool has_o, float &alpha) {
-      if (x_max > m_ref + 8.f) {
-        alpha = ex2(m_ref - x_max);
-        m_ref = x_max;
-      }
-      if (has_o) {
-        const uint64_t alpha2 = pack_f32x2(alpha, alpha);
-#pragma unroll 1
-        for (int ch = 0; ch < 8; ++ch) {
-          uint32_t v[16];
-          tmem_ld16(o_addr + ch * 16, v);
-          tmem_wait_ld();
-#pragma unroll
-          for (int i = 0; i < 16; i += 2) {
-            float lo, hi;
-            unpack_f32x2(mul_f32x2(pack_f32x2(__uint_as_float(v[i]), __uint_as_float(v[i + 1])), alpha2), lo, hi);
-            v[i] = __float_as_uint(lo);
-            v[i + 1] = __float_as_uint(hi);
-          }
-          tmem_st16(o_addr + ch * 16, v);
-        }
-      }
-    };
-    // part v of P_h is written: the product may read it
-    auto arrive = [&](int v) {
-      tmem_wait_st();
+    auto arrive = [&](uint64_t *bar) {  // this warp's tensor-memory accesses so far are ordered before it
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(&bars->p_full[v]);
+      if (lane == 0) mbar_arrive(bar);
     };
-    auto arrive_both = [&]() {
-      arrive(0);
-      if (lane == 0) mbar_arrive(&bars->p_full[1]);
-    };
-    uint32_t g = 0, nq = 0;
-    bool ok = true;
+    uint32_t g0 = 0, nt = 0;  // key steps before the present tile, tiles with key steps before it
     int4 ti;
     for (int t = 0; ok && next_tile(t, ti); ++t) {
       const int n_steps = n_steps_of(ti.y);
       const int bidx = ti.z / p.hcount, hidx = p.h0 + ti.z % p.hcount;
-      const int r = bidx * p.H + hidx;
-      const uint32_t *steps = p.steps + ((size_t)r * p.n_tiles_per_head + ti.x) * p.step_pitch;
-      // below every logit: the first step moves it (and rows without a key keep it)
-      m_ref = -3.0e38f;
-      l_run = 0.f;
-      uint32_t e_next = n_steps > 0 ? step_entry(steps, 0) : 0u;
-      for (int h = 0; h < n_steps; ++h, ++g) {
-        // whether all 128 keys of the step count for this row, or the 64 of one block (warp-uniform)
+      const uint32_t *steps = steps_of(ti.z, ti.x);
+      float m_ref = kNoReference, l_run = 0.f;  // (rows without a key keep the reference)
+      const uint32_t h0 = (w ^ g0) & 1;         // this warpgroup's first step of the tile
+      uint32_t e_next = (int)h0 < n_steps ? step_entry(steps, h0) : 0u;
+      for (int h = h0; h < n_steps; h += 2) {
+        const uint32_t g = g0 + h;
         const uint32_t e = e_next;
-        if (h + 1 < n_steps) e_next = step_entry(steps, h + 1);
-        const uint32_t qb = (warp & 3) >> 1, flags = (e >> (10 + qb)) & 0x10001u;  // (64-token blocks)
-        const bool full = B == 128 ? (int)(e + 1) * 128 <= p.N : flags == 0x10001u && !(e & 0x10001000u);
-        ok = __all_sync(0xffffffffu, mbar_wait(&bars->s_full, g & 1, abort));
-        if (!ok) break;
+        if (h + 2 < n_steps) e_next = step_entry(steps, h + 2);
+        // which halves of the step this row's query block lists, whether the step holds the ragged last block
+        const uint32_t flags = (e >> (10 + (quarter >> 1))) & 0x10001u;  // (64-token blocks)
+        const bool ragged = B == 128 ? (int)(e + 1) * 128 > p.N : (e & 0x10001000u) != 0u;
+        wait(&sh.s_full[w], (g >> 1) & 1);
+        if (g > 0) wait(&sh.m_ready[w ^ 1][quarter], ((g - 1) >> 1) & 1);  // (half a step old by now, as a rule)
         tc_fence_after();
+        const float m_prev = h > 0 ? sh.m[w ^ 1][row] : kNoReference;
         Sums sums = {0.f, 0.f, 0.f, 0.f};
-        float alpha = 1.f;
-        if (__builtin_expect(full, 1)) {
-          // All 128 keys count.  The exponentials of the first 32 keys are taken with the running reference
-          // as it stands while the row maximum is found, and once more in the rare step that moves it.
+        // Agrees on the reference of step g given the row's maximum; true if it is not the one this warp has
+        // used so far (some row).
+        auto new_reference = [&](float x_max) -> bool {
+          const bool grow = x_max > m_prev + kMaxGrowth;
+          const float m_new = grow ? x_max : m_prev;
+          sh.m[w][row] = m_new;
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&sh.m_ready[w][quarter]);
+          if (__builtin_expect(!__any_sync(0xffffffffu, m_new != m_ref), 1)) return false;
+          l_run *= ex2(m_ref - m_new);
+          m_ref = m_new;
+          if (h > 0 && __any_sync(0xffffffffu, grow)) {
+            // O changes scale: the products of the steps before have to be complete
+            if (g >= 2) wait(&sh.pv_done[w], ((g - 2) >> 1) & 1);
+            if (wait(&sh.pv_done[w ^ 1], ((g - 1) >> 1) & 1)) {
+              tc_fence_after();
+              const float alpha = ex2(m_prev - m_new);
+              const uint64_t alpha2 = pack_f32x2(alpha, alpha);
+#pragma unroll 1
+              for (int ch = 0; ch < 8; ++ch) {
+                uint32_t v[16];
+                tmem_ld16(o_addr + ch * 16, v);
+                tmem_wait_ld();
+#pragma unroll
+                for (int i = 0; i < 16; i += 2) {
+                  float lo, hi;
+                  unpack_f32x2(mul_f32x2(pack_f32x2(__uint_as_float(v[i]), __uint_as_float(v[i + 1])), alpha2), lo, hi);
+                  v[i] = __float_as_uint(lo);
+                  v[i + 1] = __float_as_uint(hi);
+                }
+                tmem_st16(o_addr + ch * 16, v);
+              }
+            }
+          }
+          return true;
+        };
+        // the product that read this warpgroup's P two steps ago is complete
+        auto p_free = [&]() {
+          if (g >= 2) wait(&sh.pv_done[w], ((g - 2) >> 1) & 1);
+          tc_fence_after();
+        };
+        if (B == 128 || flags == 0x10001u || ragged) {
+          // The exponentials of the first 32 keys are taken with the reference as it
+          // was while the row maximum is found, and once more in the rare step that moves it.
           uint32_t s[128], pk[32];
 #pragma unroll
           for (int q = 0; q < 4; ++q) tmem_ld32(s_addr + q * 32, *reinterpret_cast<uint32_t(*)[32]>(&s[q * 32]));
           tmem_wait_ld();
+          arrive(&sh.s_free[w]);
+          if (__builtin_expect(ragged, 0)) {
+            const int n0 = B == 128 ? p.N - (int)e * 128 : (flags & 1u) ? p.N - (int)(e & 0x3ff) * 64 : 0;
+            const int n1 = B == 128 ? n0 - 64 : (flags >> 16) ? p.N - (int)((e >> 16) & 0x3ff) * 64 : 0;
+#pragma unroll
+            for (int i = 0; i < 64; ++i) {
+              if (i >= n0) s[i] = 0xff800000u;  // -inf: ignored by the max, 2^-inf = 0
+              if (i >= n1) s[64 + i] = 0xff800000u;
+            }
+          }
           uint64_t neg_m2 = pack_f32x2(-m_ref, -m_ref);
           exp32(&s[0], c2, neg_m2, &pk[0], sums);
-          const float x_max = fmaxf(max64(&s[0]), max64(&s[64])) * c;
-          if (__any_sync(0xffffffffu, x_max > m_ref + 8.f)) {
-            move_reference(x_max, h > 0, alpha);
+          if (__builtin_expect(new_reference(fmaxf(max64(&s[0]), max64(&s[64])) * c), 0)) {
             neg_m2 = pack_f32x2(-m_ref, -m_ref);
             sums = {0.f, 0.f, 0.f, 0.f};
             exp32(&s[0], c2, neg_m2, &pk[0], sums);
           }
           exp32(&s[32], c2, neg_m2, &pk[16], sums);
-          tmem_st32(s_addr, pk);
+          p_free();
+          tmem_st32(p_addr, pk);
           exp32(&s[64], c2, neg_m2, &pk[0], sums);
-          tmem_st16(s_addr + 32, *reinterpret_cast<uint32_t(*)[16]>(&pk[0]));
-          arrive(0);
           exp32(&s[96], c2, neg_m2, &pk[16], sums);
-          tmem_st16(s_addr + 48, *reinterpret_cast<uint32_t(*)[16]>(&pk[16]));
-          arrive(1);
-        } else if (B == 64 && (flags == 1u || flags == 0x10000u) && !(e & 0x10001000u)) {
+          tmem_st32(p_addr + 32, pk);
+        } else if (flags != 0u) {
           // This row's query block lists one of the step's two blocks.  The product reads all 128 keys of
           // the step: zeros for the other one.
           const uint32_t v = flags >> 16;
-          const uint32_t mine = s_addr + v * 64, p_mine = s_addr + v * 32, p_other = s_addr + (32 - v * 32);
           uint32_t s[64], pk[32];
-          tmem_ld32(mine, *reinterpret_cast<uint32_t(*)[32]>(&s[0]));
-          tmem_ld32(mine + 32, *reinterpret_cast<uint32_t(*)[32]>(&s[32]));
+          tmem_ld32(s_addr + v * 64, *reinterpret_cast<uint32_t(*)[32]>(&s[0]));
+          tmem_ld32(s_addr + v * 64 + 32, *reinterpret_cast<uint32_t(*)[32]>(&s[32]));
 #pragma unroll
           for (int i = 0; i < 32; ++i) pk[i] = 0u;
           tmem_wait_ld();
-          tmem_st32(p_other, pk);
-          const float x_max = max64(s) * c;
-          if (__any_sync(0xffffffffu, x_max > m_ref + 8.f)) move_reference(x_max, h > 0, alpha);
+          arrive(&sh.s_free[w]);
+          new_reference(max64(s) * c);
+          p_free();
+          tmem_st32(p_addr + (32 - v * 32), pk);
           const uint64_t neg_m2 = pack_f32x2(-m_ref, -m_ref);
           exp32(&s[0], c2, neg_m2, &pk[0], sums);
           exp32(&s[32], c2, neg_m2, &pk[16], sums);
-          tmem_st32(p_mine, pk);
-          arrive_both();
-        } else if (B == 64 && flags == 0u) {
+          tmem_st32(p_addr + v * 32, pk);
+        } else {
           // none of the step's blocks is listed by this row's query block
           uint32_t pk[32];
 #pragma unroll
           for (int i = 0; i < 32; ++i) pk[i] = 0u;
-          tmem_st32(s_addr, pk);
-          tmem_st32(s_addr + 32, pk);
-          arrive_both();
-        } else {
-          // The ragged last block: one half at a time, the scores read twice (the weights of the first half
-          // only overwrite its own scores).
-          int lim0, lim1;  // keys of each half that count
-          if (B == 128) {
-            const int rem = p.N - (int)e * 128;
-            lim0 = min(rem, 64);
-            lim1 = max(0, min(rem - 64, 64));
-          } else {
-            lim0 = (flags & 1u) ? min(64, p.N - (int)(e & 0x3ff) * 64) : 0;
-            lim1 = (flags >> 16) ? min(64, p.N - (int)((e >> 16) & 0x3ff) * 64) : 0;
-          }
-          float x_max = -INFINITY;
-#pragma unroll 1
-          for (int pass = 0; pass < 4; ++pass) {
-            const int v = pass & 1, n = v ? lim1 : lim0;
-            uint32_t s[64], pk[32];
-            tmem_ld32(s_addr + v * 64, *reinterpret_cast<uint32_t(*)[32]>(&s[0]));
-            tmem_ld32(s_addr + v * 64 + 32, *reinterpret_cast<uint32_t(*)[32]>(&s[32]));
-            tmem_wait_ld();
-#pragma unroll
-            for (int i = 0; i < 64; ++i)
-              if (i >= n) s[i] = 0xff800000u;  // -inf: ignored by the max, 2^-inf = 0
-            if (pass < 2) {
-              x_max = fmaxf(x_max, max64(s) * c);
-            } else {
-              if (pass == 2 && __any_sync(0xffffffffu, x_max > m_ref + 8.f)) move_reference(x_max, h > 0, alpha);
-              const uint64_t neg_m2 = pack_f32x2(-m_ref, -m_ref);
-              exp32(&s[0], c2, neg_m2, &pk[0], sums);
-              exp32(&s[32], c2, neg_m2, &pk[16], sums);
-              tmem_st32(s_addr + v * 32, pk);
-              tmem_wait_st();
-            }
-          }
-          arrive_both();
+          arrive(&sh.s_free[w]);
+          new_reference(-INFINITY);
+          p_free();
+          tmem_st32(p_addr, pk);
+          tmem_st32(p_addr + 32, pk);
         }
-        l_run = l_run * alpha + ((sums.a + sums.b) + (sums.c + sums.d));
+        l_run += (sums.a + sums.b) + (sums.c + sums.d);
+        if (h == n_steps - 2) sh.l[nt & 1][row] = make_float2(l_run, m_ref);  // the partner finishes the tile
+        tmem_wait_st();
+        if (!ok) break;
+        arrive(&sh.p_full[w]);
       }
-      // epilogue: O / l, one row per thread
-      const int tok = ti.x * 128 + row;
-      const bool valid_row = tok < p.N;
-      if (ok && n_steps > 0) {
-        ok = __all_sync(0xffffffffu, mbar_wait(&bars->o_done, nq & 1, abort));
-        ++nq;
-      }
-      if (ok) {
+      if (!ok) break;
+      // epilogue: O / l, one row per thread, by the warpgroup that had the last step (a tile without key
+      // steps: by the one whose turn it is)
+      const uint32_t g_last = g0 + n_steps - 1;
+      if (n_steps > 0 ? (g_last & 1) == w : (t & 1) == (int)w) {
+        const int r = bidx * p.H + hidx, tok = ti.x * 128 + row;
+        const bool valid_row = tok < p.N;
+        if (n_steps > 0 && !wait(&sh.pv_done[w], (g_last >> 1) & 1)) break;
         tc_fence_after();
+        if (n_steps > 1) {
+          const float2 other = sh.l[nt & 1][row];
+          l_run += other.x * ex2(other.y - m_ref);
+        }
         const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
         uint16_t *orow = p.O + (long long)bidx * p.sb + (long long)hidx * p.sh + (long long)tok * p.sn;
 #pragma unroll 1
@@ -570,31 +550,32 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
               float o[8];
 #pragma unroll
               for (int i = 0; i < 8; ++i) o[i] = n_steps > 0 ? __uint_as_float(v[g4 * 8 + i]) * inv : 0.f;
-              uint4 w;
-              w.x = pack_bf16x2(o[0], o[1]);
-              w.y = pack_bf16x2(o[2], o[3]);
-              w.z = pack_bf16x2(o[4], o[5]);
-              w.w = pack_bf16x2(o[6], o[7]);
-              *reinterpret_cast<uint4 *>(orow + ch * 32 + g4 * 8) = w;
+              uint4 x;
+              x.x = pack_bf16x2(o[0], o[1]);
+              x.y = pack_bf16x2(o[2], o[3]);
+              x.z = pack_bf16x2(o[4], o[5]);
+              x.w = pack_bf16x2(o[6], o[7]);
+              *reinterpret_cast<uint4 *>(orow + ch * 32 + g4 * 8) = x;
             }
           }
         }
+        if (n_steps > 0) arrive(&sh.o_free);
         if (valid_row && p.lse != nullptr)
           p.lse[(size_t)r * p.N + tok] = l_run > 0.f ? (m_ref + log2f(l_run)) * 0.6931471805599453f : -INFINITY;
-        // (the first product of the next tile writes O only after this warp's next arrival on p_full)
       }
+      g0 += n_steps;
+      nt += n_steps > 0 ? 1 : 0;
     }
   }
 
   // ------------------------------------------------------------------ tear-down
   tc_fence_before();
   __syncthreads();
-  if (warp == kWarpMma) {
+  if (warp == kWarpQK) {
     tc_fence_after();
-    tmem_dealloc(*tmem_base, 512);
+    tmem_dealloc(tmem, 512);
   }
-  if (tid < kStreams && reinterpret_cast<AttnBars *>(smem + kOffBar + tid * kBarBytes)->abort)
-    atomicExch(p.status, HEART_ERR_DEVICE_CHECK);
+  if (tid == 0 && sh.abort) atomicExch(p.status, HEART_ERR_DEVICE_CHECK);
 }
 
 // Step lists of the tiles of a launch: one warp per tile.  The lists of the tile's query blocks (any
@@ -787,7 +768,7 @@ cudaError_t launch_bk(const Geom &g, const Workspace &w, const CUtensorMap &mq, 
                  (int)(g.N % g.block != 0), steps, tiles, firsts, prm.counter, prm.status);
   if (e != cudaSuccess) return e;
   ++*launches;
-  if (planned > kStreams * kSms) {  // up to there every tile starts at once: no order to choose
+  if (planned > kSms) {  // up to there every tile starts at once: no order to choose
     // K + V of one head beyond 32 MB (about half of one die's share of the L2): order by key locality
     const int by_first_key = (size_t)g.N * kD * 2 * 2 > (size_t)(32u << 20) ? 1 : 0;
     e = launch_pdl(tile_order_kernel, dim3((prm.n_tiles_per_head + 255) / 256, n_heads), dim3(256), 0, s,
@@ -814,7 +795,7 @@ cudaError_t launch_attention(const Geom &g, const Workspace &w, const void *Q, c
     hcount = g.H;
   }
   CUtensorMap mq, mk, mv;
-  if (!make_map(&mq, Q, g, 128, 2) || !make_map(&mk, K, g, g.block, g.block == 128 ? 2 : 1) || !make_map(&mv, V, g, 64, 2))
+  if (!make_map(&mq, Q, g, 128, 2) || !make_map(&mk, K, g, g.block, g.block == 128 ? 2 : 1) || !make_map(&mv, V, g, g.block, g.block == 128 ? 2 : 1))
     return cudaErrorInvalidValue;
   AttnParams prm = {};
   prm.O = static_cast<uint16_t *>(O);
