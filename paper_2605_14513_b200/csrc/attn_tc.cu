@@ -50,7 +50,7 @@ using namespace tc;
 
 constexpr int kAttnThreads = 384;
 constexpr int kWarpQK = 8, kWarpV = 9, kWarpK = 10, kWarpPV = 11;
-constexpr int kRegsSoftmax = 216, kRegsHelper = 72;  // 216 * 256 + 72 * 128 = the CTA's 384 x 168
+constexpr int kRegsSoftmax = 224, kRegsHelper = 56;  // 224 * 256 + 56 * 128 = the CTA's 384 x 168
 constexpr int kTileBytes = 32768;  // 128 rows x 128 dims: [2 dim halves][128 rows][64] bf16, 128-byte swizzle
 constexpr int kTileRing = 4;       // announced tiles
 constexpr int kTileReaders = 11;   // softmax warps, issuers, V producer
@@ -457,7 +457,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
           if (g >= 2) wait(&sh.pv_done[w], ((g - 2) >> 1) & 1);
           tc_fence_after();
         };
-        if (B == 128 || flags == 0x10001u || ragged) {
+        if (__builtin_expect((B == 128 || flags == 0x10001u) && !ragged, 1)) {
           // The exponentials of the first 32 keys are taken with the reference as it
           // was while the row maximum is found, and once more in the rare step that moves it.
           uint32_t s[128], pk[32];
@@ -465,15 +465,6 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
           for (int q = 0; q < 4; ++q) tmem_ld32(s_addr + q * 32, *reinterpret_cast<uint32_t(*)[32]>(&s[q * 32]));
           tmem_wait_ld();
           arrive(&sh.s_free[w]);
-          if (__builtin_expect(ragged, 0)) {
-            const int n0 = B == 128 ? p.N - (int)e * 128 : (flags & 1u) ? p.N - (int)(e & 0x3ff) * 64 : 0;
-            const int n1 = B == 128 ? n0 - 64 : (flags >> 16) ? p.N - (int)((e >> 16) & 0x3ff) * 64 : 0;
-#pragma unroll
-            for (int i = 0; i < 64; ++i) {
-              if (i >= n0) s[i] = 0xff800000u;  // -inf: ignored by the max, 2^-inf = 0
-              if (i >= n1) s[64 + i] = 0xff800000u;
-            }
-          }
           uint64_t neg_m2 = pack_f32x2(-m_ref, -m_ref);
           exp32(&s[0], c2, neg_m2, &pk[0], sums);
           if (__builtin_expect(new_reference(fmaxf(max64(&s[0]), max64(&s[64])) * c), 0)) {
@@ -487,7 +478,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
           exp32(&s[64], c2, neg_m2, &pk[0], sums);
           exp32(&s[96], c2, neg_m2, &pk[16], sums);
           tmem_st32(p_addr + 32, pk);
-        } else if (flags != 0u) {
+        } else if (B == 64 && flags != 0u && !ragged) {
           // This row's query block lists one of the step's two blocks.  The product reads all 128 keys of
           // the step: zeros for the other one.
           const uint32_t v = flags >> 16;
@@ -505,7 +496,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
           exp32(&s[0], c2, neg_m2, &pk[0], sums);
           exp32(&s[32], c2, neg_m2, &pk[16], sums);
           tmem_st32(p_addr + v * 32, pk);
-        } else {
+        } else if (B == 64 && flags == 0u) {
           // none of the step's blocks is listed by this row's query block
           uint32_t pk[32];
 #pragma unroll
@@ -515,6 +506,42 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
           p_free();
           tmem_st32(p_addr, pk);
           tmem_st32(p_addr + 32, pk);
+        } else {
+          // The ragged last block: 32 columns at a time, the scores read twice.  (Masking it in the first
+          // branch cost all steps 7 % of their clocks: 128 selects between the loads and the weights.)
+          int n0, n1;  // keys of each half that count
+          if (B == 128) {
+            n0 = p.N - (int)e * 128;
+            n1 = n0 - 64;
+          } else {
+            n0 = (flags & 1u) ? p.N - (int)(e & 0x3ff) * 64 : 0;
+            n1 = (flags >> 16) ? p.N - (int)((e >> 16) & 0x3ff) * 64 : 0;
+          }
+          float x_max = -INFINITY;
+#pragma unroll 1
+          for (int pass = 0; pass < 8; ++pass) {
+            const int q = pass & 3, n = (q & 2 ? n1 : n0) - (q & 1) * 32;
+            uint32_t s[32], pk[16];
+            tmem_ld32(s_addr + q * 32, s);
+            tmem_wait_ld();
+            float mx = -INFINITY;
+#pragma unroll
+            for (int i = 0; i < 32; ++i) {
+              if (i >= n) s[i] = 0xff800000u;  // -inf: ignored by the max, 2^-inf = 0
+              mx = fmaxf(mx, __uint_as_float(s[i]));
+            }
+            if (pass < 4) {
+              x_max = fmaxf(x_max, mx * c);
+              if (pass == 3) {
+                new_reference(x_max);
+                p_free();
+              }
+            } else {
+              exp32(s, c2, pack_f32x2(-m_ref, -m_ref), pk, sums);
+              tmem_st16(p_addr + q * 16, pk);
+            }
+          }
+          arrive(&sh.s_free[w]);
         }
         l_run += (sums.a + sums.b) + (sums.c + sums.d);
         if (h == n_steps - 2) sh.l[nt & 1][row] = make_float2(l_run, m_ref);  // the partner finishes the tile
