@@ -2,10 +2,9 @@
 // importance, retain until the accumulated importance reaches the head's threshold; the minimal
 // cumulative-mass set of Observation I).  Importance = row softmax of the block-pooled Q.K^T scores.
 //
-// Two kernels.  pooled_scores_kernel is a register-tiled fp64 contraction of the pooled means: a CTA
-// owns 64 query blocks x 128 key blocks of one head (each thread 8 x 4), the means arrive 16 dims at
-// a time by cp.async into a double-buffered shared-memory tile, and every score accumulates over the
-// 128 dims in ascending order in one fma chain.  The scores go to the workspace (they stay in L2).
+// Two kernels.  pooled_scores_kernel contracts the pooled means with the fp64 matrix instruction
+// (mma.m8n8k4.f64), the 128 dims in ascending order for every score; the means arrive by cp.async in
+// shared-memory tiles.  The scores go to the workspace (they stay in L2).
 // top_p_kernel gives each warp one row (its weights in shared memory, the loops over them rolled):
 // row max, unnormalised weights e = exp(s - max), then top-p WITHOUT a sort and without dividing by
 // the row sum z: the kept set is {e > theta} plus the lowest-index ties at theta, where theta is the
@@ -19,10 +18,7 @@
 
 namespace heart {
 
-constexpr int SI = 64;    // query blocks per CTA of the score kernel
-constexpr int SJ = 128;   // key blocks per CTA
-constexpr int TD = 16;    // dims per staged chunk
-constexpr int KLD = TD + 1;
+constexpr int kSmallScoreTiles = 148;  // 64 x 64 score tiles of a launch up to which 32 x 32 ones are used
 constexpr int kRowsPerCta = 8;  // rows (warps) per CTA of the top-p kernel
 constexpr int kMaxCand = 64;    // candidates the direct threshold evaluation takes
 
@@ -37,9 +33,9 @@ __device__ __forceinline__ double warp_max(double v) {
   return v;
 }
 
-// 8-byte asynchronous copy global -> shared; src_bytes = 0 writes zeros instead
-__device__ __forceinline__ void cp_async8(double *smem_dst, const double *src, int src_bytes) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(smem_dst)),
+// 16-byte asynchronous copy global -> shared; src_bytes = 0 writes zeros instead
+__device__ __forceinline__ void cp_async16(double *smem_dst, const double *src, int src_bytes) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(smem_dst)),
                "l"(src), "r"(src_bytes)
                : "memory");
 }
@@ -49,13 +45,31 @@ __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
-// scores[r][I][J] = scale * <mean_q[r][I], mean_k[r][J]> for the refreshed heads r.
-__global__ void __launch_bounds__(256, 2) pooled_scores_kernel(const double *__restrict__ bmean, int R, int nb,
-                                                               int pitch, double scale,
-                                                               const uint8_t *__restrict__ refresh,
-                                                               double *__restrict__ scores,
-                                                               int32_t *__restrict__ status,
-                                                               unsigned long long expect_sig) {
+// D (8 x 8) += A (8 x 4, row) * B (4 x 8, col), fp64: lane l holds A[l / 4][l % 4], B[l % 4][l / 4] and
+// D[l / 4][2 * (l % 4) + {0, 1}].
+__device__ __forceinline__ void mma_f64(double (&d)[2], double a, double b) {
+  asm("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};" : "+d"(d[0]), "+d"(d[1]) : "d"(a), "d"(b));
+}
+
+// scores[r][I][J] = scale * <mean_q[r][I], mean_k[r][J]> for the refreshed heads r.  A CTA of four warps owns
+// 2 WT x 2 WT scores of one head, a warp WT x WT; the dims come TD at a time through STAGES buffers.
+// Bound by the fp64 rate (18.5 T fma/s measured, by the matrix instruction as by plain fma).  The matrix
+// instruction is there for the operands: a warp reads 2 WT / 8 doubles per lane and k-step for (WT / 8)^2
+// products of 256 fma; with plain fma the shared-memory reads took as long as the arithmetic (8.6 T fma/s).
+// The row pitch is 4 (mod 16) doubles: the 8 x 4 fragments are read without bank conflicts.
+template <int WT, int TD, int STAGES>
+struct ScoreTile {
+  static constexpr int kRows = 4 * WT, kPitch = TD + 4;  // 2 WT query rows, then 2 WT key rows
+  static constexpr int kBytes = 8 * STAGES * kRows * kPitch;
+};
+
+template <int WT, int TD, int STAGES>
+__global__ void __launch_bounds__(128) pooled_scores_kernel(const double *__restrict__ bmean, int R, int nb, int pitch,
+                                                            double scale, const uint8_t *__restrict__ refresh,
+                                                            double *__restrict__ scores, int32_t *__restrict__ status,
+                                                            unsigned long long expect_sig) {
+  using T = ScoreTile<WT, TD, STAGES>;
+  constexpr int F = WT / 8;  // fragments per warp and side
   const int r = blockIdx.z;
   pdl_wait();  // refresh flags and block means come from the kernels before this one
   pdl_launch_dependents();
@@ -65,64 +79,65 @@ __global__ void __launch_bounds__(256, 2) pooled_scores_kernel(const double *__r
     return;
   }
   if (refresh != nullptr && refresh[r] == 0) return;  // reuse branch of Algorithm 1: nothing to predict
-  const int I0 = blockIdx.y * SI, J0 = blockIdx.x * SJ;
+  const int I0 = blockIdx.y * 2 * WT, J0 = blockIdx.x * 2 * WT;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  double *tile = reinterpret_cast<double *>(smem_raw);  // [2][SI + SJ][KLD]: query rows, then key rows
+  double *tile = reinterpret_cast<double *>(smem_raw);  // [STAGES][kRows][kPitch]
   const double *bq = bmean + ((size_t)r * nb) * kD;
   const double *bk = bmean + (((size_t)R + r) * nb) * kD;
-  const int tid = threadIdx.x;
-  constexpr int kRows = SI + SJ, kPer = kRows * TD / 256;  // 12 copies per thread and stage
-  auto stage_in = [&](int stage, int buf) {
-    const int dc = stage * TD;
-    double *dst = tile + (size_t)buf * kRows * KLD;
-#pragma unroll
-    for (int k = 0; k < kPer; ++k) {
-      const int e = tid + 256 * k, row = e / TD, dd = e % TD;
-      const int blk = row < SI ? I0 + row : J0 + row - SI;
-      const double *src = (row < SI ? bq : bk) + (size_t)min(blk, nb - 1) * kD + dc + dd;
-      cp_async8(dst + row * KLD + dd, src, blk < nb ? 8 : 0);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  auto stage_in = [&](int stage) {
+    if (stage < kD / TD) {
+      double *dst = tile + (size_t)(stage % STAGES) * T::kRows * T::kPitch;
+#pragma unroll 8
+      for (int e = tid; e < T::kRows * TD / 2; e += 128) {
+        const int row = e / (TD / 2), dd = e % (TD / 2) * 2;
+        const int blk = row < 2 * WT ? I0 + row : J0 + row - 2 * WT;
+        const double *src = (row < 2 * WT ? bq : bk) + (size_t)min(blk, nb - 1) * kD + stage * TD + dd;
+        cp_async16(dst + row * T::kPitch + dd, src, blk < nb ? 16 : 0);
+      }
     }
     cp_async_commit();
   };
-  const int rg = tid >> 5, cl = tid & 31;  // rows rg*8 .. rg*8+7, key columns cl + 32 m
-  double acc[8][4];
+  double acc[F][F][2];
 #pragma unroll
-  for (int a = 0; a < 8; ++a)
+  for (int i = 0; i < F; ++i)
 #pragma unroll
-    for (int m = 0; m < 4; ++m) acc[a][m] = 0.0;
-  stage_in(0, 0);
+    for (int j = 0; j < F; ++j) acc[i][j][0] = acc[i][j][1] = 0.0;
+#pragma unroll
+  for (int i = 0; i < STAGES - 1; ++i) stage_in(i);
+  const int ai = (warp >> 1) * WT + (lane >> 2), bj = 2 * WT + (warp & 1) * WT + (lane >> 2), kk = lane & 3;
+  const bool idle = I0 + (warp >> 1) * WT >= nb || J0 + (warp & 1) * WT >= nb;  // nothing but padding
   for (int stage = 0; stage < kD / TD; ++stage) {
-    const int buf = stage & 1;
-    if (stage + 1 < kD / TD) {
-      stage_in(stage + 1, buf ^ 1);  // its buffer was released by the barrier that ended stage - 1
-      cp_async_wait<1>();
-    } else {
-      cp_async_wait<0>();
-    }
+    stage_in(stage + STAGES - 1);  // its buffer was released by the barrier that ended stage - 1
+    cp_async_wait<STAGES - 1>();
     __syncthreads();
-    const double *Qs = tile + (size_t)buf * kRows * KLD, *Ks = Qs + SI * KLD;
+    if (!idle) {
+      const double *A = tile + (size_t)(stage % STAGES) * T::kRows * T::kPitch + ai * T::kPitch + kk;
+      const double *Bt = tile + (size_t)(stage % STAGES) * T::kRows * T::kPitch + bj * T::kPitch + kk;
 #pragma unroll 4
-    for (int dd = 0; dd < TD; ++dd) {
-      double q[8], k4[4];
+      for (int k = 0; k < TD; k += 4) {
+        double a[F], b[F];
 #pragma unroll
-      for (int a = 0; a < 8; ++a) q[a] = Qs[(rg * 8 + a) * KLD + dd];
+        for (int i = 0; i < F; ++i) a[i] = A[i * 8 * T::kPitch + k];
 #pragma unroll
-      for (int m = 0; m < 4; ++m) k4[m] = Ks[(cl + 32 * m) * KLD + dd];
+        for (int j = 0; j < F; ++j) b[j] = Bt[j * 8 * T::kPitch + k];
 #pragma unroll
-      for (int a = 0; a < 8; ++a)
+        for (int i = 0; i < F; ++i)
 #pragma unroll
-        for (int m = 0; m < 4; ++m) acc[a][m] = fma(q[a], k4[m], acc[a][m]);
+          for (int j = 0; j < F; ++j) mma_f64(acc[i][j], a[i], b[j]);
+      }
     }
     __syncthreads();  // this stage's buffer may be refilled
   }
 #pragma unroll
-  for (int a = 0; a < 8; ++a) {
-    const int I = I0 + rg * 8 + a;
+  for (int i = 0; i < F; ++i) {
+    const int I = I0 + ai + i * 8;
     if (I >= nb) continue;
+    double *srow = scores + ((size_t)r * nb + I) * pitch;
 #pragma unroll
-    for (int m = 0; m < 4; ++m) {
-      const int J = J0 + cl + 32 * m;
-      if (J < pitch) scores[((size_t)r * nb + I) * pitch + J] = acc[a][m] * scale;
+    for (int j = 0; j < F; ++j) {
+      const int J = J0 + (warp & 1) * WT + j * 8 + 2 * kk;  // (pitch is even: the pair stays inside the row)
+      if (J < pitch) *reinterpret_cast<double2 *>(srow + J) = make_double2(acc[i][j][0] * scale, acc[i][j][1] * scale);
     }
   }
 }
@@ -357,16 +372,24 @@ static cudaError_t launch_nj(const Geom &g, const Workspace &w, const double *ta
                     expect_sig);
 }
 
+template <int WT, int TD, int STAGES>
+static cudaError_t launch_scores(const Geom &g, const Workspace &w, const uint8_t *refresh, cudaStream_t s,
+                                 unsigned long long expect_sig) {
+  constexpr int smem = ScoreTile<WT, TD, STAGES>::kBytes;
+  cudaError_t e = cudaFuncSetAttribute(pooled_scores_kernel<WT, TD, STAGES>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  const unsigned t = (g.nb + 2 * WT - 1) / (2 * WT);
+  return launch_pdl(pooled_scores_kernel<WT, TD, STAGES>, dim3(t, t, g.R), dim3(128), (size_t)smem, s, (const double *)w.bmean,
+                    g.R, g.nb, ((g.nb + 31) / 32) * 32, g.scale, refresh, w.scores, w.status, expect_sig);
+}
+
 cudaError_t launch_pooled_scores(const Geom &g, const Workspace &w, const uint8_t *refresh, cudaStream_t s,
                                  int *launches, unsigned long long expect_sig) {
   ++*launches;
-  const int nj = (g.nb + 31) / 32, pitch = nj * 32;
-  const size_t smem = sizeof(double) * 2 * (SI + SJ) * KLD;
-  cudaError_t e = cudaFuncSetAttribute(pooled_scores_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  dim3 grid((g.nb + SJ - 1) / SJ, (g.nb + SI - 1) / SI, g.R);
-  return launch_pdl(pooled_scores_kernel, grid, dim3(256), smem, s, (const double *)w.bmean, g.R, g.nb, pitch, g.scale,
-                    refresh, w.scores, w.status, expect_sig);
+  // Few tiles: small ones with all dims loaded at once, so that the work spreads over the SMs.
+  const long long tiles64 = (long long)((g.nb + 63) / 64) * ((g.nb + 63) / 64) * g.R;
+  if (tiles64 <= kSmallScoreTiles) return launch_scores<16, 128, 1>(g, w, refresh, s, expect_sig);
+  return launch_scores<32, 16, 3>(g, w, refresh, s, expect_sig);
 }
 
 cudaError_t launch_top_p(const Geom &g, const Workspace &w, const double *tau, const uint8_t *refresh,
