@@ -5,22 +5,29 @@
 // Two kernels.  pooled_scores_kernel contracts the pooled means with the fp64 matrix instruction
 // (mma.m8n8k4.f64), the 128 dims in ascending order for every score; the means arrive by cp.async in
 // shared-memory tiles.  The scores go to the workspace (they stay in L2).
-// top_p_kernel gives each warp one row (its weights in shared memory, the loops over them rolled):
-// row max, unnormalised weights e = exp(s - max), then top-p WITHOUT a sort and without dividing by
-// the row sum z: the kept set is {e > theta} plus the lowest-index ties at theta, where theta is the
-// largest element value whose ">= theta" mass still reaches tau * z -- found by a search over the
-// IEEE-754 pattern of e (positive doubles order like their bit patterns): starting below the leading
-// bits that the largest and the smallest weight share, two bits a round over all blocks down to bit
-// 48, the rest directly over the few blocks that share that prefix.  Everything is fp64 so the
-// integer outputs (bit mask, ascending index list, count) agree with a plain fp64
-// sort-and-accumulate reference except when the cumulative mass is within rounding (1e-15) of tau.
+// top_p_kernel gives each warp one row and finds the kept set WITHOUT a sort and without dividing by the
+// row sum z: the blocks above a threshold plus the lowest-index ties at it, where the threshold is the
+// largest element whose ">=" mass still reaches tau * z.  It decides in fp32 first: weights
+// e = 2^((s - max) log2 e), a few rounds that narrow the threshold down, then a direct evaluation over the few blocks
+// left.  That is final when the mass misses tau * z by more than 1.5e-5 z on both sides of the cut (the
+// errors of weights and sums stay below 1.1e-5 z, derived at the kernel) and no other block shares the
+// threshold's fp32 value; otherwise (about one row in a hundred) the row is decided in fp64: e = exp(s - max) and a search
+// over the IEEE-754 pattern of e (positive doubles order like their bit patterns), starting below the
+// leading bits that the largest and the smallest weight share, two bits a round over all blocks down to
+// bit 48, the rest directly over the few blocks that share that prefix.  So the integer outputs (bit
+// mask, ascending index list, count) agree with a plain fp64 sort-and-accumulate reference except when
+// the cumulative mass is within rounding (1e-15) of tau.
 #include "common.cuh"
+#include "tc_ptx.cuh"
 
 namespace heart {
+
+using tc::ex2;
 
 constexpr int kSmallScoreTiles = 148;  // 64 x 64 score tiles of a launch up to which 32 x 32 ones are used
 constexpr int kRowsPerCta = 8;  // rows (warps) per CTA of the top-p kernel
 constexpr int kMaxCand = 64;    // candidates the direct threshold evaluation takes
+constexpr float kMassBand = 1.5e-5f;  // of z: cuts whose mass is closer to tau * z are decided in fp64
 
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
@@ -166,10 +173,11 @@ __global__ void __launch_bounds__(32 * kRowsPerCta) top_p_kernel(const double *_
     if (I >= nb) return;
     const size_t row = (size_t)r * nb + I;
     const double *srow = scores + row * pitch;
-    // The weights of the row live in shared memory (lane-major, conflict-free): rolled loops over the
-    // NJ blocks of a lane keep the kernel small enough for the instruction cache -- fully unrolled
-    // over registers it was several times slower at n_b > 512.
+    // The row lives in shared memory (lane-major, conflict-free): rolled loops over the NJ blocks of a lane
+    // keep the kernel small enough for the instruction cache -- fully unrolled over registers it was
+    // several times slower at n_b > 512.
     double *pw = weights + (size_t)warp * NJ * 32 + lane;
+    float2 *pf = reinterpret_cast<float2 *>(pw);  // (x = s - max, e = exp(x)) over the same words
     const double neg_inf = __longlong_as_double(0xfff0000000000000LL);
     double mx = neg_inf;
 #pragma unroll 4
@@ -179,18 +187,132 @@ __global__ void __launch_bounds__(32 * kRowsPerCta) top_p_kernel(const double *_
       mx = fmax(mx, pw[(j) * 32]);
     }
     mx = warp_max(mx);
+    const double tau_r = (flags & HEART_FORCE_DENSE) ? 1.0 : tau[r];
+    // Outputs: the mask words are gathered in registers (lane l keeps word l) and leave in one store.
+    auto emit = [&](auto keep_of) {
+      int base = 0;
+      uint32_t my_word = 0u;
+#pragma unroll 4
+      for (int j = 0; j < NJ; ++j) {
+        const int J = j * 32 + lane;
+        const bool keep = keep_of(j, J < nb);
+        const unsigned word = __ballot_sync(0xffffffffu, keep);
+        if (lane == j) my_word = word;
+        if (keep) kv_idx[row * idx_stride + base + __popc(word & lt_mask)] = J;
+        base += __popc(word);
+      }
+      if (lane < W) mask_bits[row * W + lane] = my_word;
+      if (lane == 0) kv_cnt[row] = base;
+    };
+
+    // fp32.  Error of a weight: x rounds by |x| 2^-24, its product with log2 e by |x| (2^-24 + 2^-25), ex2 by
+    // 2^-22 relative; over a row sum e (1.5e-7 |x| + 2.4e-7) <= 1.3e-6 z (sum e |x| <= z ln n_b).  tau * z
+    // takes 38 roundings more, 2.3e-6, the mass at a cut at most 37 + 64, 6.1e-6: 1.1e-5 z together.
+    if (tau_r > 0.0 && tau_r < 1.0) {
+      float z = 0.f;
+#pragma unroll 4
+      for (int j = 0; j < NJ; ++j) {
+        const float x = (float)(pw[(j) * 32] - mx), e = ex2(x * 1.44269504f);
+        pf[(j) * 32] = make_float2(x, e);
+        z += e;
+      }
+      auto sum = [](float v) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        return v;
+      };
+      z = sum(z);
+      const float t = (float)tau_r * z, band = kMassBand * z;
+      // The threshold lies in [lo, hi): mass(x >= lo) reaches t, mass(x >= hi) = m_hi does not.  (All blocks below
+      // -20 together hold less than 2.1e-6.)
+      float lo = -20.f, hi = 1.f, m_hi = 0.f;
+      float v1 = -10.f, v2 = -5.f, v3 = -2.5f;
+      float *cx = reinterpret_cast<float *>(cand[warp]), *ce = cx + kMaxCand;
+      int n_cand = 0;
+      for (int round = 0; round < 12; ++round) {
+        float a1 = 0.f, a2 = 0.f, a3 = 0.f;
+#pragma unroll 8
+        for (int j = 0; j < NJ; ++j) {
+          const float2 p = pf[(j) * 32];
+          if (p.x >= v1) a1 += p.y;
+          if (p.x >= v2) a2 += p.y;
+          if (p.x >= v3) a3 += p.y;
+        }
+        a1 = sum(a1);
+        a2 = sum(a2);
+        a3 = sum(a3);
+        if (a3 >= t) {
+          lo = v3;
+        } else {
+          hi = v3, m_hi = a3;
+          if (a2 >= t) {
+            lo = v2;
+          } else {
+            hi = v2, m_hi = a2;
+            if (a1 >= t) lo = v1;
+            else hi = v1, m_hi = a1;
+          }
+        }
+        const float step = 0.25f * (hi - lo);
+        v1 = lo + step;
+        v2 = lo + 2.f * step;
+        v3 = hi - step;
+        if (round < 2) continue;
+        n_cand = 0;  // collect the blocks of the interval (the first kMaxCand of them)
+        __syncwarp();
+#pragma unroll 4
+        for (int j = 0; j < NJ; ++j) {
+          const float2 p = pf[(j) * 32];
+          const bool is_c = p.x >= lo && p.x < hi;
+          const unsigned bal = __ballot_sync(0xffffffffu, is_c);
+          if (is_c) {
+            const int pos = n_cand + __popc(bal & lt_mask);
+            if (pos < kMaxCand) cx[pos] = p.x, ce[pos] = p.y;
+          }
+          n_cand += __popc(bal);
+        }
+        __syncwarp();
+        if (n_cand <= kMaxCand) break;
+      }
+      if (n_cand <= kMaxCand) {
+        // Each lane takes two candidates: is the cut at this one, clearly?
+        float x_cut = 0.f;
+        bool found = false;
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          if (k * 32 >= n_cand) break;
+          const bool have = lane + 32 * k < n_cand;
+          const float x = have ? cx[lane + 32 * k] : 0.f, e = have ? ce[lane + 32 * k] : 0.f;
+          float above = m_hi;
+          int same = 0;
+          for (int n = 0; n < n_cand; ++n) {
+            above += cx[n] > x ? ce[n] : 0.f;
+            same += cx[n] == x ? 1 : 0;
+          }
+          if (have && same == 1 && t - above > band && above + e - t > band) found = true, x_cut = x;
+        }
+        const unsigned who = __ballot_sync(0xffffffffu, found);
+        if (__popc(who) == 1) {
+          x_cut = __shfl_sync(0xffffffffu, x_cut, __ffs(who) - 1);
+          emit([&](int j, bool valid) { return valid && pf[(j) * 32].x >= x_cut; });
+          return;
+        }
+      }
+      __syncwarp();
+    }
+
+    // fp64
     double z = 0.0;
 #pragma unroll 4
     for (int j = 0; j < NJ; ++j) {
       const int J = j * 32 + lane;
-      pw[(j) * 32] = (J < nb) ? exp_nonpositive(pw[(j) * 32] - mx) : 0.0;
+      pw[(j) * 32] = (J < nb) ? exp_nonpositive(srow[J] - mx) : 0.0;
       z += pw[(j) * 32];
     }
     z = warp_sum(z);
     // From here on p holds the unnormalised weights e = exp(s - max) <= 1 and every mass is compared
     // with tau * z instead of dividing the row by z: the same ranking, the same ties and the same
     // cumulative-mass test up to rounding, at 1/3 fewer fp64 instructions per block.
-    const double tau_r = (flags & HEART_FORCE_DENSE) ? 1.0 : tau[r];
     // tau <= 0: every prefix reaches it, so the minimal one is the single largest block (lowest index
     // on ties): the smallest positive threshold gives exactly that
     const double t = (tau_r > 0.0 ? tau_r : 2.2250738585072014e-308) * z;
@@ -330,33 +452,18 @@ __global__ void __launch_bounds__(32 * kRowsPerCta) top_p_kernel(const double *_
       n_ties = nties;
     }
 
-    int base = 0, tie_seen = 0;
+    int tie_seen = 0;
     // the usual case: every block equal to theta is kept (theta = 0 when all blocks are kept)
     const bool all_ties_kept = keep_all || m_ties == n_ties;
-    // The mask words are gathered in registers (lane l keeps word l) and leave in one store.
-    uint32_t my_word = 0u;
-#pragma unroll 4
-    for (int j = 0; j < NJ; ++j) {
-      const int J = j * 32 + lane;
+    emit([&](int j, bool valid) {
       const long long b = __double_as_longlong(pw[(j) * 32]);
-      const bool valid = J < nb;
-      bool keep;
-      if (all_ties_kept) {
-        keep = valid && b >= theta;
-      } else {
-        const bool is_tie = valid && b == theta;
-        const unsigned tie_ballot = __ballot_sync(0xffffffffu, is_tie);
-        const int tie_rank = tie_seen + __popc(tie_ballot & lt_mask);
-        tie_seen += __popc(tie_ballot);
-        keep = valid && (b > theta || (is_tie && tie_rank < m_ties));
-      }
-      const unsigned word = __ballot_sync(0xffffffffu, keep);
-      if (lane == j) my_word = word;
-      if (keep) kv_idx[row * idx_stride + base + __popc(word & lt_mask)] = J;
-      base += __popc(word);
-    }
-    if (lane < W) mask_bits[row * W + lane] = my_word;
-    if (lane == 0) kv_cnt[row] = base;
+      if (all_ties_kept) return valid && b >= theta;
+      const bool is_tie = valid && b == theta;
+      const unsigned tie_ballot = __ballot_sync(0xffffffffu, is_tie);
+      const int tie_rank = tie_seen + __popc(tie_ballot & lt_mask);
+      tie_seen += __popc(tie_ballot);
+      return valid && (b > theta || (is_tie && tie_rank < m_ties));
+    });
   }
 }
 
