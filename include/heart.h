@@ -249,8 +249,8 @@ int heart_mask_iou(const heart_config *cfg, const uint32_t *mask_a, const uint32
  * y_sparse, y_dense: fp32 [C, T, H, W], contiguous, device.  weights: host, (w_LL, w_LH, w_HL, w_HH)
  * (the paper uses 1.0, 0.5, 0.01, 0.01 and eps = 1e-10).  out: device, fp64 [6] =
  * (e, E_LL, E_LH, E_HL, E_HH, denominator), energies of the unnormalised DFT, summed over channels.
- * workspace: heart_band_error_workspace_bytes(C, T, H, W) bytes of device scratch (four fp64 copies of
- * the tensor), 256-byte aligned; it need not be cleared. */
+ * workspace: heart_band_error_workspace_bytes(C, T, H, W) bytes of device scratch (two fp64 copies of
+ * the tensor and a little more), 256-byte aligned; it need not be cleared. */
 size_t heart_band_error_workspace_bytes(int32_t C, int32_t T, int32_t H, int32_t W);
 int heart_band_error(const float *y_sparse, const float *y_dense, int32_t C, int32_t T, int32_t H, int32_t W,
                      const double *weights /* host [4] */, double eps, double *out, void *workspace,

@@ -1,0 +1,23 @@
+"""The band error's axis passes at the edges: axes of length 1 and 2, lines that do not fill a CTA, axes with
+more folded samples than one shared-memory chunk holds (more than 318) or than the shared table (1024)."""
+import numpy as np
+import pytest
+import torch
+
+from parity import to_np
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("shape", [(1, 1, 1, 1), (1, 2, 1, 3), (3, 1, 7, 2), (2, 4, 1, 319), (1, 400, 3, 2), (1, 2, 1030, 4), (1, 21, 60, 104)])
+def test_band_error_axes(oracle, shape):
+    from paper_2605_14513_b200 import heart
+
+    g = torch.Generator("cuda").manual_seed(sum(shape))
+    yd = torch.randn(shape, device="cuda", generator=g)
+    ys = (yd + 0.1 * torch.randn(shape, device="cuda", generator=g)).contiguous()
+    out = to_np(heart.heart_band_error(ys, yd))
+    e, bands, denom = oracle.band_error(to_np(ys), to_np(yd))
+    # fp64 sums of at most n terms a pass: 1e-12 of the total covers n = 1030 with a wide margin
+    assert np.allclose(out[1:5], bands, rtol=1e-9, atol=1e-12 * bands.sum())
+    assert np.isclose(out[5], denom, rtol=1e-12) and np.isclose(out[0], e, rtol=1e-9)
