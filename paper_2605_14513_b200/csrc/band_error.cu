@@ -11,7 +11,7 @@
 // Each axis is a contraction with the fp64 matrix instruction.  Folding x_j +- x_{n-j} halves it: cosines see the
 // even part, sines the odd one.  x and y write their coefficients to the workspace (they stay in L2), t only
 // adds up energies.  For 16 x 21 x 60 x 104 that is 1.9e8 fma (10 us at 18.5 T fma/s) and 84 MB of L2 traffic in
-// three passes; the full circulant projections used before took 4.3e8 fma with two loads for each (0.45 ms).
+// three passes (58 us; 16 lines a warp and 8 CTAs an SM, against 64 us with 32 and 4); the full circulant projections used before took 4.3e8 fma with two loads for each (0.45 ms).
 #include <math.h>
 
 #include "common.cuh"
@@ -20,11 +20,34 @@ namespace heart {
 
 namespace {
 
-constexpr int kLines = 32;        // lines of an axis per CTA
-constexpr int kLinePitch = 36;    // 4 (mod 16) doubles: 8 x 4 fragments are read without bank conflicts
+constexpr int kLines = 16;        // lines of an axis per warp
 constexpr int kMaxChunk = 160;    // folded samples of a line in shared memory at a time
 constexpr int kMaxSharedTable = 1024;
-constexpr int kBandThreads = 128;
+constexpr int kBandThreads = 128, kBandWarps = kBandThreads / 32;
+
+// Warps of a CTA that share their lines and split the frequencies (8 at a time); the others take lines of
+// their own.
+__host__ __device__ inline int frequency_warps(int n) {
+  const int groups = (n / 2 + 1 + 7) / 8;
+  return groups <= 1 ? 1 : groups <= 2 ? 2 : kBandWarps;
+}
+__host__ __device__ inline int lines_per_cta(int n) { return kLines * (kBandWarps / frequency_warps(n)); }
+
+// Folded samples of a CTA's lines in shared memory, `rows` of them at a time (a multiple of 4): along the line
+// contiguous on the axis whose samples are (the copies then go along it), across the lines otherwise.  The
+// pitch is 4 or 12 (mod 16) doubles either way: 8 x 4 fragments are read without bank conflicts.
+struct FoldLayout {
+  int chunk, line_step, row_step, doubles;
+};
+__host__ __device__ inline FoldLayout fold_layout(int n, bool contiguous) {
+  FoldLayout f;
+  const int rows = (n / 2 + 1 + 3) / 4 * 4, lines = lines_per_cta(n);
+  f.chunk = rows < kMaxChunk ? rows : kMaxChunk;
+  f.line_step = contiguous ? f.chunk + (f.chunk % 8 == 0 ? 4 : 0) : 1;
+  f.row_step = contiguous ? 1 : lines + 4;
+  f.doubles = contiguous ? lines * f.line_step : f.chunk * f.row_step;
+  return f;
+}
 
 // tables[axis][m] = (cos, sin)(2 pi m / n) for the three axes, one after the other
 __global__ void trig_tables_kernel(int n0, int n1, int n2, double2 *__restrict__ tables) {
@@ -43,7 +66,7 @@ __device__ __forceinline__ void mma_f64(double (&d)[2], double a, double b) {
 
 // Sums over the CTA of kBandThreads threads, in a fixed order; valid in thread 0.
 template <int NV>
-__device__ __forceinline__ void cta_sums(double (&v)[NV], double *red /* [kBandThreads / 32 * NV] */) {
+__device__ __forceinline__ void cta_sums(double (&v)[NV], double *red /* [kBandWarps * NV] */) {
 #pragma unroll
   for (int q = 0; q < NV; ++q) {
 #pragma unroll
@@ -61,55 +84,70 @@ struct AxisArgs {
   const double2 *table;   // of this axis
   double *dst;            // passes 0, 1: coefficients, c_0 .. c_{n/2}, s_1 .. in place of the samples
   double *partial;        // pass 0: |y_dense|^2 per CTA; pass 2: [CTA][4] energies
-  long long lines, inner;
+  unsigned lines, inner;  // (their product with n is at most 2^31)
   int n;
   int ny, nx;             // pass 2: lengths of the other axes (inner = ny * nx)
 };
 
-// One pass over an axis of a [outer, n, inner] view; a CTA takes kLines of the outer * inner lines.
+// One pass over an axis of a [outer, n, inner] view; a CTA takes lines_per_cta(n) of the outer * inner lines.
 template <int PASS>
-__global__ void __launch_bounds__(kBandThreads) axis_kernel(const AxisArgs a) {
+__global__ void __launch_bounds__(kBandThreads, 8) axis_kernel(const AxisArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int n = a.n, h = n / 2, m = (n - 1) / 2;
-  const int rows = (h + 1 + 3) / 4 * 4, chunk = min(rows, kMaxChunk), n_chunks = (rows + chunk - 1) / chunk;
-  double *even = reinterpret_cast<double *>(smem_raw), *odd = even + chunk * kLinePitch;
-  double2 *tab = reinterpret_cast<double2 *>(odd + chunk * kLinePitch);
-  __shared__ double red[kBandThreads / 32 * 4];
-  __shared__ int line_band[kLines];      // pass 2: low along y and x | log2 of the weight << 1
+  const int fw = frequency_warps(n), lines = lines_per_cta(n);
+  const FoldLayout f = fold_layout(n, a.inner == 1);
+  const int chunk = f.chunk, n_chunks = (h + chunk) / chunk;
+  double *even = reinterpret_cast<double *>(smem_raw), *odd = even + f.doubles;
+  double2 *tab = reinterpret_cast<double2 *>(odd + f.doubles);
+  __shared__ double red[kBandWarps * 4];
+  __shared__ unsigned line_at[kLines * kBandWarps];  // offset of a line's first sample
+  __shared__ int line_band[kLines * kBandWarps];     // pass 2: low along y and x | log2 of the weight << 1
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const long long l0 = (long long)blockIdx.x * kLines;
-  const int n_lines = (int)min((long long)kLines, a.lines - l0);
+  const unsigned l0 = blockIdx.x * (unsigned)lines;
+  const int n_lines = (int)min((unsigned)lines, a.lines - l0);
   double dense = 0.0;
-  // folded samples [j0, j0 + chunk) of the lines
-  auto stage = [&](int j0) {
-    for (int e = tid; e < chunk * kLines; e += kBandThreads) {
-      const int jj = a.inner == 1 ? e % chunk : e / kLines, line = a.inner == 1 ? e / chunk : e % kLines;
-      const int j = j0 + jj;
-      double x = 0.0, y = 0.0;
-      if (line < n_lines && j <= h) {
-        const long long l = l0 + line, o = a.inner == 1 ? l : l / a.inner;
-        const long long at = o * n * a.inner + (l - o * a.inner) + (long long)j * a.inner;
-        const long long mirror = at + (long long)(n - 2 * j) * a.inner;
-        const bool pair = j >= 1 && j <= m;
-        if (PASS == 0) {
-          const double d = (double)a.yd[at];
-          x = (double)a.ys[at] - d;
-          dense = fma(d, d, dense);
-          if (pair) {
-            const double d2 = (double)a.yd[mirror];
-            y = (double)a.ys[mirror] - d2;
-            dense = fma(d2, d2, dense);
-          }
-        } else {
-          x = __ldcg(&a.src[at]);
-          if (pair) y = __ldcg(&a.src[mirror]);
-        }
-        even[jj * kLinePitch + line] = x + y;
-        odd[jj * kLinePitch + line] = pair ? x - y : 0.0;
+  for (int i = tid; i < n_lines; i += kBandThreads) {
+    const unsigned l = l0 + i, o = l / a.inner;
+    line_at[i] = o * n * a.inner + (l - o * a.inner);
+    if (PASS == 2) {
+      const int in = (int)(l - o * a.inner), iy = in / a.nx, ix = in % a.nx;
+      const int ky = iy <= a.ny / 2 ? iy : iy - a.ny / 2, kx = ix <= a.nx / 2 ? ix : ix - a.nx / 2;
+      const int wy = ky == 0 || 2 * ky == a.ny ? 0 : 1, wx = kx == 0 || 2 * kx == a.nx ? 0 : 1;
+      line_band[i] = (ky <= a.ny / 4 && kx <= a.nx / 4 ? 1 : 0) | (wy + wx) << 1;
+    }
+  }
+  __syncthreads();
+  // folded samples [j0, j0 + chunk) of the lines; consecutive threads take consecutive addresses
+  auto fold = [&](int line, int jj, int j) {
+    double x = 0.0, y = 0.0;
+    const bool pair = j >= 1 && j <= m;
+    if (line < n_lines && j <= h) {
+      const unsigned at = line_at[line] + j * a.inner, mirror = line_at[line] + (n - j) * a.inner;
+      if (PASS == 0) {
+        const float d = a.yd[at], v = a.ys[at];
+        float d2 = 0.f, v2 = 0.f;
+        if (pair) d2 = a.yd[mirror], v2 = a.ys[mirror];
+        x = (double)v - (double)d;
+        y = (double)v2 - (double)d2;
+        dense = fma((double)d, (double)d, fma((double)d2, (double)d2, dense));
       } else {
-        even[jj * kLinePitch + line] = 0.0;
-        odd[jj * kLinePitch + line] = 0.0;
+        x = __ldcg(&a.src[at]);
+        if (pair) y = __ldcg(&a.src[mirror]);
       }
+    }
+    even[jj * f.row_step + line * f.line_step] = x + y;
+    odd[jj * f.row_step + line * f.line_step] = pair ? x - y : 0.0;
+  };
+  auto stage = [&](int j0) {
+    if (a.inner == 1) {
+      // a warp per line, its lanes along the line
+      for (int jj = lane; jj < chunk; jj += 32)
+#pragma unroll 4
+        for (int line = warp; line < lines; line += kBandWarps) fold(line, jj, j0 + jj);
+    } else {
+      const int line = tid % lines;  // (lines divides the number of threads)
+#pragma unroll 4
+      for (int jj = tid / lines; jj < chunk; jj += kBandThreads / lines) fold(line, jj, j0 + jj);
     }
   };
   if (PASS == 0 && n_chunks == 1) stage(0);  // (the caller's tensors do not come from the kernel before)
@@ -121,17 +159,11 @@ __global__ void __launch_bounds__(kBandThreads) axis_kernel(const AxisArgs a) {
     for (int i = tid; i < n; i += kBandThreads) tab[i] = __ldcg(&a.table[i]);
     table = tab;
   }
-  if (PASS == 2 && tid < kLines) {
-    const int in = (int)((l0 + tid) % a.inner), iy = in / a.nx, ix = in % a.nx;
-    const int ky = iy <= a.ny / 2 ? iy : iy - a.ny / 2, kx = ix <= a.nx / 2 ? ix : ix - a.nx / 2;
-    const int wy = ky == 0 || 2 * ky == a.ny ? 0 : 1, wx = kx == 0 || 2 * kx == a.nx ? 0 : 1;
-    line_band[tid] = (ky <= a.ny / 4 && kx <= a.nx / 4 ? 1 : 0) | (wy + wx) << 1;
-  }
   __syncthreads();
   double energy[4] = {0.0, 0.0, 0.0, 0.0};  // LL, LH, HL, HH
-  const int jl = lane & 3, kl = lane >> 2;
-  for (int k0 = 0; k0 <= h; k0 += 8 * (kBandThreads / 32)) {  // warp w: frequencies k0 + 8 w ... + 7
-    const int k = k0 + 8 * warp + kl;
+  const int jl = lane & 3, kl = lane >> 2, line0 = warp / fw * kLines;
+  for (int kg = 0; kg <= h; kg += 8 * fw) {  // a warp: 8 frequencies of its 16 lines
+    const int k0 = kg + 8 * (warp % fw), k = k0 + kl;
     double c[kLines / 8][2], s[kLines / 8][2];
 #pragma unroll
     for (int i = 0; i < kLines / 8; ++i) c[i][0] = c[i][1] = s[i][0] = s[i][1] = 0.0;
@@ -143,35 +175,35 @@ __global__ void __launch_bounds__(kBandThreads) axis_kernel(const AxisArgs a) {
         __syncthreads();
         const double counted = dense;
         stage(ch * chunk);
-        if (k0 > 0) dense = counted;  // (|y_dense|^2: in the first round only)
+        if (kg > 0) dense = counted;  // (|y_dense|^2: in the first round only)
         __syncthreads();
       }
-      if (k0 + 8 * warp <= h) {
-        const double *E = even + jl * kLinePitch + kl, *O = odd + jl * kLinePitch + kl;
+      if (k0 <= h) {
+        const int at = jl * f.row_step + (line0 + kl) * f.line_step;
+        const double *E = even + at, *O = odd + at;
 #pragma unroll 2
-        for (int j = 0; j < chunk; j += 4, E += 4 * kLinePitch, O += 4 * kLinePitch) {
+        for (int j = 0; j < chunk; j += 4, E += 4 * f.row_step, O += 4 * f.row_step) {
           const double2 t = table[idx];
           idx += inc;
           idx -= idx >= n ? n : 0;
 #pragma unroll
           for (int i = 0; i < kLines / 8; ++i) {
-            mma_f64(c[i], E[8 * i], t.x);
-            mma_f64(s[i], O[8 * i], t.y);
+            mma_f64(c[i], E[8 * i * f.line_step], t.x);
+            mma_f64(s[i], O[8 * i * f.line_step], t.y);
           }
         }
       }
     }
-    if (k0 + 8 * warp > h) continue;
-    // lane: line 8 i + kl, frequencies k0 + 8 warp + 2 jl + {0, 1}
+    if (k0 > h) continue;
+    // lane: line line0 + 8 i + kl, frequencies k0 + 2 jl + {0, 1}
 #pragma unroll
     for (int i = 0; i < kLines / 8; ++i) {
-      const int line = 8 * i + kl;
+      const int line = line0 + 8 * i + kl;
       if (line >= n_lines) continue;
-      const long long l = l0 + line, o = a.inner == 1 ? l : l / a.inner;
-      double *out = PASS == 2 ? nullptr : a.dst + o * n * a.inner + (l - o * a.inner);
+      double *out = PASS == 2 ? nullptr : a.dst + line_at[line];
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
-        const int kk = k0 + 8 * warp + 2 * jl + u;
+        const int kk = k0 + 2 * jl + u;
         if (kk > h) continue;
         if (PASS == 2) {
           const int band = line_band[line];
@@ -181,15 +213,18 @@ __global__ void __launch_bounds__(kBandThreads) axis_kernel(const AxisArgs a) {
 #pragma unroll
           for (int b = 0; b < 4; ++b) energy[b] += b == q ? e : 0.0;
         } else {
-          out[(long long)kk * a.inner] = c[i][u];
-          if (kk >= 1 && kk <= m) out[(long long)(h + kk) * a.inner] = s[i][u];
+          out[kk * a.inner] = c[i][u];
+          if (kk >= 1 && kk <= m) out[(h + kk) * a.inner] = s[i][u];
         }
       }
     }
   }
   if (PASS == 2) {
     cta_sums<4>(energy, red);
-    if (tid < 4) a.partial[(size_t)blockIdx.x * 4 + tid] = energy[tid];
+    if (tid == 0) {
+#pragma unroll
+      for (int b = 0; b < 4; ++b) a.partial[(size_t)blockIdx.x * 4 + b] = energy[b];
+    }
   }
   if (PASS == 0) {
     double v[1] = {dense};
@@ -237,16 +272,15 @@ __global__ void __launch_bounds__(1024) band_final_kernel(const double *__restri
   }
 }
 
-size_t n_ctas(long long lines) { return (size_t)((lines + kLines - 1) / kLines); }
+size_t n_ctas(long long lines, int n) { return (size_t)((lines + lines_per_cta(n) - 1) / lines_per_cta(n)); }
 
 template <int PASS>
 cudaError_t launch_axis(const AxisArgs &a, cudaStream_t s) {
-  const int rows = (a.n / 2 + 1 + 3) / 4 * 4, chunk = rows < kMaxChunk ? rows : kMaxChunk;
-  const size_t smem = sizeof(double) * 2 * chunk * kLinePitch + (a.n <= kMaxSharedTable ? sizeof(double2) * a.n : 0);
-  cudaError_t e = cudaFuncSetAttribute(axis_kernel<PASS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)(sizeof(double) * 2 * kMaxChunk * kLinePitch + sizeof(double2) * kMaxSharedTable));
+  const size_t smem = sizeof(double) * 2 * fold_layout(a.n, a.inner == 1).doubles + (a.n <= kMaxSharedTable ? sizeof(double2) * a.n : 0);
+  constexpr int kMost = sizeof(double) * 2 * kMaxChunk * (kLines + 4) + sizeof(double2) * kMaxSharedTable;
+  cudaError_t e = cudaFuncSetAttribute(axis_kernel<PASS>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost);
   if (e != cudaSuccess) return e;
-  return launch_pdl(axis_kernel<PASS>, dim3((unsigned)n_ctas(a.lines)), dim3(kBandThreads), smem, s, a);
+  return launch_pdl(axis_kernel<PASS>, dim3((unsigned)n_ctas(a.lines, a.n)), dim3(kBandThreads), smem, s, a);
 }
 
 }  // namespace
@@ -254,7 +288,7 @@ cudaError_t launch_axis(const AxisArgs &a, cudaStream_t s) {
 size_t band_error_workspace_bytes(int C, int T, int H, int W) {
   const size_t n = (size_t)C * T * H * W;
   return align256(sizeof(double2) * ((size_t)T + H + W)) + 2 * align256(sizeof(double) * n) +
-         align256(sizeof(double) * 4 * n_ctas((long long)C * H * W)) + align256(sizeof(double) * n_ctas((long long)C * T * H));
+         align256(sizeof(double) * 4 * n_ctas((long long)C * H * W, T)) + align256(sizeof(double) * n_ctas((long long)C * T * H, W));
 }
 
 cudaError_t launch_band_error(const float *ys, const float *yd, int C, int T, int H, int W, const double *weights,
@@ -268,7 +302,7 @@ cudaError_t launch_band_error(const float *ys, const float *yd, int C, int T, in
   double *Bm = reinterpret_cast<double *>(p);
   p += align256(sizeof(double) * n);
   double *energies = reinterpret_cast<double *>(p);
-  p += align256(sizeof(double) * 4 * n_ctas((long long)C * H * W));
+  p += align256(sizeof(double) * 4 * n_ctas((long long)C * H * W, T));
   double *dense = reinterpret_cast<double *>(p);
   trig_tables_kernel<<<(unsigned)(((long long)T + H + W + 127) / 128), 128, 0, s>>>(W, H, T, tables);
   cudaError_t e = cudaGetLastError();
@@ -279,7 +313,7 @@ cudaError_t launch_band_error(const float *ys, const float *yd, int C, int T, in
   a.table = tables;
   a.dst = A;
   a.partial = dense;
-  a.lines = (long long)C * T * H;
+  a.lines = (unsigned)C * T * H;
   a.inner = 1;
   a.n = W;
   if ((e = launch_axis<0>(a, s)) != cudaSuccess) return e;
@@ -287,7 +321,7 @@ cudaError_t launch_band_error(const float *ys, const float *yd, int C, int T, in
   a.table = tables + W;
   a.dst = Bm;
   a.partial = nullptr;
-  a.lines = (long long)C * T * W;
+  a.lines = (unsigned)C * T * W;
   a.inner = W;
   a.n = H;
   if ((e = launch_axis<1>(a, s)) != cudaSuccess) return e;
@@ -295,14 +329,14 @@ cudaError_t launch_band_error(const float *ys, const float *yd, int C, int T, in
   a.table = tables + W + H;
   a.dst = nullptr;
   a.partial = energies;
-  a.lines = (long long)C * H * W;
-  a.inner = (long long)H * W;
+  a.lines = (unsigned)C * H * W;
+  a.inner = (unsigned)H * W;
   a.n = T;
   a.ny = H;
   a.nx = W;
   if ((e = launch_axis<2>(a, s)) != cudaSuccess) return e;
-  e = launch_pdl(band_final_kernel, dim3(1), dim3(1024), 0, s, (const double *)energies, (long long)n_ctas((long long)C * H * W),
-                 (const double *)dense, (long long)n_ctas((long long)C * T * H), (double)T * H * W, weights[0], weights[1],
+  e = launch_pdl(band_final_kernel, dim3(1), dim3(1024), 0, s, (const double *)energies, (long long)n_ctas((long long)C * H * W, T),
+                 (const double *)dense, (long long)n_ctas((long long)C * T * H, W), (double)T * H * W, weights[0], weights[1],
                  weights[2], weights[3], eps, out);
   *launches += 5;
   return e;
