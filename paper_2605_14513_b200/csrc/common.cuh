@@ -171,7 +171,7 @@ cudaError_t launch_attention(const Geom &g, const Workspace &w, const void *Q, c
                              cudaStream_t s, int *launches, int h0 = 0, int hcount = 0);
 
 cudaError_t launch_token_drift(const Geom &g, const void *Qa, const void *Ka, const void *Qb,
-                               const void *Kb, double *partial, double *drift_out, cudaStream_t s,
+                               const void *Kb, const Workspace &w, double *drift_out, cudaStream_t s,
                                int *launches);
 int token_drift_chunks(const Geom &g, int *rows_per_cta);
 cudaError_t launch_mask_iou(const Geom &g, const uint32_t *A, const uint32_t *B, double *iou,

@@ -39,11 +39,15 @@ constexpr int kRowsPerIter = 16;  // 256 threads = 16 rows x 16 chunks of 8 dims
 __global__ void __launch_bounds__(256) token_drift_partial_kernel(
     const uint16_t *__restrict__ Qa, const uint16_t *__restrict__ Ka, const uint16_t *__restrict__ Qb,
     const uint16_t *__restrict__ Kb, long long sb, long long sh, long long sn, int H, int N,
-    int rows_per_cta, double *__restrict__ partial) {
+    int rows_per_cta, double *__restrict__ partial, unsigned long long *__restrict__ sig_word) {
   const int chunk = blockIdx.x, r = blockIdx.y;
   const int c = threadIdx.x & 15, g = threadIdx.x >> 4;
   const long long head = (long long)(r / H) * sb + (long long)(r % H) * sh + c * 8;
   const int i0 = chunk * rows_per_cta, i1 = min(N, i0 + rows_per_cta);
+  pdl_wait();
+  pdl_launch_dependents();  // (the grid is one wave: the next kernel's CTAs wait where these leave)
+  // the partials overwrite the block means: the workspace no longer holds any
+  if (chunk == 0 && r == 0 && threadIdx.x == 0) *sig_word = 0;
   double acc = 0.0;
   for (int row = i0 + g; row < i1; row += 2 * kRowsPerIter) {
     const long long o0 = head + (long long)row * sn;
@@ -71,6 +75,8 @@ __global__ void __launch_bounds__(256) token_drift_final_kernel(const double *__
                                                                 int nchunks, int N,
                                                                 double *__restrict__ drift) {
   const int r = blockIdx.x;
+  pdl_wait();
+  pdl_launch_dependents();
   double s = 0.0;
   for (int i = threadIdx.x; i < nchunks; i += 256) s += partial[(size_t)r * nchunks + i];
   __shared__ double red[256];
@@ -83,37 +89,52 @@ __global__ void __launch_bounds__(256) token_drift_final_kernel(const double *__
   if (threadIdx.x == 0) drift[r] = red[0] / (double)N;
 }
 
-// One CTA per head row: popcounts of A&B and A|B over the nb*W mask words of the head.
-__global__ void __launch_bounds__(256) mask_iou_kernel(const uint32_t *__restrict__ A,
-                                                       const uint32_t *__restrict__ B, int words,
-                                                       double *__restrict__ iou,
-                                                       long long *__restrict__ counts) {
+// One CTA per head row: popcounts of A&B and A|B over the nb*W mask words of the head, four words at a time
+// where the rows allow it.  Latency bound (64 KB per CTA on the largest 64-token shape): 1024 threads with all
+// their loads in flight take 5 us there, 256 with one word each took 11.
+constexpr int kIouThreads = 1024;
+
+__global__ void __launch_bounds__(kIouThreads) mask_iou_kernel(const uint32_t *__restrict__ A,
+                                                               const uint32_t *__restrict__ B, int words,
+                                                               double *__restrict__ iou,
+                                                               long long *__restrict__ counts) {
   const int r = blockIdx.x;
+  pdl_wait();
+  pdl_launch_dependents();
   const uint32_t *a = A + (size_t)r * words, *b = B + (size_t)r * words;
-  unsigned long long inter = 0, uni = 0;
-  for (int i = threadIdx.x; i < words; i += 256) {
-    const uint32_t x = a[i], y = b[i];
+  unsigned inter = 0, uni = 0;  // (at most 2^20 pairs per head)
+  auto add = [&](uint32_t x, uint32_t y) {
     inter += __popc(x & y);
     uni += __popc(x | y);
+  };
+  const bool vec = ((reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(b)) & 15u) == 0;
+  const int quads = vec ? words / 4 : 0;
+#pragma unroll 4
+  for (int i = threadIdx.x; i < quads; i += kIouThreads) {
+    const uint4 x = reinterpret_cast<const uint4 *>(a)[i], y = reinterpret_cast<const uint4 *>(b)[i];
+    add(x.x, y.x);
+    add(x.y, y.y);
+    add(x.z, y.z);
+    add(x.w, y.w);
   }
-  __shared__ unsigned long long s_inter, s_uni;
-  if (threadIdx.x == 0) s_inter = s_uni = 0;
-  __syncthreads();
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    inter += __shfl_xor_sync(0xffffffffu, inter, o);
-    uni += __shfl_xor_sync(0xffffffffu, uni, o);
-  }
+  for (int i = 4 * quads + threadIdx.x; i < words; i += kIouThreads) add(a[i], b[i]);
+  __shared__ unsigned s_inter[kIouThreads / 32], s_uni[kIouThreads / 32];
+  inter = __reduce_add_sync(0xffffffffu, inter);
+  uni = __reduce_add_sync(0xffffffffu, uni);
   if ((threadIdx.x & 31) == 0) {
-    atomicAdd(&s_inter, inter);
-    atomicAdd(&s_uni, uni);
+    s_inter[threadIdx.x >> 5] = inter;
+    s_uni[threadIdx.x >> 5] = uni;
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    iou[r] = s_uni ? (double)s_inter / (double)s_uni : 1.0;
-    if (counts) {
-      counts[2 * r] = (long long)s_inter;
-      counts[2 * r + 1] = (long long)s_uni;
+  if (threadIdx.x < 32) {
+    inter = __reduce_add_sync(0xffffffffu, s_inter[threadIdx.x]);
+    uni = __reduce_add_sync(0xffffffffu, s_uni[threadIdx.x]);
+    if (threadIdx.x == 0) {
+      iou[r] = uni ? (double)inter / (double)uni : 1.0;
+      if (counts) {
+        counts[2 * r] = (long long)inter;
+        counts[2 * r + 1] = (long long)uni;
+      }
     }
   }
 }
@@ -130,27 +151,25 @@ int token_drift_chunks(const Geom &g, int *rows_per_cta) {
 }
 
 cudaError_t launch_token_drift(const Geom &g, const void *Qa, const void *Ka, const void *Qb,
-                               const void *Kb, double *partial, double *drift_out, cudaStream_t s,
+                               const void *Kb, const Workspace &w, double *drift_out, cudaStream_t s,
                                int *launches) {
   int rows = 0;
   const int nchunks = token_drift_chunks(g, &rows);
-  token_drift_partial_kernel<<<dim3(nchunks, g.R), 256, 0, s>>>(
-      static_cast<const uint16_t *>(Qa), static_cast<const uint16_t *>(Ka),
-      static_cast<const uint16_t *>(Qb), static_cast<const uint16_t *>(Kb), g.sb, g.sh, g.sn, g.H, g.N,
-      rows, partial);
-  cudaError_t e = cudaGetLastError();
+  double *partial = w.bmean;
+  cudaError_t e = launch_pdl(token_drift_partial_kernel, dim3(nchunks, g.R), dim3(256), 0, s, static_cast<const uint16_t *>(Qa),
+                             static_cast<const uint16_t *>(Ka), static_cast<const uint16_t *>(Qb),
+                             static_cast<const uint16_t *>(Kb), g.sb, g.sh, g.sn, g.H, g.N, rows, partial,
+                             reinterpret_cast<unsigned long long *>(w.status + kStatusSigWord));
   if (e != cudaSuccess) return e;
   ++*launches;
-  token_drift_final_kernel<<<g.R, 256, 0, s>>>(partial, nchunks, g.N, drift_out);
-  e = cudaGetLastError();
+  e = launch_pdl(token_drift_final_kernel, dim3(g.R), dim3(256), 0, s, (const double *)partial, nchunks, g.N, drift_out);
   if (e == cudaSuccess) ++*launches;
   return e;
 }
 
 cudaError_t launch_mask_iou(const Geom &g, const uint32_t *A, const uint32_t *B, double *iou,
                             long long *counts, cudaStream_t s, int *launches) {
-  mask_iou_kernel<<<g.R, 256, 0, s>>>(A, B, g.nb * g.W, iou, counts);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = launch_pdl(mask_iou_kernel, dim3(g.R), dim3(kIouThreads), 0, s, A, B, g.nb * g.W, iou, counts);
   if (e == cudaSuccess) ++*launches;
   return e;
 }

@@ -348,10 +348,7 @@ int heart_full_token_drift(const heart_config *cfg, const void *Qa, const void *
   const size_t need = (size_t)g.R * token_drift_chunks(g, &rows);  // partials live in the block-sum area
   if (need > 2 * (size_t)g.R * g.nb * kD) return HEART_ERR_INVALID;
   g_launches = 0;
-  // the partials overwrite the block means: the workspace no longer holds any
-  cudaError_t e = cudaMemsetAsync(w.status + kStatusSigWord, 0, 8, static_cast<cudaStream_t>(stream));
-  if (e != cudaSuccess) return cuda_fail(e, "token_drift");
-  e = launch_token_drift(g, Qa, Ka, Qb, Kb, w.bmean, drift_out, static_cast<cudaStream_t>(stream), &g_launches);
+  cudaError_t e = launch_token_drift(g, Qa, Ka, Qb, Kb, w, drift_out, static_cast<cudaStream_t>(stream), &g_launches);
   if (e != cudaSuccess) return cuda_fail(e, "token_drift");
   return HEART_OK;
 }
