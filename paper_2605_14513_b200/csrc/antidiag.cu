@@ -328,11 +328,13 @@ cudaError_t launch_antidiag_scores(const Geom &g, const Workspace &w, const void
     dim3 grid(row_tiles, g.R, split);
     cudaError_t e;
     if (grp == 4) {
-      e = cudaFuncSetAttribute(antidiag_scores_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+      static std::atomic<unsigned long long> done{0};
+      e = allow_shared_memory(antidiag_scores_kernel<4>, smem, done);
       if (e != cudaSuccess) return e;
       antidiag_scores_kernel<4><<<grid, kThreadsAd, smem, s>>>(mq, mk, prm);
     } else {
-      e = cudaFuncSetAttribute(antidiag_scores_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+      static std::atomic<unsigned long long> done{0};
+      e = allow_shared_memory(antidiag_scores_kernel<8>, smem, done);
       if (e != cudaSuccess) return e;
       antidiag_scores_kernel<8><<<grid, kThreadsAd, smem, s>>>(mq, mk, prm);
     }

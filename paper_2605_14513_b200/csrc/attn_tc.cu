@@ -805,7 +805,8 @@ cudaError_t launch_bk(const Geom &g, const Workspace &w, const CUtensorMap &mq, 
     ++*launches;
     prm.tiles = reinterpret_cast<const uint32_t *>(w.order);
   }
-  e = cudaFuncSetAttribute(attn_tc_kernel<B>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttnSmem);
+  static std::atomic<unsigned long long> done{0};
+  e = allow_shared_memory(attn_tc_kernel<B>, kAttnSmem, done);
   if (e != cudaSuccess) return e;
   ++*launches;
   return launch_pdl(attn_tc_kernel<B>, dim3(prm.n_tiles < kSms ? prm.n_tiles : kSms), dim3(kAttnThreads), kAttnSmem, s, mq, mk,

@@ -3,6 +3,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "heart.h"
 
 namespace heart {
@@ -123,6 +125,20 @@ __device__ __forceinline__ double exp_nonpositive(double x) {
   q = fma(q, r, 1.0);
   q = fma(q, r, 1.0);
   return __hiloint2double(__double2hiint(q) + (n << 20), __double2loint(q));
+}
+
+// Lets a kernel use `bytes` of dynamic shared memory; asked of the runtime once per kernel and device (`done` is
+// the call site's own, one bit per device).
+template <typename K>
+cudaError_t allow_shared_memory(K *kernel, int bytes, std::atomic<unsigned long long> &done) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const unsigned long long bit = dev < 64 ? 1ull << dev : 0ull;
+  if (done.load(std::memory_order_acquire) & bit) return cudaSuccess;
+  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_release);
+  return e;
 }
 
 template <typename... KArgs, typename... Args>

@@ -472,7 +472,8 @@ static cudaError_t launch_nj(const Geom &g, const Workspace &w, const double *ta
                              heart_state st, int pitch, cudaStream_t s, unsigned long long expect_sig) {
   dim3 grid((g.nb + kRowsPerCta - 1) / kRowsPerCta, g.R);
   const size_t smem = sizeof(double) * kRowsPerCta * NJ * 32;
-  cudaError_t e = cudaFuncSetAttribute(top_p_kernel<NJ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  static std::atomic<unsigned long long> done{0};
+  cudaError_t e = allow_shared_memory(top_p_kernel<NJ>, (int)smem, done);
   if (e != cudaSuccess) return e;
   return launch_pdl(top_p_kernel<NJ>, grid, dim3(32 * kRowsPerCta), smem, s, (const double *)w.scores, g.nb, pitch, tau,
                     refresh, g.flags, st.mask_bits, st.kv_idx, st.kv_cnt, g.idx_stride, g.W, (const int32_t *)w.status,
@@ -483,7 +484,8 @@ template <int WT, int TD, int STAGES>
 static cudaError_t launch_scores(const Geom &g, const Workspace &w, const uint8_t *refresh, cudaStream_t s,
                                  unsigned long long expect_sig) {
   constexpr int smem = ScoreTile<WT, TD, STAGES>::kBytes;
-  cudaError_t e = cudaFuncSetAttribute(pooled_scores_kernel<WT, TD, STAGES>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  static std::atomic<unsigned long long> done{0};
+  cudaError_t e = allow_shared_memory(pooled_scores_kernel<WT, TD, STAGES>, smem, done);
   if (e != cudaSuccess) return e;
   const unsigned t = (g.nb + 2 * WT - 1) / (2 * WT);
   return launch_pdl(pooled_scores_kernel<WT, TD, STAGES>, dim3(t, t, g.R), dim3(128), (size_t)smem, s, (const double *)w.bmean,

@@ -118,45 +118,52 @@ struct DecideArgs {
   int *ticket;  // zero between launches (used only when the layer gate is on)
 };
 
-// Layer gate over the H heads of batch entry b and the anchor update of its refreshed heads.  One
-// CTA, any block size.  The head-wise decisions, the drifts and the means were written by other CTAs
-// of the same launch: read them past L1.
-__device__ void gate_batch_entry(int b, int R, const double *mean, const DecideArgs &a,
-                                 uint8_t *sh_flags /* [2*H] */, int *cnt /* shared */) {
-  const int H = a.H;
-  if (threadIdx.x == 0) *cnt = 0;
-  __syncthreads();
-  for (int h = threadIdx.x; h < H; h += blockDim.x) {
-    const int r = b * H + h;
-    const bool rf = __ldcg(&a.pre_ws[r]) != 0;
-    sh_flags[h] = rf;
-    sh_flags[H + h] = a.has_anchor[r] != 0;
-    if (rf) atomicAdd(cnt, 1);
-  }
-  __syncthreads();
-  const double f = (double)*cnt / (double)H;
-  for (int h = threadIdx.x; h < H; h += blockDim.x) {
-    bool rf = sh_flags[h];
-    if (f < a.gate_lo) {
-      if (sh_flags[H + h]) rf = false;
-    } else if (f > a.gate_hi) {
-      rf = true;
+// Batch entries whose heads the layer gate takes together, and the shared memory that needs.
+__host__ __device__ inline int gate_group(int B, int H) { return max(1, min(B, 4096 / H)); }
+__host__ inline size_t gate_shared_bytes(int B, int H) { return (size_t)gate_group(B, H) * (sizeof(int) + 2 * (size_t)H); }
+
+// Layer gate of the batch entries and the anchor update of their refreshed heads.  One CTA, any block size.  The
+// head-wise decisions and the means were written by other CTAs of the same launch: read them past L1.
+// A chain of trips to L2: the rows of many batch entries go through each of them together.
+__device__ void apply_gate(int R, const double *mean, const DecideArgs &a, int *shared) {
+  const int H = a.H, group = gate_group(a.B, H);
+  int *cnt = shared;                                            // [group] heads that want to refresh
+  uint8_t *flags = reinterpret_cast<uint8_t *>(shared + group);  // [group * H] decision, [group * H] had an anchor
+  for (int b0 = 0; b0 < a.B; b0 += group) {
+    const int nb = min(group, a.B - b0), r0 = b0 * H, n = nb * H;
+    for (int b = threadIdx.x; b < nb; b += blockDim.x) cnt[b] = 0;
+    __syncthreads();
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+      const bool rf = __ldcg(&a.pre_ws[r0 + i]) != 0;
+      flags[i] = rf;
+      flags[n + i] = a.has_anchor[r0 + i] != 0;
+      if (rf) atomicAdd(&cnt[i / H], 1);
     }
-    sh_flags[h] = rf;
-    const int r = b * H + h;
-    a.refresh_ws[r] = rf;
-    if (a.refresh_out) a.refresh_out[r] = rf;
-    if (rf) a.has_anchor[r] = 1;
-  }
-  __syncthreads();
-  for (int e = threadIdx.x; e < H * kD; e += blockDim.x) {
-    const int h = e / kD, r = b * H + h;
-    if (sh_flags[h]) {
-      a.anchor_q[(size_t)r * kD + (e % kD)] = __ldcg(&mean[(size_t)r * kD + (e % kD)]);
-      a.anchor_k[(size_t)r * kD + (e % kD)] = __ldcg(&mean[((size_t)R + r) * kD + (e % kD)]);
+    __syncthreads();
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+      const double f = (double)cnt[i / H] / (double)H;
+      bool rf = flags[i];
+      if (f < a.gate_lo) {
+        if (flags[n + i]) rf = false;
+      } else if (f > a.gate_hi) {
+        rf = true;
+      }
+      flags[i] = rf;
+      a.refresh_ws[r0 + i] = rf;
+      if (a.refresh_out) a.refresh_out[r0 + i] = rf;
+      if (rf) a.has_anchor[r0 + i] = 1;
     }
+    __syncthreads();
+#pragma unroll 4
+    for (int e = threadIdx.x; e < n * kD; e += blockDim.x) {
+      if (flags[e / kD]) {
+        const size_t at = (size_t)r0 * kD + e;
+        a.anchor_q[at] = __ldcg(&mean[at]);
+        a.anchor_k[at] = __ldcg(&mean[(size_t)R * kD + at]);
+      }
+    }
+    __syncthreads();
   }
-  __syncthreads();
 }
 
 // One CTA per head row r, 1024 threads = 2 tensors x 4 ranges of partial sums x 128 dims.
@@ -168,10 +175,10 @@ __device__ void gate_batch_entry(int b, int R, const double *mean, const DecideA
 __global__ void __launch_bounds__(1024) mean_drift_kernel(const double *__restrict__ psum, int R, int N,
                                                           int nchunks, double *__restrict__ mean,
                                                           const DecideArgs a) {
-  extern __shared__ uint8_t sh_flags[];  // [2*H]: decision, had_anchor (gate path)
+  extern __shared__ int sh_gate[];  // gate path
   __shared__ double sm[2][4][kD];
   __shared__ double wsum[8];
-  __shared__ int last, cnt, sh_rf;
+  __shared__ int last, sh_rf;
   const int r = blockIdx.x;
   const int z = threadIdx.x >> 9, grp = (threadIdx.x >> 7) & 3, d = threadIdx.x & (kD - 1);
   const int per = (nchunks + 3) / 4;
@@ -229,7 +236,7 @@ __global__ void __launch_bounds__(1024) mean_drift_kernel(const double *__restri
   if (!last) return;
   // Every other CTA has read its old anchor and published its means and head-wise decision.
   __threadfence();
-  for (int b = 0; b < a.B; ++b) gate_batch_entry(b, R, mean, a, sh_flags, &cnt);
+  apply_gate(R, mean, a, sh_gate);
   if (threadIdx.x == 0) *a.ticket = 0;
 }
 
@@ -283,7 +290,8 @@ cudaError_t launch_decide(const Geom &g, const Workspace &w, const double *delta
   a.refresh_out = refresh_out;
   a.ticket = w.status + kStatusTicketWord;
   ++*launches;
-  return launch_pdl(mean_drift_kernel, dim3(g.R), dim3(1024), (size_t)2 * g.H, s, (const double *)w.psum, g.R, g.N,
+  const bool gate_on = g.gate_lo > 0.0 || g.gate_hi < 1.0;
+  return launch_pdl(mean_drift_kernel, dim3(g.R), dim3(1024), gate_on ? gate_shared_bytes(g.B, g.H) : 0, s, (const double *)w.psum, g.R, g.N,
                     g.nchunks, w.mean, a);
 }
 
