@@ -33,10 +33,10 @@
 // Tensor memory: O (128 columns) | S[2] (2 x 128) | P[2] (2 x 64).
 //
 // The step lists come from attn_plan_kernel (one warp per tile), which runs just before; the tiles are
-// taken head-major (the K/V of one or two heads stay in L2), within a head in the order of
-// tile_order_kernel: by the first key block of their lists once a head's K and V no longer fit one die's
-// half of the L2, except for the last two heads of the launch, whose tiles go longest-list-first so that
-// the launch does not end on a long tile that started late.
+// taken in the order of tile_order_kernel: head-major (the K/V of one or two heads stay in L2), within a
+// head by the first key block of their lists once a head's K and V no longer fit one die's half of the L2,
+// except for the last two heads of the launch, whose tiles go longest-list-first so that the launch does not
+// end on a long tile that started late.  Small launches go longest-list-first altogether.
 //
 // Every wait is bounded; a wait that runs out raises the CTA's abort flag and the status word, its roles
 // drain and stop, the other CTAs take the remaining tiles.
@@ -73,7 +73,7 @@ struct AttnShared {
   uint64_t o_free;         // O of a tile has been read
   uint64_t tile_full[kTileRing], tile_empty[kTileRing];
   uint64_t drain[2];       // abort path: the issuers' products in flight have landed
-  int4 tile[kTileRing];    // query tile of its head, listed key blocks, head of the launch, 1 (0: no tile left)
+  int4 tile[kTileRing];    // query tile of its head, listed key blocks, head, batch entry (-1: no tile left)
   float m[2][128];         // references after step g
   float2 l[2][128];        // row sum and its reference of the warpgroup without the last step, per tile & 1
   uint32_t tmem_base;
@@ -86,7 +86,7 @@ constexpr int kAttnSmem = kOffBar + sizeof(AttnShared);
 // flag: the keys do not count (the second half of the last step when the number of blocks is odd).
 struct AttnParams {
   const uint32_t *steps;  // [B*H][tiles of a head][step_pitch]
-  const uint32_t *tiles;  // [tiles of the launch] tile of the head | listed key blocks << 16, in launch order
+  const uint2 *tiles;     // [tiles of the launch] (tile of the head | listed key blocks << 16, head of the launch), in launch order
   int32_t *counter;       // tiles drawn beyond the first one of every CTA (zeroed by the plan kernel)
   uint16_t *O;
   float *lse;
@@ -182,9 +182,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
   const uint32_t tmem = sh.tmem_base;
 
   auto n_steps_of = [](int U) -> int { return B == 128 ? U : (U + 1) / 2; };
-  auto steps_of = [&](int rr, int tile) -> const uint32_t * {
-    const int r = rr / p.hcount * p.H + p.h0 + rr % p.hcount;
-    return p.steps + ((size_t)r * p.n_tiles_per_head + tile) * p.step_pitch;
+  auto steps_of = [&](const int4 &ti) -> const uint32_t * {
+    return p.steps + ((size_t)(ti.w * p.H + ti.z) * p.n_tiles_per_head + ti.x) * p.step_pitch;
   };
   auto step_entry = [&](const uint32_t *steps, int h) -> uint32_t {
     if (!p.dense) return __ldcg(&steps[h]);
@@ -207,7 +206,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     ti = sh.tile[i];
     __syncwarp();
     if (lane == 0) mbar_arrive(&sh.tile_empty[i]);
-    return ti.w != 0;
+    return ti.w >= 0;
   };
   // K or V of one key step into a 32 KB buffer
   auto load_step = [&](unsigned char *dst, const CUtensorMap *map, uint64_t *bar, uint32_t e, int hidx, int bidx) {
@@ -249,49 +248,53 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
   if (warp >= kWarpQK) setmaxnreg_dec<kRegsHelper>();
   if (warp == kWarpK) {
     if (lane == 0) {  // ===== K and Q producer
-      int t = 0, g = 0, nq = 0;  // tiles announced, key steps loaded, tiles with key steps
-      int n = blockIdx.x;        // the first tile of every CTA is fixed, the others are drawn
-      uint32_t word = 0, e = 0;  // tile n of the launch and its first key step, fetched ahead of time
-      auto fetch = [&]() {
+      int g = 0, nq = 0;     // key steps loaded, tiles with key steps
+      int4 nx;               // the tile that is announced next and its first key step, fetched ahead of time
+      uint32_t e = 0;
+      auto fetch = [&](int n) {
+        nx.w = -1;
         if (n >= p.n_tiles) return;
-        const int rr = n / p.n_tiles_per_head;
-        word = p.dense ? (uint32_t)(n - rr * p.n_tiles_per_head) | (uint32_t)p.nb << 16 : __ldcg(&p.tiles[n]);
-        if (word >> 16) e = step_entry(steps_of(rr, word & 0xffff), 0);
+        uint2 t;
+        if (p.dense) {
+          t.y = n / p.n_tiles_per_head;
+          t.x = (n - t.y * p.n_tiles_per_head) | (uint32_t)p.nb << 16;
+        } else {
+          t = __ldcg(&p.tiles[n]);
+        }
+        nx.x = t.x & 0xffff;
+        nx.y = t.x >> 16;
+        nx.w = (int)t.y / p.hcount;
+        nx.z = p.h0 + (int)t.y - nx.w * p.hcount;
+        if (nx.y > 0) e = step_entry(steps_of(nx), 0);
       };
-      fetch();
-      for (; ok; ++t) {
+      fetch(blockIdx.x);  // the first tile of every CTA is fixed, the others are drawn
+      for (int t = 0;; ++t) {
         const int i = t % kTileRing;
         if (t >= kTileRing) ok = mbar_wait(&sh.tile_empty[i], (t / kTileRing - 1) & 1, abort);
         if (!ok) break;
-        const bool none = n >= p.n_tiles;
-        const int rr = none ? 0 : n / p.n_tiles_per_head, tile = word & 0xffff, U = word >> 16;  // U = listed key blocks
-        sh.tile[i] = none ? make_int4(0, 0, 0, 0) : make_int4(tile, U, rr, 1);
+        const int4 ti = nx;
+        sh.tile[i] = ti;
         mbar_arrive(&sh.tile_full[i]);
-        if (none) break;
-        const int n_steps = n_steps_of(U), bidx = rr / p.hcount, hidx = p.h0 + rr % p.hcount;
-        const uint32_t *steps = steps_of(rr, tile);
+        if (ti.w < 0) break;
+        const int n_steps = n_steps_of(ti.y);
+        const uint32_t *steps = steps_of(ti);
         uint32_t e_now = e;
         for (int h = 0; h < n_steps; ++h, ++g) {
           const uint32_t e_next = h + 1 < n_steps ? step_entry(steps, h + 1) : 0u;
           if (g >= 2) ok = mbar_wait(&sh.s_full[g & 1], ((g - 2) >> 1) & 1, abort);
           if (!ok) break;
-          load_step(smem + kOffK + (g & 1) * kTileBytes, &map_k, &sh.k_full[g & 1], e_now, hidx, bidx);
+          load_step(smem + kOffK + (g & 1) * kTileBytes, &map_k, &sh.k_full[g & 1], e_now, ti.z, ti.w);
           if (h == 0) {
             // its buffer is free: the last step of the tile before the previous one is complete
             mbar_expect_tx(&sh.q_full[nq & 1], kTileBytes);
-            tma_load_5d(smem + kOffQ + (nq & 1) * kTileBytes, &map_q, &sh.q_full[nq & 1], 0, tile * 128, 0, hidx, bidx);
+            tma_load_5d(smem + kOffQ + (nq & 1) * kTileBytes, &map_q, &sh.q_full[nq & 1], 0, ti.x * 128, 0, ti.z, ti.w);
             ++nq;
+            fetch(gridDim.x + atomicAdd(p.counter, 1));
           }
           e_now = e_next;
-          if (h == 0) {
-            n = gridDim.x + atomicAdd(p.counter, 1);
-            fetch();
-          }
         }
-        if (U == 0) {
-          n = gridDim.x + atomicAdd(p.counter, 1);
-          fetch();
-        }
+        if (!ok) break;
+        if (n_steps == 0) fetch(gridDim.x + atomicAdd(p.counter, 1));
       }
       if (*abort) {
         settle_pair(sh.q_full, nq);
@@ -303,8 +306,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     int g = 0;
     int4 ti;
     for (int t = 0; ok && next_tile(t, ti); ++t) {
-      const int n_steps = n_steps_of(ti.y), bidx = ti.z / p.hcount, hidx = p.h0 + ti.z % p.hcount;
-      const uint32_t *steps = steps_of(ti.z, ti.x);
+      const int n_steps = n_steps_of(ti.y);
+      const uint32_t *steps = steps_of(ti);
       uint32_t e_next = n_steps > 0 ? step_entry(steps, 0) : 0u;
       for (int h = 0; h < n_steps; ++h, ++g) {
         const uint32_t e = e_next;
@@ -315,7 +318,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
         // waits that depend on it run out and the abort path is taken.
         if (p.test_skip_v && blockIdx.x == 0 && g == 1) continue;
 #endif
-        if (lane == 0) load_step(smem + kOffV + (g & 1) * kTileBytes, &map_v, &sh.v_full[g & 1], e, hidx, bidx);
+        if (lane == 0) load_step(smem + kOffV + (g & 1) * kTileBytes, &map_v, &sh.v_full[g & 1], e, ti.z, ti.w);
       }
     }
     if (*abort && lane == 0) settle_pair(sh.v_full, g);
@@ -399,8 +402,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     int4 ti;
     for (int t = 0; ok && next_tile(t, ti); ++t) {
       const int n_steps = n_steps_of(ti.y);
-      const int bidx = ti.z / p.hcount, hidx = p.h0 + ti.z % p.hcount;
-      const uint32_t *steps = steps_of(ti.z, ti.x);
+      const uint32_t *steps = steps_of(ti);
       float m_ref = kNoReference, l_run = 0.f;  // (rows without a key keep the reference)
       const uint32_t h0 = (w ^ g0) & 1;         // this warpgroup's first step of the tile
       uint32_t e_next = (int)h0 < n_steps ? step_entry(steps, h0) : 0u;
@@ -554,7 +556,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
       // steps: by the one whose turn it is)
       const uint32_t g_last = g0 + n_steps - 1;
       if (n_steps > 0 ? (g_last & 1) == w : (t & 1) == (int)w) {
-        const int r = bidx * p.H + hidx, tok = ti.x * 128 + row;
+        const int tok = ti.x * 128 + row;
         const bool valid_row = tok < p.N;
         if (n_steps > 0 && !wait(&sh.pv_done[w], (g_last >> 1) & 1)) break;
         tc_fence_after();
@@ -563,7 +565,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
           l_run += other.x * ex2(other.y - m_ref);
         }
         const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
-        uint16_t *orow = p.O + (long long)bidx * p.sb + (long long)hidx * p.sh + (long long)tok * p.sn;
+        uint16_t *orow = p.O + (long long)ti.w * p.sb + (long long)ti.z * p.sh + (long long)tok * p.sn;
 #pragma unroll 1
         for (int ch = 0; ch < 4; ++ch) {  // 32 output dims at a time
           uint32_t v[32];
@@ -588,7 +590,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
         }
         if (n_steps > 0) arrive(&sh.o_free);
         if (valid_row && p.lse != nullptr)
-          p.lse[(size_t)r * p.N + tok] = l_run > 0.f ? (m_ref + log2f(l_run)) * 0.6931471805599453f : -INFINITY;
+          p.lse[(size_t)(ti.w * p.H + ti.z) * p.N + tok] = l_run > 0.f ? (m_ref + log2f(l_run)) * 0.6931471805599453f : -INFINITY;
       }
       g0 += n_steps;
       nt += n_steps > 0 ? 1 : 0;
@@ -616,7 +618,7 @@ template <int B>
 __global__ void __launch_bounds__(32 * kPlanWarps)
     attn_plan_kernel(const int32_t *__restrict__ kv_idx, const int32_t *__restrict__ kv_cnt, int nb, int ncph, int idx_stride,
                      int H, int h0, int hcount, int n_tiles, int step_pitch, int ragged, uint32_t *__restrict__ steps,
-                     uint32_t *__restrict__ tiles, uint32_t *__restrict__ firsts, int32_t *__restrict__ counter,
+                     uint2 *__restrict__ tiles, uint32_t *__restrict__ firsts, int32_t *__restrict__ counter,
                      int32_t *__restrict__ status) {
   constexpr int QBT = 128 / B;  // query blocks per tile
   __shared__ uint32_t sets[kPlanWarps][QBT][32];
@@ -710,47 +712,48 @@ __global__ void __launch_bounds__(32 * kPlanWarps)
   const int src = has ? __ffs(has) - 1 : 0;
   const int first = __shfl_sync(0xffffffffu, lane * 32 + __ffs(any) - 1, src);
   if (lane == 0) {
-    tiles[n] = (uint32_t)t | (uint32_t)U << 16;
+    tiles[n] = make_uint2((uint32_t)t | (uint32_t)U << 16, rr);
     firsts[n] = has ? first : 0x3ff;
   }
 }
 
-// Order of the tiles of every head of a launch: rank by counting over at most 1024 distinct keys, 256
-// tiles per CTA.  Heads before the last two: index order while a head's K and V fit the L2 comfortably;
-// beyond that ascending by the first key block that the tile's lists name (ties by tile index) -- tiles
-// that read the same region of K and V run together.  The last two heads: descending by the number of
-// listed key blocks.
-__global__ void __launch_bounds__(256) tile_order_kernel(const uint32_t *__restrict__ tiles, const uint32_t *__restrict__ firsts,
-                                                         int ncph, int n_heads, int by_first_key, uint32_t *__restrict__ order) {
+// Order of the tiles of a launch: every group of `per_group` tiles (a head's, or all of a small launch) is
+// ranked by counting over at most 1024 distinct keys, 256 tiles per CTA.  Groups before the last
+// `n_by_length`: index order while a head's K and V fit the L2 comfortably; beyond that ascending by the
+// first key block that the tile's lists name (ties by tile index) -- tiles that read the same region of K and
+// V run together.  The last ones: descending by the number of listed key blocks.
+__global__ void __launch_bounds__(256) tile_order_kernel(const uint2 *__restrict__ tiles, const uint32_t *__restrict__ firsts,
+                                                         int per_group, int n_by_length, int by_first_key,
+                                                         uint2 *__restrict__ order) {
   __shared__ __align__(16) uint32_t key[1024];
-  const int rr = blockIdx.y, t = blockIdx.x * 256 + threadIdx.x;
+  const int group = blockIdx.y, t = blockIdx.x * 256 + threadIdx.x;
   pdl_wait();
   pdl_launch_dependents();
-  const bool by_length = rr >= n_heads - 2;
-  const size_t base = (size_t)rr * ncph;
+  const bool by_length = group >= (int)gridDim.y - n_by_length;
+  const size_t base = (size_t)group * per_group;
   if (!by_length && !by_first_key) {
-    if (t < ncph) order[base + t] = __ldcg(&tiles[base + t]);
+    if (t < per_group) order[base + t] = __ldcg(&tiles[base + t]);
     return;
   }
-  uint32_t my_word = 0u;
+  uint2 my_word = make_uint2(0u, 0u);
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     const int u = threadIdx.x + k * 256;
     uint32_t v = 0xffffffffu;
-    if (u < ncph) {
-      const uint32_t w = __ldcg(&tiles[base + u]);
+    if (u < per_group) {
+      const uint2 w = __ldcg(&tiles[base + u]);
       if (u == t) my_word = w;
-      v = (by_length ? 0xffffu - (w >> 16) : __ldcg(&firsts[base + u])) << 10 | (uint32_t)u;
+      v = (by_length ? 0xffffu - (w.x >> 16) : __ldcg(&firsts[base + u])) << 10 | (uint32_t)u;
     }
     key[u] = v;
   }
   __syncthreads();
-  if (t >= ncph) return;
+  if (t >= per_group) return;
   const uint32_t mine = key[t];
   int rank = 0;
   const uint4 *k4 = reinterpret_cast<const uint4 *>(key);
 #pragma unroll 4
-  for (int u = 0; u < (ncph + 3) / 4; ++u) {
+  for (int u = 0; u < (per_group + 3) / 4; ++u) {
     const uint4 w = k4[u];
     rank += (w.x < mine ? 1 : 0) + (w.y < mine ? 1 : 0) + (w.z < mine ? 1 : 0) + (w.w < mine ? 1 : 0);
   }
@@ -782,11 +785,13 @@ cudaError_t launch_bk(const Geom &g, const Workspace &w, const CUtensorMap &mq, 
   cudaError_t e;
   const int n_heads = g.B * prm.hcount;
   prm.n_tiles = n_heads * prm.n_tiles_per_head;
-  // the plan lives where the pooled scores of the mask predictor were: [R][tiles][steps], then two words per tile
-  uint32_t *steps = reinterpret_cast<uint32_t *>(w.scores);
+  // the plan lives where the pooled scores of the mask predictor were: (word, head) per tile in plan order and in
+  // launch order, [R][tiles][steps], the first key block per tile
+  const size_t all_tiles = (size_t)g.R * prm.n_tiles_per_head;
+  uint2 *tiles = reinterpret_cast<uint2 *>(w.scores), *order = tiles + all_tiles;
+  uint32_t *steps = reinterpret_cast<uint32_t *>(order + all_tiles);
   prm.step_pitch = B == 128 ? g.nb : (g.nb + 1) / 2;
-  uint32_t *tiles = steps + (size_t)g.R * prm.n_tiles_per_head * prm.step_pitch;
-  uint32_t *firsts = tiles + (size_t)g.R * prm.n_tiles_per_head;
+  uint32_t *firsts = steps + all_tiles * prm.step_pitch;
   prm.steps = steps;
   prm.tiles = tiles;
   const int planned = prm.dense ? 0 : prm.n_tiles;  // (dense: the kernel only zeroes the counter)
@@ -796,14 +801,16 @@ cudaError_t launch_bk(const Geom &g, const Workspace &w, const CUtensorMap &mq, 
   if (e != cudaSuccess) return e;
   ++*launches;
   if (planned > kSms) {  // up to there every tile starts at once: no order to choose
+    // Up to 1024 tiles (7 rounds of the SMs): longest first over all heads.  Their K and V stay in L2 anyway.
+    const bool small = planned <= 1024;
+    const int per_group = small ? planned : prm.n_tiles_per_head, groups = small ? 1 : n_heads;
     // K + V of one head beyond 32 MB (about half of one die's share of the L2): order by key locality
     const int by_first_key = (size_t)g.N * kD * 2 * 2 > (size_t)(32u << 20) ? 1 : 0;
-    e = launch_pdl(tile_order_kernel, dim3((prm.n_tiles_per_head + 255) / 256, n_heads), dim3(256), 0, s,
-                   (const uint32_t *)tiles, (const uint32_t *)firsts, prm.n_tiles_per_head, n_heads, by_first_key,
-                   reinterpret_cast<uint32_t *>(w.order));
+    e = launch_pdl(tile_order_kernel, dim3((per_group + 255) / 256, groups), dim3(256), 0, s, (const uint2 *)tiles,
+                   (const uint32_t *)firsts, per_group, small ? 1 : 2, by_first_key, order);
     if (e != cudaSuccess) return e;
     ++*launches;
-    prm.tiles = reinterpret_cast<const uint32_t *>(w.order);
+    prm.tiles = order;
   }
   static std::atomic<unsigned long long> done{0};
   e = allow_shared_memory(attn_tc_kernel<B>, kAttnSmem, done);

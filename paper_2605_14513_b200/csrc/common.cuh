@@ -47,9 +47,9 @@ struct Workspace {
   uint8_t *pre;       // [R]            head-wise decision before the gate
   uint8_t *refresh;   // [R]            final decision of the current step
   double *drift;      // [R]
-  int32_t *order;     // [R * ceil(N / 128)] order in which an attention launch takes the tiles of each head
   double *scores;     // [R][nb][pitch] pooled scores of the refreshed heads, pitch = nb rounded up to 32;
-                      //        afterwards the step lists of the attention launch (at most half of the area)
+                      //        afterwards the plan of the attention launch (2 words + 2 words + steps + 1 word per tile:
+                      //        at most 4 n_b + 20 bytes per query block, against 8 pitch)
   void *pairs;        // strided antidiagonal estimator only (HEART_ESTIMATOR_ANTIDIAG in the flags):
                       // float2 [R][N/16][nb], a (max, sum) pair per (query group, key block)
   size_t bytes_drift;  // what heart_drift alone touches (everything above `scores`)
@@ -76,8 +76,6 @@ __host__ inline Workspace carve(const Geom &g, void *base) {
   off += align256((size_t)g.R);
   w.drift = reinterpret_cast<double *>(p + off);
   off += align256(sizeof(double) * (size_t)g.R);
-  w.order = reinterpret_cast<int32_t *>(p + off);
-  off += align256(sizeof(int32_t) * (size_t)g.R * (size_t)((g.N + 127) / 128));
   w.bytes_drift = off;
   w.scores = reinterpret_cast<double *>(p + off);
   off += align256(sizeof(double) * (size_t)g.R * g.nb * (size_t)(((g.nb + 31) / 32) * 32));
