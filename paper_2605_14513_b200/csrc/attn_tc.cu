@@ -26,7 +26,7 @@
 //   warp 8      issues S_g = Q K_g^T once step g - 2 has emptied the buffer, warp 11 O += P_g V_g.
 //   warp 9      V producer, warp 10 K and Q producer (draws the tiles and announces them): TMA loads
 //               (cp.async.bulk.tensor, 128-byte swizzle, completion on mbarriers), two 32 KB buffers each.
-// The reference: m_g = m_{g-1} unless the row's maximum of step g exceeds it by more than 2^32.  Each warp
+// The reference: m_g = m_{g-1} unless the row's maximum of step g exceeds it by more than 2^64.  Each warp
 // publishes the references of its 32 rows after the maximum of every step and reads those of the step
 // before; a row whose reference moved gets its part of O rescaled by the warp that moved it, once the
 // products of the steps before are complete, and both partners rescale their own row sums.
@@ -56,12 +56,13 @@ constexpr int kTileRing = 4;       // announced tiles
 constexpr int kTileReaders = 11;   // softmax warps, issuers, V producer
 constexpr float kNoReference = -3.0e38f;  // below every logit: the first step moves it
 // A row's reference moves when its maximum exceeds it by this much (log2).  Weights, sums and O are floating
-// point with 8 exponent bits throughout, so a scale of up to 2^32 costs no precision and leaves 2^95 of
-// range; a move costs a rescale of O behind the products in flight.
-constexpr float kMaxGrowth = 32.f;
+// point with 8 exponent bits throughout, so a scale of up to 2^64 costs no precision, and 2^17 such weights
+// leave room for values up to 2^46.  A move costs a rescale of O behind the products in flight.
+constexpr float kMaxGrowth = 64.f;
 
 // Shared-memory plan (the dynamic allocation itself is 1024-byte aligned).
-constexpr int kOffQ = 0, kOffK = 2 * kTileBytes, kOffV = 4 * kTileBytes, kOffBar = 6 * kTileBytes;
+constexpr int kOutBytes = 2048;  // per softmax warp: 32 rows x 32 dims of the output
+constexpr int kOffQ = 0, kOffK = 2 * kTileBytes, kOffV = 4 * kTileBytes, kOffOut = 6 * kTileBytes, kOffBar = kOffOut + 8 * kOutBytes;
 
 struct AttnShared {
   uint64_t q_full[2], k_full[2], v_full[2];  // TMA -> issuer
@@ -86,7 +87,8 @@ constexpr int kAttnSmem = kOffBar + sizeof(AttnShared);
 // flag: the keys do not count (the second half of the last step when the number of blocks is odd).
 struct AttnParams {
   const uint32_t *steps;  // [B*H][tiles of a head][step_pitch]
-  const uint2 *tiles;     // [tiles of the launch] (tile of the head | listed key blocks << 16, head of the launch), in launch order
+  const uint4 *tiles;     // [tiles of the launch] (tile of the head | listed key blocks << 16, head of the launch,
+                          // first step, first key block), in launch order
   int32_t *counter;       // tiles drawn beyond the first one of every CTA (zeroed by the plan kernel)
   uint16_t *O;
   float *lse;
@@ -254,18 +256,19 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
       auto fetch = [&](int n) {
         nx.w = -1;
         if (n >= p.n_tiles) return;
-        uint2 t;
+        uint4 t;
         if (p.dense) {
           t.y = n / p.n_tiles_per_head;
           t.x = (n - t.y * p.n_tiles_per_head) | (uint32_t)p.nb << 16;
+          t.z = step_entry(nullptr, 0);
         } else {
           t = __ldcg(&p.tiles[n]);
         }
+        e = t.z;
         nx.x = t.x & 0xffff;
         nx.y = t.x >> 16;
         nx.w = (int)t.y / p.hcount;
         nx.z = p.h0 + (int)t.y - nx.w * p.hcount;
-        if (nx.y > 0) e = step_entry(steps_of(nx), 0);
       };
       fetch(blockIdx.x);  // the first tile of every CTA is fixed, the others are drawn
       for (int t = 0;; ++t) {
@@ -565,30 +568,45 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
           l_run += other.x * ex2(other.y - m_ref);
         }
         const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
-        uint16_t *orow = p.O + (long long)ti.w * p.sb + (long long)ti.z * p.sh + (long long)tok * p.sn;
-#pragma unroll 1
-        for (int ch = 0; ch < 4; ++ch) {  // 32 output dims at a time
-          uint32_t v[32];
-          if (n_steps > 0) {
-            tmem_ld32(o_addr + ch * 32, v);
-            tmem_wait_ld();
-          }
-          if (valid_row) {
+        uint32_t v[128];
+        if (n_steps > 0) {
 #pragma unroll
-            for (int g4 = 0; g4 < 4; ++g4) {
-              float o[8];
+          for (int ch = 0; ch < 4; ++ch) tmem_ld32(o_addr + ch * 32, *reinterpret_cast<uint32_t(*)[32]>(&v[ch * 32]));
+          tmem_wait_ld();
+          arrive(&sh.o_free);
+        } else {
 #pragma unroll
-              for (int i = 0; i < 8; ++i) o[i] = n_steps > 0 ? __uint_as_float(v[g4 * 8 + i]) * inv : 0.f;
-              uint4 x;
-              x.x = pack_bf16x2(o[0], o[1]);
-              x.y = pack_bf16x2(o[2], o[3]);
-              x.z = pack_bf16x2(o[4], o[5]);
-              x.w = pack_bf16x2(o[6], o[7]);
-              *reinterpret_cast<uint4 *>(orow + ch * 32 + g4 * 8) = x;
-            }
-          }
+          for (int i = 0; i < 128; ++i) v[i] = 0u;
         }
-        if (n_steps > 0) arrive(&sh.o_free);
+        // A row per thread would touch 32 lines with every store (2700-5000 clocks for a tile, during which the
+        // partner runs out of work): 32 dims at a time go through shared memory, so that four lanes write 64
+        // bytes of a row.
+        unsigned char *out = smem + kOffOut + warp * kOutBytes;
+        uint16_t *tile_out = p.O + (long long)ti.w * p.sb + (long long)ti.z * p.sh + (long long)(ti.x * 128 + quarter * 32) * p.sn;
+        const int rows = p.N - (ti.x * 128 + (int)quarter * 32);  // of this warp that exist
+#pragma unroll
+        for (int ch = 0; ch < 4; ++ch) {
+#pragma unroll
+          for (int g4 = 0; g4 < 4; ++g4) {
+            float o[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) o[i] = __uint_as_float(v[ch * 32 + g4 * 8 + i]) * inv;
+            uint4 x;
+            x.x = pack_bf16x2(o[0], o[1]);
+            x.y = pack_bf16x2(o[2], o[3]);
+            x.z = pack_bf16x2(o[4], o[5]);
+            x.w = pack_bf16x2(o[6], o[7]);
+            *reinterpret_cast<uint4 *>(out + lane * 64 + ((g4 ^ (lane >> 1)) & 3) * 16) = x;
+          }
+          __syncwarp();
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const int rr = i * 8 + (lane >> 2), g4 = lane & 3;
+            const uint4 x = *reinterpret_cast<const uint4 *>(out + rr * 64 + ((g4 ^ (rr >> 1)) & 3) * 16);
+            if (rr < rows) *reinterpret_cast<uint4 *>(tile_out + (long long)rr * p.sn + ch * 32 + g4 * 8) = x;
+          }
+          __syncwarp();
+        }
         if (valid_row && p.lse != nullptr)
           p.lse[(size_t)(ti.w * p.H + ti.z) * p.N + tok] = l_run > 0.f ? (m_ref + log2f(l_run)) * 0.6931471805599453f : -INFINITY;
       }
@@ -618,7 +636,7 @@ template <int B>
 __global__ void __launch_bounds__(32 * kPlanWarps)
     attn_plan_kernel(const int32_t *__restrict__ kv_idx, const int32_t *__restrict__ kv_cnt, int nb, int ncph, int idx_stride,
                      int H, int h0, int hcount, int n_tiles, int step_pitch, int ragged, uint32_t *__restrict__ steps,
-                     uint2 *__restrict__ tiles, uint32_t *__restrict__ firsts, int32_t *__restrict__ counter,
+                     uint4 *__restrict__ tiles, int32_t *__restrict__ counter,
                      int32_t *__restrict__ status) {
   constexpr int QBT = 128 / B;  // query blocks per tile
   __shared__ uint32_t sets[kPlanWarps][QBT][32];
@@ -711,10 +729,8 @@ __global__ void __launch_bounds__(32 * kPlanWarps)
   const unsigned has = __ballot_sync(0xffffffffu, any != 0u);
   const int src = has ? __ffs(has) - 1 : 0;
   const int first = __shfl_sync(0xffffffffu, lane * 32 + __ffs(any) - 1, src);
-  if (lane == 0) {
-    tiles[n] = make_uint2((uint32_t)t | (uint32_t)U << 16, rr);
-    firsts[n] = has ? first : 0x3ff;
-  }
+  __syncwarp();  // the first step, written by some lane, is read back
+  if (lane == 0) tiles[n] = make_uint4((uint32_t)t | (uint32_t)U << 16, rr, has ? *(volatile uint32_t *)out : 0u, has ? first : 0x3ff);
 }
 
 // Order of the tiles of a launch: every group of `per_group` tiles (a head's, or all of a small launch) is
@@ -722,9 +738,8 @@ __global__ void __launch_bounds__(32 * kPlanWarps)
 // `n_by_length`: index order while a head's K and V fit the L2 comfortably; beyond that ascending by the
 // first key block that the tile's lists name (ties by tile index) -- tiles that read the same region of K and
 // V run together.  The last ones: descending by the number of listed key blocks.
-__global__ void __launch_bounds__(256) tile_order_kernel(const uint2 *__restrict__ tiles, const uint32_t *__restrict__ firsts,
-                                                         int per_group, int n_by_length, int by_first_key,
-                                                         uint2 *__restrict__ order) {
+__global__ void __launch_bounds__(256) tile_order_kernel(const uint4 *__restrict__ tiles, int per_group,
+                                                         int n_by_length, int by_first_key, uint4 *__restrict__ order) {
   __shared__ __align__(16) uint32_t key[1024];
   const int group = blockIdx.y, t = blockIdx.x * 256 + threadIdx.x;
   pdl_wait();
@@ -735,15 +750,15 @@ __global__ void __launch_bounds__(256) tile_order_kernel(const uint2 *__restrict
     if (t < per_group) order[base + t] = __ldcg(&tiles[base + t]);
     return;
   }
-  uint2 my_word = make_uint2(0u, 0u);
+  uint4 my_word = make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     const int u = threadIdx.x + k * 256;
     uint32_t v = 0xffffffffu;
     if (u < per_group) {
-      const uint2 w = __ldcg(&tiles[base + u]);
+      const uint4 w = __ldcg(&tiles[base + u]);
       if (u == t) my_word = w;
-      v = (by_length ? 0xffffu - (w.x >> 16) : __ldcg(&firsts[base + u])) << 10 | (uint32_t)u;
+      v = (by_length ? 0xffffu - (w.x >> 16) : w.w) << 10 | (uint32_t)u;
     }
     key[u] = v;
   }
@@ -785,19 +800,18 @@ cudaError_t launch_bk(const Geom &g, const Workspace &w, const CUtensorMap &mq, 
   cudaError_t e;
   const int n_heads = g.B * prm.hcount;
   prm.n_tiles = n_heads * prm.n_tiles_per_head;
-  // the plan lives where the pooled scores of the mask predictor were: (word, head) per tile in plan order and in
-  // launch order, [R][tiles][steps], the first key block per tile
+  // the plan lives where the pooled scores of the mask predictor were: four words per tile in plan order and in
+  // launch order, [R][tiles][steps]
   const size_t all_tiles = (size_t)g.R * prm.n_tiles_per_head;
-  uint2 *tiles = reinterpret_cast<uint2 *>(w.scores), *order = tiles + all_tiles;
+  uint4 *tiles = reinterpret_cast<uint4 *>(w.scores), *order = tiles + all_tiles;
   uint32_t *steps = reinterpret_cast<uint32_t *>(order + all_tiles);
   prm.step_pitch = B == 128 ? g.nb : (g.nb + 1) / 2;
-  uint32_t *firsts = steps + all_tiles * prm.step_pitch;
   prm.steps = steps;
   prm.tiles = tiles;
   const int planned = prm.dense ? 0 : prm.n_tiles;  // (dense: the kernel only zeroes the counter)
   e = launch_pdl(attn_plan_kernel<B>, dim3(planned ? (planned + kPlanWarps - 1) / kPlanWarps : 1), dim3(32 * kPlanWarps), 0, s,
                  kv_idx, kv_cnt, g.nb, prm.n_tiles_per_head, g.idx_stride, g.H, prm.h0, prm.hcount, planned, prm.step_pitch,
-                 (int)(g.N % g.block != 0), steps, tiles, firsts, prm.counter, prm.status);
+                 (int)(g.N % g.block != 0), steps, tiles, prm.counter, prm.status);
   if (e != cudaSuccess) return e;
   ++*launches;
   if (planned > kSms) {  // up to there every tile starts at once: no order to choose
@@ -806,8 +820,7 @@ cudaError_t launch_bk(const Geom &g, const Workspace &w, const CUtensorMap &mq, 
     const int per_group = small ? planned : prm.n_tiles_per_head, groups = small ? 1 : n_heads;
     // K + V of one head beyond 32 MB (about half of one die's share of the L2): order by key locality
     const int by_first_key = (size_t)g.N * kD * 2 * 2 > (size_t)(32u << 20) ? 1 : 0;
-    e = launch_pdl(tile_order_kernel, dim3((per_group + 255) / 256, groups), dim3(256), 0, s, (const uint2 *)tiles,
-                   (const uint32_t *)firsts, per_group, small ? 1 : 2, by_first_key, order);
+    e = launch_pdl(tile_order_kernel, dim3((per_group + 255) / 256, groups), dim3(256), 0, s, (const uint4 *)tiles, per_group, small ? 1 : 2, by_first_key, order);
     if (e != cudaSuccess) return e;
     ++*launches;
     prm.tiles = order;

@@ -48,8 +48,8 @@ struct Workspace {
   uint8_t *refresh;   // [R]            final decision of the current step
   double *drift;      // [R]
   double *scores;     // [R][nb][pitch] pooled scores of the refreshed heads, pitch = nb rounded up to 32;
-                      //        afterwards the plan of the attention launch (2 words + 2 words + steps + 1 word per tile:
-                      //        at most 4 n_b + 20 bytes per query block, against 8 pitch)
+                      //        afterwards the plan of the attention launch (two times four words and the steps per tile: at
+                      //        most 4 n_b + 32 bytes per query block, against 8 pitch >= 256)
   void *pairs;        // strided antidiagonal estimator only (HEART_ESTIMATOR_ANTIDIAG in the flags):
                       // float2 [R][N/16][nb], a (max, sum) pair per (query group, key block)
   size_t bytes_drift;  // what heart_drift alone touches (everything above `scores`)
