@@ -75,6 +75,8 @@ struct AttnShared {
   uint64_t tile_full[kTileRing], tile_empty[kTileRing];
   uint64_t drain[2];       // abort path: the issuers' products in flight have landed
   int4 tile[kTileRing];    // query tile of its head, listed key blocks, head, batch entry (-1: no tile left)
+  uint32_t entry[4];       // the key steps in flight, for the softmax warps: entry[g & 3] is written before K_g is asked
+                           // for and read before the scores of step g are handed back, which K_{g+4} waits for
   float m[2][128];         // references after step g
   float2 l[2][128];        // row sum and its reference of the warpgroup without the last step, per tile & 1
   uint32_t tmem_base;
@@ -286,6 +288,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
           const uint32_t e_next = h + 1 < n_steps ? step_entry(steps, h + 1) : 0u;
           if (g >= 2) ok = mbar_wait(&sh.s_full[g & 1], ((g - 2) >> 1) & 1, abort);
           if (!ok) break;
+          sh.entry[g & 3] = e_now;
           load_step(smem + kOffK + (g & 1) * kTileBytes, &map_k, &sh.k_full[g & 1], e_now, ti.z, ti.w);
           if (h == 0) {
             // its buffer is free: the last step of the tile before the previous one is complete
@@ -405,18 +408,15 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     int4 ti;
     for (int t = 0; ok && next_tile(t, ti); ++t) {
       const int n_steps = n_steps_of(ti.y);
-      const uint32_t *steps = steps_of(ti);
       float m_ref = kNoReference, l_run = 0.f;  // (rows without a key keep the reference)
       const uint32_t h0 = (w ^ g0) & 1;         // this warpgroup's first step of the tile
-      uint32_t e_next = (int)h0 < n_steps ? step_entry(steps, h0) : 0u;
       for (int h = h0; h < n_steps; h += 2) {
         const uint32_t g = g0 + h;
-        const uint32_t e = e_next;
-        if (h + 2 < n_steps) e_next = step_entry(steps, h + 2);
+        wait(&sh.s_full[w], (g >> 1) & 1);
+        const uint32_t e = sh.entry[g & 3];
         // which halves of the step this row's query block lists, whether the step holds the ragged last block
         const uint32_t flags = (e >> (10 + (quarter >> 1))) & 0x10001u;  // (64-token blocks)
         const bool ragged = B == 128 ? (int)(e + 1) * 128 > p.N : (e & 0x10001000u) != 0u;
-        wait(&sh.s_full[w], (g >> 1) & 1);
         if (g > 0) wait(&sh.m_ready[w ^ 1][quarter], ((g - 1) >> 1) & 1);  // (half a step old by now, as a rule)
         tc_fence_after();
         const float m_prev = h > 0 ? sh.m[w ^ 1][row] : kNoReference;
@@ -462,28 +462,56 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
           if (g >= 2) wait(&sh.pv_done[w], ((g - 2) >> 1) & 1);
           tc_fence_after();
         };
-        if (__builtin_expect((B == 128 || flags == 0x10001u) && !ragged, 1)) {
-          // The exponentials of the first 32 keys are taken with the reference as it
-          // was while the row maximum is found, and once more in the rare step that moves it.
+        if (__builtin_expect(ragged, 0)) {
+          // Keys that do not count get a score of -inf in tensor memory, where a loop over columns is a loop;
+          // the step is then like any other.  (As 128 selects between the loads and the weights it slowed all
+          // steps by 7 %; a branch of its own, 32 columns at a time, took 5000-9000 clocks instead of 2600.)
+          int n0, n1;  // keys of each half that count
+          if (B == 128) {
+            n0 = p.N - (int)e * 128;
+            n1 = n0 - 64;
+          } else {
+            n0 = (flags & 1u) ? p.N - (int)(e & 0x3ff) * 64 : 0;
+            n1 = (flags >> 16) ? p.N - (int)((e >> 16) & 0x3ff) * 64 : 0;
+          }
+#pragma unroll 1
+          for (int col = 0; col < 128; col += 8) {
+            const int n = (col < 64 ? n0 : n1 + 64) - col;  // columns of these eight that count
+            if (n <= 0) {
+              tmem_st8_fill(s_addr + col, 0xff800000u);
+            } else {
+#pragma unroll 1
+              for (int i = n; i < 8; ++i) tmem_st1(s_addr + col + i, 0xff800000u);
+            }
+          }
+          tmem_wait_st();
+        }
+        if (__builtin_expect(B == 128 || flags == 0x10001u || ragged, 1)) {
+          // The exponentials of the first 32 keys are taken with the reference as it was while the row maximum is
+          // found, and once more, by the same instructions, in the rare step that moves it (a tile's first ones:
+          // a copy of its own for them cost 2 % of the clocks of a tile with 10-20 steps, from cold instructions).
           uint32_t s[128], pk[32];
 #pragma unroll
           for (int q = 0; q < 4; ++q) tmem_ld32(s_addr + q * 32, *reinterpret_cast<uint32_t(*)[32]>(&s[q * 32]));
           tmem_wait_ld();
           arrive(&sh.s_free[w]);
-          uint64_t neg_m2 = pack_f32x2(-m_ref, -m_ref);
-          exp32(&s[0], c2, neg_m2, &pk[0], sums);
-          if (__builtin_expect(new_reference(fmaxf(max64(&s[0]), max64(&s[64])) * c), 0)) {
+          uint64_t neg_m2;
+          bool again = false;
+#pragma unroll 1
+          do {
             neg_m2 = pack_f32x2(-m_ref, -m_ref);
             sums = {0.f, 0.f, 0.f, 0.f};
             exp32(&s[0], c2, neg_m2, &pk[0], sums);
-          }
+            const float x_max = fmaxf(max64(&s[0]), max64(&s[64])) * c;
+            again = !again && new_reference(x_max);
+          } while (__builtin_expect(again, 0));
           exp32(&s[32], c2, neg_m2, &pk[16], sums);
           p_free();
           tmem_st32(p_addr, pk);
           exp32(&s[64], c2, neg_m2, &pk[0], sums);
           exp32(&s[96], c2, neg_m2, &pk[16], sums);
           tmem_st32(p_addr + 32, pk);
-        } else if (B == 64 && flags != 0u && !ragged) {
+        } else if (flags != 0u) {
           // This row's query block lists one of the step's two blocks.  The product reads all 128 keys of
           // the step: zeros for the other one.
           const uint32_t v = flags >> 16;
@@ -501,7 +529,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
           exp32(&s[0], c2, neg_m2, &pk[0], sums);
           exp32(&s[32], c2, neg_m2, &pk[16], sums);
           tmem_st32(p_addr + v * 32, pk);
-        } else if (B == 64 && flags == 0u) {
+        } else {
           // none of the step's blocks is listed by this row's query block
           uint32_t pk[32];
 #pragma unroll
@@ -511,42 +539,6 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
           p_free();
           tmem_st32(p_addr, pk);
           tmem_st32(p_addr + 32, pk);
-        } else {
-          // The ragged last block: 32 columns at a time, the scores read twice.  (Masking it in the first
-          // branch cost all steps 7 % of their clocks: 128 selects between the loads and the weights.)
-          int n0, n1;  // keys of each half that count
-          if (B == 128) {
-            n0 = p.N - (int)e * 128;
-            n1 = n0 - 64;
-          } else {
-            n0 = (flags & 1u) ? p.N - (int)(e & 0x3ff) * 64 : 0;
-            n1 = (flags >> 16) ? p.N - (int)((e >> 16) & 0x3ff) * 64 : 0;
-          }
-          float x_max = -INFINITY;
-#pragma unroll 1
-          for (int pass = 0; pass < 8; ++pass) {
-            const int q = pass & 3, n = (q & 2 ? n1 : n0) - (q & 1) * 32;
-            uint32_t s[32], pk[16];
-            tmem_ld32(s_addr + q * 32, s);
-            tmem_wait_ld();
-            float mx = -INFINITY;
-#pragma unroll
-            for (int i = 0; i < 32; ++i) {
-              if (i >= n) s[i] = 0xff800000u;  // -inf: ignored by the max, 2^-inf = 0
-              mx = fmaxf(mx, __uint_as_float(s[i]));
-            }
-            if (pass < 4) {
-              x_max = fmaxf(x_max, mx * c);
-              if (pass == 3) {
-                new_reference(x_max);
-                p_free();
-              }
-            } else {
-              exp32(s, c2, pack_f32x2(-m_ref, -m_ref), pk, sums);
-              tmem_st16(p_addr + q * 16, pk);
-            }
-          }
-          arrive(&sh.s_free[w]);
         }
         l_run += (sums.a + sums.b) + (sums.c + sums.d);
         if (h == n_steps - 2) sh.l[nt & 1][row] = make_float2(l_run, m_ref);  // the partner finishes the tile
