@@ -36,7 +36,8 @@
 // taken in the order of tile_order_kernel: head-major (the K/V of one or two heads stay in L2), within a
 // head by the first key block of their lists once a head's K and V no longer fit one die's half of the L2,
 // except for the last two heads of the launch, whose tiles go longest-list-first so that the launch does not
-// end on a long tile that started late.  Small launches go longest-list-first altogether.
+// end on a long tile that started late.  Launches of at most 1024 tiles go longest-list-first altogether
+// (tile_order_small_kernel).
 //
 // Every wait is bounded; a wait that runs out raises the CTA's abort flag and the status word, its roles
 // drain and stop, the other CTAs take the remaining tiles.
@@ -644,25 +645,35 @@ __global__ void __launch_bounds__(32 * kPlanWarps)
   for (int q = 0; q < QBT; ++q) sets[warp][q][lane] = 0u;
   __syncwarp();
   bool bad = false;
+  // The counts and the first 64 entries of the lists are asked for together (entries beyond the count are not
+  // looked at): one trip to memory for a short list instead of one for each query block's count and list.
+  int cnt[QBT], head[QBT][2];
 #pragma unroll
   for (int q = 0; q < QBT; ++q) {
-    const int I = t * QBT + q;
-    if (I >= nb) break;
-    const size_t row = (size_t)r * nb + I;
-    int cnt = __ldcg(&kv_cnt[row]);
-    if (cnt < 0 || cnt > idx_stride) {
+    const size_t row = (size_t)r * nb + t * QBT + q;
+    const bool real = t * QBT + q < nb;
+    cnt[q] = real ? __ldcg(&kv_cnt[row]) : 0;
+#pragma unroll
+    for (int i = 0; i < 2; ++i) head[q][i] = real && lane + 32 * i < idx_stride ? __ldcg(&kv_idx[row * idx_stride + lane + 32 * i]) : 0;
+  }
+#pragma unroll
+  for (int q = 0; q < QBT; ++q) {
+    if (cnt[q] < 0 || cnt[q] > idx_stride) {
       bad = true;
-      cnt = cnt < 0 ? 0 : idx_stride;
+      cnt[q] = cnt[q] < 0 ? 0 : idx_stride;
     }
-    const int32_t *list = kv_idx + row * idx_stride;
-#pragma unroll 4
-    for (int k = lane; k < cnt; k += 32) {
-      const int J = __ldcg(&list[k]);
+    auto list = [&](int J) {
       if (J < 0 || J >= nb)
         bad = true;  // skipped, reported
       else
         atomicOr(&sets[warp][q][J >> 5], 1u << (J & 31));
-    }
+    };
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+      if (lane + 32 * i < cnt[q]) list(head[q][i]);
+    const int32_t *row = kv_idx + ((size_t)r * nb + t * QBT + q) * idx_stride;
+#pragma unroll 4
+    for (int k = lane + 64; k < cnt[q]; k += 32) list(__ldcg(&row[k]));
   }
   __syncwarp();
   if (bad) atomicExch(status, HEART_ERR_DEVICE_CHECK);
@@ -725,9 +736,50 @@ __global__ void __launch_bounds__(32 * kPlanWarps)
   if (lane == 0) tiles[n] = make_uint4((uint32_t)t | (uint32_t)U << 16, rr, has ? *(volatile uint32_t *)out : 0u, has ? first : 0x3ff);
 }
 
-// Order of the tiles of a launch: every group of `per_group` tiles (a head's, or all of a small launch) is
-// ranked by counting over at most 1024 distinct keys, 256 tiles per CTA.  Groups before the last
-// `n_by_length`: index order while a head's K and V fit the L2 comfortably; beyond that ascending by the
+// Order of a launch of at most 1024 tiles: longest list first, one thread per tile, by counting the tiles of each
+// length (ties in any order).  Ranking every tile against all others took 7.6 us for 1024 tiles, this takes 1.1.
+__global__ void __launch_bounds__(1024) tile_order_small_kernel(const uint4 *__restrict__ tiles, int n_tiles, uint4 *__restrict__ order) {
+  __shared__ int count[1024], warp_sum[32];
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  count[t] = 0;
+  __syncthreads();
+  pdl_wait();
+  pdl_launch_dependents();
+  uint4 word = make_uint4(0u, 0u, 0u, 0u);
+  int bin = 0, among = 0;  // 1023 - length, place among the tiles of that length
+  if (t < n_tiles) {
+    word = __ldcg(&tiles[t]);
+    bin = 1023 - min((int)(word.x >> 16), 1023);
+    among = atomicAdd(&count[bin], 1);
+  }
+  __syncthreads();
+  const int mine = count[t];
+  int before = mine;  // tiles in the bins up to this thread's, first of the warp's bins, then of all
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int u = __shfl_up_sync(0xffffffffu, before, o);
+    if (lane >= o) before += u;
+  }
+  if (lane == 31) warp_sum[warp] = before;
+  __syncthreads();
+  if (warp == 0) {
+    const int own = warp_sum[lane];
+    int v = own;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int u = __shfl_up_sync(0xffffffffu, v, o);
+      if (lane >= o) v += u;
+    }
+    warp_sum[lane] = v - own;
+  }
+  __syncthreads();
+  count[t] = before - mine + warp_sum[warp];
+  __syncthreads();
+  if (t < n_tiles) order[count[bin] + among] = word;
+}
+
+// Order of the tiles of a larger launch: the tiles of a head are ranked by counting over at most 1024 distinct
+// keys, 256 tiles per CTA.  Heads before the last `n_by_length`: index order while a head's K and V fit the L2 comfortably; beyond that ascending by the
 // first key block that the tile's lists name (ties by tile index) -- tiles that read the same region of K and
 // V run together.  The last ones: descending by the number of listed key blocks.
 __global__ void __launch_bounds__(256) tile_order_kernel(const uint4 *__restrict__ tiles, int per_group,
@@ -807,12 +859,14 @@ cudaError_t launch_bk(const Geom &g, const Workspace &w, const CUtensorMap &mq, 
   if (e != cudaSuccess) return e;
   ++*launches;
   if (planned > kSms) {  // up to there every tile starts at once: no order to choose
-    // Up to 1024 tiles (7 rounds of the SMs): longest first over all heads.  Their K and V stay in L2 anyway.
-    const bool small = planned <= 1024;
-    const int per_group = small ? planned : prm.n_tiles_per_head, groups = small ? 1 : n_heads;
-    // K + V of one head beyond 32 MB (about half of one die's share of the L2): order by key locality
-    const int by_first_key = (size_t)g.N * kD * 2 * 2 > (size_t)(32u << 20) ? 1 : 0;
-    e = launch_pdl(tile_order_kernel, dim3((per_group + 255) / 256, groups), dim3(256), 0, s, (const uint4 *)tiles, per_group, small ? 1 : 2, by_first_key, order);
+    if (planned <= 1024) {  // (7 rounds of the SMs): over all heads, whose K and V stay in L2 anyway
+      e = launch_pdl(tile_order_small_kernel, dim3(1), dim3(1024), 0, s, (const uint4 *)tiles, planned, order);
+    } else {
+      // K + V of one head beyond 32 MB (about half of one die's share of the L2): order by key locality
+      const int by_first_key = (size_t)g.N * kD * 2 * 2 > (size_t)(32u << 20) ? 1 : 0;
+      e = launch_pdl(tile_order_kernel, dim3((prm.n_tiles_per_head + 255) / 256, n_heads), dim3(256), 0, s, (const uint4 *)tiles,
+                     prm.n_tiles_per_head, 2, by_first_key, order);
+    }
     if (e != cudaSuccess) return e;
     ++*launches;
     prm.tiles = order;
