@@ -35,9 +35,8 @@
 // The step lists come from attn_plan_kernel (one warp per tile), which runs just before; the tiles are
 // taken in the order of tile_order_kernel: head-major (the K/V of one or two heads stay in L2), within a
 // head by the first key block of their lists once a head's K and V no longer fit one die's half of the L2,
-// except for the last two heads of the launch, whose tiles go longest-list-first so that the launch does not
-// end on a long tile that started late.  Launches of at most 1024 tiles go longest-list-first altogether
-// (tile_order_small_kernel).
+// except for the launch's last tiles (up to 1024; all of a small launch), which go longest-list-first so that the
+// launch does not end on a long tile that started late.
 //
 // Every wait is bounded; a wait that runs out raises the CTA's abort flag and the status word, its roles
 // drain and stop, the other CTAs take the remaining tiles.
@@ -296,8 +295,10 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
             mbar_expect_tx(&sh.q_full[nq & 1], kTileBytes);
             tma_load_5d(smem + kOffQ + (nq & 1) * kTileBytes, &map_q, &sh.q_full[nq & 1], 0, ti.x * 128, 0, ti.z, ti.w);
             ++nq;
-            fetch(gridDim.x + atomicAdd(p.counter, 1));
           }
+          // The next tile is drawn at the last moment that hides the trip to memory: drawn with the first step, a
+          // CTA on a long tile already owned another one while others ran out (2 x 12 x 2465: 56.9 us against 55.2).
+          if (h == n_steps - 1) fetch(gridDim.x + atomicAdd(p.counter, 1));
           e_now = e_next;
         }
         if (!ok) break;
@@ -736,24 +737,50 @@ __global__ void __launch_bounds__(32 * kPlanWarps)
   if (lane == 0) tiles[n] = make_uint4((uint32_t)t | (uint32_t)U << 16, rr, has ? *(volatile uint32_t *)out : 0u, has ? first : 0x3ff);
 }
 
-// Order of a launch of at most 1024 tiles: longest list first, one thread per tile, by counting the tiles of each
-// length (ties in any order).  Ranking every tile against all others took 7.6 us for 1024 tiles, this takes 1.1.
-__global__ void __launch_bounds__(1024) tile_order_small_kernel(const uint4 *__restrict__ tiles, int n_tiles, uint4 *__restrict__ order) {
-  __shared__ int count[1024], warp_sum[32];
+// Order of the tiles of a launch, one CTA per head and one for the launch's last tiles (at most 1024, whole heads;
+// a small launch is all of it).
+// Heads: index order while a head's K and V fit the L2 comfortably; beyond that ascending by the first key block that
+// a tile's lists name (ties by tile index), every tile ranked against all others: tiles that read the same region
+// of K and V run together.
+// The last tiles: longest list first over all their heads, by counting the tiles of each length (ties in any order),
+// so that the launch does not end on a long tile that started late.  (Head by head, the longest tile of the last head,
+// 249 steps of 40 x 33k, started when 65 steps a CTA were left.  Ranking 1024 tiles against all others took 7.6 us,
+// counting takes 1.1.)
+__global__ void __launch_bounds__(1024) tile_order_kernel(const uint4 *__restrict__ tiles, int n_tiles, int per_head,
+                                                          int by_first_key, uint4 *__restrict__ order) {
+  __shared__ __align__(16) uint32_t key[1024];
+  __shared__ int warp_sum[32];
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-  count[t] = 0;
+  const bool tail = blockIdx.x == gridDim.x - 1;
+  const int base = blockIdx.x * per_head, n = tail ? n_tiles - base : per_head;
+  key[t] = tail ? 0u : 0xffffffffu;
   __syncthreads();
   pdl_wait();
   pdl_launch_dependents();
   uint4 word = make_uint4(0u, 0u, 0u, 0u);
-  int bin = 0, among = 0;  // 1023 - length, place among the tiles of that length
-  if (t < n_tiles) {
-    word = __ldcg(&tiles[t]);
-    bin = 1023 - min((int)(word.x >> 16), 1023);
-    among = atomicAdd(&count[bin], 1);
+  if (t < n) word = __ldcg(&tiles[base + t]);
+  if (!tail) {
+    int rank = t;
+    if (by_first_key) {
+      const uint32_t mine = word.w << 10 | (uint32_t)t;
+      if (t < n) key[t] = mine;
+      __syncthreads();
+      rank = 0;
+      const uint4 *k4 = reinterpret_cast<const uint4 *>(key);
+#pragma unroll 4
+      for (int u = 0; u < (n + 3) / 4; ++u) {
+        const uint4 k = k4[u];
+        rank += (k.x < mine ? 1 : 0) + (k.y < mine ? 1 : 0) + (k.z < mine ? 1 : 0) + (k.w < mine ? 1 : 0);
+      }
+    }
+    if (t < n) order[base + rank] = word;
+    return;
   }
+  const int bin = 1023 - min((int)(word.x >> 16), 1023);
+  uint32_t among = 0;  // place among the tiles of that length
+  if (t < n) among = atomicAdd(&key[bin], 1u);
   __syncthreads();
-  const int mine = count[t];
+  const int mine = (int)key[t];
   int before = mine;  // tiles in the bins up to this thread's, first of the warp's bins, then of all
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
@@ -773,50 +800,9 @@ __global__ void __launch_bounds__(1024) tile_order_small_kernel(const uint4 *__r
     warp_sum[lane] = v - own;
   }
   __syncthreads();
-  count[t] = before - mine + warp_sum[warp];
+  key[t] = (uint32_t)(before - mine + warp_sum[warp]);
   __syncthreads();
-  if (t < n_tiles) order[count[bin] + among] = word;
-}
-
-// Order of the tiles of a larger launch: the tiles of a head are ranked by counting over at most 1024 distinct
-// keys, 256 tiles per CTA.  Heads before the last `n_by_length`: index order while a head's K and V fit the L2 comfortably; beyond that ascending by the
-// first key block that the tile's lists name (ties by tile index) -- tiles that read the same region of K and
-// V run together.  The last ones: descending by the number of listed key blocks.
-__global__ void __launch_bounds__(256) tile_order_kernel(const uint4 *__restrict__ tiles, int per_group,
-                                                         int n_by_length, int by_first_key, uint4 *__restrict__ order) {
-  __shared__ __align__(16) uint32_t key[1024];
-  const int group = blockIdx.y, t = blockIdx.x * 256 + threadIdx.x;
-  pdl_wait();
-  pdl_launch_dependents();
-  const bool by_length = group >= (int)gridDim.y - n_by_length;
-  const size_t base = (size_t)group * per_group;
-  if (!by_length && !by_first_key) {
-    if (t < per_group) order[base + t] = __ldcg(&tiles[base + t]);
-    return;
-  }
-  uint4 my_word = make_uint4(0u, 0u, 0u, 0u);
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const int u = threadIdx.x + k * 256;
-    uint32_t v = 0xffffffffu;
-    if (u < per_group) {
-      const uint4 w = __ldcg(&tiles[base + u]);
-      if (u == t) my_word = w;
-      v = (by_length ? 0xffffu - (w.x >> 16) : w.w) << 10 | (uint32_t)u;
-    }
-    key[u] = v;
-  }
-  __syncthreads();
-  if (t >= per_group) return;
-  const uint32_t mine = key[t];
-  int rank = 0;
-  const uint4 *k4 = reinterpret_cast<const uint4 *>(key);
-#pragma unroll 4
-  for (int u = 0; u < (per_group + 3) / 4; ++u) {
-    const uint4 w = k4[u];
-    rank += (w.x < mine ? 1 : 0) + (w.y < mine ? 1 : 0) + (w.z < mine ? 1 : 0) + (w.w < mine ? 1 : 0);
-  }
-  order[base + rank] = my_word;
+  if (t < n) order[base + key[bin] + among] = word;
 }
 
 // ---------------------------------------------------------------------- host side
@@ -859,14 +845,11 @@ cudaError_t launch_bk(const Geom &g, const Workspace &w, const CUtensorMap &mq, 
   if (e != cudaSuccess) return e;
   ++*launches;
   if (planned > kSms) {  // up to there every tile starts at once: no order to choose
-    if (planned <= 1024) {  // (7 rounds of the SMs): over all heads, whose K and V stay in L2 anyway
-      e = launch_pdl(tile_order_small_kernel, dim3(1), dim3(1024), 0, s, (const uint4 *)tiles, planned, order);
-    } else {
-      // K + V of one head beyond 32 MB (about half of one die's share of the L2): order by key locality
-      const int by_first_key = (size_t)g.N * kD * 2 * 2 > (size_t)(32u << 20) ? 1 : 0;
-      e = launch_pdl(tile_order_kernel, dim3((prm.n_tiles_per_head + 255) / 256, n_heads), dim3(256), 0, s, (const uint4 *)tiles,
-                     prm.n_tiles_per_head, 2, by_first_key, order);
-    }
+    // K + V of one head beyond 32 MB (about half of one die's share of the L2): order by key locality
+    const int by_first_key = (size_t)g.N * kD * 2 * 2 > (size_t)(32u << 20) ? 1 : 0;
+    const int tail_heads = 1024 / prm.n_tiles_per_head;  // (a head has at most 1024 tiles)
+    const int heads = n_heads > tail_heads ? n_heads - tail_heads : 0;
+    e = launch_pdl(tile_order_kernel, dim3(heads + 1), dim3(1024), 0, s, (const uint4 *)tiles, planned, prm.n_tiles_per_head, by_first_key, order);
     if (e != cudaSuccess) return e;
     ++*launches;
     prm.tiles = order;
