@@ -10,8 +10,8 @@
 // largest element whose ">=" mass still reaches tau * z.  It decides in fp32 first: weights
 // e = 2^((s - max) log2 e), a few rounds that narrow the threshold down, then a direct evaluation over the few blocks
 // left.  That is final when the mass misses tau * z by more than 1.5e-5 z on both sides of the cut (the
-// errors of weights and sums stay below 1.1e-5 z, derived at the kernel) and no other block shares the
-// threshold's fp32 value; otherwise (about one row in a hundred) the row is decided in fp64: e = exp(s - max) and a search
+// errors of weights and sums stay below 1.2e-5 z, derived at the kernel) and no other block shares the
+// threshold's fp32 value; otherwise (a few rows in a hundred) the row is decided in fp64: e = exp(s - max) and a search
 // over the IEEE-754 pattern of e (positive doubles order like their bit patterns), starting below the
 // leading bits that the largest and the smallest weight share, two bits a round over all blocks down to
 // bit 48, the rest directly over the few blocks that share that prefix.  So the integer outputs (bit
@@ -25,7 +25,11 @@ namespace heart {
 using tc::ex2;
 
 constexpr int kSmallScoreTiles = 148;  // 64 x 64 score tiles of a launch up to which 32 x 32 ones are used
-constexpr int kRowsPerCta = 8;  // rows (warps) per CTA of the top-p kernel
+// Rows (warps) per CTA of the top-p kernel.  A row that needs the fp64 search takes many times longer than the
+// others and holds its CTA: 22296 such rows take 121 us with eight rows a CTA,
+// 108 with two; short rows gain nothing and pay for the CTAs.
+template <int NJ>
+constexpr int kRowsPerCta = NJ >= 24 ? 2 : 8;
 constexpr int kMaxCand = 64;    // candidates the direct threshold evaluation takes
 constexpr float kMassBand = 1.5e-5f;  // of z: cuts whose mass is closer to tau * z are decided in fp64
 
@@ -150,7 +154,7 @@ __global__ void __launch_bounds__(128) pooled_scores_kernel(const double *__rest
 }
 
 template <int NJ>  // NJ*32 >= n_b
-__global__ void __launch_bounds__(32 * kRowsPerCta) top_p_kernel(const double *__restrict__ scores, int nb, int pitch,
+__global__ void __launch_bounds__(32 * kRowsPerCta<NJ>) top_p_kernel(const double *__restrict__ scores, int nb, int pitch,
                                                                  const double *__restrict__ tau,
                                                                  const uint8_t *__restrict__ refresh,
                                                                  unsigned flags, uint32_t *__restrict__ mask_bits,
@@ -165,28 +169,31 @@ __global__ void __launch_bounds__(32 * kRowsPerCta) top_p_kernel(const double *_
   if (refresh != nullptr && refresh[r] == 0) return;  // reuse branch of Algorithm 1: mask untouched
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   extern __shared__ __align__(16) unsigned char smem_top[];
-  double *weights = reinterpret_cast<double *>(smem_top);  // [kRowsPerCta][NJ * 32]
-  __shared__ double cand[kRowsPerCta][kMaxCand];
+  double *weights = reinterpret_cast<double *>(smem_top);  // [kRowsPerCta<NJ>][NJ * 32]
+  __shared__ double cand[kRowsPerCta<NJ>][kMaxCand];
   const unsigned lt_mask = (1u << lane) - 1u;
   {
-    const int I = blockIdx.x * kRowsPerCta + warp;
+    const int I = blockIdx.x * kRowsPerCta<NJ> + warp;
     if (I >= nb) return;
     const size_t row = (size_t)r * nb + I;
     const double *srow = scores + row * pitch;
-    // The row lives in shared memory (lane-major, conflict-free): rolled loops over the NJ blocks of a lane
-    // keep the kernel small enough for the instruction cache -- fully unrolled over registers it was
-    // several times slower at n_b > 512.
+    // fp64 search: the row lives in shared memory (lane-major, conflict-free), and rolled loops over the NJ blocks
+    // of a lane keep the kernel small -- fully unrolled over registers it was several times slower at n_b > 512.
     double *pw = weights + (size_t)warp * NJ * 32 + lane;
-    float2 *pf = reinterpret_cast<float2 *>(pw);  // (x = s - max, e = exp(x)) over the same words
     const double neg_inf = __longlong_as_double(0xfff0000000000000LL);
+    // fp32 search: in registers (from shared memory with rolled loops: 121 us instead of 115 for 22296 rows of 929).
+    float x[NJ], e[NJ];  // s - max, exp of it
     double mx = neg_inf;
-#pragma unroll 4
-    for (int j = 0; j < NJ; ++j) {
-      const int J = j * 32 + lane;
-      pw[(j) * 32] = (J < nb) ? srow[J] : neg_inf;
-      mx = fmax(mx, pw[(j) * 32]);
+    {
+      double v[NJ];
+#pragma unroll
+      for (int j = 0; j < NJ; ++j) v[j] = (j * 32 + lane < nb) ? srow[j * 32 + lane] : neg_inf;
+#pragma unroll
+      for (int j = 0; j < NJ; ++j) mx = fmax(mx, v[j]);
+      mx = warp_max(mx);
+#pragma unroll
+      for (int j = 0; j < NJ; ++j) x[j] = (float)(v[j] - mx);
     }
-    mx = warp_max(mx);
     const double tau_r = (flags & HEART_FORCE_DENSE) ? 1.0 : tau[r];
     // Outputs: the mask words are gathered in registers (lane l keeps word l) and leave in one store.
     auto emit = [&](auto keep_of) {
@@ -207,14 +214,14 @@ __global__ void __launch_bounds__(32 * kRowsPerCta) top_p_kernel(const double *_
 
     // fp32.  Error of a weight: x rounds by |x| 2^-24, its product with log2 e by |x| (2^-24 + 2^-25), ex2 by
     // 2^-22 relative; over a row sum e (1.5e-7 |x| + 2.4e-7) <= 1.3e-6 z (sum e |x| <= z ln n_b).  tau * z
-    // takes 38 roundings more, 2.3e-6, the mass at a cut at most 37 + 64, 6.1e-6: 1.1e-5 z together.
+    // takes 38 roundings more, 2.3e-6, the mass at a cut at most 37 + 38 + 64 (row, list,
+    // candidates), 8.3e-6: 1.2e-5 z together.
     if (tau_r > 0.0 && tau_r < 1.0) {
       float z = 0.f;
-#pragma unroll 4
+#pragma unroll
       for (int j = 0; j < NJ; ++j) {
-        const float x = (float)(pw[(j) * 32] - mx), e = ex2(x * 1.44269504f);
-        pf[(j) * 32] = make_float2(x, e);
-        z += e;
+        e[j] = ex2(x[j] * 1.44269504f);
+        z += e[j];
       }
       auto sum = [](float v) {
 #pragma unroll
@@ -227,20 +234,7 @@ __global__ void __launch_bounds__(32 * kRowsPerCta) top_p_kernel(const double *_
       // -20 together hold less than 2.1e-6.)
       float lo = -20.f, hi = 1.f, m_hi = 0.f;
       float v1 = -10.f, v2 = -5.f, v3 = -2.5f;
-      float *cx = reinterpret_cast<float *>(cand[warp]), *ce = cx + kMaxCand;
-      int n_cand = 0;
-      for (int round = 0; round < 12; ++round) {
-        float a1 = 0.f, a2 = 0.f, a3 = 0.f;
-#pragma unroll 8
-        for (int j = 0; j < NJ; ++j) {
-          const float2 p = pf[(j) * 32];
-          if (p.x >= v1) a1 += p.y;
-          if (p.x >= v2) a2 += p.y;
-          if (p.x >= v3) a3 += p.y;
-        }
-        a1 = sum(a1);
-        a2 = sum(a2);
-        a3 = sum(a3);
+      auto narrow = [&](float a1, float a2, float a3) {  // by the masses at v1 < v2 < v3
         if (a3 >= t) {
           lo = v3;
         } else {
@@ -257,22 +251,53 @@ __global__ void __launch_bounds__(32 * kRowsPerCta) top_p_kernel(const double *_
         v1 = lo + step;
         v2 = lo + 2.f * step;
         v3 = hi - step;
-        if (round < 2) continue;
-        n_cand = 0;  // collect the blocks of the interval (the first kMaxCand of them)
-        __syncwarp();
-#pragma unroll 4
+      };
+      for (int round = 0; round < 2; ++round) {
+        float a1 = 0.f, a2 = 0.f, a3 = 0.f;
+#pragma unroll
         for (int j = 0; j < NJ; ++j) {
-          const float2 p = pf[(j) * 32];
-          const bool is_c = p.x >= lo && p.x < hi;
+          a1 += x[j] >= v1 ? e[j] : 0.f;
+          a2 += x[j] >= v2 ? e[j] : 0.f;
+          a3 += x[j] >= v3 ? e[j] : 0.f;
+        }
+        narrow(sum(a1), sum(a2), sum(a3));
+      }
+      // The blocks of that interval (a tenth of the row, as a rule) go to shared memory, where the search goes on.
+      float2 *list = reinterpret_cast<float2 *>(weights + (size_t)warp * NJ * 32);
+      int n_list = 0;
+#pragma unroll
+      for (int j = 0; j < NJ; ++j) {
+        const bool is_c = x[j] >= lo && x[j] < hi;
+        const unsigned bal = __ballot_sync(0xffffffffu, is_c);
+        if (is_c) list[n_list + __popc(bal & lt_mask)] = make_float2(x[j], e[j]);
+        n_list += __popc(bal);
+      }
+      __syncwarp();
+      float *cx = reinterpret_cast<float *>(cand[warp]), *ce = cx + kMaxCand;
+      int n_cand = 0;
+      const float m_list = m_hi;  // mass above the list
+      for (int round = 0; round < 12; ++round) {
+        n_cand = 0;
+#pragma unroll 4
+        for (int k = lane; k - lane < n_list; k += 32) {
+          const float2 c = k < n_list ? list[k] : make_float2(-INFINITY, 0.f);
+          const bool is_c = c.x >= lo && c.x < hi;
           const unsigned bal = __ballot_sync(0xffffffffu, is_c);
-          if (is_c) {
-            const int pos = n_cand + __popc(bal & lt_mask);
-            if (pos < kMaxCand) cx[pos] = p.x, ce[pos] = p.y;
-          }
+          const int pos = n_cand + __popc(bal & lt_mask);
+          if (is_c && pos < kMaxCand) cx[pos] = c.x, ce[pos] = c.y;
           n_cand += __popc(bal);
         }
         __syncwarp();
         if (n_cand <= kMaxCand) break;
+        float a1 = 0.f, a2 = 0.f, a3 = 0.f;
+#pragma unroll 4
+        for (int k = lane; k < n_list; k += 32) {
+          const float2 c = list[k];
+          a1 += c.x >= v1 ? c.y : 0.f;
+          a2 += c.x >= v2 ? c.y : 0.f;
+          a3 += c.x >= v3 ? c.y : 0.f;
+        }
+        narrow(m_list + sum(a1), m_list + sum(a2), m_list + sum(a3));
       }
       if (n_cand <= kMaxCand) {
         // Each lane takes two candidates: is the cut at this one, clearly?
@@ -282,19 +307,30 @@ __global__ void __launch_bounds__(32 * kRowsPerCta) top_p_kernel(const double *_
         for (int k = 0; k < 2; ++k) {
           if (k * 32 >= n_cand) break;
           const bool have = lane + 32 * k < n_cand;
-          const float x = have ? cx[lane + 32 * k] : 0.f, e = have ? ce[lane + 32 * k] : 0.f;
+          const float xk = have ? cx[lane + 32 * k] : 0.f, ek = have ? ce[lane + 32 * k] : 0.f;
           float above = m_hi;
           int same = 0;
           for (int n = 0; n < n_cand; ++n) {
-            above += cx[n] > x ? ce[n] : 0.f;
-            same += cx[n] == x ? 1 : 0;
+            above += cx[n] > xk ? ce[n] : 0.f;
+            same += cx[n] == xk ? 1 : 0;
           }
-          if (have && same == 1 && t - above > band && above + e - t > band) found = true, x_cut = x;
+          if (have && same == 1 && t - above > band && above + ek - t > band) found = true, x_cut = xk;
         }
         const unsigned who = __ballot_sync(0xffffffffu, found);
         if (__popc(who) == 1) {
           x_cut = __shfl_sync(0xffffffffu, x_cut, __ffs(who) - 1);
-          emit([&](int j, bool valid) { return valid && pf[(j) * 32].x >= x_cut; });
+          int base = 0;
+          uint32_t my_word = 0u;
+#pragma unroll
+          for (int j = 0; j < NJ; ++j) {
+            const bool keep = j * 32 + lane < nb && x[j] >= x_cut;
+            const unsigned word = __ballot_sync(0xffffffffu, keep);
+            my_word = lane == j ? word : my_word;
+            if (keep) kv_idx[row * idx_stride + base + __popc(word & lt_mask)] = j * 32 + lane;
+            base += __popc(word);
+          }
+          if (lane < W) mask_bits[row * W + lane] = my_word;
+          if (lane == 0) kv_cnt[row] = base;
           return;
         }
       }
@@ -470,12 +506,12 @@ __global__ void __launch_bounds__(32 * kRowsPerCta) top_p_kernel(const double *_
 template <int NJ>
 static cudaError_t launch_nj(const Geom &g, const Workspace &w, const double *tau, const uint8_t *refresh,
                              heart_state st, int pitch, cudaStream_t s, unsigned long long expect_sig) {
-  dim3 grid((g.nb + kRowsPerCta - 1) / kRowsPerCta, g.R);
-  const size_t smem = sizeof(double) * kRowsPerCta * NJ * 32;
+  dim3 grid((g.nb + kRowsPerCta<NJ> - 1) / kRowsPerCta<NJ>, g.R);
+  const size_t smem = sizeof(double) * kRowsPerCta<NJ> * NJ * 32;
   static std::atomic<unsigned long long> done{0};
   cudaError_t e = allow_shared_memory(top_p_kernel<NJ>, (int)smem, done);
   if (e != cudaSuccess) return e;
-  return launch_pdl(top_p_kernel<NJ>, grid, dim3(32 * kRowsPerCta), smem, s, (const double *)w.scores, g.nb, pitch, tau,
+  return launch_pdl(top_p_kernel<NJ>, grid, dim3(32 * kRowsPerCta<NJ>), smem, s, (const double *)w.scores, g.nb, pitch, tau,
                     refresh, g.flags, st.mask_bits, st.kv_idx, st.kv_cnt, g.idx_stride, g.W, (const int32_t *)w.status,
                     expect_sig);
 }
@@ -505,6 +541,7 @@ cudaError_t launch_top_p(const Geom &g, const Workspace &w, const double *tau, c
                          heart_state st, cudaStream_t s, int *launches, unsigned long long expect_sig) {
   ++*launches;
   const int nj = (g.nb + 31) / 32, pitch = nj * 32;
+  if (nj <= 2) return launch_nj<2>(g, w, tau, refresh, st, pitch, s, expect_sig);
   if (nj <= 8) return launch_nj<8>(g, w, tau, refresh, st, pitch, s, expect_sig);
   if (nj <= 16) return launch_nj<16>(g, w, tau, refresh, st, pitch, s, expect_sig);
   if (nj <= 24) return launch_nj<24>(g, w, tau, refresh, st, pitch, s, expect_sig);
