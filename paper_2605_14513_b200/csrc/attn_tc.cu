@@ -38,6 +38,12 @@
 // except for the launch's last tiles (up to 1024; all of a small launch), which go longest-list-first so that the
 // launch does not end on a long tile that started late.
 //
+// Small launches (a tile per CTA at most) have an instance of their own, which plans its tile itself and, while tiles
+// are few, shares its key steps among a cluster of 2 or 4 CTAs: their O and row sums meet in shared memory, and each CTA
+// puts together its share of the rows.  2 heads x 2k, 32 tiles of up to 13 steps: 19.0 us with a plan kernel before it,
+// 17.9 without, 16.5 with two CTAs a tile, 15.5 with four.  (Reading the parts takes 2.8 us of it, at 9 bytes a clock
+// and SM between SMs: more CTAs would not pay.)
+//
 // Every wait is bounded; a wait that runs out raises the CTA's abort flag and the status word, its roles
 // drain and stop, the other CTAs take the remaining tiles.
 #include <cuda.h>
@@ -59,6 +65,7 @@ constexpr float kNoReference = -3.0e38f;  // below every logit: the first step m
 // point with 8 exponent bits throughout, so a scale of up to 2^64 costs no precision, and 2^17 such weights
 // leave room for values up to 2^46.  A move costs a rescale of O behind the products in flight.
 constexpr float kMaxGrowth = 64.f;
+constexpr int kMaxSplit = 4;  // CTAs that share a tile in a small launch
 
 // Shared-memory plan (the dynamic allocation itself is 1024-byte aligned).
 constexpr int kOutBytes = 2048;  // per softmax warp: 32 rows x 32 dims of the output
@@ -81,6 +88,10 @@ struct AttnShared {
   float2 l[2][128];        // row sum and its reference of the warpgroup without the last step, per tile & 1
   uint32_t tmem_base;
   int abort;
+  // small launches: the tile's plan
+  uint4 word;
+  uint32_t sets[2][32];
+  uint32_t steps[HEART_MAX_BLOCKS];
 };
 constexpr int kAttnSmem = kOffBar + sizeof(AttnShared);
 
@@ -99,6 +110,7 @@ struct AttnParams {
   int H, N, nb, n_tiles, n_tiles_per_head, step_pitch, dense;
   int h0, hcount;  // this launch covers heads [h0, h0 + hcount) of every batch entry
   float scale_log2;
+  int split;        // small launches: CTAs (one cluster) that share the key steps of a tile
   int test_skip_v;  // test-hook builds only: CTA 0 leaves out the V copy of its second key step
 };
 
@@ -135,10 +147,142 @@ __device__ __forceinline__ float max64(const uint32_t *s) {
   return fmaxf(fmaxf(m[0], m[1]), fmaxf(m[2], m[3]));
 }
 
+struct PlanParams {
+  const int32_t *kv_idx, *kv_cnt;  // [B*H][nb][idx_stride], [B*H][nb]
+  int nb, ncph, idx_stride;        // ncph: tiles of a head
+  int H, h0, hcount;
+  int ragged;                      // the last block is not whole
+  int32_t *status;
+};
+// The step list of tile n of a launch, by one warp; it goes to out_of(tile among all heads).  The lists of the tile's query blocks (any
+// order; entries out of range are skipped and reported, duplicates merged) become bit sets, and those the
+// list of key steps.  64-token blocks: key blocks that both query blocks list come first, then blocks of
+// query block 0 paired with blocks of query block 1, so that in such a step every row has 64 exponentials
+// to take instead of half of the rows 128; ascending within each group.
+// Returns the tile's word (see AttnParams), in lane 0.
+template <int B, typename OutOf>
+__device__ __forceinline__ uint4 plan_tile(const PlanParams &p, int n, int lane, uint32_t (*sets)[32], OutOf out_of) {
+  constexpr int QBT = 128 / B;  // query blocks per tile
+  const int rr = n / p.ncph, t = n % p.ncph;
+  const int r = (rr / p.hcount) * p.H + p.h0 + rr % p.hcount;
+#pragma unroll
+  for (int q = 0; q < QBT; ++q) sets[q][lane] = 0u;
+  __syncwarp();
+  bool bad = false;
+  // The counts and the first 64 entries of the lists are asked for together (entries beyond the count are not
+  // looked at): one trip to memory for a short list instead of one for each query block's count and list.
+  int cnt[QBT], head[QBT][2];
+#pragma unroll
+  for (int q = 0; q < QBT; ++q) {
+    const size_t row = (size_t)r * p.nb + t * QBT + q;
+    const bool real = t * QBT + q < p.nb;
+    cnt[q] = real ? __ldcg(&p.kv_cnt[row]) : 0;
+#pragma unroll
+    for (int i = 0; i < 2; ++i) head[q][i] = real && lane + 32 * i < p.idx_stride ? __ldcg(&p.kv_idx[row * p.idx_stride + lane + 32 * i]) : 0;
+  }
+#pragma unroll
+  for (int q = 0; q < QBT; ++q) {
+    if (cnt[q] < 0 || cnt[q] > p.idx_stride) {
+      bad = true;
+      cnt[q] = cnt[q] < 0 ? 0 : p.idx_stride;
+    }
+    auto list = [&](int J) {
+      if (J < 0 || J >= p.nb)
+        bad = true;  // skipped, reported
+      else
+        atomicOr(&sets[q][J >> 5], 1u << (J & 31));
+    };
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+      if (lane + 32 * i < cnt[q]) list(head[q][i]);
+    const int32_t *row = p.kv_idx + ((size_t)r * p.nb + t * QBT + q) * p.idx_stride;
+#pragma unroll 4
+    for (int k = lane + 64; k < cnt[q]; k += 32) list(__ldcg(&row[k]));
+  }
+  __syncwarp();
+  if (bad) atomicExch(p.status, HEART_ERR_DEVICE_CHECK);
+  // exclusive prefix over the lanes of a count per lane
+  auto prefix = [lane](int v) {
+    int s = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int u = __shfl_up_sync(0xffffffffu, s, o);
+      if (lane >= o) s += u;
+    }
+    return s - v;
+  };
+  auto sum = [](int v) { return (int)__reduce_add_sync(0xffffffffu, (unsigned)v); };
+  uint32_t *out = out_of(r * p.ncph + t);
+  const uint32_t a = sets[0][lane], b = QBT == 2 ? sets[QBT - 1][lane] : 0u;
+  const uint32_t any = a | b;
+  const int U = sum(__popc(any));
+  if (B == 128) {
+    int pos = prefix(__popc(a));
+    for (uint32_t m = a; m; m &= m - 1) out[pos++] = lane * 32 + __ffs(m) - 1;
+  } else {
+    uint16_t *out16 = reinterpret_cast<uint16_t *>(out);
+    // the word of key block J, listed by the query blocks in `flags`
+    auto word = [&](int J, int flags) { return (uint16_t)(J | flags << 10 | (p.ragged && J == p.nb - 1 ? 1 << 12 : 0)); };
+    int last = -1;  // the last listed block, in the lane that writes it
+    const int D = sum(__popc(a & b));
+    int pos = prefix(__popc(a & b));
+    for (uint32_t m = a & b; m; m &= m - 1) {
+      const int J = lane * 32 + __ffs(m) - 1;
+      last = pos == U - 1 ? J : last;
+      out16[pos++] = word(J, 3);
+    }
+    int S[2] = {sum(__popc(a & ~b)), sum(__popc(b & ~a))};
+    int start = D, skip[2] = {0, 0};
+    if ((D & 1) && S[0] + S[1] > 0) {  // one single next to the last shared block; pairs start on a step
+      const int x = S[0] >= S[1] ? 0 : 1;
+      skip[x] = 1;
+      --S[x];
+      ++start;
+    }
+    const int paired = min(S[0], S[1]);
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const uint32_t only = q ? b & ~a : a & ~b;
+      int k = prefix(__popc(only)) - skip[q];
+      for (uint32_t m = only; m; m &= m - 1, ++k) {
+        const int at = k < 0 ? D : k < paired ? start + 2 * k + q : start + paired + k;
+        const int J = lane * 32 + __ffs(m) - 1;
+        last = at == U - 1 ? J : last;
+        out16[at] = word(J, 1 << q);
+      }
+    }
+    if ((U & 1) && last >= 0) out16[U] = (uint16_t)last;  // second half of the last step: the same block, without flags
+  }
+  const unsigned has = __ballot_sync(0xffffffffu, any != 0u);
+  const int src = has ? __ffs(has) - 1 : 0;
+  const int first = __shfl_sync(0xffffffffu, lane * 32 + __ffs(any) - 1, src);
+  __syncwarp();  // the first step, written by some lane, is read back
+  return make_uint4((uint32_t)t | (uint32_t)U << 16, rr, has ? *(volatile uint32_t *)out : 0u, has ? first : 0x3ff);
+}
+
+// Plans of all tiles of a launch, one warp per tile (a launch of at most one tile per SM makes them in the
+// attention kernel instead).
+constexpr int kPlanWarps = 8;
+
 template <int B>
+__global__ void __launch_bounds__(32 * kPlanWarps)
+    attn_plan_kernel(const PlanParams p, int n_tiles, int step_pitch, uint32_t *__restrict__ steps, uint4 *__restrict__ tiles,
+                     int32_t *__restrict__ counter) {
+  __shared__ uint32_t sets[kPlanWarps][128 / B][32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int n = blockIdx.x * kPlanWarps + warp;
+  pdl_wait();  // the lists come from the kernel before this one
+  pdl_launch_dependents();
+  if (blockIdx.x == 0 && threadIdx.x == 0) *counter = 0;
+  if (n >= n_tiles) return;
+  const uint4 word = plan_tile<B>(p, n, lane, sets[warp], [&](int tile) { return steps + (size_t)tile * step_pitch; });
+  if (lane == 0) tiles[n] = word;
+}
+
+template <int B, bool Small>
 __global__ void __launch_bounds__(kAttnThreads, 1)
     attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
-                   const __grid_constant__ CUtensorMap map_v, const AttnParams p) {
+                   const __grid_constant__ CUtensorMap map_v, const AttnParams p, const PlanParams plan) {
   extern __shared__ __align__(1024) unsigned char smem[];
   AttnShared &sh = *reinterpret_cast<AttnShared *>(smem + kOffBar);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -180,17 +324,26 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
   // CTA of this launch has started: its CTAs then fill the SMs that finish first.
   pdl_wait();
   pdl_launch_dependents();
+  if (Small && !p.dense && warp == 0) {
+    const uint4 word = plan_tile<B>(plan, blockIdx.x / p.split, lane, sh.sets, [&](int) { return sh.steps; });
+    if (lane == 0) sh.word = word;
+  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = sh.tmem_base;
 
-  auto n_steps_of = [](int U) -> int { return B == 128 ? U : (U + 1) / 2; };
+  // Key steps of a tile with U listed key blocks that this CTA takes, and the first one of them.
+  const int rank = Small ? (int)cluster_ctarank() : 0;
+  auto first_step = [&](int U, int part) -> int { return Small ? (B == 128 ? U : (U + 1) / 2) * part / p.split : 0; };
+  auto n_steps_of = [&](int U) -> int { return Small ? first_step(U, rank + 1) - first_step(U, rank) : B == 128 ? U : (U + 1) / 2; };
   auto steps_of = [&](const int4 &ti) -> const uint32_t * {
+    if (Small) return sh.steps + first_step(ti.y, rank);
     return p.steps + ((size_t)(ti.w * p.H + ti.z) * p.n_tiles_per_head + ti.x) * p.step_pitch;
   };
   auto step_entry = [&](const uint32_t *steps, int h) -> uint32_t {
-    if (!p.dense) return __ldcg(&steps[h]);
+    if (!p.dense) return Small ? steps[h] : __ldcg(&steps[h]);
+    if (Small) h += first_step(p.nb, rank);
     if (B == 128) return h;
     const uint32_t ragged = (p.N & 63) ? p.nb - 1 : 0x3ff + 1, a = 2 * h, b = 2 * h + 1;
     return (a | 3u << 10 | (a == ragged ? 1u << 12 : 0u)) | (b < (uint32_t)p.nb ? b | 3u << 10 | (b == ragged ? 1u << 12 : 0u) : a) << 16;
@@ -264,15 +417,18 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
           t.x = (n - t.y * p.n_tiles_per_head) | (uint32_t)p.nb << 16;
           t.z = step_entry(nullptr, 0);
         } else {
-          t = __ldcg(&p.tiles[n]);
+          t = Small ? sh.word : __ldcg(&p.tiles[n]);
         }
         e = t.z;
         nx.x = t.x & 0xffff;
         nx.y = t.x >> 16;
         nx.w = (int)t.y / p.hcount;
         nx.z = p.h0 + (int)t.y - nx.w * p.hcount;
+        if (Small && n_steps_of(nx.y) > 0) e = step_entry(steps_of(nx), 0);
       };
-      fetch(blockIdx.x);  // the first tile of every CTA is fixed, the others are drawn
+      // the first tile of every CTA is fixed, the others are drawn (a small launch has no others)
+      fetch(Small ? blockIdx.x / p.split : blockIdx.x);
+      auto draw = [&]() { fetch(Small ? p.n_tiles : gridDim.x + atomicAdd(p.counter, 1)); };
       for (int t = 0;; ++t) {
         const int i = t % kTileRing;
         if (t >= kTileRing) ok = mbar_wait(&sh.tile_empty[i], (t / kTileRing - 1) & 1, abort);
@@ -298,11 +454,11 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
           }
           // The next tile is drawn at the last moment that hides the trip to memory: drawn with the first step, a
           // CTA on a long tile already owned another one while others ran out (2 x 12 x 2465: 56.9 us against 55.2).
-          if (h == n_steps - 1) fetch(gridDim.x + atomicAdd(p.counter, 1));
+          if (h == n_steps - 1) draw();
           e_now = e_next;
         }
         if (!ok) break;
-        if (n_steps == 0) fetch(gridDim.x + atomicAdd(p.counter, 1));
+        if (n_steps == 0) draw();
       }
       if (*abort) {
         settle_pair(sh.q_full, nq);
@@ -561,7 +717,6 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
           const float2 other = sh.l[nt & 1][row];
           l_run += other.x * ex2(other.y - m_ref);
         }
-        const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
         uint32_t v[128];
         if (n_steps > 0) {
 #pragma unroll
@@ -572,6 +727,15 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
 #pragma unroll
           for (int i = 0; i < 128; ++i) v[i] = 0u;
         }
+        if (Small && p.split > 1) {  // O as it is, where the keys were, with its row sums: the parts are put together below
+          float4 *part = reinterpret_cast<float4 *>(smem + kOffK + row * 512);
+#pragma unroll
+          for (int i = 0; i < 32; ++i)
+            part[i ^ (row & 7)] = make_float4(__uint_as_float(v[4 * i]), __uint_as_float(v[4 * i + 1]), __uint_as_float(v[4 * i + 2]), __uint_as_float(v[4 * i + 3]));
+          sh.l[0][row] = make_float2(l_run, m_ref);
+          break;
+        }
+        const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
         // A row per thread would touch 32 lines with every store (2700-5000 clocks for a tile, during which the
         // partner runs out of work): 32 dims at a time go through shared memory, so that four lanes write 64
         // bytes of a row.
@@ -607,6 +771,65 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
       g0 += n_steps;
       nt += n_steps > 0 ? 1 : 0;
     }
+    if (Small && p.split > 1) {
+      // ===== the parts of a tile, one in every CTA of the cluster: each CTA puts together 128 / split rows
+      const int n = blockIdx.x / p.split, rows = 128 / p.split;
+      uint4 word;
+      if (p.dense) {
+        word.y = n / p.n_tiles_per_head;
+        word.x = n - word.y * p.n_tiles_per_head;
+      } else {
+        word = sh.word;
+      }
+      const int b = (int)word.y / p.hcount, hd = p.h0 + (int)word.y - b * p.hcount, tok0 = (word.x & 0xffff) * 128;
+      const uint32_t off_l = smem_u32(&sh.l[0][0]) - smem_u32(smem), off_abort = smem_u32(const_cast<int *>(&sh.abort)) - smem_u32(smem);
+      uint32_t base[kMaxSplit], gave_up = 0u;
+      cluster_sync();
+#pragma unroll
+      for (int i = 0; i < kMaxSplit; ++i) {
+        base[i] = cluster_address(smem_u32(smem), i < p.split ? i : 0);
+        gave_up |= cluster_ld1(base[i] + off_abort);
+      }
+#pragma unroll 2
+      for (int row = rank * rows + warp; row < (rank + 1) * rows; row += 8) {
+        float l[kMaxSplit], m[kMaxSplit], m_all = kNoReference, l_all = 0.f;
+        float4 x[kMaxSplit], o = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int i = 0; i < kMaxSplit; ++i) {
+          if (i >= p.split) break;
+          const float2 lm = cluster_ld2(base[i] + off_l + row * 8);
+          x[i] = cluster_ld4(base[i] + kOffK + row * 512 + ((lane ^ (row & 7)) << 4));
+          l[i] = lm.x;
+          m[i] = lm.x > 0.f ? lm.y : kNoReference;
+          m_all = fmaxf(m_all, m[i]);
+        }
+#pragma unroll
+        for (int i = 0; i < kMaxSplit; ++i) {
+          if (i >= p.split) break;
+          if (l[i] > 0.f) {  // (a part without keys has zeros)
+            const float f = ex2(m[i] - m_all);
+            l_all = fmaf(l[i], f, l_all);
+            o.x = fmaf(x[i].x, f, o.x);
+            o.y = fmaf(x[i].y, f, o.y);
+            o.z = fmaf(x[i].z, f, o.z);
+            o.w = fmaf(x[i].w, f, o.w);
+          }
+        }
+        const float inv = l_all > 0.f ? 1.f / l_all : 0.f;
+        const int tok = tok0 + row;
+        if (tok < p.N && gave_up == 0u) {  // (a tile of which a part gave up is not written)
+          const uint2 y = make_uint2(pack_bf16x2(o.x * inv, o.y * inv), pack_bf16x2(o.z * inv, o.w * inv));
+          *reinterpret_cast<uint2 *>(p.O + (long long)b * p.sb + (long long)hd * p.sh + (long long)tok * p.sn + lane * 4) = y;
+          if (lane == 0 && p.lse != nullptr)
+            p.lse[(size_t)(b * p.H + hd) * p.N + tok] = l_all > 0.f ? (m_all + log2f(l_all)) * 0.6931471805599453f : -INFINITY;
+        }
+      }
+      cluster_sync();  // shared memory stays until everyone has read it
+    }
+  }
+  if (Small && p.split > 1 && warp >= kWarpQK) {
+    cluster_sync();
+    cluster_sync();
   }
 
   // ------------------------------------------------------------------ tear-down
@@ -617,124 +840,6 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     tmem_dealloc(tmem, 512);
   }
   if (tid == 0 && sh.abort) atomicExch(p.status, HEART_ERR_DEVICE_CHECK);
-}
-
-// Step lists of the tiles of a launch: one warp per tile.  The lists of the tile's query blocks (any
-// order; entries out of range are skipped and reported, duplicates merged) become bit sets, and those the
-// list of key steps.  64-token blocks: key blocks that both query blocks list come first, then blocks of
-// query block 0 paired with blocks of query block 1, so that in such a step every row has 64 exponentials
-// to take instead of half of the rows 128; ascending within each group.
-constexpr int kPlanWarps = 8;
-
-template <int B>
-__global__ void __launch_bounds__(32 * kPlanWarps)
-    attn_plan_kernel(const int32_t *__restrict__ kv_idx, const int32_t *__restrict__ kv_cnt, int nb, int ncph, int idx_stride,
-                     int H, int h0, int hcount, int n_tiles, int step_pitch, int ragged, uint32_t *__restrict__ steps,
-                     uint4 *__restrict__ tiles, int32_t *__restrict__ counter,
-                     int32_t *__restrict__ status) {
-  constexpr int QBT = 128 / B;  // query blocks per tile
-  __shared__ uint32_t sets[kPlanWarps][QBT][32];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int n = blockIdx.x * kPlanWarps + warp;
-  pdl_wait();  // the lists come from the kernel before this one
-  pdl_launch_dependents();
-  if (blockIdx.x == 0 && threadIdx.x == 0) *counter = 0;
-  if (n >= n_tiles) return;
-  const int rr = n / ncph, t = n % ncph;
-  const int r = (rr / hcount) * H + h0 + rr % hcount;
-#pragma unroll
-  for (int q = 0; q < QBT; ++q) sets[warp][q][lane] = 0u;
-  __syncwarp();
-  bool bad = false;
-  // The counts and the first 64 entries of the lists are asked for together (entries beyond the count are not
-  // looked at): one trip to memory for a short list instead of one for each query block's count and list.
-  int cnt[QBT], head[QBT][2];
-#pragma unroll
-  for (int q = 0; q < QBT; ++q) {
-    const size_t row = (size_t)r * nb + t * QBT + q;
-    const bool real = t * QBT + q < nb;
-    cnt[q] = real ? __ldcg(&kv_cnt[row]) : 0;
-#pragma unroll
-    for (int i = 0; i < 2; ++i) head[q][i] = real && lane + 32 * i < idx_stride ? __ldcg(&kv_idx[row * idx_stride + lane + 32 * i]) : 0;
-  }
-#pragma unroll
-  for (int q = 0; q < QBT; ++q) {
-    if (cnt[q] < 0 || cnt[q] > idx_stride) {
-      bad = true;
-      cnt[q] = cnt[q] < 0 ? 0 : idx_stride;
-    }
-    auto list = [&](int J) {
-      if (J < 0 || J >= nb)
-        bad = true;  // skipped, reported
-      else
-        atomicOr(&sets[warp][q][J >> 5], 1u << (J & 31));
-    };
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-      if (lane + 32 * i < cnt[q]) list(head[q][i]);
-    const int32_t *row = kv_idx + ((size_t)r * nb + t * QBT + q) * idx_stride;
-#pragma unroll 4
-    for (int k = lane + 64; k < cnt[q]; k += 32) list(__ldcg(&row[k]));
-  }
-  __syncwarp();
-  if (bad) atomicExch(status, HEART_ERR_DEVICE_CHECK);
-  // exclusive prefix over the lanes of a count per lane
-  auto prefix = [lane](int v) {
-    int s = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int u = __shfl_up_sync(0xffffffffu, s, o);
-      if (lane >= o) s += u;
-    }
-    return s - v;
-  };
-  auto sum = [](int v) { return (int)__reduce_add_sync(0xffffffffu, (unsigned)v); };
-  uint32_t *out = steps + ((size_t)r * ncph + t) * step_pitch;
-  const uint32_t a = sets[warp][0][lane], b = QBT == 2 ? sets[warp][QBT - 1][lane] : 0u;
-  const uint32_t any = a | b;
-  const int U = sum(__popc(any));
-  if (B == 128) {
-    int pos = prefix(__popc(a));
-    for (uint32_t m = a; m; m &= m - 1) out[pos++] = lane * 32 + __ffs(m) - 1;
-  } else {
-    uint16_t *out16 = reinterpret_cast<uint16_t *>(out);
-    // the word of key block J, listed by the query blocks in `flags`
-    auto word = [&](int J, int flags) { return (uint16_t)(J | flags << 10 | (ragged && J == nb - 1 ? 1 << 12 : 0)); };
-    int last = -1;  // the last listed block, in the lane that writes it
-    const int D = sum(__popc(a & b));
-    int pos = prefix(__popc(a & b));
-    for (uint32_t m = a & b; m; m &= m - 1) {
-      const int J = lane * 32 + __ffs(m) - 1;
-      last = pos == U - 1 ? J : last;
-      out16[pos++] = word(J, 3);
-    }
-    int S[2] = {sum(__popc(a & ~b)), sum(__popc(b & ~a))};
-    int start = D, skip[2] = {0, 0};
-    if ((D & 1) && S[0] + S[1] > 0) {  // one single next to the last shared block; pairs start on a step
-      const int x = S[0] >= S[1] ? 0 : 1;
-      skip[x] = 1;
-      --S[x];
-      ++start;
-    }
-    const int paired = min(S[0], S[1]);
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      const uint32_t only = q ? b & ~a : a & ~b;
-      int k = prefix(__popc(only)) - skip[q];
-      for (uint32_t m = only; m; m &= m - 1, ++k) {
-        const int at = k < 0 ? D : k < paired ? start + 2 * k + q : start + paired + k;
-        const int J = lane * 32 + __ffs(m) - 1;
-        last = at == U - 1 ? J : last;
-        out16[at] = word(J, 1 << q);
-      }
-    }
-    if ((U & 1) && last >= 0) out16[U] = (uint16_t)last;  // second half of the last step: the same block, without flags
-  }
-  const unsigned has = __ballot_sync(0xffffffffu, any != 0u);
-  const int src = has ? __ffs(has) - 1 : 0;
-  const int first = __shfl_sync(0xffffffffu, lane * 32 + __ffs(any) - 1, src);
-  __syncwarp();  // the first step, written by some lane, is read back
-  if (lane == 0) tiles[n] = make_uint4((uint32_t)t | (uint32_t)U << 16, rr, has ? *(volatile uint32_t *)out : 0u, has ? first : 0x3ff);
 }
 
 // Order of the tiles of a launch, one CTA per head and one for the launch's last tiles (at most 1024, whole heads;
@@ -809,6 +914,7 @@ __global__ void __launch_bounds__(1024) tile_order_kernel(const uint4 *__restric
 namespace {
 
 constexpr int kSms = 148;
+constexpr int kSplitCtas = 128;  // clusters of four do not fill the last SMs of every group of SMs
 
 // bf16 [B,H,N,128] with element strides (sb, sh, sn, 1) as (64 dims, token, dim half, head, batch): box =
 // 64 dims x `rows` tokens x `halves` dim halves, 128-byte swizzle, out-of-range rows read as zero.
@@ -838,13 +944,36 @@ cudaError_t launch_bk(const Geom &g, const Workspace &w, const CUtensorMap &mq, 
   prm.step_pitch = B == 128 ? g.nb : (g.nb + 1) / 2;
   prm.steps = steps;
   prm.tiles = tiles;
+  PlanParams plan = {};
+  plan.kv_idx = kv_idx;
+  plan.kv_cnt = kv_cnt;
+  plan.nb = g.nb;
+  plan.ncph = prm.n_tiles_per_head;
+  plan.idx_stride = g.idx_stride;
+  plan.H = g.H;
+  plan.h0 = prm.h0;
+  plan.hcount = prm.hcount;
+  plan.ragged = (int)(g.N % g.block != 0);
+  plan.status = prm.status;
+  if (prm.n_tiles <= kSms) {
+    // Shared among CTAs as far as there are SMs, with at least two key steps each if all are listed.  By the tiles of all
+    // heads, not of this launch: a call that runs its heads in groups gives the same bits.
+    prm.split = 1;
+    for (int n = kMaxSplit; n >= 2 && prm.split == 1; n /= 2)
+      if (all_tiles * n <= kSplitCtas && prm.step_pitch >= 2 * n) prm.split = n;
+    static std::atomic<unsigned long long> done{0};
+    e = allow_shared_memory(attn_tc_kernel<B, true>, kAttnSmem, done);
+    if (e != cudaSuccess) return e;
+    ++*launches;
+    return launch_pdl(attn_tc_kernel<B, true>, dim3(prm.n_tiles * prm.split), dim3(kAttnThreads), kAttnSmem, s, Cluster{prm.split}, mq, mk,
+                      mv, prm, plan);
+  }
   const int planned = prm.dense ? 0 : prm.n_tiles;  // (dense: the kernel only zeroes the counter)
-  e = launch_pdl(attn_plan_kernel<B>, dim3(planned ? (planned + kPlanWarps - 1) / kPlanWarps : 1), dim3(32 * kPlanWarps), 0, s,
-                 kv_idx, kv_cnt, g.nb, prm.n_tiles_per_head, g.idx_stride, g.H, prm.h0, prm.hcount, planned, prm.step_pitch,
-                 (int)(g.N % g.block != 0), steps, tiles, prm.counter, prm.status);
+  e = launch_pdl(attn_plan_kernel<B>, dim3(planned ? (planned + kPlanWarps - 1) / kPlanWarps : 1), dim3(32 * kPlanWarps), 0, s, plan,
+                 planned, prm.step_pitch, steps, tiles, prm.counter);
   if (e != cudaSuccess) return e;
   ++*launches;
-  if (planned > kSms) {  // up to there every tile starts at once: no order to choose
+  if (planned) {
     // K + V of one head beyond 32 MB (about half of one die's share of the L2): order by key locality
     const int by_first_key = (size_t)g.N * kD * 2 * 2 > (size_t)(32u << 20) ? 1 : 0;
     const int tail_heads = 1024 / prm.n_tiles_per_head;  // (a head has at most 1024 tiles)
@@ -855,11 +984,10 @@ cudaError_t launch_bk(const Geom &g, const Workspace &w, const CUtensorMap &mq, 
     prm.tiles = order;
   }
   static std::atomic<unsigned long long> done{0};
-  e = allow_shared_memory(attn_tc_kernel<B>, kAttnSmem, done);
+  e = allow_shared_memory(attn_tc_kernel<B, false>, kAttnSmem, done);
   if (e != cudaSuccess) return e;
   ++*launches;
-  return launch_pdl(attn_tc_kernel<B>, dim3(prm.n_tiles < kSms ? prm.n_tiles : kSms), dim3(kAttnThreads), kAttnSmem, s, mq, mk,
-                    mv, prm);
+  return launch_pdl(attn_tc_kernel<B, false>, dim3(kSms), dim3(kAttnThreads), kAttnSmem, s, mq, mk, mv, prm, plan);
 }
 
 }  // namespace
