@@ -10,15 +10,19 @@
 // The contraction is a bf16 GEMM per head on the very memory of Q and K: row a of the left operand
 // is the 16 tokens of group a laid end to end (16 x 128 values), row c of the right operand the 16
 // tokens of group c in reverse order.  A 5-D tensor map (dim, token in group, group, head, batch)
-// lets one TMA box fetch "token t of 128 (or 256) consecutive groups", which is exactly a K-major
-// operand tile; reversing the key tokens is a change of one box coordinate.
+// lets one TMA box fetch "token t of 128 consecutive groups", which is exactly a K-major operand tile;
+// reversing the key tokens is a change of one box coordinate.
 //
-// antidiag_scores_kernel: one CTA per (128 groups of queries, head); it walks over all key groups,
-// 256 at a time.  Warp 0 issues the TMA loads into a four-stage ring (one stage = 64 dims of one
-// token position: 16 KB of Q + 32 KB of K), warp 1 issues tcgen05.mma (M = 128, N = 256, 4 x K = 16
-// per stage, 32 stages per tile) into one of two 256-column accumulators in tensor memory, warps
-// 2-5 drain the other accumulator: one thread per query group, and for every key block of the tile
-// the pair (max, sum of 2^(x - max)) over the block's 4 or 8 groups goes to the workspace.
+// antidiag_scores_kernel: a tile is 256 query groups x 256 key groups of a head, the work of two CTAs of a cluster
+// (cta_group::2): each loads its half of both operands, holds its half of the rows of the result and drains it.
+// One CTA per SM; the tiles are dealt to the pairs, and the pipeline runs on across them.  Warp 0 issues the TMA
+// loads into a six-stage ring (one stage = 64 dims of one token position: 16 KB of Q + 16 KB of K per CTA), warp 1 of
+// the even CTA issues tcgen05.mma (M = 256, N = 256, 4 x K = 16 per stage, 32 stages per tile) into one of two
+// 256-column accumulators in tensor memory, warps 2-5 drain the other accumulator: one thread per query group, and for
+// every key block of the tile the pair (max, sum of 2^(x - max)) over the block's 4 or 8 groups goes to the workspace.
+// What bounds it: a 128 x 256 tile per CTA asks the L2 for 96 bytes a clock and SM, which it does not give (197 us for
+// 12 heads of 2048 groups); the pair asks for 64.  140 us now, 1470 TFLOP/s, the tensor pipe 81 % busy at the 1.5 GHz
+// that the power limit leaves.
 // antidiag_reduce_kernel (fp64) turns the pairs of the groups of one query block into the log of
 // the block importances, which top_p_kernel consumes like pooled scores.
 #include <cuda.h>
@@ -32,15 +36,16 @@ using namespace tc;
 namespace {
 
 constexpr int kS = HEART_ANTIDIAG_STRIDE;  // tokens per group
-constexpr int kMt = 128;                   // query groups per CTA
-constexpr int kNt = 256;                   // key groups per accumulator tile
-constexpr int kStagesAd = 4;
-constexpr int kABytes = kMt * 128, kBBytes = kNt * 128, kStageBytes = kABytes + kBBytes;
+constexpr int kMt = 256;                   // query groups per tile: 128 in each CTA of a pair
+constexpr int kNt = 256;                   // key groups per tile
+constexpr int kStagesAd = 6;
+constexpr int kHalfBytes = 128 * 128;      // 128 groups x 64 dims: a CTA's half of either operand of a stage
+constexpr int kStageBytes = 2 * kHalfBytes;
 constexpr int kKSteps = kS * 2;            // ring stages per tile: 16 token positions x 2 halves of the head dim
 constexpr int kThreadsAd = 192;
 
 struct AdBars {
-  uint64_t full[kStagesAd], empty[kStagesAd];
+  uint64_t full[kStagesAd], empty[kStagesAd];  // full, acc_empty: the even CTA's count for both
   uint64_t acc_full[2], acc_empty[2];
   uint64_t drain;
   uint32_t tmem_base;
@@ -51,7 +56,7 @@ struct AdParams {
   float2 *pairs;          // [R][Ns][nb]: (max, sum) in the log2 domain per (query group, key block)
   const uint8_t *refresh;
   int32_t *status;
-  int H, Ns, nb, g;       // g = groups per block
+  int H, R, Ns, nb;
   float c2;               // (scale / s) * log2(e)
 };
 
@@ -59,22 +64,24 @@ template <int G>  // groups per block: 4 (64-token blocks) or 8 (128-token block
 __global__ void __launch_bounds__(kThreadsAd, 1)
     antidiag_scores_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                            const AdParams p) {
-  const int r = blockIdx.y;
-  if (p.refresh != nullptr && p.refresh[r] == 0) return;  // reuse branch of Algorithm 1: nothing to predict
   extern __shared__ unsigned char smem_dyn[];
   unsigned char *smem = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) &
                                                           ~static_cast<uintptr_t>(1023));
   AdBars *bars = reinterpret_cast<AdBars *>(smem + kStagesAd * kStageBytes);
   volatile int *abort = &bars->abort;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int bidx = r / p.H, hidx = r % p.H;
-  const int a0 = blockIdx.x * kMt;
-  // The key groups are dealt to gridDim.z CTAs per (row tile, head): every key block's pair is written
-  // by exactly one of them, so nothing has to be combined.  This CTA takes tiles [tile0, tile0 + n_tiles).
-  const int all_tiles = (p.Ns + kNt - 1) / kNt;
-  const int tile0 = (int)((long long)all_tiles * blockIdx.z / gridDim.z);
-  const int n_tiles = (int)((long long)all_tiles * (blockIdx.z + 1) / gridDim.z) - tile0;
-  const int n_steps = n_tiles * kKSteps;
+  const uint32_t rank = cluster_ctarank();  // of the pair
+  // Tiles of the refreshed heads (the others: reuse branch of Algorithm 1, nothing to predict), column tiles of a row
+  // first, dealt to the pairs in turn.  Every role walks the same list.
+  const int row_tiles = (p.Ns + kMt - 1) / kMt, col_tiles = (p.Ns + kNt - 1) / kNt, n_tiles = p.R * row_tiles * col_tiles;
+  const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
+  auto each_tile = [&](auto body) {  // body(head, row tile, column tile) -> go on?
+    for (int u = pair; u < n_tiles; u += n_pairs) {
+      const int row = u / col_tiles, r = row / row_tiles;
+      if (p.refresh != nullptr && p.refresh[r] == 0) continue;
+      if (!body(r, row - r * row_tiles, u - row * col_tiles)) break;
+    }
+  };
 
   if (tid == 0) {
     for (int i = 0; i < kStagesAd; ++i) {
@@ -83,18 +90,15 @@ __global__ void __launch_bounds__(kThreadsAd, 1)
     }
     for (int i = 0; i < 2; ++i) {
       mbar_init(&bars->acc_full[i], 1);
-      mbar_init(&bars->acc_empty[i], 4);  // one arrival per draining warp
+      mbar_init(&bars->acc_empty[i], 8);  // one arrival per draining warp of the pair
     }
     mbar_init(&bars->drain, 1);
     bars->abort = 0;
     mbar_fence_init();
   }
-  if (warp == 1) {
-    tmem_alloc(&bars->tmem_base, 512);
-    tmem_relinquish();
-  }
+  if (warp == 1) tmem_alloc_pair(&bars->tmem_base, 512);
   tc_fence_before();
-  __syncthreads();
+  cluster_sync();  // (the other CTA's barriers are there)
   tc_fence_after();
   const uint32_t tmem = bars->tmem_base;
   auto settle = [&](uint64_t *bar, uint32_t parity) {
@@ -107,72 +111,72 @@ __global__ void __launch_bounds__(kThreadsAd, 1)
     if (lane == 0) {  // ===== TMA producer
       tma_prefetch_desc(&map_q);
       tma_prefetch_desc(&map_k);
-      int issued = 0;
-      for (int it = 0; it < n_steps; ++it) {
-        const int st = it % kStagesAd, n = it / kStagesAd;
-        if (n >= 1 && !mbar_wait_relaxed(&bars->empty[st], (n - 1) & 1, abort)) break;
-        const int tile = it / kKSteps, ks = it % kKSteps, t = ks >> 1, dh = ks & 1;
-        unsigned char *dst = smem + st * kStageBytes;
-        mbar_expect_tx(&bars->full[st], kStageBytes);
-        // token t of the query groups a0 .. a0+127; token s-1-t of the key groups of this tile
-        tma_load_5d(dst, &map_q, &bars->full[st], dh * 64, t, a0, hidx, bidx);
-        tma_load_5d(dst + kABytes, &map_k, &bars->full[st], dh * 64, kS - 1 - t, (tile0 + tile) * kNt, hidx, bidx);
-        issued = it + 1;
-      }
-      if (*abort)  // shared memory must not be released under a copy in flight
-        for (int it = (issued > kStagesAd ? issued - kStagesAd : 0); it < issued; ++it)
-          settle(&bars->full[it % kStagesAd], (it / kStagesAd) & 1);
+      int it = 0;
+      each_tile([&](int r, int row, int col) {
+        const int bidx = r / p.H, hidx = r % p.H;
+        for (int ks = 0; ks < kKSteps; ++ks, ++it) {
+          const int st = it % kStagesAd, n = it / kStagesAd, t = ks >> 1, dh = ks & 1;
+          if (n >= 1 && !mbar_wait(&bars->empty[st], (n - 1) & 1, abort)) return false;
+          unsigned char *dst = smem + st * kStageBytes;
+          if (rank == 0) mbar_expect_tx(&bars->full[st], 2 * kStageBytes);
+          // this CTA's half of token t of the query groups, of token s-1-t of the key groups of the tile
+          tma_load_5d_pair(dst, &map_q, &bars->full[st], dh * 64, t, row * kMt + rank * 128, hidx, bidx);
+          tma_load_5d_pair(dst + kHalfBytes, &map_k, &bars->full[st], dh * 64, kS - 1 - t, col * kNt + rank * 128, hidx, bidx);
+        }
+        return true;
+      });
     }
   } else if (warp == 1) {
-    // ===== MMA issuer: the whole warp runs the loop, one elected lane issues
-    constexpr uint32_t idesc = idesc_bf16_f32(kMt, kNt, false, false);
-    auto at = [](uint64_t desc, uint32_t off16) -> uint64_t {
-      return (desc & 0xffffffff00000000ull) | (uint32_t)((uint32_t)desc + off16);
-    };
-    const bool leader = elect_one();
-    const uint64_t a_desc0 = smem_desc_sw128(smem_u32(smem), 16, 1024);
-    const uint64_t b_desc0 = smem_desc_sw128(smem_u32(smem + kABytes), 16, 1024);
-    bool ok = true;
-    int it = 0;
-    for (int tile = 0; tile < n_tiles && ok; ++tile) {
-      const int buf = tile & 1, m = tile >> 1;
-      if (m >= 1) ok = mbar_wait(&bars->acc_empty[buf], (m - 1) & 1, abort);
-      if (!ok) break;
-      tc_fence_after();
-      const uint32_t d = tmem + buf * kNt;
-      for (int ks = 0; ks < kKSteps && ok; ++ks, ++it) {
-        const int st = it % kStagesAd, n = it / kStagesAd;
-        ok = mbar_wait(&bars->full[st], n & 1, abort);
-        if (!ok) break;
+    // ===== MMA issuer of the pair: the whole warp runs the loop, one elected lane issues
+    if (rank == 0) {
+      constexpr uint32_t idesc = idesc_bf16_f32(kMt, kNt, false, false);
+      auto at = [](uint64_t desc, uint32_t off16) -> uint64_t {
+        return (desc & 0xffffffff00000000ull) | (uint32_t)((uint32_t)desc + off16);
+      };
+      const bool leader = elect_one();
+      const uint64_t a_desc0 = smem_desc_sw128(smem_u32(smem), 16, 1024);
+      const uint64_t b_desc0 = smem_desc_sw128(smem_u32(smem + kHalfBytes), 16, 1024);
+      int it = 0, tile = 0;
+      each_tile([&](int, int, int) {
+        const int buf = tile & 1, m = tile >> 1;
+        ++tile;
+        if (m >= 1 && !__all_sync(0xffffffffu, mbar_wait(&bars->acc_empty[buf], (m - 1) & 1, abort))) return false;
         tc_fence_after();
-        const uint64_t a_desc = at(a_desc0, st * (kStageBytes >> 4)), b_desc = at(b_desc0, st * (kStageBytes >> 4));
-        if (leader) {
+        const uint32_t d = tmem + buf * kNt;
+        for (int ks = 0; ks < kKSteps; ++ks, ++it) {
+          const int st = it % kStagesAd, n = it / kStagesAd;
+          if (!__all_sync(0xffffffffu, mbar_wait(&bars->full[st], n & 1, abort))) return false;
+          tc_fence_after();
+          const uint64_t a_desc = at(a_desc0, st * (kStageBytes >> 4)), b_desc = at(b_desc0, st * (kStageBytes >> 4));
+          if (leader) {
 #pragma unroll
-          for (int k = 0; k < 4; ++k) mma_ss(d, at(a_desc, k * 2), at(b_desc, k * 2), idesc, (ks > 0 || k > 0) ? 1u : 0u);
-          tc_commit(&bars->empty[st]);
-          if (ks == kKSteps - 1) tc_commit(&bars->acc_full[buf]);
+            for (int k = 0; k < 4; ++k) mma_ss_pair(d, at(a_desc, k * 2), at(b_desc, k * 2), idesc, (ks > 0 || k > 0) ? 1u : 0u);
+            tc_commit_pair(&bars->empty[st]);
+            if (ks == kKSteps - 1) tc_commit_pair(&bars->acc_full[buf]);
+          }
+          __syncwarp();
         }
+        return true;
+      });
+      if (*abort) {  // tensor memory must not be released under a product in flight
+        if (leader) tc_commit_pair(&bars->drain);
         __syncwarp();
+        settle(&bars->drain, 0);
       }
-    }
-    if (*abort) {  // tensor memory must not be released under a product in flight
-      if (leader) tc_commit(&bars->drain);
-      __syncwarp();
-      settle(&bars->drain, 0);
     }
   } else {
     // ===== drain: thread = one query group; per key block of the tile a (max, sum) pair
     const int q = warp & 3;  // the lane quarter of tensor memory this warp may read
-    const int a = a0 + q * 32 + lane;
     const uint32_t lane_addr = tmem + ((uint32_t)(q * 32) << 16);
-    float2 *out = p.pairs + ((size_t)r * p.Ns + (a < p.Ns ? a : 0)) * p.nb;
-    bool ok = true;
-    for (int tile = 0; tile < n_tiles && ok; ++tile) {
+    int tile = 0;
+    each_tile([&](int r, int row, int col) {
       const int buf = tile & 1, m = tile >> 1;
-      ok = __all_sync(0xffffffffu, mbar_wait(&bars->acc_full[buf], m & 1, abort));
-      if (!ok) break;
+      ++tile;
+      const int a = row * kMt + rank * 128 + q * 32 + lane;
+      float2 *out = p.pairs + ((size_t)r * p.Ns + (a < p.Ns ? a : 0)) * p.nb;
+      if (!__all_sync(0xffffffffu, mbar_wait(&bars->acc_full[buf], m & 1, abort))) return false;
       tc_fence_after();
-      const int c0 = (tile0 + tile) * kNt;
+      const int c0 = col * kNt;
 #pragma unroll 1
       for (int ch = 0; ch < kNt / 32; ++ch) {
         if (c0 + ch * 32 >= p.Ns) break;  // (uniform) nothing but padding from here on
@@ -196,14 +200,24 @@ __global__ void __launch_bounds__(kThreadsAd, 1)
       }
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(&bars->acc_empty[buf]);
-    }
+      if (lane == 0) mbar_arrive_in(&bars->acc_empty[buf], 0);
+      return true;
+    });
   }
   tc_fence_before();
-  __syncthreads();
+  // Neither CTA leaves while the other one's products read its shared memory or arrivals are under way; after an
+  // abort in either, copies in flight get time to land (bounded: a copy takes microseconds).
+  cluster_sync();
+  const uint32_t off_abort = smem_u32(&bars->abort);
+  if ((cluster_ld1(cluster_address(off_abort, 0)) | cluster_ld1(cluster_address(off_abort, 1))) != 0u) {
+    const long long t0 = clock64();
+    while (clock64() - t0 < 2000000LL) {
+    }
+  }
+  cluster_sync();
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc(tmem, 512);
+    tmem_dealloc_pair(tmem, 512);
   }
   if (tid == 0 && bars->abort) atomicExch(p.status, HEART_ERR_DEVICE_CHECK);
 }
@@ -288,6 +302,26 @@ bool make_group_map(CUtensorMap *m, const void *base, const Geom &g, int Ns, int
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+template <int G>
+cudaError_t launch_scores(const CUtensorMap &mq, const CUtensorMap &mk, const AdParams &prm, long long tiles, int smem, cudaStream_t s) {
+  static std::atomic<unsigned long long> done{0};
+  cudaError_t e = allow_shared_memory(antidiag_scores_kernel<G>, smem, done);
+  if (e != cudaSuccess) return e;
+  const int pairs = (int)(tiles < 74 ? tiles : 74);  // two of the 148 SMs each
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(2 * pairs);
+  cfg.blockDim = dim3(kThreadsAd);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 2;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, antidiag_scores_kernel<G>, mq, mk, prm);
+}
+
 }  // namespace
 
 size_t antidiag_pairs_bytes(const Geom &g) {
@@ -299,7 +333,7 @@ cudaError_t launch_antidiag_scores(const Geom &g, const Workspace &w, const void
   const int Ns = g.N / kS, grp = g.block / kS, pitch = ((g.nb + 31) / 32) * 32;
   if (Ns > 0) {
     CUtensorMap mq, mk;
-    if (!make_group_map(&mq, Q, g, Ns, kMt) || !make_group_map(&mk, K, g, Ns, kNt)) return cudaErrorInvalidValue;
+    if (!make_group_map(&mq, Q, g, Ns, 128) || !make_group_map(&mk, K, g, Ns, 128)) return cudaErrorInvalidValue;
     AdParams prm;
     prm.pairs = reinterpret_cast<float2 *>(w.pairs);
     prm.refresh = refresh;
@@ -307,39 +341,13 @@ cudaError_t launch_antidiag_scores(const Geom &g, const Workspace &w, const void
     prm.H = g.H;
     prm.Ns = Ns;
     prm.nb = g.nb;
-    prm.g = grp;
+    prm.R = g.R;
     prm.c2 = (float)(g.scale / (double)kS * 1.4426950408889634);
     const int smem = kStagesAd * kStageBytes + 1024 + 256;
-    // Split the key range over up to four CTAs per (row tile, head) when that fills the 148 SMs' waves
-    // better (one CTA per SM); a shape-only rule.
-    const int row_tiles = (Ns + kMt - 1) / kMt, col_tiles = (Ns + kNt - 1) / kNt;
-    int split = 1;
-    double best_eff = 0.0;
-    for (int c = 1; c <= 4 && c <= col_tiles; ++c) {
-      const long long ctas = (long long)row_tiles * g.R * c;
-      const double waves = (double)((ctas + 147) / 148);
-      const int longest = (col_tiles + c - 1) / c;  // column tiles of the busiest CTA
-      const double eff = (double)ctas / (148.0 * waves) * ((double)col_tiles / c) / longest;
-      if (eff > best_eff + 0.02) {
-        best_eff = eff;
-        split = c;
-      }
-    }
-    dim3 grid(row_tiles, g.R, split);
-    cudaError_t e;
-    if (grp == 4) {
-      static std::atomic<unsigned long long> done{0};
-      e = allow_shared_memory(antidiag_scores_kernel<4>, smem, done);
-      if (e != cudaSuccess) return e;
-      antidiag_scores_kernel<4><<<grid, kThreadsAd, smem, s>>>(mq, mk, prm);
-    } else {
-      static std::atomic<unsigned long long> done{0};
-      e = allow_shared_memory(antidiag_scores_kernel<8>, smem, done);
-      if (e != cudaSuccess) return e;
-      antidiag_scores_kernel<8><<<grid, kThreadsAd, smem, s>>>(mq, mk, prm);
-    }
+    const long long tiles = (long long)g.R * ((Ns + kMt - 1) / kMt) * ((Ns + kNt - 1) / kNt);
+    cudaError_t e = grp == 4 ? launch_scores<4>(mq, mk, prm, tiles, smem, s) : launch_scores<8>(mq, mk, prm, tiles, smem, s);
+    if (e != cudaSuccess) return e;
     ++*launches;
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   const float2 *pairs = reinterpret_cast<const float2 *>(w.pairs);
   const dim3 rgrid(g.nb, g.R);
