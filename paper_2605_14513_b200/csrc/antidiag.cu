@@ -97,6 +97,8 @@ __global__ void __launch_bounds__(kThreadsAd, 1)
     mbar_fence_init();
   }
   if (warp == 1) tmem_alloc_pair(&bars->tmem_base, 512);
+  pdl_wait();  // refresh flags, and the workspace that the kernel before this one may still read
+  pdl_launch_dependents();
   tc_fence_before();
   cluster_sync();  // (the other CTA's barriers are there)
   tc_fence_after();
@@ -226,15 +228,17 @@ __global__ void __launch_bounds__(kThreadsAd, 1)
 // scores[r][I][J] = ln(importance(I, J)) (-inf for importance 0), which the top-p kernel reads like
 // pooled scores.  A query block without a full group gets equal scores (uniform importance).
 // One warp per group of the block (at most 8): row maximum and row sum by shuffles, the weights of
-// the lane's key blocks stay in registers in between; the groups are then added into the block's
-// weights one after the other.  Every reduction has a fixed shape: bit-reproducible.
+// the lane's key blocks stay in registers in between; they meet in shared memory, where a thread adds up
+// the groups of a key block one after the other.  Every reduction has a fixed shape: bit-reproducible.
 template <int NJ>  // NJ * 32 >= n_b
 __global__ void __launch_bounds__(256, 2) antidiag_reduce_kernel(const float2 *__restrict__ pairs, int Ns, int nb,
                                                                  int g, int pitch, const uint8_t *__restrict__ refresh,
                                                                  double *__restrict__ scores) {
   const int I = blockIdx.x, r = blockIdx.y;
+  pdl_wait();
+  pdl_launch_dependents();
   if (refresh != nullptr && refresh[r] == 0) return;
-  __shared__ double wgt[HEART_MAX_BLOCKS];
+  extern __shared__ __align__(16) double wgt[];  // [g][NJ * 32]
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int a0 = I * g, a1 = min(a0 + g, Ns);
   const int nJ = (Ns + g - 1) / g;  // key blocks that hold at least one full group
@@ -243,11 +247,9 @@ __global__ void __launch_bounds__(256, 2) antidiag_reduce_kernel(const float2 *_
     for (int J = tid; J < pitch; J += 256) srow[J] = 0.0;
     return;
   }
-  for (int J = tid; J < nb; J += 256) wgt[J] = 0.0;
   constexpr int kPerLane = NJ;
   const double ln2 = 0.6931471805599453;
   double e[kPerLane];
-  double inv_z = 0.0;
   const int a = a0 + warp;  // this warp's group (g <= 8 warps have one)
   if (warp < g && a < a1) {
     const float2 *prow = pairs + ((size_t)r * Ns + a) * nb;
@@ -270,20 +272,16 @@ __global__ void __launch_bounds__(256, 2) antidiag_reduce_kernel(const float2 *_
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
-    inv_z = 1.0 / z;
+    const double inv_z = 1.0 / z;
+#pragma unroll
+    for (int k = 0; k < kPerLane; ++k) wgt[(warp * kPerLane + k) * 32 + lane] = e[k] * inv_z;
   }
   __syncthreads();
-  for (int aa = 0; aa < g; ++aa) {  // groups in ascending order: a fixed summation order
-    if (warp == aa && a < a1) {
-#pragma unroll
-      for (int k = 0; k < kPerLane; ++k)
-        if (lane + 32 * k < nJ) wgt[lane + 32 * k] += e[k] * inv_z;
-    }
-    __syncthreads();
-  }
   const double inv = 1.0 / (double)(a1 - a0);
   for (int J = tid; J < pitch; J += 256) {
-    const double w = (J < nJ) ? wgt[J] * inv : 0.0;
+    double w = 0.0;
+    for (int n = 0; n < a1 - a0; ++n) w += wgt[n * kPerLane * 32 + J];  // groups in ascending order: a fixed summation order
+    w = (J < nJ) ? w * inv : 0.0;
     srow[J] = (w > 0.0) ? log(w) : -INFINITY;
   }
 }
@@ -308,18 +306,18 @@ cudaError_t launch_scores(const CUtensorMap &mq, const CUtensorMap &mk, const Ad
   cudaError_t e = allow_shared_memory(antidiag_scores_kernel<G>, smem, done);
   if (e != cudaSuccess) return e;
   const int pairs = (int)(tiles < 74 ? tiles : 74);  // two of the 148 SMs each
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(2 * pairs);
-  cfg.blockDim = dim3(kThreadsAd);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = 2;
-  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, antidiag_scores_kernel<G>, mq, mk, prm);
+  return launch_pdl(antidiag_scores_kernel<G>, dim3(2 * pairs), dim3(kThreadsAd), smem, s, Cluster{2}, mq, mk, prm);
+}
+
+template <int NJ>
+cudaError_t launch_reduce(const Geom &g, const float2 *pairs, int Ns, int grp, int pitch, const uint8_t *refresh, double *scores,
+                          cudaStream_t s) {
+  const int smem = grp * NJ * 32 * (int)sizeof(double);
+  static std::atomic<unsigned long long> done{0};
+  cudaError_t e = allow_shared_memory(antidiag_reduce_kernel<NJ>, 8 * NJ * 32 * (int)sizeof(double), done);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(antidiag_reduce_kernel<NJ>, dim3(g.nb, g.R), dim3(256), (size_t)smem, s, pairs, Ns, g.nb, grp, pitch, refresh,
+                    scores);
 }
 
 }  // namespace
@@ -350,18 +348,13 @@ cudaError_t launch_antidiag_scores(const Geom &g, const Workspace &w, const void
     ++*launches;
   }
   const float2 *pairs = reinterpret_cast<const float2 *>(w.pairs);
-  const dim3 rgrid(g.nb, g.R);
   const int nj = (g.nb + 31) / 32;
-  if (nj <= 8)
-    antidiag_reduce_kernel<8><<<rgrid, 256, 0, s>>>(pairs, Ns, g.nb, grp, pitch, refresh, w.scores);
-  else if (nj <= 16)
-    antidiag_reduce_kernel<16><<<rgrid, 256, 0, s>>>(pairs, Ns, g.nb, grp, pitch, refresh, w.scores);
-  else if (nj <= 24)
-    antidiag_reduce_kernel<24><<<rgrid, 256, 0, s>>>(pairs, Ns, g.nb, grp, pitch, refresh, w.scores);
-  else
-    antidiag_reduce_kernel<32><<<rgrid, 256, 0, s>>>(pairs, Ns, g.nb, grp, pitch, refresh, w.scores);
+  cudaError_t e = nj <= 8    ? launch_reduce<8>(g, pairs, Ns, grp, pitch, refresh, w.scores, s)
+                  : nj <= 16 ? launch_reduce<16>(g, pairs, Ns, grp, pitch, refresh, w.scores, s)
+                  : nj <= 24 ? launch_reduce<24>(g, pairs, Ns, grp, pitch, refresh, w.scores, s)
+                             : launch_reduce<32>(g, pairs, Ns, grp, pitch, refresh, w.scores, s);
   ++*launches;
-  return cudaGetLastError();
+  return e;
 }
 
 }  // namespace heart
