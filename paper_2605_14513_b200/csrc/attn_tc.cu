@@ -41,7 +41,7 @@
 // Small launches (a tile per CTA at most) have an instance of their own, which plans its tile itself and, while tiles
 // are few, shares its key steps among a cluster of 2 or 4 CTAs: their O and row sums meet in shared memory, and each CTA
 // puts together its share of the rows.  2 heads x 2k, 32 tiles of up to 13 steps: 19.0 us with a plan kernel before it,
-// 17.9 without, 16.5 with two CTAs a tile, 15.5 with four.  (Reading the parts takes 2.8 us of it, at 9 bytes a clock
+// 17.9 without, 16.5 with two CTAs a tile, 15.5 with four (14.7 since the plan is shorter).  (Reading the parts takes 2.8 us of it, at 9 bytes a clock
 // and SM between SMs: more CTAs would not pay.)
 //
 // Every wait is bounded; a wait that runs out raises the CTA's abort flag and the status word, its roles
@@ -201,59 +201,60 @@ __device__ __forceinline__ uint4 plan_tile(const PlanParams &p, int n, int lane,
   }
   __syncwarp();
   if (bad) atomicExch(p.status, HEART_ERR_DEVICE_CHECK);
-  // exclusive prefix over the lanes of a count per lane
-  auto prefix = [lane](int v) {
-    int s = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int u = __shfl_up_sync(0xffffffffu, s, o);
-      if (lane >= o) s += u;
-    }
-    return s - v;
-  };
   auto sum = [](int v) { return (int)__reduce_add_sync(0xffffffffu, (unsigned)v); };
   uint32_t *out = out_of(r * p.ncph + t);
   const uint32_t a = sets[0][lane], b = QBT == 2 ? sets[QBT - 1][lane] : 0u;
   const uint32_t any = a | b;
   const int U = sum(__popc(any));
+  // 32 key blocks at a time, one per lane.  (A lane per word of the set, bit after bit, made the whole call 15.6 us
+  // instead of 14.7 for 2 heads of 32 key blocks and 55.2 instead of 51.3 for 24 of 39; sparse lists over 512 and more
+  // take the same time either way.)
+  const unsigned has = __ballot_sync(0xffffffffu, any != 0u);  // words of the set that are not empty
+  const uint32_t bit = 1u << lane, below = bit - 1u;
   if (B == 128) {
-    int pos = prefix(__popc(a));
-    for (uint32_t m = a; m; m &= m - 1) out[pos++] = lane * 32 + __ffs(m) - 1;
+    int pos = 0;
+    for (unsigned todo = has; todo; todo &= todo - 1) {
+      const int n = __ffs(todo) - 1;
+      const uint32_t m = __shfl_sync(0xffffffffu, a, n);
+      if (m & bit) out[pos + __popc(m & below)] = n * 32 + lane;
+      pos += __popc(m);
+    }
   } else {
     uint16_t *out16 = reinterpret_cast<uint16_t *>(out);
-    // the word of key block J, listed by the query blocks in `flags`
-    auto word = [&](int J, int flags) { return (uint16_t)(J | flags << 10 | (p.ragged && J == p.nb - 1 ? 1 << 12 : 0)); };
-    int last = -1;  // the last listed block, in the lane that writes it
     const int D = sum(__popc(a & b));
-    int pos = prefix(__popc(a & b));
-    for (uint32_t m = a & b; m; m &= m - 1) {
-      const int J = lane * 32 + __ffs(m) - 1;
-      last = pos == U - 1 ? J : last;
-      out16[pos++] = word(J, 3);
-    }
-    int S[2] = {sum(__popc(a & ~b)), sum(__popc(b & ~a))};
-    int start = D, skip[2] = {0, 0};
-    if ((D & 1) && S[0] + S[1] > 0) {  // one single next to the last shared block; pairs start on a step
-      const int x = S[0] >= S[1] ? 0 : 1;
-      skip[x] = 1;
-      --S[x];
+    int S0 = sum(__popc(a & ~b)), S1 = sum(__popc(b & ~a));
+    int start = D;
+    int n_both = 0, n_a = 0, n_b = 0;  // blocks of each kind so far; the one that goes to D is number -1
+    if ((D & 1) && S0 + S1 > 0) {      // one single next to the last shared block; pairs start on a step
+      if (S0 >= S1) {
+        n_a = -1;
+        --S0;
+      } else {
+        n_b = -1;
+        --S1;
+      }
       ++start;
     }
-    const int paired = min(S[0], S[1]);
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      const uint32_t only = q ? b & ~a : a & ~b;
-      int k = prefix(__popc(only)) - skip[q];
-      for (uint32_t m = only; m; m &= m - 1, ++k) {
-        const int at = k < 0 ? D : k < paired ? start + 2 * k + q : start + paired + k;
-        const int J = lane * 32 + __ffs(m) - 1;
+    const int paired = min(S0, S1);
+    int last = -1;  // the last listed block, in the lane that writes it
+    for (unsigned todo = has; todo; todo &= todo - 1) {
+      const int n = __ffs(todo) - 1;
+      const uint32_t wa = __shfl_sync(0xffffffffu, a, n), wb = __shfl_sync(0xffffffffu, b, n);
+      const uint32_t both = wa & wb, only_a = wa & ~wb, only_b = wb & ~wa;
+      if ((wa | wb) & bit) {
+        const int J = n * 32 + lane, q = (only_b & bit) ? 1 : 0;
+        const int k = q ? n_b + __popc(only_b & below) : n_a + __popc(only_a & below);
+        const int at = (both & bit) ? n_both + __popc(both & below) : k < 0 ? D : k < paired ? start + 2 * k + q : start + paired + k;
+        const int flags = ((wa & bit) ? 1 : 0) | ((wb & bit) ? 2 : 0);
+        out16[at] = (uint16_t)(J | flags << 10 | (p.ragged && J == p.nb - 1 ? 1 << 12 : 0));
         last = at == U - 1 ? J : last;
-        out16[at] = word(J, 1 << q);
       }
+      n_both += __popc(both);
+      n_a += __popc(only_a);
+      n_b += __popc(only_b);
     }
     if ((U & 1) && last >= 0) out16[U] = (uint16_t)last;  // second half of the last step: the same block, without flags
   }
-  const unsigned has = __ballot_sync(0xffffffffu, any != 0u);
   const int src = has ? __ffs(has) - 1 : 0;
   const int first = __shfl_sync(0xffffffffu, lane * 32 + __ffs(any) - 1, src);
   __syncwarp();  // the first step, written by some lane, is read back
