@@ -811,13 +811,13 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
           const float2 lm = cluster_ld2(base[i] + off_l + row * 8);
           x[i] = cluster_ld4(base[i] + kOffK + row * 512 + ((lane ^ (row & 7)) << 4));
           l[i] = lm.x;
-          m[i] = lm.x > 0.f ? lm.y : kNoReference;
+          m[i] = lm.x != 0.f ? lm.y : kNoReference;
           m_all = fmaxf(m_all, m[i]);
         }
 #pragma unroll
         for (int i = 0; i < kMaxSplit; ++i) {
           if (i >= p.split) break;
-          if (l[i] > 0.f) {  // (a part without keys has zeros)
+          if (l[i] != 0.f) {  // (a part without keys has zeros; a sum that is not a number goes into the row's result)
             const float f = ex2(m[i] - m_all);
             l_all = fmaf(l[i], f, l_all);
             o.x = fmaf(x[i].x, f, o.x);
