@@ -152,6 +152,8 @@ int heart_predict_mask(const heart_config *cfg, const void *Q, const void *K, co
  *   For query token i of block I:  o_i = sum_j softmax_j(scale * <q_i,k_j>) v_j over the real keys
  *   (j < N) of the key blocks kv_idx[r,I,0..kv_cnt[r,I]).  bf16 in, fp32 accumulate, bf16 out (RNE).
  *   An empty list gives zeros (lse = -inf).  Rows i >= N are never written.
+ *   Unnormalised sums stay below 2^8 * (listed keys) * max |v|: finite for |v| up to 2^102 whatever the lists and the
+ *   logits.  Weights below 2^-102 of a row's largest may count as zero.
  *   lse [R, N] fp32 natural-log sum-exp of the scaled logits, or NULL.
  *   Lists must hold distinct block indices in [0, n_b); entries out of range are skipped and
  *   reported as HEART_ERR_DEVICE_CHECK through heart_get_status. */

@@ -26,7 +26,7 @@
 //   warp 8      issues S_g = Q K_g^T once step g - 2 has emptied the buffer, warp 11 O += P_g V_g.
 //   warp 9      V producer, warp 10 K and Q producer (draws the tiles and announces them): TMA loads
 //               (cp.async.bulk.tensor, 128-byte swizzle, completion on mbarriers), two 32 KB buffers each.
-// The reference: m_g = m_{g-1} unless the row's maximum of step g exceeds it by more than 2^64.  Each warp
+// The reference: m_g = m_{g-1} unless the row's maximum of step g exceeds it by more than 2^8.  Each warp
 // publishes the references of its 32 rows after the maximum of every step and reads those of the step
 // before; a row whose reference moved gets its part of O rescaled by the warp that moved it, once the
 // products of the steps before are complete, and both partners rescale their own row sums.
@@ -61,10 +61,12 @@ constexpr int kTileBytes = 32768;  // 128 rows x 128 dims: [2 dim halves][128 ro
 constexpr int kTileRing = 4;       // announced tiles
 constexpr int kTileReaders = 11;   // softmax warps, issuers, V producer
 constexpr float kNoReference = -3.0e38f;  // below every logit: the first step moves it
-// A row's reference moves when its maximum exceeds it by this much (log2).  Weights, sums and O are floating
-// point with 8 exponent bits throughout, so a scale of up to 2^64 costs no precision, and 2^17 such weights
-// leave room for values up to 2^46.  A move costs a rescale of O behind the products in flight.
-constexpr float kMaxGrowth = 64.f;
+// A row's reference is set kHeadroom (log2) above the row's maximum, and moves when a maximum exceeds it by kMaxGrowth.
+// A move costs a rescale of O behind the products in flight, so a row should climb far before its next one: 40 x 33k
+// takes 3.47 ms if it moves 2^8 above the last maximum, 2.77 at 2^16, 2.69 at 2^24 and beyond.  Most of the room lies
+// below 1: weights are at most 2^8, so n keys with values up to 2^120 / n cannot overflow O (all of it above 1, with
+// weights up to 2^64, left 2^64 / n), and a weight of 2^-110 of the largest is still a normal number.
+constexpr float kHeadroom = 16.f, kMaxGrowth = 8.f;
 constexpr int kMaxSplit = 4;  // CTAs that share a tile in a small launch
 
 // Shared-memory plan (the dynamic allocation itself is 1024-byte aligned).
@@ -591,7 +593,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
         // used so far (some row).
         auto new_reference = [&](float x_max) -> bool {
           const bool grow = x_max > m_prev + kMaxGrowth;
-          const float m_new = grow ? x_max : m_prev;
+          const float m_new = grow ? x_max + kHeadroom : m_prev;
           sh.m[w][row] = m_new;
           __syncwarp();
           if (lane == 0) mbar_arrive(&sh.m_ready[w][quarter]);

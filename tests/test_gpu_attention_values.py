@@ -4,7 +4,9 @@ import numpy as np
 import pytest
 import torch
 
-from parity import to_np
+from paper_2605_14513_b200 import inputs
+
+from parity import check_attention, to_np
 
 pytestmark = pytest.mark.gpu
 
@@ -47,3 +49,47 @@ def test_a_value_that_is_not_a_number_reaches_the_rows_that_use_it_and_no_others
         hit[0] = True if dense else (np.arange(N) // block) % 2 == 0
         assert np.isnan(On[hit]).all() and not np.isfinite(lse_n[hit]).any()
         assert np.array_equal(On[~hit], O[~hit]) and np.array_equal(lse_n[~hit], lse[~hit])
+
+
+def staircase(rs, H, N, v_scale=1.0):
+    """Q, K, V whose rows see their maximum climb and fall from one key step to the next by amounts on both sides of
+    those at which the kernel moves a row's reference, in 64 patterns a head that are dealt to the rows at random.
+    Pattern c of a row is read off dims c and c + 64 of the keys (a coarse and a fine part of the logit)."""
+    levels = rs.uniform(-60, 60, (H, 64, 1)) + np.cumsum(
+        rs.choice([-40, -5, -1, 0, 1, 2, 3, 5, 7, 9, 29, 31, 33, 61], (H, 64, (N + 63) // 64),
+                  p=[.04, .08, .1, .1, .1, .1, .1, .08, .05, .05, .05, .05, .05, .05]), axis=2)
+    logit = (np.repeat(levels, 64, axis=2)[:, :, :N] - rs.uniform(0, 3, (H, 64, N))) * np.log(2.0)
+    logit = torch.from_numpy(np.moveaxis(logit, 1, 2).copy())  # [H, N, 64]
+    coarse = logit.to(torch.bfloat16)
+    K = torch.cat([coarse, (logit - coarse.double()).to(torch.bfloat16)], dim=2)
+    pattern = torch.from_numpy(rs.randint(0, 64, (H, N, 1)))
+    Q = torch.zeros((H, N, 128), dtype=torch.bfloat16)
+    Q.scatter_(2, pattern, 1.0)
+    Q.scatter_(2, pattern + 64, 1.0)
+    V = (torch.from_numpy(rs.standard_normal((H, N, 128))) * v_scale).to(torch.bfloat16)
+    return tuple(x[None].cuda().contiguous() for x in (Q, K, V))
+
+
+@pytest.mark.parametrize("block", [64, 128])
+@pytest.mark.parametrize("v_scale", [1.0, 2.0 ** 100])
+@pytest.mark.parametrize("H,N", [(2, 2045), (4, 1029), (8, 1000), (12, 1700)])
+def test_row_maxima_that_climb_from_step_to_step(oracle, block, v_scale, H, N):
+    """Contributions from before a move of the reference still count after it (a maximum that climbs by 31 and then by
+    2 powers of two, say), the moves fall on even and odd key steps of rows next to each other, and values of V near
+    the top of the range do not overflow on the way: a result is a mean of them."""
+    from paper_2605_14513_b200 import heart
+
+    rs = np.random.RandomState(H * N + block)
+    Q, K, V = staircase(rs, H, N, v_scale)
+    nb = heart.n_blocks(N, block)
+    idx, cnt = np.zeros((H, nb, nb), np.int32), np.zeros((H, nb), np.int32)
+    for r in range(H):
+        for I in range(nb):
+            sel = np.sort(rs.permutation(nb)[: rs.choice([nb, nb - 1, (nb + 1) // 2])])
+            cnt[r, I], idx[r, I, : len(sel)] = len(sel), sel
+    O, lse = attend(heart, heart.make_config(1, H, N, block, scale=1.0), Q, K, V, (torch.from_numpy(idx).cuda(), torch.from_numpy(cnt).cuda()))
+    ref, lse_ref = oracle.block_sparse_attn(*(inputs.bits(t) for t in (Q, K, V)), block, idx, cnt, scale=1.0, want_lse=True)
+    ref, lse_ref = np.asarray(ref).reshape(H, N, 128), np.asarray(lse_ref).reshape(H, N)
+    check_attention(O.astype(np.float64) / v_scale, ref / v_scale)
+    # fp32 scores up to 2^10 (2^-14) and bf16-rounded weights (2^-9 relative each) in the sum behind the logarithm
+    assert np.allclose(lse, lse_ref, rtol=0, atol=2.0 ** -8)
