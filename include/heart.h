@@ -91,14 +91,18 @@ typedef struct {
 } heart_state;
 
 /* Bytes of scratch every compute call needs (block means, token means, flags, status
- * word, and the pooled scores of the mask predictor: 8 * R * n_b * roundup(n_b, 32) bytes,
+ * words; the plan of the attention call, 32 + 2 * n_b (block 64) or 32 + 4 * n_b bytes for each of the
+ * R * ceil(N / 128) tiles; the pooled scores of the mask predictor: 8 * R * n_b * roundup(n_b, 32) bytes,
  * by far the largest part; with HEART_ESTIMATOR_ANTIDIAG in cfg->flags another
  * 8 * R * floor(N / 16) * n_b bytes).  Host-only; returns 0 for an invalid or unsupported config.
- * The caller allocates it once (256-byte aligned) and zero-fills it before first use. */
+ * The caller allocates it once (256-byte aligned) and zero-fills it before first use.
+ * A workspace serves one call at a time: calls that share one are ordered, by a stream or by events.  What may
+ * overlap all the same is heart_block_sparse_attn with one of heart_drift and heart_predict_mask: it touches
+ * the status words and its plan only, they touch neither but to report an error. */
 size_t heart_workspace_bytes(const heart_config *cfg /* host */);
 
-/* The leading part of that workspace which heart_drift alone reads and writes (everything
- * but the pooled scores).  A caller that only ever calls heart_drift may allocate just this
+/* The leading part of that workspace without the pooled scores: all that heart_drift reads and writes
+ * lies in it.  A caller that only ever calls heart_drift may allocate just this
  * much.  Host-only; 0 for an invalid or unsupported config. */
 size_t heart_drift_workspace_bytes(const heart_config *cfg /* host */);
 
@@ -205,7 +209,7 @@ int heart_step_host(const heart_config *cfg, const void *Q_host, const void *K_h
  *
  * Same arguments, results and error codes as heart_drift (an invalid cfg gives heart_drift's code), except:
  *   - no `workspace`; st->mask_bits / kv_idx / kv_cnt may be NULL (they are not touched);
- *   - a shape whose heart_drift_workspace_bytes exceeds HEART_STATIC_SCRATCH_BYTES is rejected with
+ *   - a shape whose drift scratch (block means and what goes with them) exceeds HEART_STATIC_SCRATCH_BYTES is rejected with
  *     HEART_ERR_TOO_LARGE before anything is launched;
  *   - the per-block means it leaves behind are in the built-in array, not in a caller workspace,
  *     so a following heart_predict_mask recomputes them (it always does).

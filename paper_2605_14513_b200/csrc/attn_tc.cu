@@ -949,12 +949,10 @@ cudaError_t launch_bk(const Geom &g, const Workspace &w, const CUtensorMap &mq, 
   cudaError_t e;
   const int n_heads = g.B * prm.hcount;
   prm.n_tiles = n_heads * prm.n_tiles_per_head;
-  // the plan lives where the pooled scores of the mask predictor were: four words per tile in plan order and in
-  // launch order, [R][tiles][steps]
   const size_t all_tiles = (size_t)g.R * prm.n_tiles_per_head;
-  uint4 *tiles = reinterpret_cast<uint4 *>(w.scores), *order = tiles + all_tiles;
+  uint4 *tiles = static_cast<uint4 *>(w.plan), *order = tiles + all_tiles;
   uint32_t *steps = reinterpret_cast<uint32_t *>(order + all_tiles);
-  prm.step_pitch = B == 128 ? g.nb : (g.nb + 1) / 2;
+  prm.step_pitch = (int)plan_steps_per_tile(g);
   prm.steps = steps;
   prm.tiles = tiles;
   PlanParams plan = {};

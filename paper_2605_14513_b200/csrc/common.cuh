@@ -35,24 +35,30 @@ __host__ inline void set_chunks(Geom &g) {
   g.nchunks = (g.nb + g.bpc - 1) / g.bpc;
 }
 
+// Plan of an attention call: two words of 16 bytes per 128-row tile (in plan and in launch order) and the tile's key
+// steps, 4 bytes each (one or two key blocks).
+__host__ inline size_t plan_steps_per_tile(const Geom &g) { return g.block == 128 ? g.nb : (g.nb + 1) / 2; }
+__host__ inline size_t plan_bytes(const Geom &g) { return (size_t)g.R * ((g.N + 127) / 128) * (32 + 4 * plan_steps_per_tile(g)); }
+
 // Workspace layout (all offsets 256-byte aligned).
 struct Workspace {
   int32_t *status;    // [64]   word 0: sticky device-check code; word 1: detail; word 8: ticket counter
                       //        of the drift kernel (zero between launches); words 10-11: signature of
                       //        the (Q, K, shape) whose block means the workspace holds (0: none); word 12:
-                      //        tiles that the streams of an attention launch have drawn
+                      //        tiles of an attention launch drawn beyond the first one of every CTA
   double *bmean;      // [2][R][nb][D]  per-block (pooled) means of Q (0) and K (1)
   double *psum;       // [2][R][nchunks][D]  per-CTA partial token sums
   double *mean;       // [2][R][D]      token means of the current step
   uint8_t *pre;       // [R]            head-wise decision before the gate
   uint8_t *refresh;   // [R]            final decision of the current step
   double *drift;      // [R]
-  double *scores;     // [R][nb][pitch] pooled scores of the refreshed heads, pitch = nb rounded up to 32;
-                      //        afterwards the plan of the attention launch (two times four words and the steps per tile: at
-                      //        most 4 n_b + 32 bytes per query block, against 8 pitch >= 256)
+  void *plan;         // of an attention call, which besides it touches the status words only (a mask prediction for
+                      // another layer may run beside it): two times four words per tile, [R][tiles][steps]
+  double *scores;     // [R][nb][pitch] pooled scores of the refreshed heads, pitch = nb rounded up to 32
   void *pairs;        // strided antidiagonal estimator only (HEART_ESTIMATOR_ANTIDIAG in the flags):
                       // float2 [R][N/16][nb], a (max, sum) pair per (query group, key block)
-  size_t bytes_drift;  // what heart_drift alone touches (everything above `scores`)
+  size_t bytes_drift;      // what heart_drift alone touches (everything above `plan`)
+  size_t bytes_no_scores;  // everything above `scores`
   size_t bytes;
 };
 
@@ -77,6 +83,9 @@ __host__ inline Workspace carve(const Geom &g, void *base) {
   w.drift = reinterpret_cast<double *>(p + off);
   off += align256(sizeof(double) * (size_t)g.R);
   w.bytes_drift = off;
+  w.plan = p + off;
+  off += align256(plan_bytes(g));
+  w.bytes_no_scores = off;
   w.scores = reinterpret_cast<double *>(p + off);
   off += align256(sizeof(double) * (size_t)g.R * g.nb * (size_t)(((g.nb + 31) / 32) * 32));
   w.pairs = p + off;

@@ -43,11 +43,11 @@ int heart_drift_static(const heart_config *cfg, const void *Q, const void *K, co
                        heart_state *st, double *drift_out, uint8_t *refresh_out, heart_stream_t stream) {
   if (cfg == nullptr) return HEART_ERR_INVALID;
   // Size check first, from the same accounting the caller-allocated path uses (the part of the
-  // workspace that the drift kernels touch: the pooled-score area of the mask predictor lies behind it).
+  // workspace that the drift kernels touch: the attention plan and the pooled scores lie behind it).
   Geom geom;
   const int shape_rc = make_geom(cfg, &geom);
   if (shape_rc != HEART_OK) return shape_rc;  // the code heart_drift gives for this cfg
-  const size_t need = heart_drift_workspace_bytes(cfg);
+  const size_t need = carve(geom, nullptr).bytes_drift;
   if (need > (size_t)HEART_STATIC_SCRATCH_BYTES) return HEART_ERR_TOO_LARGE;
   if (!Q || !K || !delta || !st || !st->anchor_q || !st->anchor_k || !st->has_anchor) return HEART_ERR_INVALID;
   if ((reinterpret_cast<uintptr_t>(Q) & 15u) || (reinterpret_cast<uintptr_t>(K) & 15u)) return HEART_ERR_INVALID;

@@ -99,7 +99,7 @@ size_t heart_workspace_bytes(const heart_config *cfg) {
 size_t heart_drift_workspace_bytes(const heart_config *cfg) {
   Geom g;
   if (make_geom(cfg, &g) != HEART_OK) return 0;
-  return carve(g, nullptr).bytes_drift;
+  return carve(g, nullptr).bytes_no_scores;
 }
 
 int heart_state_reset(const heart_config *cfg, heart_state *st, heart_stream_t stream) {
