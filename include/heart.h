@@ -97,8 +97,9 @@ typedef struct {
  * 8 * R * floor(N / 16) * n_b bytes).  Host-only; returns 0 for an invalid or unsupported config.
  * The caller allocates it once (256-byte aligned) and zero-fills it before first use.
  * A workspace serves one call at a time: calls that share one are ordered, by a stream or by events.  What may
- * overlap all the same is heart_block_sparse_attn with one of heart_drift and heart_predict_mask: it touches
- * the status words and its plan only, they touch neither but to report an error. */
+ * overlap all the same is heart_block_sparse_attn with one of heart_drift and heart_predict_mask (it touches
+ * the status words and its plan only, they touch neither but to report an error), and heart_block_sparse_attn
+ * calls of which at most one has lists (under HEART_FORCE_DENSE it writes the status word alone, on errors). */
 size_t heart_workspace_bytes(const heart_config *cfg /* host */);
 
 /* The leading part of that workspace without the pooled scores: all that heart_drift reads and writes

@@ -429,9 +429,11 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
         nx.z = p.h0 + (int)t.y - nx.w * p.hcount;
         if (Small && n_steps_of(nx.y) > 0) e = step_entry(steps_of(nx), 0);
       };
-      // the first tile of every CTA is fixed, the others are drawn (a small launch has no others)
-      fetch(Small ? blockIdx.x / p.split : blockIdx.x);
-      auto draw = [&]() { fetch(Small ? p.n_tiles : gridDim.x + atomicAdd(p.counter, 1)); };
+      // The first tile of every CTA is fixed, the others are drawn (a small launch has no others).  Dense tiles are all
+      // of one length: dealt in turn, so that dense calls share nothing and may overlap on one workspace.
+      int mine = Small ? blockIdx.x / p.split : blockIdx.x;
+      fetch(mine);
+      auto draw = [&]() { fetch(Small ? p.n_tiles : p.dense ? mine += gridDim.x : gridDim.x + atomicAdd(p.counter, 1)); };
       for (int t = 0;; ++t) {
         const int i = t % kTileRing;
         if (t >= kTileRing) ok = mbar_wait(&sh.tile_empty[i], (t / kTileRing - 1) & 1, abort);
@@ -979,17 +981,16 @@ cudaError_t launch_bk(const Geom &g, const Workspace &w, const CUtensorMap &mq, 
     return launch_pdl(attn_tc_kernel<B, true>, dim3(prm.n_tiles * prm.split), dim3(kAttnThreads), kAttnSmem, s, Cluster{prm.split}, mq, mk,
                       mv, prm, plan);
   }
-  const int planned = prm.dense ? 0 : prm.n_tiles;  // (dense: the kernel only zeroes the counter)
-  e = launch_pdl(attn_plan_kernel<B>, dim3(planned ? (planned + kPlanWarps - 1) / kPlanWarps : 1), dim3(32 * kPlanWarps), 0, s, plan,
-                 planned, prm.step_pitch, steps, tiles, prm.counter);
-  if (e != cudaSuccess) return e;
-  ++*launches;
-  if (planned) {
+  if (!prm.dense) {
+    e = launch_pdl(attn_plan_kernel<B>, dim3((prm.n_tiles + kPlanWarps - 1) / kPlanWarps), dim3(32 * kPlanWarps), 0, s, plan, prm.n_tiles,
+                   prm.step_pitch, steps, tiles, prm.counter);
+    if (e != cudaSuccess) return e;
+    ++*launches;
     // K + V of one head beyond 32 MB (about half of one die's share of the L2): order by key locality
     const int by_first_key = (size_t)g.N * kD * 2 * 2 > (size_t)(32u << 20) ? 1 : 0;
     const int tail_heads = 1024 / prm.n_tiles_per_head;  // (a head has at most 1024 tiles)
     const int heads = n_heads > tail_heads ? n_heads - tail_heads : 0;
-    e = launch_pdl(tile_order_kernel, dim3(heads + 1), dim3(1024), 0, s, (const uint4 *)tiles, planned, prm.n_tiles_per_head, by_first_key, order);
+    e = launch_pdl(tile_order_kernel, dim3(heads + 1), dim3(1024), 0, s, (const uint4 *)tiles, prm.n_tiles, prm.n_tiles_per_head, by_first_key, order);
     if (e != cudaSuccess) return e;
     ++*launches;
     prm.tiles = order;

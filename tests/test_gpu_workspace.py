@@ -1,5 +1,5 @@
 """What a call leaves alone in the workspace: a mask prediction for one layer may run on a second stream beside the
-attention of another on the same workspace."""
+attention of another on the same workspace, and so may a dense attention."""
 import numpy as np
 import pytest
 import torch
@@ -79,3 +79,31 @@ def test_mask_prediction_beside_attention_on_one_workspace(block):
         assert heart.heart_get_status(ws) == 0
         assert torch.equal(O.view(torch.int16), want.view(torch.int16))
         assert torch.equal(st.kv_cnt, st_want.kv_cnt) and torch.equal(st.mask_bits, st_want.mask_bits)
+
+
+@pytest.mark.parametrize("block", [64, 128])
+def test_dense_attention_beside_attention_on_one_workspace(block):
+    from paper_2605_14513_b200 import heart
+
+    H, N = 8, 8100
+    Q, K, V = tensors(H, N, 3)
+    idx, cnt = lists(np.random.RandomState(1), H, heart.n_blocks(N, block), 0.5)
+    cfg, dense = heart.make_config(1, H, N, block), heart.make_config(1, H, N, block, flags=heart.FORCE_DENSE)
+    ws = heart.new_workspace(cfg)
+    want, want_dense = torch.empty_like(Q), torch.empty_like(Q)
+    heart.heart_block_sparse_attn(dense, Q, K, V, None, None, want_dense, ws)
+    assert not ws.any()  # nothing is kept there, so nothing can be in another call's way
+    heart.heart_block_sparse_attn(cfg, Q, K, V, idx, cnt, want, ws)
+    torch.cuda.synchronize()
+    side = [torch.cuda.Stream() for _ in range(2)]
+    for _ in range(5):
+        O, dense_out = torch.empty_like(Q), [torch.empty_like(Q) for _ in side]
+        torch.cuda.synchronize()
+        heart.heart_block_sparse_attn(cfg, Q, K, V, idx, cnt, O, ws)
+        for s, out in zip(side, dense_out):
+            with torch.cuda.stream(s):
+                heart.heart_block_sparse_attn(dense, Q, K, V, None, None, out, ws)
+        torch.cuda.synchronize()
+        assert heart.heart_get_status(ws) == 0
+        assert torch.equal(O.view(torch.int16), want.view(torch.int16))
+        assert all(torch.equal(out.view(torch.int16), want_dense.view(torch.int16)) for out in dense_out)
