@@ -10,8 +10,8 @@
 // largest element whose ">=" mass still reaches tau * z.  It decides in fp32 first: weights
 // e = 2^((s - max) log2 e), a few rounds that narrow the threshold down, then a direct evaluation over the few blocks
 // left.  That is final when the mass misses tau * z by more than 1.5e-5 z on both sides of the cut (the
-// errors of weights and sums stay below 1.2e-5 z, derived at the kernel) and no other block shares the
-// threshold's fp32 value; otherwise (a few rows in a hundred) the row is decided in fp64: e = exp(s - max) and a search
+// errors of weights and sums stay below 1.2e-5 z, derived at the kernel) and no other block may share the
+// threshold's weight; otherwise (a few rows in a hundred) the row is decided in fp64: e = exp(s - max) and a search
 // over the IEEE-754 pattern of e (positive doubles order like their bit patterns), starting below the
 // leading bits that the largest and the smallest weight share, two bits a round over all blocks down to
 // bit 48, the rest directly over the few blocks that share that prefix.  So the integer outputs (bit
@@ -32,6 +32,10 @@ template <int NJ>
 constexpr int kRowsPerCta = NJ >= 24 ? 2 : 8;
 constexpr int kMaxCand = 64;    // candidates the direct threshold evaluation takes
 constexpr float kMassBand = 1.5e-5f;  // of z: cuts whose mass is closer to tau * z are decided in fp64
+// Blocks are ranked by their weight, lowest index first among equals.  Weights exp(s - max) round to the same double
+// where s - max differ by less than 2^-52, and the fp32 value of s - max may then be the same or one step off: a cut with
+// another block within two steps of fp32 or 2^-51 is decided in fp64.
+constexpr float kTieRel = 2.38418579e-7f, kTieAbs = 4.44089210e-16f;  // 2^-22, 2^-51
 
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
@@ -308,13 +312,14 @@ __global__ void __launch_bounds__(32 * kRowsPerCta<NJ>) top_p_kernel(const doubl
           if (k * 32 >= n_cand) break;
           const bool have = lane + 32 * k < n_cand;
           const float xk = have ? cx[lane + 32 * k] : 0.f, ek = have ? ce[lane + 32 * k] : 0.f;
+          const float near = fmaf(fabsf(xk), kTieRel, kTieAbs);  // (with the interval's ends: no block outside is as near)
           float above = m_hi;
           int same = 0;
           for (int n = 0; n < n_cand; ++n) {
             above += cx[n] > xk ? ce[n] : 0.f;
-            same += cx[n] == xk ? 1 : 0;
+            same += fabsf(cx[n] - xk) <= near ? 1 : 0;
           }
-          if (have && same == 1 && t - above > band && above + ek - t > band) found = true, x_cut = xk;
+          if (have && same == 1 && xk - near >= lo && xk + near < hi && t - above > band && above + ek - t > band) found = true, x_cut = xk;
         }
         const unsigned who = __ballot_sync(0xffffffffu, found);
         if (__popc(who) == 1) {

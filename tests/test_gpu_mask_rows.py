@@ -31,3 +31,31 @@ def test_thresholds_next_to_a_cumulative_mass(oracle, nb, H):
     oracle.predict_mask(p.Qb, p.Kb, wl.block, tau, p.ost)
     # fp64 on both sides: cuts 1e-9 apart are told apart
     assert check_masks(p.gst, p.ost, range(H), tau, p.probs_row) == 0
+
+
+@pytest.mark.parametrize("base,step", [(0.0, 2.0 ** -57), (0.0, 2.0 ** -54), (0.75, 2.0 ** -53), (0.75, 2.0 ** -49)])
+@pytest.mark.parametrize("nb", [4, 40, 600])
+def test_scores_a_rounding_apart(oracle, base, step, nb):
+    """Scores base + {0 .. 3} * step: where exp(score - max) is the same double the lowest index comes first, although
+    the fp32 values of score - max differ; where it is not, the larger score does."""
+    from paper_2605_14513_b200 import heart
+
+    rs = np.random.RandomState(nb)
+    times = rs.randint(0, 4, nb)
+    times[:4] = [0, 1, 2, 0]
+    N = 64 * nb
+    K = torch.zeros((1, 1, nb, 64, 128))
+    K[..., 0] = base
+    K[..., 1] = torch.from_numpy(times * step).float()[None, None, :, None]
+    K = K.view(1, 1, N, 128).to(torch.bfloat16).cuda()
+    Q = torch.zeros((1, 1, N, 128))
+    Q[..., :2] = 1.0
+    Q = Q.to(torch.bfloat16).cuda()
+    cfg = heart.make_config(1, 1, N, 64, scale=1.0)
+    # (weights equal to 1e-14: cuts lie near k / nb, where a mass is within rounding of tau; these stay 2e-4 away)
+    for tau in (0.3137, 0.4231, 0.7139, 0.9173):
+        st, ost, ws = heart.State(cfg), oracle.State(1, 1, N, 128, 64), heart.new_workspace(cfg)
+        heart.heart_predict_mask(cfg, Q, K, torch.tensor([tau], dtype=torch.float64, device="cuda"), st, ws)
+        oracle.predict_mask(inputs.bits(Q), inputs.bits(K), 64, np.array([tau]), ost, scale=1.0)
+        assert np.array_equal(st.kv_cnt.cpu().numpy(), ost.kv_cnt)
+        assert np.array_equal(st.mask_bits.cpu().numpy().view(np.uint32), ost.mask_bits)
