@@ -34,8 +34,9 @@ constexpr int kMaxCand = 64;    // candidates the direct threshold evaluation ta
 constexpr float kMassBand = 1.5e-5f;  // of z: cuts whose mass is closer to tau * z are decided in fp64
 // Blocks are ranked by their weight, lowest index first among equals.  Weights exp(s - max) round to the same double
 // where s - max differ by less than 2^-52, and the fp32 value of s - max may then be the same or one step off: a cut with
-// another block within two steps of fp32 or 2^-51 is decided in fp64.
-constexpr float kTieRel = 2.38418579e-7f, kTieAbs = 4.44089210e-16f;  // 2^-22, 2^-51
+// another block within a step of fp32 or 2^-51 is decided in fp64.  (One such row costs a launch of a few waves 10 us:
+// 2^-22, two to three steps, sent one row in 20000 of nearly equal scores there.)
+constexpr float kTieRel = 1.19209290e-7f, kTieAbs = 4.44089210e-16f;  // 2^-23, 2^-51
 
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
