@@ -294,6 +294,9 @@ __global__ void __launch_bounds__(32 * kRowsPerCta<NJ>) top_p_kernel(const doubl
         }
         __syncwarp();
         if (n_cand <= kMaxCand) break;
+        // More than the direct evaluation takes.  Equal ones (the first 64, at least) are left to fp64 at once: quarters do
+        // not part them (12 rounds on rows of equal scores: 1147 us for 22296 of 929, 852 now; fp64 alone, before: 902).
+        if (__all_sync(0xffffffffu, cx[lane] == cx[0] && cx[lane + 32] == cx[0])) break;
         float a1 = 0.f, a2 = 0.f, a3 = 0.f;
 #pragma unroll 4
         for (int k = lane; k < n_list; k += 32) {

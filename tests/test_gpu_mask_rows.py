@@ -59,3 +59,31 @@ def test_scores_a_rounding_apart(oracle, base, step, nb):
         oracle.predict_mask(inputs.bits(Q), inputs.bits(K), 64, np.array([tau]), ost, scale=1.0)
         assert np.array_equal(st.kv_cnt.cpu().numpy(), ost.kv_cnt)
         assert np.array_equal(st.mask_bits.cpu().numpy().view(np.uint32), ost.mask_bits)
+
+
+@pytest.mark.parametrize("nb", [3, 64, 65, 130, 700])
+def test_rows_of_equal_scores(oracle, nb):
+    """All blocks equal, all but one, half of them, and equal ones below the cut: more than 64 candidates that no
+    threshold parts."""
+    from paper_2605_14513_b200 import heart
+
+    N = 64 * nb
+    rs = np.random.RandomState(nb)
+    score = np.zeros((4, nb))
+    score[1, nb // 2] = 3.0
+    score[2, rs.permutation(nb)[: nb // 2]] = 1.5
+    score[3] = np.where(np.arange(nb) % 3 == 0, -2.0, rs.uniform(-1, 1, nb))
+    K = torch.zeros((1, 4, nb, 64, 128))
+    K[..., 0] = torch.from_numpy(score).float()[None, :, :, None]
+    K = K.view(1, 4, N, 128).to(torch.bfloat16).cuda()
+    Q = torch.zeros((1, 4, N, 128))
+    Q[..., 0] = 1.0
+    Q = Q.to(torch.bfloat16).cuda()
+    cfg = heart.make_config(1, 4, N, 64, scale=1.0)
+    for tau in (0.0137, 0.3137, 0.7139, 0.9773):  # (not within rounding of k / nb, where the mass of equal blocks is)
+        tau = np.full(4, tau)
+        st, ost, ws = heart.State(cfg), oracle.State(1, 4, N, 128, 64), heart.new_workspace(cfg)
+        heart.heart_predict_mask(cfg, Q, K, torch.from_numpy(tau).cuda(), st, ws)
+        oracle.predict_mask(inputs.bits(Q), inputs.bits(K), 64, tau, ost, scale=1.0)
+        assert np.array_equal(st.kv_cnt.cpu().numpy(), ost.kv_cnt)
+        assert np.array_equal(st.mask_bits.cpu().numpy().view(np.uint32), ost.mask_bits)
