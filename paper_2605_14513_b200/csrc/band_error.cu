@@ -83,13 +83,14 @@ struct AxisArgs {
   const float *ys, *yd;   // pass 0: err = ys - yd
   const double2 *table;   // of this axis
   double *dst;            // passes 0, 1: coefficients, c_0 .. c_{n/2}, s_1 .. in place of the samples
-  double *partial;        // pass 0: |y_dense|^2 per CTA; pass 2: [CTA][4] energies
+  double *partial;        // pass 0: |y_dense|^2 per CTA of the first frequencies; pass 2: [CTA][4] energies
   unsigned lines, inner;  // (their product with n is at most 2^31)
   int n;
   int ny, nx;             // pass 2: lengths of the other axes (inner = ny * nx)
 };
 
-// One pass over an axis of a [outer, n, inner] view; a CTA takes lines_per_cta(n) of the outer * inner lines.
+// One pass over an axis of a [outer, n, inner] view; a CTA takes lines_per_cta(n) of the outer * inner lines and, of their
+// rounds of 8 * frequency_warps(n) frequencies, every gridDim.y-th.
 template <int PASS>
 __global__ void __launch_bounds__(kBandThreads, 8) axis_kernel(const AxisArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -162,7 +163,7 @@ __global__ void __launch_bounds__(kBandThreads, 8) axis_kernel(const AxisArgs a)
   __syncthreads();
   double energy[4] = {0.0, 0.0, 0.0, 0.0};  // LL, LH, HL, HH
   const int jl = lane & 3, kl = lane >> 2, line0 = warp / fw * kLines;
-  for (int kg = 0; kg <= h; kg += 8 * fw) {  // a warp: 8 frequencies of its 16 lines
+  for (int kg = 8 * fw * blockIdx.y; kg <= h; kg += 8 * fw * gridDim.y) {  // a warp: 8 frequencies of its 16 lines
     const int k0 = kg + 8 * (warp % fw), k = k0 + kl;
     double c[kLines / 8][2], s[kLines / 8][2];
 #pragma unroll
@@ -223,13 +224,13 @@ __global__ void __launch_bounds__(kBandThreads, 8) axis_kernel(const AxisArgs a)
     cta_sums<4>(energy, red);
     if (tid == 0) {
 #pragma unroll
-      for (int b = 0; b < 4; ++b) a.partial[(size_t)blockIdx.x * 4 + b] = energy[b];
+      for (int b = 0; b < 4; ++b) a.partial[((size_t)blockIdx.y * gridDim.x + blockIdx.x) * 4 + b] = energy[b];
     }
   }
   if (PASS == 0) {
     double v[1] = {dense};
     cta_sums<1>(v, red);
-    if (tid == 0) a.partial[blockIdx.x] = v[0];
+    if (tid == 0 && blockIdx.y == 0) a.partial[blockIdx.x] = v[0];
   }
 }
 
@@ -274,6 +275,15 @@ __global__ void __launch_bounds__(1024) band_final_kernel(const double *__restri
 
 size_t n_ctas(long long lines, int n) { return (size_t)((lines + lines_per_cta(n) - 1) / lines_per_cta(n)); }
 
+// CTAs that share the frequencies of a set of lines: as many as there are rounds, while lines alone leave SMs without a
+// CTA.  (One line of 4096 samples, 65 rounds over 13 chunks: 6466 us in one CTA.)
+int frequency_splits(long long lines, int n) {
+  const size_t ctas = n_ctas(lines, n), per_round = 8 * frequency_warps(n), rounds = (n / 2 + per_round) / per_round;
+  return ctas >= 148 ? 1 : (int)(rounds < 296 / ctas ? rounds : 296 / ctas);
+}
+// CTAs of the pass over t: each leaves four sums.
+size_t n_energies(int C, int T, int H, int W) { return n_ctas((long long)C * H * W, T) * frequency_splits((long long)C * H * W, T); }
+
 template <int PASS>
 cudaError_t launch_axis(const AxisArgs &a, cudaStream_t s) {
   const size_t smem = sizeof(double) * 2 * fold_layout(a.n, a.inner == 1).doubles + (a.n <= kMaxSharedTable ? sizeof(double2) * a.n : 0);
@@ -281,7 +291,8 @@ cudaError_t launch_axis(const AxisArgs &a, cudaStream_t s) {
   static std::atomic<unsigned long long> done{0};
   cudaError_t e = allow_shared_memory(axis_kernel<PASS>, kMost, done);
   if (e != cudaSuccess) return e;
-  return launch_pdl(axis_kernel<PASS>, dim3((unsigned)n_ctas(a.lines, a.n)), dim3(kBandThreads), smem, s, a);
+  const dim3 grid((unsigned)n_ctas(a.lines, a.n), (unsigned)frequency_splits(a.lines, a.n));
+  return launch_pdl(axis_kernel<PASS>, grid, dim3(kBandThreads), smem, s, a);
 }
 
 }  // namespace
@@ -289,7 +300,7 @@ cudaError_t launch_axis(const AxisArgs &a, cudaStream_t s) {
 size_t band_error_workspace_bytes(int C, int T, int H, int W) {
   const size_t n = (size_t)C * T * H * W;
   return align256(sizeof(double2) * ((size_t)T + H + W)) + 2 * align256(sizeof(double) * n) +
-         align256(sizeof(double) * 4 * n_ctas((long long)C * H * W, T)) + align256(sizeof(double) * n_ctas((long long)C * T * H, W));
+         align256(sizeof(double) * 4 * n_energies(C, T, H, W)) + align256(sizeof(double) * n_ctas((long long)C * T * H, W));
 }
 
 cudaError_t launch_band_error(const float *ys, const float *yd, int C, int T, int H, int W, const double *weights,
@@ -303,7 +314,7 @@ cudaError_t launch_band_error(const float *ys, const float *yd, int C, int T, in
   double *Bm = reinterpret_cast<double *>(p);
   p += align256(sizeof(double) * n);
   double *energies = reinterpret_cast<double *>(p);
-  p += align256(sizeof(double) * 4 * n_ctas((long long)C * H * W, T));
+  p += align256(sizeof(double) * 4 * n_energies(C, T, H, W));
   double *dense = reinterpret_cast<double *>(p);
   trig_tables_kernel<<<(unsigned)(((long long)T + H + W + 127) / 128), 128, 0, s>>>(W, H, T, tables);
   cudaError_t e = cudaGetLastError();
@@ -336,7 +347,7 @@ cudaError_t launch_band_error(const float *ys, const float *yd, int C, int T, in
   a.ny = H;
   a.nx = W;
   if ((e = launch_axis<2>(a, s)) != cudaSuccess) return e;
-  e = launch_pdl(band_final_kernel, dim3(1), dim3(1024), 0, s, (const double *)energies, (long long)n_ctas((long long)C * H * W, T),
+  e = launch_pdl(band_final_kernel, dim3(1), dim3(1024), 0, s, (const double *)energies, (long long)n_energies(C, T, H, W),
                  (const double *)dense, (long long)n_ctas((long long)C * T * H, W), (double)T * H * W, weights[0], weights[1],
                  weights[2], weights[3], eps, out);
   *launches += 5;

@@ -21,3 +21,9 @@ def test_band_error_axes(oracle, shape):
     # fp64 sums of at most n terms a pass: 1e-12 of the total covers n = 1030 with a wide margin
     assert np.allclose(out[1:5], bands, rtol=1e-9, atol=1e-12 * bands.sum())
     assert np.isclose(out[5], denom, rtol=1e-12) and np.isclose(out[0], e, rtol=1e-9)
+
+
+@pytest.mark.parametrize("shape", [(1, 1, 1, 4097), (5, 700, 2, 3), (1, 3, 2048, 1), (146, 1, 64, 65)])
+def test_few_long_lines(oracle, shape):
+    """Axes whose lines are fewer than the SMs: CTAs share their frequencies (one to 65 shares of them, uneven ones)."""
+    test_band_error_axes(oracle, shape)
