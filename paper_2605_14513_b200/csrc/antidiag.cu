@@ -302,8 +302,7 @@ bool make_group_map(CUtensorMap *m, const void *base, const Geom &g, int Ns, int
 
 template <int G>
 cudaError_t launch_scores(const CUtensorMap &mq, const CUtensorMap &mk, const AdParams &prm, long long tiles, int smem, cudaStream_t s) {
-  static std::atomic<unsigned long long> done{0};
-  cudaError_t e = allow_shared_memory(antidiag_scores_kernel<G>, smem, done);
+  cudaError_t e = allow_shared_memory(antidiag_scores_kernel<G>, smem);
   if (e != cudaSuccess) return e;
   const int pairs = (int)(tiles < 74 ? tiles : 74);  // two of the 148 SMs each
   return launch_pdl(antidiag_scores_kernel<G>, dim3(2 * pairs), dim3(kThreadsAd), smem, s, Cluster{2}, mq, mk, prm);
@@ -313,8 +312,7 @@ template <int NJ>
 cudaError_t launch_reduce(const Geom &g, const float2 *pairs, int Ns, int grp, int pitch, const uint8_t *refresh, double *scores,
                           cudaStream_t s) {
   const int smem = grp * NJ * 32 * (int)sizeof(double);
-  static std::atomic<unsigned long long> done{0};
-  cudaError_t e = allow_shared_memory(antidiag_reduce_kernel<NJ>, 8 * NJ * 32 * (int)sizeof(double), done);
+  cudaError_t e = allow_shared_memory(antidiag_reduce_kernel<NJ>, 8 * NJ * 32 * (int)sizeof(double));
   if (e != cudaSuccess) return e;
   return launch_pdl(antidiag_reduce_kernel<NJ>, dim3(g.nb, g.R), dim3(256), (size_t)smem, s, pairs, Ns, g.nb, grp, pitch, refresh,
                     scores);

@@ -974,8 +974,7 @@ cudaError_t launch_bk(const Geom &g, const Workspace &w, const CUtensorMap &mq, 
     prm.split = 1;
     for (int n = kMaxSplit; n >= 2 && prm.split == 1; n /= 2)
       if (all_tiles * n <= kSplitCtas && prm.step_pitch >= 2 * n) prm.split = n;
-    static std::atomic<unsigned long long> done{0};
-    e = allow_shared_memory(attn_tc_kernel<B, true>, kAttnSmem, done);
+    e = allow_shared_memory(attn_tc_kernel<B, true>, kAttnSmem);
     if (e != cudaSuccess) return e;
     ++*launches;
     return launch_pdl(attn_tc_kernel<B, true>, dim3(prm.n_tiles * prm.split), dim3(kAttnThreads), kAttnSmem, s, Cluster{prm.split}, mq, mk,
@@ -995,8 +994,7 @@ cudaError_t launch_bk(const Geom &g, const Workspace &w, const CUtensorMap &mq, 
     ++*launches;
     prm.tiles = order;
   }
-  static std::atomic<unsigned long long> done{0};
-  e = allow_shared_memory(attn_tc_kernel<B, false>, kAttnSmem, done);
+  e = allow_shared_memory(attn_tc_kernel<B, false>, kAttnSmem);
   if (e != cudaSuccess) return e;
   ++*launches;
   return launch_pdl(attn_tc_kernel<B, false>, dim3(kSms), dim3(kAttnThreads), kAttnSmem, s, mq, mk, mv, prm, plan);

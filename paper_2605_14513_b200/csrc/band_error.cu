@@ -288,8 +288,7 @@ template <int PASS>
 cudaError_t launch_axis(const AxisArgs &a, cudaStream_t s) {
   const size_t smem = sizeof(double) * 2 * fold_layout(a.n, a.inner == 1).doubles + (a.n <= kMaxSharedTable ? sizeof(double2) * a.n : 0);
   constexpr int kMost = sizeof(double) * 2 * kMaxChunk * (kLines + 4) + sizeof(double2) * kMaxSharedTable;
-  static std::atomic<unsigned long long> done{0};
-  cudaError_t e = allow_shared_memory(axis_kernel<PASS>, kMost, done);
+  cudaError_t e = allow_shared_memory(axis_kernel<PASS>, kMost);
   if (e != cudaSuccess) return e;
   const dim3 grid((unsigned)n_ctas(a.lines, a.n), (unsigned)frequency_splits(a.lines, a.n));
   return launch_pdl(axis_kernel<PASS>, grid, dim3(kBandThreads), smem, s, a);

@@ -3,8 +3,6 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#include <atomic>
-
 #include "heart.h"
 
 namespace heart {
@@ -134,18 +132,11 @@ __device__ __forceinline__ double exp_nonpositive(double x) {
   return __hiloint2double(__double2hiint(q) + (n << 20), __double2loint(q));
 }
 
-// Lets a kernel use `bytes` of dynamic shared memory; asked of the runtime once per kernel and device (`done` is
-// the call site's own, one bit per device).
+// Lets a kernel use `bytes` of dynamic shared memory.  Asked of the runtime on every call (60 ns): the answer belongs to the
+// context, of which a device may have several, one after the other or side by side.
 template <typename K>
-cudaError_t allow_shared_memory(K *kernel, int bytes, std::atomic<unsigned long long> &done) {
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  const unsigned long long bit = dev < 64 ? 1ull << dev : 0ull;
-  if (done.load(std::memory_order_acquire) & bit) return cudaSuccess;
-  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_release);
-  return e;
+cudaError_t allow_shared_memory(K *kernel, int bytes) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
 }
 
 struct Cluster {

@@ -517,8 +517,7 @@ static cudaError_t launch_nj(const Geom &g, const Workspace &w, const double *ta
                              heart_state st, int pitch, cudaStream_t s, unsigned long long expect_sig) {
   dim3 grid((g.nb + kRowsPerCta<NJ> - 1) / kRowsPerCta<NJ>, g.R);
   const size_t smem = sizeof(double) * kRowsPerCta<NJ> * NJ * 32;
-  static std::atomic<unsigned long long> done{0};
-  cudaError_t e = allow_shared_memory(top_p_kernel<NJ>, (int)smem, done);
+  cudaError_t e = allow_shared_memory(top_p_kernel<NJ>, (int)smem);
   if (e != cudaSuccess) return e;
   return launch_pdl(top_p_kernel<NJ>, grid, dim3(32 * kRowsPerCta<NJ>), smem, s, (const double *)w.scores, g.nb, pitch, tau,
                     refresh, g.flags, st.mask_bits, st.kv_idx, st.kv_cnt, g.idx_stride, g.W, (const int32_t *)w.status,
@@ -529,8 +528,7 @@ template <int WT, int TD, int STAGES>
 static cudaError_t launch_scores(const Geom &g, const Workspace &w, const uint8_t *refresh, cudaStream_t s,
                                  unsigned long long expect_sig) {
   constexpr int smem = ScoreTile<WT, TD, STAGES>::kBytes;
-  static std::atomic<unsigned long long> done{0};
-  cudaError_t e = allow_shared_memory(pooled_scores_kernel<WT, TD, STAGES>, smem, done);
+  cudaError_t e = allow_shared_memory(pooled_scores_kernel<WT, TD, STAGES>, smem);
   if (e != cudaSuccess) return e;
   const unsigned t = (g.nb + 2 * WT - 1) / (2 * WT);
   return launch_pdl(pooled_scores_kernel<WT, TD, STAGES>, dim3(t, t, g.R), dim3(128), (size_t)smem, s, (const double *)w.bmean,
