@@ -45,7 +45,8 @@
 // and SM between SMs: more CTAs would not pay.)
 //
 // Every wait is bounded; a wait that runs out raises the CTA's abort flag and the status word, its roles
-// drain and stop, the other CTAs take the remaining tiles.
+// drain and stop.  The tile it worked on and those it had drawn already, or was dealt, stay unwritten (as does a tile that a
+// cluster shares); the other CTAs take the rest.
 #include <cuda.h>
 
 #include "common.cuh"

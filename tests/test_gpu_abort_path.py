@@ -65,3 +65,71 @@ def test_a_wait_that_runs_out_is_reported_and_the_context_stays_usable():
     O_prod, status, _, _ = dense_attention(h, TEST_SKIP_V, Q, K, V, wl)
     assert status == 0
     assert torch.equal(O_prod.view(torch.int16), O_ref.view(torch.int16))
+
+
+@pytest.fixture
+def hooks():
+    from paper_2605_14513_b200 import heart as h
+
+    product = h.lib()
+    h._lib = h.load(heart_build.build_test_hooks())
+    yield h
+    h._lib = product
+
+
+@pytest.mark.parametrize("block", [64, 128])
+@pytest.mark.parametrize("H,N", [(2, 420), (80, 257)])  # tiles shared by a cluster; 240 tiles of 2 or 3 steps for 148 CTAs
+def test_other_tiles_are_complete_after_an_abort(hooks, block, H, N):
+    h = hooks
+    g = torch.Generator("cuda").manual_seed(N)
+    Q, K, V = (torch.randn((1, H, N, 128), generator=g, device="cuda").to(torch.bfloat16) for _ in range(3))
+    nb, tiles = h.n_blocks(N, block), (N + 127) // 128
+    idx = torch.arange(nb, dtype=torch.int32, device="cuda").expand(H, nb, nb).contiguous()
+    cnt = torch.full((H, nb), nb, dtype=torch.int32, device="cuda")
+    for dense in (True, False):
+        cfg = h.make_config(1, H, N, block, flags=h.FORCE_DENSE if dense else 0)
+        use = (None, None) if dense else (idx, cnt)
+        ws = h.new_workspace(cfg)
+        ref, bad, again = (torch.full_like(Q, float("nan")) for _ in range(3))
+        h.heart_block_sparse_attn(cfg, Q, K, V, *use, ref, ws)
+        assert h.heart_get_status(ws) == 0 and not ref.isnan().any()
+        cfg.flags |= TEST_SKIP_V
+        t0 = time.perf_counter()
+        h.heart_block_sparse_attn(cfg, Q, K, V, *use, bad, ws)
+        assert h.heart_get_status(ws) == h.ERR_DEVICE_CHECK
+        assert time.perf_counter() - t0 < 5.0
+        lost = [(head, t) for head in range(H) for t in range(tiles) if bad[0, head, 128 * t].isnan().any()]
+        if H * tiles <= 148 or dense:  # the tiles of CTA 0 are known
+            assert lost == [divmod(n, tiles) for n in range(0, H * tiles, 148)]
+        else:  # its first one, and the next if that was drawn already
+            assert 1 <= len(lost) <= 2
+        for head, t in lost:
+            assert bad[0, head, 128 * t : 128 * t + 128].isnan().all()
+            bad[0, head, 128 * t : 128 * t + 128] = ref[0, head, 128 * t : 128 * t + 128]
+        assert torch.equal(bad.view(torch.int16), ref.view(torch.int16))
+        cfg.flags &= ~TEST_SKIP_V
+        h.heart_block_sparse_attn(cfg, Q, K, V, *use, again, ws)
+        assert h.heart_get_status(ws) == 0
+        assert torch.equal(again.view(torch.int16), ref.view(torch.int16))
+
+
+@pytest.mark.parametrize("block", [64, 128])
+@pytest.mark.parametrize("H,N", [(2, 600), (100, 600), (3, 9000)])  # a tile a pair; more tiles than pairs; 9 tiles a head
+def test_antidiagonal_pair_that_gives_up(hooks, block, H, N):
+    h = hooks
+    g = torch.Generator("cuda").manual_seed(N)
+    Q, K = (torch.randn((1, H, N, 128), generator=g, device="cuda").to(torch.bfloat16) for _ in range(2))
+    cfg = h.make_config(1, H, N, block, flags=h.ESTIMATOR_ANTIDIAG)
+    tau = torch.full((H,), 0.9, dtype=torch.float64, device="cuda")
+    ws, ref, bad, again = h.new_workspace(cfg), h.State(cfg), h.State(cfg), h.State(cfg)
+    h.heart_predict_mask(cfg, Q, K, tau, ref, ws)
+    assert h.heart_get_status(ws) == 0
+    cfg.flags |= TEST_SKIP_V
+    t0 = time.perf_counter()
+    h.heart_predict_mask(cfg, Q, K, tau, bad, ws)
+    assert h.heart_get_status(ws) == h.ERR_DEVICE_CHECK
+    assert time.perf_counter() - t0 < 5.0
+    cfg.flags &= ~TEST_SKIP_V
+    h.heart_predict_mask(cfg, Q, K, tau, again, ws)
+    assert h.heart_get_status(ws) == 0
+    assert torch.equal(again.kv_cnt, ref.kv_cnt) and torch.equal(again.mask_bits, ref.mask_bits)
