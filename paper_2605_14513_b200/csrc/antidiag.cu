@@ -115,6 +115,7 @@ __global__ void __launch_bounds__(kThreadsAd, 1)
       tma_prefetch_desc(&map_q);
       tma_prefetch_desc(&map_k);
       int it = 0;
+      const uint32_t even_full = cluster_address(smem_u32(bars->full), 0);
       each_tile([&](int r, int row, int col) {
         const int bidx = r / p.H, hidx = r % p.H;
         for (int ks = 0; ks < kKSteps; ++ks, ++it) {
@@ -128,8 +129,8 @@ __global__ void __launch_bounds__(kThreadsAd, 1)
           if (p.test_skip_copy && blockIdx.x == 0 && it == 1) continue;
 #endif
           // this CTA's half of token t of the query groups, of token s-1-t of the key groups of the tile
-          tma_load_5d_pair(dst, &map_q, &bars->full[st], dh * 64, t, row * kMt + rank * 128, hidx, bidx);
-          tma_load_5d_pair(dst + kHalfBytes, &map_k, &bars->full[st], dh * 64, kS - 1 - t, col * kNt + rank * 128, hidx, bidx);
+          tma_load_5d_pair(dst, &map_q, even_full + 8 * st, dh * 64, t, row * kMt + rank * 128, hidx, bidx);
+          tma_load_5d_pair(dst + kHalfBytes, &map_k, even_full + 8 * st, dh * 64, kS - 1 - t, col * kNt + rank * 128, hidx, bidx);
         }
         return true;
       });
@@ -325,10 +326,6 @@ cudaError_t launch_reduce(const Geom &g, const float2 *pairs, int Ns, int grp, i
 }
 
 }  // namespace
-
-size_t antidiag_pairs_bytes(const Geom &g) {
-  return sizeof(float2) * (size_t)g.R * (size_t)(g.N / kS) * (size_t)g.nb;
-}
 
 cudaError_t launch_antidiag_scores(const Geom &g, const Workspace &w, const void *Q, const void *K,
                                    const uint8_t *refresh, cudaStream_t s, int *launches) {

@@ -15,10 +15,13 @@
 #include <math.h>
 
 #include "common.cuh"
+#include "tc_ptx.cuh"
 
 namespace heart {
 
 namespace {
+
+using tc::mma_f64;
 
 constexpr int kLines = 16;        // lines of an axis per warp
 constexpr int kMaxChunk = 160;    // folded samples of a line in shared memory at a time
@@ -58,10 +61,6 @@ __global__ void trig_tables_kernel(int n0, int n1, int n2, double2 *__restrict__
   double sn, cs;
   sincospi(2.0 * (double)m / (double)n, &sn, &cs);
   tables[i] = make_double2(cs, sn);
-}
-
-__device__ __forceinline__ void mma_f64(double (&d)[2], double a, double b) {
-  asm("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};" : "+d"(d[0]), "+d"(d[1]) : "d"(a), "d"(b));
 }
 
 // Sums over the CTA of kBandThreads threads, in a fixed order; valid in thread 0.

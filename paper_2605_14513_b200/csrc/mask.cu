@@ -23,11 +23,13 @@
 namespace heart {
 
 using tc::ex2;
+using tc::mma_f64;
 
 constexpr int kSmallScoreTiles = 148;  // 64 x 64 score tiles of a launch up to which 32 x 32 ones are used
 // Rows (warps) per CTA of the top-p kernel.  A row that needs the fp64 search takes many times longer than the
-// others and holds its CTA: 22296 such rows take 121 us with eight rows a CTA,
-// 108 with two; short rows gain nothing and pay for the CTAs.
+// others and holds its CTA: 22296 rows of 929 take 121 us with eight rows a CTA,
+// 108 with two; from 513 blocks on two are no slower anywhere (whole call, tau 0.97: 40 x 591 blocks 268 against 274 us, 16 x 735
+// 161 against 167); short rows gain nothing and pay for the CTAs.
 template <int NJ>
 constexpr int kRowsPerCta = NJ >= 24 ? 2 : 8;
 constexpr int kMaxCand = 64;    // candidates the direct threshold evaluation takes
@@ -59,12 +61,6 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N>
 __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
-
-// D (8 x 8) += A (8 x 4, row) * B (4 x 8, col), fp64: lane l holds A[l / 4][l % 4], B[l % 4][l / 4] and
-// D[l / 4][2 * (l % 4) + {0, 1}].
-__device__ __forceinline__ void mma_f64(double (&d)[2], double a, double b) {
-  asm("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};" : "+d"(d[0]), "+d"(d[1]) : "d"(a), "d"(b));
 }
 
 // scores[r][I][J] = scale * <mean_q[r][I], mean_k[r][J]> for the refreshed heads r.  A CTA of four warps owns

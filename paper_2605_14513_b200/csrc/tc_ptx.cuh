@@ -247,19 +247,25 @@ __device__ __forceinline__ void tc_commit_pair(uint64_t *bar) {
                "h"((uint16_t)3)
                : "memory");
 }
-// A box into this CTA's shared memory whose bytes count on the even CTA's barrier (an address with the bit of the odd
-// CTA cleared).
-__device__ __forceinline__ void tma_load_5d_pair(void *smem_dst, const CUtensorMap *map, uint64_t *bar, int c0, int c1, int c2,
+// A box into this CTA's shared memory whose bytes count on a barrier of the pair (`bar`: its address in the cluster).
+__device__ __forceinline__ void tma_load_5d_pair(void *smem_dst, const CUtensorMap *map, uint32_t bar, int c0, int c1, int c2,
                                                  int c3, int c4) {
   asm volatile(
       "cp.async.bulk.tensor.5d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6, %7}], [%2];"
-      ::"r"(smem_u32(smem_dst)), "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_u32(bar) & 0xfeffffffu), "r"(c0), "r"(c1),
+      ::"r"(smem_u32(smem_dst)), "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(c0), "r"(c1),
       "r"(c2), "r"(c3), "r"(c4)
       : "memory");
 }
 // Arrival on the barrier at this address in CTA `rank` of the cluster.
 __device__ __forceinline__ void mbar_arrive_in(uint64_t *bar, uint32_t rank) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_address(smem_u32(bar), rank)) : "memory");
+}
+
+// ---------------------------------------------------------------- fp64 matrix instruction
+// D (8 x 8) += A (8 x 4, row) * B (4 x 8, col): lane l holds A[l / 4][l % 4], B[l % 4][l / 4] and
+// D[l / 4][2 * (l % 4) + {0, 1}].
+__device__ __forceinline__ void mma_f64(double (&d)[2], double a, double b) {
+  asm("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};" : "+d"(d[0]), "+d"(d[1]) : "d"(a), "d"(b));
 }
 
 // ---------------------------------------------------------------- descriptors

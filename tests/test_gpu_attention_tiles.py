@@ -1,7 +1,7 @@
 """The attention kernel's step lists and tile queue at their edges: odd numbers of listed blocks, key
 blocks that only one of a tile's two query blocks lists, the ragged last block in either half of a step,
 query blocks without any key block (runs of them longer than the announcement ring), and more tiles than
-there are streams (296), so that tiles are drawn from the counter."""
+there are CTAs (148), so that tiles are drawn from the counter."""
 import numpy as np
 import pytest
 import torch
@@ -32,8 +32,8 @@ def make_lists(rs, R, nb, kind, block):
 
 @pytest.mark.parametrize("block", [64, 128])
 @pytest.mark.parametrize("kind,H,N", [
-    ("random", 3, 700),        # 6 tiles: every stream at most one
-    ("random", 110, 330),      # 330 tiles of 3 a head: some streams draw a second tile; ragged last tile and block
+    ("random", 3, 700),        # 6 tiles: every CTA at most one
+    ("random", 110, 330),      # 330 tiles of 3 a head: CTAs draw a second and a third tile; ragged last tile and block
     ("disjoint", 2, 64 * 9 + 5),
     ("one_sided", 2, 64 * 8 - 3),
     ("empty_runs", 160, 257),  # 480 tiles, runs of 18 empty ones
