@@ -436,7 +436,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
         if (Small && n_steps_of(nx.y) > 0) e = step_entry(steps_of(nx), 0);
       };
       // The first tile of every CTA is fixed, the others are drawn (a small launch has no others).  Dense tiles are all
-      // of one length: dealt in turn, so that dense calls share nothing and may overlap on one workspace.
+      // of one length: dealt in turn, so that dense calls share nothing and may overlap on one workspace.  (Drawn, the faster
+      // SMs take the odd tiles: 12 x 33k 5604 us, dealt 5721.)
       int mine = Small ? blockIdx.x / p.split : blockIdx.x;
       fetch(mine);
       auto draw = [&]() { fetch(Small ? p.n_tiles : p.dense ? mine += gridDim.x : gridDim.x + atomicAdd(p.counter, 1)); };
