@@ -11,7 +11,8 @@
 // Each axis is a contraction with the fp64 matrix instruction.  Folding x_j +- x_{n-j} halves it: cosines see the
 // even part, sines the odd one.  x and y write their coefficients to the workspace (they stay in L2), t only
 // adds up energies.  For 16 x 21 x 60 x 104 that is 1.9e8 fma (10 us at 18.5 T fma/s) and 84 MB of L2 traffic in
-// three passes (58 us; 16 lines a warp and 8 CTAs an SM, against 64 us with 32 and 4); the full circulant projections used before took 4.3e8 fma with two loads for each (0.45 ms).
+// three passes (58 us; 16 lines a warp and 8 CTAs an SM, against 64 us with 32 and 4); the full circulant projections used
+// before took 4.3e8 fma with two loads for each (0.45 ms).
 #include <math.h>
 
 #include "common.cuh"
