@@ -9,10 +9,9 @@
 // its own coefficients (no subtraction of energies).  Low along an axis: k <= floor(n/4).
 //
 // Each axis is a contraction with the fp64 matrix instruction.  Folding x_j +- x_{n-j} halves it: cosines see the
-// even part, sines the odd one.  x and y write their coefficients to the workspace (they stay in L2), t only
-// adds up energies.  For 16 x 21 x 60 x 104 that is 1.9e8 fma (10 us at 18.5 T fma/s) and 84 MB of L2 traffic in
-// three passes (58 us; 16 lines a warp and 8 CTAs an SM, against 64 us with 32 and 4); the full circulant projections used
-// before took 4.3e8 fma with two loads for each (0.45 ms).
+// even part, sines the odd one.  For 16 x 21 x 60 x 104 that is 1.9e8 fma (10 us at 18.5 T fma/s).  Two ways through it:
+// planes that a CTA holds are transformed along y and x in one kernel, another goes over t (40 us); any other shape goes
+// axis by axis through the workspace, in five launches (55 us for that one).
 #include <math.h>
 
 #include "common.cuh"
@@ -273,6 +272,379 @@ __global__ void __launch_bounds__(1024) band_final_kernel(const double *__restri
   }
 }
 
+// ------------------------------------------------------------------ planes that fit in shared memory
+// The usual latent: a [y, x] plane of one channel and time is transformed along both of its axes by two CTAs, one for
+// the part that is even along y and one for the odd one, without a trip to the workspace in between; a second kernel
+// goes over t, and its last CTA puts the result together.  Two launches instead of five, 34 MB of traffic in the L2 less:
+// 16 x 21 x 60 x 104 takes 40.5 us instead of 55.3.  Neither kernel is near a rate (fp64 matrix pipe 33 and 13 % busy,
+// issue slots 44 and 47 %): 672 CTAs, three an SM, fold, wait and multiply in turn.  (With 64-bit remainders and the
+// cosine and sine of an entry side by side, so that a warp's entries collide in twice as many banks: 50.2 us.)
+
+constexpr int kPlaneThreads = 256, kPlaneWarps = kPlaneThreads / 32;
+constexpr int kPlaneMaxShared = 200 * 1024;  // of a CTA, in bytes
+constexpr int kTimeThreads = 128, kTimeLines = 64, kTimePitch = kTimeLines + 4, kTimeMax = 96, kTimeCtas = 148 * 4;
+
+__host__ __device__ inline int round_up(int v, int m) { return (v + m - 1) / m * m; }
+
+// A: folded rows, [rows rounded to 8][even part along x | odd part], B: [x coefficients rounded to 8][rows].  The pitches are
+// 4 (mod 8) doubles: 8 x 4 fragments are read without bank conflicts.
+struct PlaneLayout {
+  int even_cols, pitch_a, rows, pitch_b, doubles;
+};
+__host__ __device__ inline PlaneLayout plane_layout(int ny, int nx) {
+  PlaneLayout f;
+  f.even_cols = round_up(nx / 2 + 1, 4);
+  const int cols = f.even_cols + round_up((nx - 1) / 2, 4);
+  f.pitch_a = cols + (cols % 8 == 0 ? 4 : 0);
+  f.rows = round_up(ny / 2 + 1, 8);
+  f.pitch_b = f.rows + 4;
+  f.doubles = f.rows * f.pitch_a + round_up(nx, 8) * f.pitch_b;
+  return f;
+}
+inline size_t plane_shared_bytes(int ny, int nx) { return sizeof(double) * plane_layout(ny, nx).doubles + sizeof(double2) * ((size_t)ny + nx); }
+
+// cos 2 pi m / n, then sin 2 pi m / n (apart: a warp's entries collide in fewer banks); entry i0 of the CTA's first thread
+__device__ __forceinline__ void fill_trig_table(double *tab, int n, int i0 = 0) {
+  for (int m = (int)threadIdx.x - i0; m < n; m += blockDim.x)
+    if (m >= 0) sincospi(2.0 * (double)m / (double)n, &tab[n + m], &tab[m]);
+}
+
+__device__ __forceinline__ int mod_small(int v, int n) {  // v mod n for 0 <= v < 3 n
+  v -= v >= n ? n : 0;
+  return v - (v >= n ? n : 0);
+}
+// acc[i] = lines of tile t0 + i (of n_tiles, 8 lines each) times 8 frequencies over `samples` samples, the first of which is
+// sample j0 (0 or 1) of the axis; tab: the cosines or the sines of the axis.  lane: frequency k <= n / 2.
+template <int TILES>
+__device__ __forceinline__ void contract(double (&acc)[TILES][2], const double *lines, int pitch, int t0, int n_tiles, int samples,
+                                         const double *tab, int n, int k, int j0) {
+  const int lane = threadIdx.x & 31, jl = lane & 3;
+  const double *a = lines + (t0 * 8 + (lane >> 2)) * pitch + jl;
+  int idx = mod_small(k * (j0 + jl), n);  // (at most n / 2 * 4)
+  const int inc = mod_small(4 * k, n);
+#pragma unroll
+  for (int i = 0; i < TILES; ++i) acc[i][0] = acc[i][1] = 0.0;
+  if (t0 + TILES <= n_tiles) {
+#pragma unroll 2
+    for (int j = 0; j < samples; j += 4) {
+      const double t = tab[idx];
+      idx += inc;
+      idx -= idx >= n ? n : 0;
+#pragma unroll
+      for (int i = 0; i < TILES; ++i) mma_f64(acc[i], a[i * 8 * pitch + j], t);
+    }
+  } else {
+    for (int j = 0; j < samples; j += 4) {
+      const double t = tab[idx];
+      idx += inc;
+      idx -= idx >= n ? n : 0;
+#pragma unroll
+      for (int i = 0; i < TILES; ++i)
+        if (t0 + i < n_tiles) mma_f64(acc[i], a[i * 8 * pitch + j], t);
+    }
+  }
+}
+
+// CTA 2 * plane + parity along y.
+__global__ void __launch_bounds__(kPlaneThreads, 3) plane_kernel(const float *__restrict__ ys, const float *__restrict__ yd, int ny, int nx,
+                                                                 double *__restrict__ dst, double *__restrict__ dense_out,
+                                                                 int *__restrict__ ticket) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const PlaneLayout f = plane_layout(ny, nx);
+  double *tab_x = reinterpret_cast<double *>(smem_raw), *tab_y = tab_x + 2 * nx;
+  double *A = tab_y + 2 * ny, *Bm = A + f.rows * f.pitch_a;
+  __shared__ double red[kPlaneWarps];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int odd = blockIdx.x & 1;
+  const size_t plane = (size_t)(blockIdx.x >> 1) * ny * nx;
+  const int hx = nx / 2, mx = (nx - 1) / 2, hy = ny / 2, my = (ny - 1) / 2;
+  const int rows = odd ? my : hy + 1;  // samples along y of this parity: odd ones start at 1
+  fill_trig_table(tab_x, nx);
+  fill_trig_table(tab_y, ny, nx < kPlaneThreads ? nx : 0);  // (by the threads that have no entry of x)
+  pdl_wait();
+  pdl_launch_dependents();
+  if (blockIdx.x == 0 && threadIdx.x == 0) *ticket = 0;
+
+  // folded along both axes, a warp per row; the loads of four rows at a time
+  double dense = 0.0;
+  const int row_tiles = (rows + 7) / 8, odd_cols = round_up(mx, 4);
+  const float *s0 = ys + plane, *d0 = yd + plane;
+  for (int j = lane; j < f.even_cols; j += 32) {
+    const bool in = j <= hx, xpair = j >= 1 && j <= mx;
+#pragma unroll 2
+    for (int i = warp; i < row_tiles * 8; i += kPlaneWarps) {
+      const int jy = i + odd;
+      const bool real = in && i < rows, pair = real && jy >= 1 && jy <= my;
+      const int at = jy * nx, mirror = (ny - jy) * nx;
+      float s1[4], d1[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int off = (q < 2 ? at : mirror) + ((q & 1) ? nx - j : j);
+        const bool load = (q < 2 ? real : pair) && ((q & 1) == 0 || xpair);
+        s1[q] = load ? __ldg(&s0[off]) : 0.f;
+        d1[q] = load ? __ldg(&d0[off]) : 0.f;
+      }
+      double e[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const double d = (double)d1[q];
+        e[q] = (double)s1[q] - d;
+        dense = fma(d, d, dense);
+      }
+      const double u = odd ? e[0] - e[2] : e[0] + e[2], v = odd ? e[1] - e[3] : e[1] + e[3];
+      double *row = A + i * f.pitch_a;
+      row[j] = u + v;
+      if (xpair) row[f.even_cols + j - 1] = u - v;  // (zeros in the rows that fill the last tile)
+    }
+  }
+  for (int i = warp; i < row_tiles * 8; i += kPlaneWarps)
+    for (int j = mx + lane; j < odd_cols; j += 32) A[i * f.pitch_a + f.even_cols + j] = 0.0;
+  if (!odd) {  // |y_dense|^2 of the plane
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) dense += __shfl_xor_sync(0xffffffffu, dense, o);
+    if (lane == 0) red[warp] = dense;
+  }
+  __syncthreads();
+  if (!odd && threadIdx.x == 0) {
+    double sum = 0.0;
+#pragma unroll
+    for (int i = 0; i < kPlaneWarps; ++i) sum += red[i];
+    dense_out[blockIdx.x >> 1] = sum;
+  }
+
+  // along x: lines are the rows; cosines of the even part, then sines of the odd one
+  constexpr int TX = 4, TY = 7;  // tiles of 8 lines that share the table entries of a warp
+  const int cos_x = (hx + 8) / 8, sin_x = (mx + 7) / 8;
+  for (int t0 = 0; t0 < row_tiles; t0 += TX) {
+    for (int kt = warp; kt < cos_x + sin_x; kt += kPlaneWarps) {
+      const bool sine = kt >= cos_x;
+      const int k0 = sine ? 1 + (kt - cos_x) * 8 : kt * 8, k_last = sine ? mx : hx;
+      double acc[TX][2];
+      contract<TX>(acc, A + (sine ? f.even_cols : 0), f.pitch_a, t0, row_tiles, sine ? odd_cols : f.even_cols, tab_x + (sine ? nx : 0), nx,
+                   min(k0 + (lane >> 2), k_last), sine ? 1 : 0);
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int k = k0 + 2 * (lane & 3) + u;
+        if (k > k_last) continue;
+        double *col = Bm + (sine ? hx + k : k) * f.pitch_b + t0 * 8 + (lane >> 2);
+#pragma unroll
+        for (int i = 0; i < TX; ++i)
+          if (t0 + i < row_tiles) col[i * 8] = acc[i][u];
+      }
+    }
+  }
+  __syncthreads();
+
+  // along y: lines are the coefficients of x
+  const int kts = odd ? (my + 7) / 8 : (hy + 8) / 8, col_tiles = (nx + 7) / 8, k_last = odd ? my : hy;
+  const int samples = round_up(rows, 4);
+  for (int e = warp; e < kts * ((col_tiles + TY - 1) / TY); e += kPlaneWarps) {
+    const int t0 = e / kts * TY, k0 = e % kts * 8 + odd;
+    double acc[TY][2];
+    contract<TY>(acc, Bm, f.pitch_b, t0, col_tiles, samples, tab_y + (odd ? ny : 0), ny, min(k0 + (lane >> 2), k_last), odd);
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int k = k0 + 2 * (lane & 3) + u, col = t0 * 8 + (lane >> 2);
+      if (k > k_last) continue;
+      double *out = dst + plane + (size_t)((odd ? hy + k : k) * nx + col);
+#pragma unroll
+      for (int i = 0; i < TY; ++i)
+        if (col + i * 8 < nx) out[i * 8] = acc[i][u];
+    }
+  }
+}
+
+struct TimeArgs {
+  const double *src;    // [C][n][inner]
+  double *energies;     // [gridDim.x][4]
+  const double *dense;  // [planes]
+  int *ticket;
+  double *out;
+  int n, ny, nx, units_per_c, units, planes;
+  double n_freq, w0, w1, w2, w3, eps;
+};
+
+// The pass over t: 64 lines at a time, their samples brought in while those before are worked on; the energies are added
+// up over all of a CTA's lines, and the CTA that finishes last adds those of all CTAs in a fixed order and writes the result.
+__global__ void __launch_bounds__(kTimeThreads, 4) time_kernel(const TimeArgs a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int n = a.n, h = n / 2, m = (n - 1) / 2, inner = a.ny * a.nx;
+  double *tab = reinterpret_cast<double *>(smem_raw), *raw = tab + 2 * n;  // samples: [2][n + 1][kTimePitch], the last row zero
+  const int stage = (n + 1) * kTimePitch;
+  __shared__ int line_band[2][kTimeLines];  // low along y and x | log2 of the weight << 1 (no line: 0x100)
+  __shared__ double red[(kTimeThreads / 32) * 5];
+  __shared__ int last;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  fill_trig_table(tab, n);
+  for (int i = tid; i < kTimePitch; i += kTimeThreads) raw[n * kTimePitch + i] = raw[stage + n * kTimePitch + i] = 0.0;
+  const int line = tid & (kTimeLines - 1), part = tid / kTimeLines;
+  pdl_wait();
+  pdl_launch_dependents();
+  auto bring = [&](int unit, int buf) {
+    if (unit < a.units) {
+      const int c = unit / a.units_per_c, in = (unit - c * a.units_per_c) * kTimeLines + line;
+      const bool real = in < inner;
+      const double *src = a.src + (size_t)c * n * inner + (real ? in : 0);
+      const uint32_t dst = (uint32_t)__cvta_generic_to_shared(raw + buf * stage + line);
+      for (int j = part; j < n; j += kTimeThreads / kTimeLines)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst + j * kTimePitch * 8), "l"(src + (size_t)j * inner), "r"(real ? 8 : 0) : "memory");
+      if (part == 0) {
+        const int iy = in / a.nx, ix = in - iy * a.nx;
+        const int ky = iy <= a.ny / 2 ? iy : iy - a.ny / 2, kx = ix <= a.nx / 2 ? ix : ix - a.nx / 2;
+        const int wy = ky == 0 || 2 * ky == a.ny ? 0 : 1, wx = kx == 0 || 2 * kx == a.nx ? 0 : 1;
+        line_band[buf][line] = real ? (ky <= a.ny / 4 && kx <= a.nx / 4 ? 1 : 0) | (wy + wx) << 1 : 0x100;
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  double energy[4] = {0.0, 0.0, 0.0, 0.0};  // LL, LH, HL, HH
+  const int l0 = warp * 16 + (lane >> 2), jl = lane & 3;
+  bring(blockIdx.x, 0);
+  int buf = 0;
+  for (int unit = blockIdx.x; unit < a.units; unit += gridDim.x, buf ^= 1) {
+    bring(unit + gridDim.x, buf ^ 1);  // (free since the barrier that ended the unit before)
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+    __syncthreads();
+    // a warp: 16 lines; cosines and sines of 8 frequencies at a time
+    const double *x = raw + buf * stage + l0;
+    double low[2] = {0.0, 0.0}, high[2] = {0.0, 0.0};  // energy below and above n / 4, per line
+    for (int k0 = 0; k0 <= h; k0 += 8) {
+      const int k = min(k0 + (lane >> 2), h);
+      double cs[2][2] = {}, sn[2][2] = {};
+      int idx = mod_small(k * jl, n);
+      const int inc = mod_small(4 * k, n);
+#pragma unroll 3
+      for (int j = jl; j - jl <= h; j += 4) {
+        const bool pair = j >= 1 && j <= m;
+        const double *p = x + (j <= h ? j : n) * kTimePitch, *q = x + (pair ? n - j : n) * kTimePitch;
+        const double c = tab[idx], s = tab[n + idx];
+        idx += inc;
+        idx -= idx >= n ? n : 0;
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          const double u = p[8 * i], v = q[8 * i];
+          mma_f64(cs[i], u + v, c);
+          mma_f64(sn[i], pair ? u - v : 0.0, s);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int kk = k0 + 2 * jl + u;
+        if (kk > h) continue;
+        const double w = kk == 0 || 2 * kk == n ? 1.0 : 2.0;
+        const bool sine = kk >= 1 && kk <= m, below = kk <= n / 4;
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          const double e = sine ? fma(cs[i][u], cs[i][u], sn[i][u] * sn[i][u]) : cs[i][u] * cs[i][u];
+          if (below) low[i] = fma(w, e, low[i]);
+          else high[i] = fma(w, e, high[i]);
+        }
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const int band = line_band[buf][l0 + 8 * i];
+      if (band >> 8) continue;
+      const double w = (double)(1 << (band >> 1));
+      if (band & 1) {
+        energy[0] = fma(w, low[i], energy[0]);
+        energy[2] = fma(w, high[i], energy[2]);
+      } else {
+        energy[1] = fma(w, low[i], energy[1]);
+        energy[3] = fma(w, high[i], energy[3]);
+      }
+    }
+    __syncthreads();
+  }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  __syncthreads();
+  auto sums = [&](auto &v, int nv) {  // over the CTA, in a fixed order; valid in thread 0
+#pragma unroll
+    for (int q = 0; q < nv; ++q) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_xor_sync(0xffffffffu, v[q], o);
+      if (lane == 0) red[warp * nv + q] = v[q];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < nv; ++q) v[q] = (red[q] + red[nv + q]) + (red[2 * nv + q] + red[3 * nv + q]);
+  };
+  sums(energy, 4);
+  if (tid == 0) {
+#pragma unroll
+    for (int b = 0; b < 4; ++b) __stcg(&a.energies[(size_t)blockIdx.x * 4 + b], energy[b]);
+    __threadfence();
+    last = atomicAdd(a.ticket, 1) == (int)gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  double tot[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+#pragma unroll 4
+  for (int i = tid; i < (int)gridDim.x; i += kTimeThreads) {
+    const double2 x = __ldcg(reinterpret_cast<const double2 *>(a.energies) + 2 * i), y = __ldcg(reinterpret_cast<const double2 *>(a.energies) + 2 * i + 1);
+    tot[0] += x.x, tot[1] += x.y, tot[2] += y.x, tot[3] += y.y;
+  }
+#pragma unroll 4
+  for (int i = tid; i < a.planes; i += kTimeThreads) tot[4] += __ldcg(&a.dense[i]);
+  sums(tot, 5);
+  if (tid == 0) {
+    const double denom = tot[4] * a.n_freq + a.eps;
+    a.out[0] = (a.w0 * tot[0] + a.w1 * tot[1] + a.w2 * tot[2] + a.w3 * tot[3]) / denom;
+    a.out[1] = tot[0];
+    a.out[2] = tot[1];
+    a.out[3] = tot[2];
+    a.out[4] = tot[3];
+    a.out[5] = denom;
+  }
+}
+
+// Planes of 512 points and more that a CTA holds, and time axes whose samples of 64 lines it holds.  (Smaller planes do
+// not fill a CTA's warps, longer time axes go through the general pass in parts.)
+bool planes_fit(int T, int H, int W) {
+  return (long long)H * W >= 512 && (long long)H * W <= kPlaneMaxShared / 8 && plane_shared_bytes(H, W) <= kPlaneMaxShared && T <= kTimeMax;
+}
+int time_units(int C, int H, int W) { return C * ((H * W + kTimeLines - 1) / kTimeLines); }
+int time_ctas(int C, int H, int W) { return time_units(C, H, W) < kTimeCtas ? time_units(C, H, W) : kTimeCtas; }
+size_t time_shared_bytes(int n) { return sizeof(double) * (2 * n + 2 * (n + 1) * kTimePitch); }
+
+cudaError_t launch_planes(const float *ys, const float *yd, int C, int T, int H, int W, const double *weights, double eps, double *out,
+                          char *p, cudaStream_t s, int *launches) {
+  TimeArgs a = {};
+  a.ticket = reinterpret_cast<int *>(p);
+  p += 256;
+  double *coef = reinterpret_cast<double *>(p);
+  p += align256(sizeof(double) * (size_t)C * T * H * W);
+  a.energies = reinterpret_cast<double *>(p);
+  p += align256(sizeof(double) * 4 * time_ctas(C, H, W));
+  double *dense = reinterpret_cast<double *>(p);
+  cudaError_t e = allow_shared_memory(plane_kernel, kPlaneMaxShared);
+  if (e != cudaSuccess) return e;
+  e = launch_pdl(plane_kernel, dim3(2u * C * T), dim3(kPlaneThreads), plane_shared_bytes(H, W), s, ys, yd, H, W, coef, dense, a.ticket);
+  if (e != cudaSuccess) return e;
+  ++*launches;
+  a.src = coef;
+  a.dense = dense;
+  a.out = out;
+  a.n = T;
+  a.ny = H;
+  a.nx = W;
+  a.units_per_c = time_units(1, H, W);
+  a.units = time_units(C, H, W);
+  a.planes = C * T;
+  a.n_freq = (double)T * H * W;
+  a.w0 = weights[0];
+  a.w1 = weights[1];
+  a.w2 = weights[2];
+  a.w3 = weights[3];
+  a.eps = eps;
+  e = allow_shared_memory(time_kernel, (int)time_shared_bytes(kTimeMax));
+  if (e != cudaSuccess) return e;
+  e = launch_pdl(time_kernel, dim3(time_ctas(C, H, W)), dim3(kTimeThreads), time_shared_bytes(T), s, a);
+  ++*launches;
+  return e;
+}
+
 size_t n_ctas(long long lines, int n) { return (size_t)((lines + lines_per_cta(n) - 1) / lines_per_cta(n)); }
 
 // CTAs that share the frequencies of a set of lines: as many as there are rounds, while lines alone leave SMs without a
@@ -298,6 +670,8 @@ cudaError_t launch_axis(const AxisArgs &a, cudaStream_t s) {
 
 size_t band_error_workspace_bytes(int C, int T, int H, int W) {
   const size_t n = (size_t)C * T * H * W;
+  if (planes_fit(T, H, W))
+    return 256 + align256(sizeof(double) * n) + align256(sizeof(double) * 4 * time_ctas(C, H, W)) + align256(sizeof(double) * (size_t)C * T);
   return align256(sizeof(double2) * ((size_t)T + H + W)) + 2 * align256(sizeof(double) * n) +
          align256(sizeof(double) * 4 * n_energies(C, T, H, W)) + align256(sizeof(double) * n_ctas((long long)C * T * H, W));
 }
@@ -306,6 +680,7 @@ cudaError_t launch_band_error(const float *ys, const float *yd, int C, int T, in
                               double eps, double *out, void *workspace, cudaStream_t s, int *launches) {
   const long long n = (long long)C * T * H * W;
   char *p = static_cast<char *>(workspace);
+  if (planes_fit(T, H, W)) return launch_planes(ys, yd, C, T, H, W, weights, eps, out, p, s, launches);
   double2 *tables = reinterpret_cast<double2 *>(p);  // of x, y, t
   p += align256(sizeof(double2) * ((size_t)T + H + W));
   double *A = reinterpret_cast<double *>(p);

@@ -27,3 +27,11 @@ def test_band_error_axes(oracle, shape):
 def test_few_long_lines(oracle, shape):
     """Axes whose lines are fewer than the SMs: CTAs share their frequencies (one to 65 shares of them, uneven ones)."""
     test_band_error_axes(oracle, shape)
+
+
+@pytest.mark.parametrize("shape", [(1, 1, 8, 64), (2, 3, 23, 23), (1, 5, 1, 512), (3, 2, 512, 1), (1, 4, 2, 257), (1, 2, 257, 2), (3, 96, 16, 33),
+                                   (1, 97, 16, 33), (2, 2, 96, 170), (1, 3, 97, 169), (1, 1, 110, 215), (1, 1, 7, 73), (40, 1, 30, 41)])
+def test_planes_in_shared_memory(oracle, shape):
+    """Planes on both sides of what a CTA takes (512 points, its shared memory, 96 steps of time), axes that fill their
+    tiles of eight lines and frequencies and axes that do not."""
+    test_band_error_axes(oracle, shape)
