@@ -43,7 +43,8 @@ struct Workspace {
   int32_t *status;    // [64]   word 0: sticky device-check code; word 1: detail; word 8: ticket counter
                       //        of the drift kernel (zero between launches); words 10-11: signature of
                       //        the (Q, K, shape) whose block means the workspace holds (0: none); word 12:
-                      //        tiles of an attention launch drawn beyond the first one of every CTA
+                      //        tiles of an attention launch drawn beyond the first one of every CTA; words
+                      //        16-63: ticket counters of the heads in a small heart_step (zero between launches)
   double *bmean;      // [2][R][nb][D]  per-block (pooled) means of Q (0) and K (1)
   double *psum;       // [2][R][nchunks][D]  per-CTA partial token sums
   double *mean;       // [2][R][D]      token means of the current step
@@ -93,7 +94,20 @@ __host__ inline Workspace carve(const Geom &g, void *base) {
   return w;
 }
 
-constexpr int kStatusTicketWord = 8, kStatusSigWord = 10, kStatusTileWord = 12;
+constexpr int kStatusTicketWord = 8, kStatusSigWord = 10, kStatusTileWord = 12, kStatusHeadTicketWord = 16, kStatusHeadTickets = 48;
+
+// Decision inputs of the drift kernels.
+struct DecideArgs {
+  int B, H;
+  const double *delta;
+  double gate_lo, gate_hi;
+  unsigned flags;
+  double *anchor_q, *anchor_k;
+  uint8_t *has_anchor, *refresh_ws, *pre_ws;
+  double *drift_out;
+  uint8_t *refresh_out;
+  int *ticket;  // zero between launches (the layer gate's counter, or one a head)
+};
 
 #ifdef __CUDACC__
 // Programmatic dependent launch: a kernel launched with the stream-serialisation attribute may be
@@ -130,6 +144,36 @@ __device__ __forceinline__ double exp_nonpositive(double x) {
   q = fma(q, r, 1.0);
   q = fma(q, r, 1.0);
   return __hiloint2double(__double2hiint(q) + (n << 20), __double2loint(q));
+}
+
+// Partial sums of one dim (`stride` kD) in four ascending ranges, s[q] that of range q, each added up in order.  All loads of a
+// range of up to eight chunks are in flight together (one after the other, as a rolled loop takes them, 32 chunks took 3 us).
+__device__ __forceinline__ double sum_range(const double *__restrict__ src, int i0, int i1) {
+  double s = 0.0;
+  for (int i = i0; i < i1; i += 8) {
+    double v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = __ldcg(&src[(size_t)min(i + u, i1 - 1) * kD]);
+#pragma unroll
+    for (int u = 0; u < 8; ++u) s = i + u < i1 ? s + v[u] : s;
+  }
+  return s;
+}
+__device__ __forceinline__ void sum_chunks(double (&s)[4], const double *__restrict__ src, int n) {
+  const int per = (n + 3) / 4;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) s[q] = 0.0;
+  for (int i = 0; i < per; i += 8) {
+    double v[4][8];
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+      for (int u = 0; u < 8; ++u) v[q][u] = __ldcg(&src[(size_t)min(q * per + i + u, n - 1) * kD]);
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+      for (int u = 0; u < 8; ++u) s[q] = i + u < per && q * per + i + u < n ? s[q] + v[q][u] : s[q];
+  }
 }
 
 // Lets a kernel use `bytes` of dynamic shared memory.  Asked of the runtime on every call (60 ns): the answer belongs to the
@@ -176,6 +220,12 @@ cudaError_t launch_block_sums(const Geom &g, const void *Q, const void *K, const
                               cudaStream_t s, int *launches);
 cudaError_t launch_decide(const Geom &g, const Workspace &w, const double *delta, heart_state st,
                           double *drift_out, uint8_t *refresh_out, cudaStream_t s, int *launches);
+DecideArgs decide_args(const Geom &g, const Workspace &w, const double *delta, heart_state st, double *drift_out, uint8_t *refresh_out);
+cudaError_t launch_decide(const Geom &g, const Workspace &w, const DecideArgs &a, cudaStream_t s);
+// Small layer-steps: masks of the refreshed heads in one kernel, with the decision unless the layer gate needs its own.
+bool rows_kernel_fits(const Geom &g);
+cudaError_t launch_decide_and_predict(const Geom &g, const Workspace &w, const DecideArgs &decide, const double *tau, heart_state st,
+                                      cudaStream_t s, int *launches);
 // expect_sig != 0: the block means were left by an earlier call; the kernels check the workspace's
 // signature against it and report HEART_ERR_DEVICE_CHECK (masks untouched) on a mismatch.
 cudaError_t launch_predict_mask(const Geom &g, const Workspace &w, const double *tau,

@@ -67,10 +67,14 @@ bool state_ok(const heart_state *st) {
 }
 
 // Mask prediction inside a layer-step (the refresh flags are the ones the decision kernel just wrote).
-cudaError_t predict_for_step(const Geom &g, const Workspace &w, const void *Q, const void *K, const double *tau,
-                             heart_state st, cudaStream_t s) {
+// The steps between the block sums and the attention: drift, decision, masks of the refreshed heads.
+cudaError_t decide_for_step(const Geom &g, const Workspace &w, const void *Q, const void *K, const double *delta, const double *tau,
+                            heart_state st, double *drift_out, uint8_t *refresh_out, cudaStream_t s) {
+  if (rows_kernel_fits(g)) return launch_decide_and_predict(g, w, decide_args(g, w, delta, st, drift_out, refresh_out), tau, st, s, &g_launches);
+  cudaError_t e = launch_decide(g, w, delta, st, drift_out, refresh_out, s, &g_launches);
+  if (e != cudaSuccess) return e;
   if (g.flags & HEART_ESTIMATOR_ANTIDIAG) {
-    cudaError_t e = launch_antidiag_scores(g, w, Q, K, w.refresh, s, &g_launches);
+    e = launch_antidiag_scores(g, w, Q, K, w.refresh, s, &g_launches);
     if (e != cudaSuccess) return e;
     return launch_top_p(g, w, tau, w.refresh, st, s, &g_launches, 0);
   }
@@ -210,10 +214,8 @@ int heart_step(const heart_config *cfg, const void *Q, const void *K, const void
   }
   e = launch_block_sums(g, Q, K, w, s, &g_launches);
   if (e != cudaSuccess) return cuda_fail(e, "block_sums");
-  e = launch_decide(g, w, delta, *st, drift_out, refresh_out, s, &g_launches);
-  if (e != cudaSuccess) return cuda_fail(e, "decide");
-  e = predict_for_step(g, w, Q, K, tau, *st, s);
-  if (e != cudaSuccess) return cuda_fail(e, "predict_mask");
+  e = decide_for_step(g, w, Q, K, delta, tau, *st, drift_out, refresh_out, s);
+  if (e != cudaSuccess) return cuda_fail(e, "decide, predict_mask");
   e = launch_attention(g, w, Q, K, V, st->kv_idx, st->kv_cnt, false, O, lse, s, &g_launches);
   if (e != cudaSuccess) return cuda_fail(e, "attention");
   return HEART_OK;
@@ -295,10 +297,8 @@ int heart_step_host(const heart_config *cfg, const void *Q_host, const void *K_h
   } else {
     e = launch_block_sums(g, Q_dev, K_dev, w, s, &g_launches);
     if (e != cudaSuccess) return cuda_fail(e, "block_sums");
-    e = launch_decide(g, w, delta, *st, w.drift, nullptr, s, &g_launches);
-    if (e != cudaSuccess) return cuda_fail(e, "decide");
-    e = predict_for_step(g, w, Q_dev, K_dev, tau, *st, s);
-    if (e != cudaSuccess) return cuda_fail(e, "predict_mask");
+    e = decide_for_step(g, w, Q_dev, K_dev, delta, tau, *st, w.drift, nullptr, s);
+    if (e != cudaSuccess) return cuda_fail(e, "decide, predict_mask");
   }
   const int groups = g.H < kHostGroups ? g.H : kHostGroups;
   for (int gi = 0; gi < groups; ++gi) {

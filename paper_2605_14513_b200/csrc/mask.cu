@@ -32,6 +32,8 @@ constexpr int kSmallScoreTiles = 148;  // 64 x 64 score tiles of a launch up to 
 // 161 against 167); short rows gain nothing and pay for the CTAs.
 template <int NJ>
 constexpr int kRowsPerCta = NJ >= 24 ? 2 : 8;
+template <int NJ>
+constexpr int kCtasPerSm = NJ >= 32 ? 10 : NJ >= 24 ? 12 : NJ >= 8 ? 4 : 5;  // (the registers that leaves: 96, 80, 64, 48)
 constexpr int kMaxCand = 64;    // candidates the direct threshold evaluation takes
 constexpr float kMassBand = 1.5e-5f;  // of z: cuts whose mass is closer to tau * z are decided in fp64
 // Blocks are ranked by their weight, lowest index first among equals.  Weights exp(s - max) round to the same double
@@ -154,8 +156,352 @@ __global__ void __launch_bounds__(128) pooled_scores_kernel(const double *__rest
   }
 }
 
+// The kept set of one row of scores, by one warp.  `weights`: NJ * 32 doubles of shared memory, `cand`: kMaxCand of them.
 template <int NJ>  // NJ*32 >= n_b
-__global__ void __launch_bounds__(32 * kRowsPerCta<NJ>) top_p_kernel(const double *__restrict__ scores, int nb, int pitch,
+__device__ __forceinline__ void top_p_row(const double *__restrict__ srow, int nb, double tau_r, double *weights, double *cand,
+                                          uint32_t *__restrict__ mask_row, int W, int32_t *__restrict__ idx_row, int32_t *cnt) {
+  const int lane = threadIdx.x & 31;
+  const unsigned lt_mask = (1u << lane) - 1u;
+  // fp64 search: the row lives in shared memory (lane-major, conflict-free), and rolled loops over the NJ blocks
+  // of a lane keep the kernel small -- fully unrolled over registers it was several times slower at n_b > 512.
+  double *pw = weights + lane;
+  const double neg_inf = __longlong_as_double(0xfff0000000000000LL);
+  // fp32 search: in registers (from shared memory with rolled loops: 121 us instead of 115 for 22296 rows of 929).
+  float x[NJ], e[NJ];  // s - max, exp of it
+  double mx = neg_inf;
+  {
+    double v[NJ];
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) v[j] = (j * 32 + lane < nb) ? srow[j * 32 + lane] : neg_inf;
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) mx = fmax(mx, v[j]);
+    mx = warp_max(mx);
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) x[j] = (float)(v[j] - mx);
+  }
+  // Outputs: the mask words are gathered in registers (lane l keeps word l) and leave in one store.
+  auto emit = [&](auto keep_of) {
+    int base = 0;
+    uint32_t my_word = 0u;
+#pragma unroll 4
+    for (int j = 0; j < NJ; ++j) {
+      const int J = j * 32 + lane;
+      const bool keep = keep_of(j, J < nb);
+      const unsigned word = __ballot_sync(0xffffffffu, keep);
+      if (lane == j) my_word = word;
+      if (keep) idx_row[base + __popc(word & lt_mask)] = J;
+      base += __popc(word);
+    }
+    if (lane < W) mask_row[lane] = my_word;
+    if (lane == 0) *cnt = base;
+  };
+
+  // fp32.  Error of a weight: x rounds by |x| 2^-24, its product with log2 e by |x| (2^-24 + 2^-25), ex2 by
+  // 2^-22 relative; over a row sum e (1.5e-7 |x| + 2.4e-7) <= 1.3e-6 z (sum e |x| <= z ln n_b).  tau * z
+  // takes 38 roundings more, 2.3e-6, the mass at a cut at most 37 + 38 + 64 (row, list,
+  // candidates), 8.3e-6: 1.2e-5 z together.
+  if (tau_r > 0.0 && tau_r < 1.0) {
+    float z = 0.f;
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) {
+      e[j] = ex2(x[j] * 1.44269504f);
+      z += e[j];
+    }
+    auto sum = [](float v) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      return v;
+    };
+    z = sum(z);
+    const float t = (float)tau_r * z, band = kMassBand * z;
+    // The threshold lies in [lo, hi): mass(x >= lo) reaches t, mass(x >= hi) = m_hi does not.  (All blocks below
+    // -20 together hold less than 2.1e-6.)
+    float lo = -20.f, hi = 1.f, m_hi = 0.f;
+    float v1 = -10.f, v2 = -5.f, v3 = -2.5f;
+    auto narrow = [&](float a1, float a2, float a3) {  // by the masses at v1 < v2 < v3
+      if (a3 >= t) {
+        lo = v3;
+      } else {
+        hi = v3, m_hi = a3;
+        if (a2 >= t) {
+          lo = v2;
+        } else {
+          hi = v2, m_hi = a2;
+          if (a1 >= t) lo = v1;
+          else hi = v1, m_hi = a1;
+        }
+      }
+      const float step = 0.25f * (hi - lo);
+      v1 = lo + step;
+      v2 = lo + 2.f * step;
+      v3 = hi - step;
+    };
+    for (int round = 0; round < 2; ++round) {
+      float a1 = 0.f, a2 = 0.f, a3 = 0.f;
+#pragma unroll
+      for (int j = 0; j < NJ; ++j) {
+        a1 += x[j] >= v1 ? e[j] : 0.f;
+        a2 += x[j] >= v2 ? e[j] : 0.f;
+        a3 += x[j] >= v3 ? e[j] : 0.f;
+      }
+      narrow(sum(a1), sum(a2), sum(a3));
+    }
+    // The blocks of that interval (a tenth of the row, as a rule) go to shared memory, where the search goes on.
+    float2 *list = reinterpret_cast<float2 *>(weights);
+    int n_list = 0;
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) {
+      const bool is_c = x[j] >= lo && x[j] < hi;
+      const unsigned bal = __ballot_sync(0xffffffffu, is_c);
+      if (is_c) list[n_list + __popc(bal & lt_mask)] = make_float2(x[j], e[j]);
+      n_list += __popc(bal);
+    }
+    __syncwarp();
+    float2 *close = reinterpret_cast<float2 *>(cand);
+    int n_cand = 0;
+    const float m_list = m_hi;  // mass above the list
+    for (int round = 0; round < 12; ++round) {
+      n_cand = 0;
+#pragma unroll 4
+      for (int k = lane; k - lane < n_list; k += 32) {
+        const float2 c = k < n_list ? list[k] : make_float2(-INFINITY, 0.f);
+        const bool is_c = c.x >= lo && c.x < hi;
+        const unsigned bal = __ballot_sync(0xffffffffu, is_c);
+        const int pos = n_cand + __popc(bal & lt_mask);
+        if (is_c && pos < kMaxCand) close[pos] = c;
+        n_cand += __popc(bal);
+      }
+      __syncwarp();
+      if (n_cand <= kMaxCand) break;
+      // More than the direct evaluation takes.  Equal ones (the first 64, at least) are left to fp64 at once: quarters do
+      // not part them (12 rounds on rows of equal scores: 1147 us for 22296 of 929, 852 now; fp64 alone, before: 902).
+      if (__all_sync(0xffffffffu, close[lane].x == close[0].x && close[lane + 32].x == close[0].x)) break;
+      float a1 = 0.f, a2 = 0.f, a3 = 0.f;
+#pragma unroll 4
+      for (int k = lane; k < n_list; k += 32) {
+        const float2 c = list[k];
+        a1 += c.x >= v1 ? c.y : 0.f;
+        a2 += c.x >= v2 ? c.y : 0.f;
+        a3 += c.x >= v3 ? c.y : 0.f;
+      }
+      narrow(m_list + sum(a1), m_list + sum(a2), m_list + sum(a3));
+    }
+    if (n_cand <= kMaxCand) {
+      // Each lane takes two candidates: is the cut at this one, clearly?
+      if (lane == 0 && (n_cand & 1)) close[n_cand] = make_float2(-INFINITY, 0.f);  // (read in pairs; cand has room for one more)
+      __syncwarp();
+      float x_cut = 0.f;
+      bool found = false;
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        if (k * 32 >= n_cand) break;
+        const bool have = lane + 32 * k < n_cand;
+        const float2 mine = close[have ? lane + 32 * k : 0];
+        float above = m_hi;
+#pragma unroll 4
+        for (int n = 0; n < n_cand; n += 2) {
+          const float4 c = *reinterpret_cast<const float4 *>(&close[n]);
+          above += c.x > mine.x ? c.y : 0.f;
+          above += c.z > mine.x ? c.w : 0.f;
+        }
+        if (have && t - above > band && above + mine.y - t > band) found = true, x_cut = mine.x;
+      }
+      const unsigned who = __ballot_sync(0xffffffffu, found);
+      bool clear = __popc(who) == 1;
+      if (clear) {
+        // ... and no other block may share its weight (with the interval's ends: no block outside is as near)
+        x_cut = __shfl_sync(0xffffffffu, x_cut, __ffs(who) - 1);
+        const float near = fmaf(fabsf(x_cut), kTieRel, kTieAbs);
+        const unsigned same0 = __ballot_sync(0xffffffffu, lane < n_cand && fabsf(close[lane].x - x_cut) <= near);
+        const unsigned same1 = __ballot_sync(0xffffffffu, lane + 32 < n_cand && fabsf(close[lane + 32].x - x_cut) <= near);
+        clear = __popc(same0) + __popc(same1) == 1 && x_cut - near >= lo && x_cut + near < hi;
+      }
+      if (clear) {
+        int base = 0;
+        uint32_t my_word = 0u;
+#pragma unroll
+        for (int j = 0; j < NJ; ++j) {
+          const bool keep = j * 32 + lane < nb && x[j] >= x_cut;
+          const unsigned word = __ballot_sync(0xffffffffu, keep);
+          my_word = lane == j ? word : my_word;
+          if (keep) idx_row[base + __popc(word & lt_mask)] = j * 32 + lane;
+          base += __popc(word);
+        }
+        if (lane < W) mask_row[lane] = my_word;
+        if (lane == 0) *cnt = base;
+        return;
+      }
+    }
+    __syncwarp();
+  }
+
+  // fp64
+  double z = 0.0;
+#pragma unroll 4
+  for (int j = 0; j < NJ; ++j) {
+    const int J = j * 32 + lane;
+    pw[(j) * 32] = (J < nb) ? exp_nonpositive(srow[J] - mx) : 0.0;
+    z += pw[(j) * 32];
+  }
+  z = warp_sum(z);
+  // From here on p holds the unnormalised weights e = exp(s - max) <= 1 and every mass is compared
+  // with tau * z instead of dividing the row by z: the same ranking, the same ties and the same
+  // cumulative-mass test up to rounding, at 1/3 fewer fp64 instructions per block.
+  // tau <= 0: every prefix reaches it, so the minimal one is the single largest block (lowest index
+  // on ties): the smallest positive threshold gives exactly that
+  const double t = (tau_r > 0.0 ? tau_r : 2.2250738585072014e-308) * z;
+  const bool keep_all = !(tau_r < 1.0) || !(z >= t);
+  long long theta = 0;
+  int m_ties = 0, n_ties = 0;
+  if (!keep_all) {
+    // Rounds over all blocks, two bits of theta each: three trial thresholds per round, their three
+    // reductions side by side (fixed split of the sums: same order on every run).
+    auto round2 = [&](int bit) {
+      // trial patterns theta | 01, 10, 11 at bits (bit+1, bit): the mass is non-increasing in them
+      // (bit >= 32: the low words of the patterns are zero, so comparing the high words decides)
+      const long long c1 = theta | (1LL << bit), c2 = theta | (2LL << bit), c3 = theta | (3LL << bit);
+      const int h1 = (int)(c1 >> 32), h2 = (int)(c2 >> 32), h3 = (int)(c3 >> 32);
+      double a1 = 0.0, a2 = 0.0, a3 = 0.0, b1 = 0.0, b2 = 0.0, b3 = 0.0;
+#pragma unroll 2
+      for (int j = 0; j < NJ; j += 2) {
+        const int k0 = __double2hiint(pw[(j) * 32]), k1 = __double2hiint(pw[(j + 1) * 32]);
+        if (k0 >= h1) a1 += pw[(j) * 32];
+        if (k0 >= h2) a2 += pw[(j) * 32];
+        if (k0 >= h3) a3 += pw[(j) * 32];
+        if (k1 >= h1) b1 += pw[(j + 1) * 32];
+        if (k1 >= h2) b2 += pw[(j + 1) * 32];
+        if (k1 >= h3) b3 += pw[(j + 1) * 32];
+      }
+      double m1 = a1 + b1, m2 = a2 + b2, m3 = a3 + b3;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        m1 += __shfl_xor_sync(0xffffffffu, m1, o);
+        m2 += __shfl_xor_sync(0xffffffffu, m2, o);
+        m3 += __shfl_xor_sync(0xffffffffu, m3, o);
+      }
+      theta = (m3 >= t) ? c3 : (m2 >= t) ? c2 : (m1 >= t) ? c1 : theta;
+    };
+    static_assert(NJ % 2 == 0, "two blocks per step");
+    // The exponent and the top four mantissa bits first (bits 61..48; bit 62 is clear for p <= 1) ...
+    constexpr int low = 48;  // bits [low, 62) of theta are decided over all blocks
+    static_assert(low >= 32, "the full-width rounds compare high words only");
+    // theta is the value of one of the blocks, so it shares the leading bits that the largest and
+    // the smallest weight of the row have in common: the rounds start below them.
+    int first_bit = 60;
+    {
+      int hmax = 0, hmin = 0x7fffffff;
+#pragma unroll 4
+      for (int j = 0; j < NJ; ++j) {
+        const int h = __double2hiint(pw[(j) * 32]);
+        hmax = max(hmax, h);
+        if (j * 32 + lane < nb) hmin = min(hmin, h);
+      }
+      hmax = __reduce_max_sync(0xffffffffu, hmax);
+      hmin = __reduce_min_sync(0xffffffffu, hmin);
+      const int top = 63 - __clz(hmax ^ hmin);  // highest bit (of the 64) in which they differ; 31 if none in the high word
+      first_bit = min(60, top & ~1);            // the round at `bit` decides bits (bit + 1, bit)
+      if (first_bit + 2 < 62) theta = ((long long)hmax << 32) & ~((1LL << (first_bit + 2)) - 1);
+    }
+    for (int bit = first_bit; bit >= low; bit -= 2) round2(bit);
+    if (first_bit < low) theta &= ~((1LL << low) - 1);  // the whole searched prefix is common
+    // ... then only the blocks whose pattern shares that prefix can still decide the remaining bits:
+    // they are compacted into shared memory (the first kMaxCand of them; more than that takes the
+    // slow path below, which does not read the list).  Blocks above the prefix enter as one constant.
+    const long long hi = theta >> low;
+    double *scr = cand;
+    double ab0 = 0.0, ab1 = 0.0;
+    int n_cand = 0;
+    __syncwarp();
+#pragma unroll 4
+    for (int j = 0; j < NJ; ++j) {
+      const long long kh = __double_as_longlong(pw[(j) * 32]) >> low;
+      if (kh > hi) {
+        if (j & 1) ab1 += pw[(j) * 32]; else ab0 += pw[(j) * 32];
+      }
+      const bool is_c = (kh == hi) && (j * 32 + lane < nb);
+      const unsigned bal = __ballot_sync(0xffffffffu, is_c);
+      if (is_c) {
+        const int pos = n_cand + __popc(bal & lt_mask);
+        if (pos < kMaxCand) scr[pos] = pw[(j) * 32];
+      }
+      n_cand += __popc(bal);
+    }
+    const double mass_above = warp_sum(ab0 + ab1);
+    __syncwarp();
+    if (n_cand <= kMaxCand) {
+      // Few candidates: each lane takes two of them and adds up, over all candidates, the mass at
+      // or above its own value; theta is the largest candidate whose mass still reaches tau (the
+      // smallest candidate always does: that is what the prefix search established).
+      const double c0 = (lane < n_cand) ? scr[lane] : 0.0, c1 = (lane + 32 < n_cand) ? scr[lane + 32] : 0.0;
+      const long long k0 = __double_as_longlong(c0), k1 = __double_as_longlong(c1);
+      double g0 = mass_above, g1 = mass_above;
+      long long k_min = 0x7fffffffffffffffLL;
+      for (int n = 0; n < n_cand; ++n) {
+        const double v = scr[n];
+        const long long kv = __double_as_longlong(v);
+        if (kv >= k0) g0 += v;
+        if (kv >= k1) g1 += v;
+        k_min = kv < k_min ? kv : k_min;
+      }
+      long long best = k_min;
+      if (lane < n_cand && g0 >= t && k0 > best) best = k0;
+      if (lane + 32 < n_cand && g1 >= t && k1 > best) best = k1;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const long long other = __shfl_xor_sync(0xffffffffu, best, o);
+        best = other > best ? other : best;
+      }
+      theta = best;
+    } else {  // many near-equal blocks: keep searching over all of them, a bit at a time
+      for (int bit = low - 1; bit >= 0; --bit) {
+        const long long cnd = theta | (1LL << bit);
+        double g0 = 0.0, g1 = 0.0, g2 = 0.0, g3 = 0.0;  // fixed 4-way split: same order on every run
+#pragma unroll 1
+        for (int j = 0; j < NJ; j += 4) {
+          if (__double_as_longlong(pw[(j) * 32]) >= cnd) g0 += pw[(j) * 32];
+          if (j + 1 < NJ && __double_as_longlong(pw[(j + 1) * 32]) >= cnd) g1 += pw[(j + 1) * 32];
+          if (j + 2 < NJ && __double_as_longlong(pw[(j + 2) * 32]) >= cnd) g2 += pw[(j + 2) * 32];
+          if (j + 3 < NJ && __double_as_longlong(pw[(j + 3) * 32]) >= cnd) g3 += pw[(j + 3) * 32];
+        }
+        if (warp_sum((g0 + g1) + (g2 + g3)) >= t) theta = cnd;
+      }
+    }
+    double above = 0.0;
+    int nties = 0;
+#pragma unroll 4
+    for (int j = 0; j < NJ; ++j) {
+      const long long b = __double_as_longlong(pw[(j) * 32]);
+      if (b > theta) above += pw[(j) * 32];
+      nties += (b == theta && j * 32 + lane < nb) ? 1 : 0;
+    }
+    above = warp_sum(above);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) nties += __shfl_xor_sync(0xffffffffu, nties, o);
+    const double th = __longlong_as_double(theta);
+    double c = above;
+    do {  // ties enter in ascending index order, one at a time, until the mass reaches tau
+      c += th;
+      ++m_ties;
+    } while (c < t && m_ties < nties);
+    n_ties = nties;
+  }
+
+  int tie_seen = 0;
+  // the usual case: every block equal to theta is kept (theta = 0 when all blocks are kept)
+  const bool all_ties_kept = keep_all || m_ties == n_ties;
+  emit([&](int j, bool valid) {
+    const long long b = __double_as_longlong(pw[(j) * 32]);
+    if (all_ties_kept) return valid && b >= theta;
+    const bool is_tie = valid && b == theta;
+    const unsigned tie_ballot = __ballot_sync(0xffffffffu, is_tie);
+    const int tie_rank = tie_seen + __popc(tie_ballot & lt_mask);
+    tie_seen += __popc(tie_ballot);
+    return valid && (b > theta || (is_tie && tie_rank < m_ties));
+  });
+}
+
+template <int NJ>  // NJ*32 >= n_b
+__global__ void __launch_bounds__(32 * kRowsPerCta<NJ>, kCtasPerSm<NJ>) top_p_kernel(const double *__restrict__ scores, int nb, int pitch,
                                                                  const double *__restrict__ tau,
                                                                  const uint8_t *__restrict__ refresh,
                                                                  unsigned flags, uint32_t *__restrict__ mask_bits,
@@ -168,343 +514,126 @@ __global__ void __launch_bounds__(32 * kRowsPerCta<NJ>) top_p_kernel(const doubl
   if (expect_sig != 0 && *reinterpret_cast<const unsigned long long *>(status + kStatusSigWord) != expect_sig)
     return;  // reported by the score kernel
   if (refresh != nullptr && refresh[r] == 0) return;  // reuse branch of Algorithm 1: mask untouched
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int warp = threadIdx.x >> 5;
   extern __shared__ __align__(16) unsigned char smem_top[];
   double *weights = reinterpret_cast<double *>(smem_top);  // [kRowsPerCta<NJ>][NJ * 32]
-  __shared__ double cand[kRowsPerCta<NJ>][kMaxCand];
-  const unsigned lt_mask = (1u << lane) - 1u;
+  __shared__ __align__(16) double cand[kRowsPerCta<NJ>][kMaxCand];
+  const int I = blockIdx.x * kRowsPerCta<NJ> + warp;
+  if (I >= nb) return;
+  const size_t row = (size_t)r * nb + I;
+  top_p_row<NJ>(scores + row * pitch, nb, (flags & HEART_FORCE_DENSE) ? 1.0 : tau[r], weights + (size_t)warp * NJ * 32, cand[warp],
+                mask_bits + row * W, W, kv_idx + row * idx_stride, kv_cnt + row);
+}
+
+// Small layer-steps: a CTA takes eight query blocks of a head from the pooled means to the lists, a warp per row, so that one
+// launch does the work of two or three (whole steps: 2 x 2048 tokens 26.7 us with three, 24.5 with one; 2 x 12 x 2465 with the
+// gate 71.4 and 68.6).  Bound by latency.  DECIDE (no layer gate, a ticket for every head): every CTA of a head adds up the head's token means and decides for itself, bit for bit like mean_drift_kernel; the CTA that took the
+// last of the head's tickets, when all of them have read the old anchor, moves it.
+struct RowArgs {
+  const double *bmean, *tau;
+  int R, nb;
+  double scale;
+  unsigned flags;
+  const uint8_t *refresh;  // without DECIDE
+  uint32_t *mask_bits;
+  int32_t *kv_idx, *kv_cnt;
+  int idx_stride, W;
+  const double *psum;  // DECIDE
+  int N, nchunks;
+  DecideArgs decide;
+};
+constexpr int kRowsKernelThreads = 256, kRowsKernelPitch = kD + 4;
+__host__ __device__ inline int rows_kernel_doubles(int nj, int nb) { return (8 + (nb + 7) / 8 * 8) * kRowsKernelPitch + 2 * 8 * nj * 32; }
+
+template <int NJ, bool DECIDE>
+__global__ void __launch_bounds__(kRowsKernelThreads) mask_rows_kernel(const RowArgs a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int nb = a.nb, keys = (nb + 7) / 8 * 8, r = blockIdx.y, I0 = blockIdx.x * 8;
+  double *tile = reinterpret_cast<double *>(smem_raw);  // 8 query rows, then the key rows
+  double *scores = tile + (8 + keys) * kRowsKernelPitch, *weights = scores + 8 * NJ * 32;
+  __shared__ __align__(16) double cand[8][kMaxCand];
+  __shared__ double wsum[8], mean[2 * kD];
+  __shared__ int sh_refresh;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  double anc = 0.0, dl = 0.0;
+  bool had = false;
+  if (DECIDE) {  // what does not come from the block-sum pass
+    anc = ((tid >> 7) ? a.decide.anchor_k : a.decide.anchor_q)[(size_t)r * kD + (tid & (kD - 1))];
+    if (tid == 0) {
+      had = a.decide.has_anchor[r] != 0;
+      dl = a.decide.delta[r];
+    }
+  }
+  pdl_wait();
+  pdl_launch_dependents();
+  if (!DECIDE && a.refresh[r] == 0) return;  // (decided by mean_drift_kernel, which has the layer gate)
+  const double *bq = a.bmean + (size_t)r * nb * kD, *bk = a.bmean + ((size_t)a.R + r) * nb * kD;
+#pragma unroll 8
+  for (int e = tid; e < (8 + keys) * (kD / 2); e += kRowsKernelThreads) {
+    const int row = e / (kD / 2), dd = e % (kD / 2) * 2, blk = row < 8 ? I0 + row : row - 8;
+    cp_async16(tile + row * kRowsKernelPitch + dd, (row < 8 ? bq : bk) + (size_t)min(blk, nb - 1) * kD + dd, blk < nb ? 16 : 0);
+  }
+  cp_async_commit();
+  if (DECIDE) {
+    double s[4];
+    sum_chunks(s, a.psum + ((size_t)(tid >> 7) * a.R + r) * a.nchunks * kD + (tid & (kD - 1)), a.nchunks);
+    const double m = (((s[0] + s[1]) + s[2]) + s[3]) / (double)a.N;
+    mean[tid] = m;
+    double v = fabs(anc - m);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (lane == 0) wsum[warp] = v;
+    __syncthreads();
+    if (tid == 0) {
+      const double pq = (wsum[0] + wsum[1]) + (wsum[2] + wsum[3]), pk = (wsum[4] + wsum[5]) + (wsum[6] + wsum[7]);
+      const double dr = had ? (pq + pk) : __longlong_as_double(0x7ff0000000000000LL);
+      const bool rf = !had || dr > dl || (a.decide.flags & HEART_FORCE_REFRESH) != 0;
+      if (blockIdx.x == 0) {
+        if (a.decide.drift_out) a.decide.drift_out[r] = dr;
+        if (a.decide.refresh_out) a.decide.refresh_out[r] = rf;
+        a.decide.refresh_ws[r] = rf;
+      }
+      sh_refresh = rf;
+    }
+  }
+  cp_async_wait<0>();
+  __syncthreads();
+  if (DECIDE && !sh_refresh) return;
+  int last = 0;
+  if (DECIDE && warp == 7 && lane == 0) {
+    // every warp has read its part of the anchor; asked for here, the answer has come when the lists are out
+    __threadfence();
+    last = atomicAdd(&a.decide.ticket[r], 1) == (int)gridDim.x - 1;
+  }
+  // 8 x 8 scores at a time, the 128 dims in ascending order as everywhere
   {
-    const int I = blockIdx.x * kRowsPerCta<NJ> + warp;
-    if (I >= nb) return;
-    const size_t row = (size_t)r * nb + I;
-    const double *srow = scores + row * pitch;
-    // fp64 search: the row lives in shared memory (lane-major, conflict-free), and rolled loops over the NJ blocks
-    // of a lane keep the kernel small -- fully unrolled over registers it was several times slower at n_b > 512.
-    double *pw = weights + (size_t)warp * NJ * 32 + lane;
-    const double neg_inf = __longlong_as_double(0xfff0000000000000LL);
-    // fp32 search: in registers (from shared memory with rolled loops: 121 us instead of 115 for 22296 rows of 929).
-    float x[NJ], e[NJ];  // s - max, exp of it
-    double mx = neg_inf;
-    {
-      double v[NJ];
+    const double *A = tile + (lane >> 2) * kRowsKernelPitch + (lane & 3), *B = A + (8 + warp * 8) * kRowsKernelPitch;
+    double acc[(NJ + 1) / 2][2];
 #pragma unroll
-      for (int j = 0; j < NJ; ++j) v[j] = (j * 32 + lane < nb) ? srow[j * 32 + lane] : neg_inf;
+    for (int i = 0; i < (NJ + 1) / 2; ++i) acc[i][0] = acc[i][1] = 0.0;
+#pragma unroll 8
+    for (int k = 0; k < kD; k += 4) {
+      const double q = A[k];
 #pragma unroll
-      for (int j = 0; j < NJ; ++j) mx = fmax(mx, v[j]);
-      mx = warp_max(mx);
-#pragma unroll
-      for (int j = 0; j < NJ; ++j) x[j] = (float)(v[j] - mx);
+      for (int i = 0; i < (NJ + 1) / 2; ++i)
+        if ((warp + 8 * i) * 8 < keys) mma_f64(acc[i], q, B[i * 64 * kRowsKernelPitch + k]);
     }
-    const double tau_r = (flags & HEART_FORCE_DENSE) ? 1.0 : tau[r];
-    // Outputs: the mask words are gathered in registers (lane l keeps word l) and leave in one store.
-    auto emit = [&](auto keep_of) {
-      int base = 0;
-      uint32_t my_word = 0u;
-#pragma unroll 4
-      for (int j = 0; j < NJ; ++j) {
-        const int J = j * 32 + lane;
-        const bool keep = keep_of(j, J < nb);
-        const unsigned word = __ballot_sync(0xffffffffu, keep);
-        if (lane == j) my_word = word;
-        if (keep) kv_idx[row * idx_stride + base + __popc(word & lt_mask)] = J;
-        base += __popc(word);
-      }
-      if (lane < W) mask_bits[row * W + lane] = my_word;
-      if (lane == 0) kv_cnt[row] = base;
-    };
-
-    // fp32.  Error of a weight: x rounds by |x| 2^-24, its product with log2 e by |x| (2^-24 + 2^-25), ex2 by
-    // 2^-22 relative; over a row sum e (1.5e-7 |x| + 2.4e-7) <= 1.3e-6 z (sum e |x| <= z ln n_b).  tau * z
-    // takes 38 roundings more, 2.3e-6, the mass at a cut at most 37 + 38 + 64 (row, list,
-    // candidates), 8.3e-6: 1.2e-5 z together.
-    if (tau_r > 0.0 && tau_r < 1.0) {
-      float z = 0.f;
 #pragma unroll
-      for (int j = 0; j < NJ; ++j) {
-        e[j] = ex2(x[j] * 1.44269504f);
-        z += e[j];
-      }
-      auto sum = [](float v) {
+    for (int i = 0; i < (NJ + 1) / 2; ++i)
+      if ((warp + 8 * i) * 8 < keys)
+        *reinterpret_cast<double2 *>(scores + (lane >> 2) * NJ * 32 + (warp + 8 * i) * 8 + 2 * (lane & 3)) =
+            make_double2(acc[i][0] * a.scale, acc[i][1] * a.scale);
+  }
+  __syncthreads();
+  const int I = I0 + warp;
+  const size_t row = (size_t)r * nb + I;
+  if (I < nb)
+    top_p_row<NJ>(scores + warp * NJ * 32, nb, (a.flags & HEART_FORCE_DENSE) ? 1.0 : a.tau[r], weights + warp * NJ * 32, cand[warp],
+                  a.mask_bits + row * a.W, a.W, a.kv_idx + row * a.idx_stride, a.kv_cnt + row);
+  if (DECIDE && warp == 7 && __shfl_sync(0xffffffffu, last, 0)) {
+    if (lane == 0) a.decide.ticket[r] = 0, a.decide.has_anchor[r] = 1;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        return v;
-      };
-      z = sum(z);
-      const float t = (float)tau_r * z, band = kMassBand * z;
-      // The threshold lies in [lo, hi): mass(x >= lo) reaches t, mass(x >= hi) = m_hi does not.  (All blocks below
-      // -20 together hold less than 2.1e-6.)
-      float lo = -20.f, hi = 1.f, m_hi = 0.f;
-      float v1 = -10.f, v2 = -5.f, v3 = -2.5f;
-      auto narrow = [&](float a1, float a2, float a3) {  // by the masses at v1 < v2 < v3
-        if (a3 >= t) {
-          lo = v3;
-        } else {
-          hi = v3, m_hi = a3;
-          if (a2 >= t) {
-            lo = v2;
-          } else {
-            hi = v2, m_hi = a2;
-            if (a1 >= t) lo = v1;
-            else hi = v1, m_hi = a1;
-          }
-        }
-        const float step = 0.25f * (hi - lo);
-        v1 = lo + step;
-        v2 = lo + 2.f * step;
-        v3 = hi - step;
-      };
-      for (int round = 0; round < 2; ++round) {
-        float a1 = 0.f, a2 = 0.f, a3 = 0.f;
-#pragma unroll
-        for (int j = 0; j < NJ; ++j) {
-          a1 += x[j] >= v1 ? e[j] : 0.f;
-          a2 += x[j] >= v2 ? e[j] : 0.f;
-          a3 += x[j] >= v3 ? e[j] : 0.f;
-        }
-        narrow(sum(a1), sum(a2), sum(a3));
-      }
-      // The blocks of that interval (a tenth of the row, as a rule) go to shared memory, where the search goes on.
-      float2 *list = reinterpret_cast<float2 *>(weights + (size_t)warp * NJ * 32);
-      int n_list = 0;
-#pragma unroll
-      for (int j = 0; j < NJ; ++j) {
-        const bool is_c = x[j] >= lo && x[j] < hi;
-        const unsigned bal = __ballot_sync(0xffffffffu, is_c);
-        if (is_c) list[n_list + __popc(bal & lt_mask)] = make_float2(x[j], e[j]);
-        n_list += __popc(bal);
-      }
-      __syncwarp();
-      float *cx = reinterpret_cast<float *>(cand[warp]), *ce = cx + kMaxCand;
-      int n_cand = 0;
-      const float m_list = m_hi;  // mass above the list
-      for (int round = 0; round < 12; ++round) {
-        n_cand = 0;
-#pragma unroll 4
-        for (int k = lane; k - lane < n_list; k += 32) {
-          const float2 c = k < n_list ? list[k] : make_float2(-INFINITY, 0.f);
-          const bool is_c = c.x >= lo && c.x < hi;
-          const unsigned bal = __ballot_sync(0xffffffffu, is_c);
-          const int pos = n_cand + __popc(bal & lt_mask);
-          if (is_c && pos < kMaxCand) cx[pos] = c.x, ce[pos] = c.y;
-          n_cand += __popc(bal);
-        }
-        __syncwarp();
-        if (n_cand <= kMaxCand) break;
-        // More than the direct evaluation takes.  Equal ones (the first 64, at least) are left to fp64 at once: quarters do
-        // not part them (12 rounds on rows of equal scores: 1147 us for 22296 of 929, 852 now; fp64 alone, before: 902).
-        if (__all_sync(0xffffffffu, cx[lane] == cx[0] && cx[lane + 32] == cx[0])) break;
-        float a1 = 0.f, a2 = 0.f, a3 = 0.f;
-#pragma unroll 4
-        for (int k = lane; k < n_list; k += 32) {
-          const float2 c = list[k];
-          a1 += c.x >= v1 ? c.y : 0.f;
-          a2 += c.x >= v2 ? c.y : 0.f;
-          a3 += c.x >= v3 ? c.y : 0.f;
-        }
-        narrow(m_list + sum(a1), m_list + sum(a2), m_list + sum(a3));
-      }
-      if (n_cand <= kMaxCand) {
-        // Each lane takes two candidates: is the cut at this one, clearly?
-        float x_cut = 0.f;
-        bool found = false;
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-          if (k * 32 >= n_cand) break;
-          const bool have = lane + 32 * k < n_cand;
-          const float xk = have ? cx[lane + 32 * k] : 0.f, ek = have ? ce[lane + 32 * k] : 0.f;
-          const float near = fmaf(fabsf(xk), kTieRel, kTieAbs);  // (with the interval's ends: no block outside is as near)
-          float above = m_hi;
-          int same = 0;
-          for (int n = 0; n < n_cand; ++n) {
-            above += cx[n] > xk ? ce[n] : 0.f;
-            same += fabsf(cx[n] - xk) <= near ? 1 : 0;
-          }
-          if (have && same == 1 && xk - near >= lo && xk + near < hi && t - above > band && above + ek - t > band) found = true, x_cut = xk;
-        }
-        const unsigned who = __ballot_sync(0xffffffffu, found);
-        if (__popc(who) == 1) {
-          x_cut = __shfl_sync(0xffffffffu, x_cut, __ffs(who) - 1);
-          int base = 0;
-          uint32_t my_word = 0u;
-#pragma unroll
-          for (int j = 0; j < NJ; ++j) {
-            const bool keep = j * 32 + lane < nb && x[j] >= x_cut;
-            const unsigned word = __ballot_sync(0xffffffffu, keep);
-            my_word = lane == j ? word : my_word;
-            if (keep) kv_idx[row * idx_stride + base + __popc(word & lt_mask)] = j * 32 + lane;
-            base += __popc(word);
-          }
-          if (lane < W) mask_bits[row * W + lane] = my_word;
-          if (lane == 0) kv_cnt[row] = base;
-          return;
-        }
-      }
-      __syncwarp();
-    }
-
-    // fp64
-    double z = 0.0;
-#pragma unroll 4
-    for (int j = 0; j < NJ; ++j) {
-      const int J = j * 32 + lane;
-      pw[(j) * 32] = (J < nb) ? exp_nonpositive(srow[J] - mx) : 0.0;
-      z += pw[(j) * 32];
-    }
-    z = warp_sum(z);
-    // From here on p holds the unnormalised weights e = exp(s - max) <= 1 and every mass is compared
-    // with tau * z instead of dividing the row by z: the same ranking, the same ties and the same
-    // cumulative-mass test up to rounding, at 1/3 fewer fp64 instructions per block.
-    // tau <= 0: every prefix reaches it, so the minimal one is the single largest block (lowest index
-    // on ties): the smallest positive threshold gives exactly that
-    const double t = (tau_r > 0.0 ? tau_r : 2.2250738585072014e-308) * z;
-    const bool keep_all = !(tau_r < 1.0) || !(z >= t);
-    long long theta = 0;
-    int m_ties = 0, n_ties = 0;
-    if (!keep_all) {
-      // Rounds over all blocks, two bits of theta each: three trial thresholds per round, their three
-      // reductions side by side (fixed split of the sums: same order on every run).
-      auto round2 = [&](int bit) {
-        // trial patterns theta | 01, 10, 11 at bits (bit+1, bit): the mass is non-increasing in them
-        // (bit >= 32: the low words of the patterns are zero, so comparing the high words decides)
-        const long long c1 = theta | (1LL << bit), c2 = theta | (2LL << bit), c3 = theta | (3LL << bit);
-        const int h1 = (int)(c1 >> 32), h2 = (int)(c2 >> 32), h3 = (int)(c3 >> 32);
-        double a1 = 0.0, a2 = 0.0, a3 = 0.0, b1 = 0.0, b2 = 0.0, b3 = 0.0;
-#pragma unroll 2
-        for (int j = 0; j < NJ; j += 2) {
-          const int k0 = __double2hiint(pw[(j) * 32]), k1 = __double2hiint(pw[(j + 1) * 32]);
-          if (k0 >= h1) a1 += pw[(j) * 32];
-          if (k0 >= h2) a2 += pw[(j) * 32];
-          if (k0 >= h3) a3 += pw[(j) * 32];
-          if (k1 >= h1) b1 += pw[(j + 1) * 32];
-          if (k1 >= h2) b2 += pw[(j + 1) * 32];
-          if (k1 >= h3) b3 += pw[(j + 1) * 32];
-        }
-        double m1 = a1 + b1, m2 = a2 + b2, m3 = a3 + b3;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          m1 += __shfl_xor_sync(0xffffffffu, m1, o);
-          m2 += __shfl_xor_sync(0xffffffffu, m2, o);
-          m3 += __shfl_xor_sync(0xffffffffu, m3, o);
-        }
-        theta = (m3 >= t) ? c3 : (m2 >= t) ? c2 : (m1 >= t) ? c1 : theta;
-      };
-      static_assert(NJ % 2 == 0, "two blocks per step");
-      // The exponent and the top four mantissa bits first (bits 61..48; bit 62 is clear for p <= 1) ...
-      constexpr int low = 48;  // bits [low, 62) of theta are decided over all blocks
-      static_assert(low >= 32, "the full-width rounds compare high words only");
-      // theta is the value of one of the blocks, so it shares the leading bits that the largest and
-      // the smallest weight of the row have in common: the rounds start below them.
-      int first_bit = 60;
-      {
-        int hmax = 0, hmin = 0x7fffffff;
-#pragma unroll 4
-        for (int j = 0; j < NJ; ++j) {
-          const int h = __double2hiint(pw[(j) * 32]);
-          hmax = max(hmax, h);
-          if (j * 32 + lane < nb) hmin = min(hmin, h);
-        }
-        hmax = __reduce_max_sync(0xffffffffu, hmax);
-        hmin = __reduce_min_sync(0xffffffffu, hmin);
-        const int top = 63 - __clz(hmax ^ hmin);  // highest bit (of the 64) in which they differ; 31 if none in the high word
-        first_bit = min(60, top & ~1);            // the round at `bit` decides bits (bit + 1, bit)
-        if (first_bit + 2 < 62) theta = ((long long)hmax << 32) & ~((1LL << (first_bit + 2)) - 1);
-      }
-      for (int bit = first_bit; bit >= low; bit -= 2) round2(bit);
-      if (first_bit < low) theta &= ~((1LL << low) - 1);  // the whole searched prefix is common
-      // ... then only the blocks whose pattern shares that prefix can still decide the remaining bits:
-      // they are compacted into shared memory (the first kMaxCand of them; more than that takes the
-      // slow path below, which does not read the list).  Blocks above the prefix enter as one constant.
-      const long long hi = theta >> low;
-      double *scr = cand[warp];
-      double ab0 = 0.0, ab1 = 0.0;
-      int n_cand = 0;
-      __syncwarp();
-#pragma unroll 4
-      for (int j = 0; j < NJ; ++j) {
-        const long long kh = __double_as_longlong(pw[(j) * 32]) >> low;
-        if (kh > hi) {
-          if (j & 1) ab1 += pw[(j) * 32]; else ab0 += pw[(j) * 32];
-        }
-        const bool is_c = (kh == hi) && (j * 32 + lane < nb);
-        const unsigned bal = __ballot_sync(0xffffffffu, is_c);
-        if (is_c) {
-          const int pos = n_cand + __popc(bal & lt_mask);
-          if (pos < kMaxCand) scr[pos] = pw[(j) * 32];
-        }
-        n_cand += __popc(bal);
-      }
-      const double mass_above = warp_sum(ab0 + ab1);
-      __syncwarp();
-      if (n_cand <= kMaxCand) {
-        // Few candidates: each lane takes two of them and adds up, over all candidates, the mass at
-        // or above its own value; theta is the largest candidate whose mass still reaches tau (the
-        // smallest candidate always does: that is what the prefix search established).
-        const double c0 = (lane < n_cand) ? scr[lane] : 0.0, c1 = (lane + 32 < n_cand) ? scr[lane + 32] : 0.0;
-        const long long k0 = __double_as_longlong(c0), k1 = __double_as_longlong(c1);
-        double g0 = mass_above, g1 = mass_above;
-        long long k_min = 0x7fffffffffffffffLL;
-        for (int n = 0; n < n_cand; ++n) {
-          const double v = scr[n];
-          const long long kv = __double_as_longlong(v);
-          if (kv >= k0) g0 += v;
-          if (kv >= k1) g1 += v;
-          k_min = kv < k_min ? kv : k_min;
-        }
-        long long best = k_min;
-        if (lane < n_cand && g0 >= t && k0 > best) best = k0;
-        if (lane + 32 < n_cand && g1 >= t && k1 > best) best = k1;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          const long long other = __shfl_xor_sync(0xffffffffu, best, o);
-          best = other > best ? other : best;
-        }
-        theta = best;
-      } else {  // many near-equal blocks: keep searching over all of them, a bit at a time
-        for (int bit = low - 1; bit >= 0; --bit) {
-          const long long cnd = theta | (1LL << bit);
-          double g0 = 0.0, g1 = 0.0, g2 = 0.0, g3 = 0.0;  // fixed 4-way split: same order on every run
-#pragma unroll 1
-          for (int j = 0; j < NJ; j += 4) {
-            if (__double_as_longlong(pw[(j) * 32]) >= cnd) g0 += pw[(j) * 32];
-            if (j + 1 < NJ && __double_as_longlong(pw[(j + 1) * 32]) >= cnd) g1 += pw[(j + 1) * 32];
-            if (j + 2 < NJ && __double_as_longlong(pw[(j + 2) * 32]) >= cnd) g2 += pw[(j + 2) * 32];
-            if (j + 3 < NJ && __double_as_longlong(pw[(j + 3) * 32]) >= cnd) g3 += pw[(j + 3) * 32];
-          }
-          if (warp_sum((g0 + g1) + (g2 + g3)) >= t) theta = cnd;
-        }
-      }
-      double above = 0.0;
-      int nties = 0;
-#pragma unroll 4
-      for (int j = 0; j < NJ; ++j) {
-        const long long b = __double_as_longlong(pw[(j) * 32]);
-        if (b > theta) above += pw[(j) * 32];
-        nties += (b == theta && j * 32 + lane < nb) ? 1 : 0;
-      }
-      above = warp_sum(above);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) nties += __shfl_xor_sync(0xffffffffu, nties, o);
-      const double th = __longlong_as_double(theta);
-      double c = above;
-      do {  // ties enter in ascending index order, one at a time, until the mass reaches tau
-        c += th;
-        ++m_ties;
-      } while (c < t && m_ties < nties);
-      n_ties = nties;
-    }
-
-    int tie_seen = 0;
-    // the usual case: every block equal to theta is kept (theta = 0 when all blocks are kept)
-    const bool all_ties_kept = keep_all || m_ties == n_ties;
-    emit([&](int j, bool valid) {
-      const long long b = __double_as_longlong(pw[(j) * 32]);
-      if (all_ties_kept) return valid && b >= theta;
-      const bool is_tie = valid && b == theta;
-      const unsigned tie_ballot = __ballot_sync(0xffffffffu, is_tie);
-      const int tie_rank = tie_seen + __popc(tie_ballot & lt_mask);
-      tie_seen += __popc(tie_ballot);
-      return valid && (b > theta || (is_tie && tie_rank < m_ties));
-    });
+    for (int i = lane; i < 2 * kD; i += 32) (i >= kD ? a.decide.anchor_k : a.decide.anchor_q)[(size_t)r * kD + (i & (kD - 1))] = mean[i];
   }
 }
 
@@ -549,6 +678,60 @@ cudaError_t launch_top_p(const Geom &g, const Workspace &w, const double *tau, c
   if (nj <= 16) return launch_nj<16>(g, w, tau, refresh, st, pitch, s, expect_sig);
   if (nj <= 24) return launch_nj<24>(g, w, tau, refresh, st, pitch, s, expect_sig);
   return launch_nj<32>(g, w, tau, refresh, st, pitch, s, expect_sig);
+}
+
+// One wave of CTAs (by their shared memory: five an SM at 32 blocks, two at 64, one at 128): a second wave would read every
+// head's key means once more for each eight rows, which the tiles of pooled_scores_kernel do not.
+bool rows_kernel_fits(const Geom &g) {
+  const int nj = (g.nb + 31) / 32;
+  if (nj > 4 || (g.flags & HEART_ESTIMATOR_ANTIDIAG)) return false;
+  const size_t bytes = sizeof(double) * rows_kernel_doubles(nj <= 2 ? 2 : 4, g.nb);
+  const long long per_sm = (long long)(224 * 1024 / (bytes + 8 * 1024));
+  return (long long)g.R * ((g.nb + 7) / 8) <= 148 * per_sm;
+}
+
+template <int NJ, bool DECIDE>
+static cudaError_t launch_rows(const Geom &g, const RowArgs &a, cudaStream_t s) {
+  const int smem = (int)sizeof(double) * rows_kernel_doubles(NJ, g.nb);
+  cudaError_t e = allow_shared_memory(mask_rows_kernel<NJ, DECIDE>, (int)sizeof(double) * rows_kernel_doubles(NJ, NJ * 32));
+  if (e != cudaSuccess) return e;
+  return launch_pdl(mask_rows_kernel<NJ, DECIDE>, dim3((g.nb + 7) / 8, g.R), dim3(kRowsKernelThreads), (size_t)smem, s, a);
+}
+
+static RowArgs row_args(const Geom &g, const Workspace &w, const double *tau, heart_state st) {
+  RowArgs a = {};
+  a.bmean = w.bmean;
+  a.tau = tau;
+  a.R = g.R;
+  a.nb = g.nb;
+  a.scale = g.scale;
+  a.flags = g.flags;
+  a.mask_bits = st.mask_bits;
+  a.kv_idx = st.kv_idx;
+  a.kv_cnt = st.kv_cnt;
+  a.idx_stride = g.idx_stride;
+  a.W = g.W;
+  return a;
+}
+
+cudaError_t launch_decide_and_predict(const Geom &g, const Workspace &w, const DecideArgs &decide, const double *tau, heart_state st,
+                                      cudaStream_t s, int *launches) {
+  RowArgs a = row_args(g, w, tau, st);
+  const bool gate_on = g.gate_lo > 0.0 || g.gate_hi < 1.0;
+  ++*launches;
+  if (gate_on || g.R > kStatusHeadTickets) {
+    cudaError_t e = launch_decide(g, w, decide, s);
+    if (e != cudaSuccess) return e;
+    ++*launches;
+    a.refresh = w.refresh;
+    return g.nb <= 64 ? launch_rows<2, false>(g, a, s) : launch_rows<4, false>(g, a, s);
+  }
+  a.psum = w.psum;
+  a.N = g.N;
+  a.nchunks = g.nchunks;
+  a.decide = decide;
+  a.decide.ticket = w.status + kStatusHeadTicketWord;
+  return g.nb <= 64 ? launch_rows<2, true>(g, a, s) : launch_rows<4, true>(g, a, s);
 }
 
 cudaError_t launch_predict_mask(const Geom &g, const Workspace &w, const double *tau,

@@ -105,19 +105,6 @@ __global__ void __launch_bounds__(256, 5) block_sums_kernel(const uint16_t *__re
   if (threadIdx.x < kD) psum[(((size_t)z * R + r) * gridDim.x + chunk) * kD + threadIdx.x] = total;
 }
 
-// Decision inputs of mean_drift_kernel.
-struct DecideArgs {
-  int B, H;
-  const double *delta;
-  double gate_lo, gate_hi;
-  unsigned flags;
-  double *anchor_q, *anchor_k;
-  uint8_t *has_anchor, *refresh_ws, *pre_ws;
-  double *drift_out;
-  uint8_t *refresh_out;
-  int *ticket;  // zero between launches (used only when the layer gate is on)
-};
-
 // Batch entries whose heads the layer gate takes together, and the shared memory that needs.
 __host__ __device__ inline int gate_group(int B, int H) { return max(1, min(B, 4096 / H)); }
 __host__ inline size_t gate_shared_bytes(int B, int H) { return (size_t)gate_group(B, H) * (sizeof(int) + 2 * (size_t)H); }
@@ -195,10 +182,7 @@ __global__ void __launch_bounds__(1024) mean_drift_kernel(const double *__restri
   }
   pdl_wait();  // the partial sums come from the kernel before this one
   pdl_launch_dependents();
-  double s = 0.0;
-#pragma unroll 8
-  for (int i = i0; i < i1; ++i) s += src[(size_t)i * kD];
-  sm[z][grp][d] = s;
+  sm[z][grp][d] = sum_range(src, i0, i1);
   __syncthreads();
   double m = 0.0;
   if (threadIdx.x < 2 * kD) {
@@ -272,8 +256,7 @@ cudaError_t launch_block_sums(const Geom &g, const void *Q, const void *K, const
                     w.bmean, w.psum, sig_word, sig);
 }
 
-cudaError_t launch_decide(const Geom &g, const Workspace &w, const double *delta, heart_state st,
-                          double *drift_out, uint8_t *refresh_out, cudaStream_t s, int *launches) {
+DecideArgs decide_args(const Geom &g, const Workspace &w, const double *delta, heart_state st, double *drift_out, uint8_t *refresh_out) {
   DecideArgs a;
   a.B = g.B;
   a.H = g.H;
@@ -289,7 +272,15 @@ cudaError_t launch_decide(const Geom &g, const Workspace &w, const double *delta
   a.drift_out = drift_out;
   a.refresh_out = refresh_out;
   a.ticket = w.status + kStatusTicketWord;
+  return a;
+}
+
+cudaError_t launch_decide(const Geom &g, const Workspace &w, const double *delta, heart_state st,
+                          double *drift_out, uint8_t *refresh_out, cudaStream_t s, int *launches) {
   ++*launches;
+  return launch_decide(g, w, decide_args(g, w, delta, st, drift_out, refresh_out), s);
+}
+cudaError_t launch_decide(const Geom &g, const Workspace &w, const DecideArgs &a, cudaStream_t s) {
   const bool gate_on = g.gate_lo > 0.0 || g.gate_hi < 1.0;
   return launch_pdl(mean_drift_kernel, dim3(g.R), dim3(1024), gate_on ? gate_shared_bytes(g.B, g.H) : 0, s, (const double *)w.psum, g.R, g.N,
                     g.nchunks, w.mean, a);
