@@ -38,11 +38,11 @@
 // except for the launch's last tiles (up to 1024; all of a small launch), which go longest-list-first so that the
 // launch does not end on a long tile that started late.
 //
-// Small launches (a tile per CTA at most) have an instance of their own, which plans its tile itself and, while tiles
-// are few, shares its key steps among a cluster of 2 or 4 CTAs: their O and row sums meet in shared memory, and each CTA
-// puts together its share of the rows.  2 heads x 2k, 32 tiles of up to 13 steps: 19.0 us with a plan kernel before it,
-// 17.9 without, 16.5 with two CTAs a tile, 15.5 with four (14.7 since the plan is shorter).  (Reading the parts takes 2.8 us of it, at 9 bytes a clock
-// and SM between SMs: more CTAs would not pay.)
+// Small launches (a tile per CTA at most) have an instance of their own, which plans its tile itself while Q comes in and, while
+// tiles are few, shares its key steps among a cluster of 2 or 4 CTAs: each CTA copies the others their share of the rows of its
+// part of O as soon as it has it, and puts its own share together.  2 heads x 2k, 32 tiles of up to 13 steps, from the end
+// of the kernel before: 23.0 k clocks when the CTAs read one another's parts behind a barrier, with the roles' first
+// instructions and Q fetched behind the plan, 18.9 k now; 2.3 k of them are the plan, 4 k the exchange of 48 KB each way.
 //
 // Every wait is bounded; a wait that runs out raises the CTA's abort flag and the status word, its roles
 // drain and stop.  The tile it worked on and those it had drawn already, or was dealt, stay unwritten (as does a tile that a
@@ -91,8 +91,10 @@ struct AttnShared {
   float2 l[2][128];        // row sum and its reference of the warpgroup without the last step, per tile & 1
   uint32_t tmem_base;
   int abort;
-  // small launches: the tile's plan
-  uint4 word;
+  // small launches: the parts of a tile that this CTA puts together, the tile's plan
+  uint64_t parts_full;     // the other CTAs' parts have arrived
+  alignas(16) float2 part_l[128];      // row sums and references of this CTA's part (a row sum of -1: it gave up)
+  alignas(16) float2 in_l[kMaxSplit - 1][128 / 2];  // of the rows that this CTA puts together, from the other CTAs
   uint32_t sets[2][32];
   uint32_t steps[HEART_MAX_BLOCKS];
 };
@@ -283,6 +285,61 @@ __global__ void __launch_bounds__(32 * kPlanWarps)
   if (lane == 0) tiles[n] = word;
 }
 
+// Small launches: rows [rank * rows, (rank + 1) * rows) of a shared tile from the parts of the cluster's CTAs, by the
+// softmax warps.  A function that a kernel calls twice, the first time while it waits for the kernel before it, without
+// writing (`real` false): every CTA runs this code once, and from cold instructions it took 3 us.
+struct PartAddresses {
+  uint32_t own, own_l, slot, slot2, in_l;  // in shared memory
+};
+__device__ __noinline__ void merge_parts(const PartAddresses at, int rank, int split, int valid_rows, bool real, uint16_t *out, long long sn,
+                                         float *lse) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, rows = 128 / split;
+  // a warp: four rows at a time, eight lanes each, lane q of them pieces q, q + 8, q + 16 and q + 24 of four dims
+#pragma unroll 1
+  for (int i0 = warp * 4 + (lane >> 3); i0 < (real ? rows : 32); i0 += 32) {
+    const int row = rank * rows + i0, q = lane & 7;
+    float l[kMaxSplit], m[kMaxSplit], m_all = kNoReference, l_all = 0.f;
+    uint32_t src[kMaxSplit];
+    bool gave_up = false;
+#pragma unroll
+    for (int i = 0; i < kMaxSplit; ++i) {
+      // parts are held in the order of the CTAs behind this one, its own last
+      const int place = (i - rank - 1 + split) & (split - 1);
+      const bool own = place == split - 1;
+      src[i] = own ? at.own + row * 512 : (place < 2 ? at.slot + place * (kTileBytes / 2) : at.slot2) + i0 * 512;
+      const float2 lm = lds2(own ? at.own_l + row * 8 : at.in_l + place * (128 / 2 * 8) + i0 * 8);
+      l[i] = i < split ? lm.x : 0.f;
+      m[i] = l[i] != 0.f ? lm.y : kNoReference;  // (a part without keys)
+      gave_up |= l[i] == -1.f;
+      m_all = fmaxf(m_all, m[i]);
+    }
+    float4 o[4] = {};
+#pragma unroll
+    for (int i = 0; i < kMaxSplit; ++i) {
+      if (i >= split) break;
+      if (l[i] != 0.f) {  // (a part without keys has zeros; a sum that is not a number goes into the row's result)
+        const float f = ex2(m[i] - m_all);
+        l_all = fmaf(l[i], f, l_all);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const float4 x = lds4(src[i] + (((q + 8 * k) ^ (row & 7)) << 4));
+          o[k].x = fmaf(x.x, f, o[k].x);
+          o[k].y = fmaf(x.y, f, o[k].y);
+          o[k].z = fmaf(x.z, f, o[k].z);
+          o[k].w = fmaf(x.w, f, o[k].w);
+        }
+      }
+    }
+    const float inv = l_all > 0.f ? 1.f / l_all : 0.f;
+    if (real && row < valid_rows && !gave_up) {  // (a tile of which a part gave up is not written)
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        *reinterpret_cast<uint2 *>(out + row * sn + (q + 8 * k) * 4) = make_uint2(pack_bf16x2(o[k].x * inv, o[k].y * inv), pack_bf16x2(o[k].z * inv, o[k].w * inv));
+      if (q == 0 && lse != nullptr) lse[row] = l_all > 0.f ? (m_all + log2f(l_all)) * 0.6931471805599453f : -INFINITY;
+    }
+  }
+}
+
 template <int B, bool Small>
 __global__ void __launch_bounds__(kAttnThreads, 1)
     attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
@@ -311,6 +368,11 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     mbar_init(&sh.o_free, 4);
     mbar_init(&sh.drain[0], 1);
     mbar_init(&sh.drain[1], 1);
+    mbar_init(&sh.parts_full, 1);
+    if (Small) {  // this CTA's only tile, but for the number of its key blocks
+      const int n = blockIdx.x / p.split, hr = n / p.n_tiles_per_head, b = hr / p.hcount;
+      sh.tile[0] = make_int4(n - hr * p.n_tiles_per_head, p.nb, p.h0 + hr - b * p.hcount, b);
+    }
     sh.abort = 0;
     mbar_fence_init();
   }
@@ -323,15 +385,23 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     tma_prefetch_desc(&map_k);
     tma_prefetch_desc(&map_v);
   }
+  const int rank = Small ? (int)cluster_ctarank() : 0;
+  const PartAddresses parts = {smem_u32(smem + kOffK), smem_u32(sh.part_l), smem_u32(smem + kOffQ + kTileBytes), smem_u32(smem + kOffOut),
+                               smem_u32(sh.in_l)};
+  if (Small) {  // the barriers are initialised: for the Q copy below, and for the other CTAs' parts
+    if (p.split > 1) {
+      if (warp < 8) merge_parts(parts, rank, p.split, 0, false, nullptr, 0, nullptr);
+      cluster_sync();
+    } else {
+      __syncthreads();
+    }
+  }
   // Launched with programmatic stream serialisation: everything above overlaps the end of the kernels
   // before it.  A kernel that follows (the next layer-step's block-sum pass) may be scheduled once every
   // CTA of this launch has started: its CTAs then fill the SMs that finish first.
-  pdl_wait();
+  // (In a small launch the roles wait where their code is: fetched only behind the plan, its first lines took 1 us.)
+  if (!Small) pdl_wait();
   pdl_launch_dependents();
-  if (Small && !p.dense && warp == 0) {
-    const uint4 word = plan_tile<B>(plan, blockIdx.x / p.split, lane, sh.sets, [&](int) { return sh.steps; });
-    if (lane == 0) sh.word = word;
-  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -340,11 +410,9 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
   // Key steps of a tile with U listed key blocks that this CTA takes, and the first one of them.  (A tile of one step is not
   // shared: its cluster's first CTA takes it and the others leave.  2 x 2048 tokens: 8.6 us against 12.4 with one key block
   // listed, 5.9 against 9.5 with none.)
-  const int rank = Small ? (int)cluster_ctarank() : 0;
-  const int tile_blocks = !Small ? 0 : p.dense ? p.nb : (int)(sh.word.x >> 16);
-  const bool shared_tile = Small && p.split > 1 && tile_blocks > (B == 128 ? 1 : 2);
-  const int parts = shared_tile ? p.split : 1;
-  auto first_step = [&](int U, int part) -> int { return Small ? (B == 128 ? U : (U + 1) / 2) * part / parts : 0; };
+  bool shared_tile = false, at_barrier = false;
+  int parts_of_tile = 1;
+  auto first_step = [&](int U, int part) -> int { return Small ? (B == 128 ? U : (U + 1) / 2) * part / parts_of_tile : 0; };
   auto n_steps_of = [&](int U) -> int { return Small ? first_step(U, rank + 1) - first_step(U, rank) : B == 128 ? U : (U + 1) / 2; };
   auto steps_of = [&](const int4 &ti) -> const uint32_t * {
     if (Small) return sh.steps + first_step(ti.y, rank);
@@ -365,8 +433,18 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     if (__builtin_expect(!complete(bar, parity), 0)) ok = __all_sync(0xffffffffu, mbar_wait(bar, parity, abort)) && ok;
     return ok;
   };
+  auto small_tile = [&](int U) {
+    shared_tile = p.split > 1 && U > (B == 128 ? 1 : 2);
+    parts_of_tile = shared_tile ? p.split : 1;
+  };
   // The announced tile t; false: none left (or abort).  Every lane of the warp gets the same answer.
   auto next_tile = [&](int t, int4 &ti) -> bool {
+    if (Small) {
+      if (t > 0 || !wait(&sh.tile_full[0], 0)) return false;
+      ti = sh.tile[0];
+      small_tile(ti.y);
+      return rank < parts_of_tile;
+    }
     const int i = t % kTileRing;
     if (!wait(&sh.tile_full[i], (t / kTileRing) & 1)) return false;
     ti = sh.tile[i];
@@ -413,35 +491,54 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
   // ------------------------------------------------------------------ roles
   if (warp >= kWarpQK) setmaxnreg_dec<kRegsHelper>();
   if (warp == kWarpK) {
+    if (Small) pdl_wait();
     if (lane == 0) {  // ===== K and Q producer
       int g = 0, nq = 0;     // key steps loaded, tiles with key steps
+      if (Small) {
+        // the launch's only tile of this CTA is known before its plan is: its Q comes in meanwhile
+        int4 ti = sh.tile[0];
+        mbar_expect_tx(&sh.q_full[0], kTileBytes);
+        tma_load_5d(smem + kOffQ, &map_q, &sh.q_full[0], 0, ti.x * 128, 0, ti.z, ti.w);
+        ok = mbar_wait(&sh.tile_full[0], 0, abort);
+        ti = sh.tile[0];
+        small_tile(ti.y);
+        const int n_steps = ok && rank < parts_of_tile ? n_steps_of(ti.y) : 0;
+        const uint32_t *steps = steps_of(ti);
+#pragma unroll 1
+        for (; g < n_steps; ++g) {
+          if (g >= 2) ok = mbar_wait(&sh.s_full[g & 1], ((g - 2) >> 1) & 1, abort);
+          if (!ok) break;
+          const uint32_t e = step_entry(steps, g);
+          sh.entry[g & 3] = e;
+          load_step(smem + kOffK + (g & 1) * kTileBytes, &map_k, &sh.k_full[g & 1], e, ti.z, ti.w);
+        }
+      }
       int4 nx;               // the tile that is announced next and its first key step, fetched ahead of time
       uint32_t e = 0;
       auto fetch = [&](int n) {
         nx.w = -1;
-        if (n >= p.n_tiles || rank >= parts) return;
+        if (n >= p.n_tiles) return;
         uint4 t;
         if (p.dense) {
           t.y = n / p.n_tiles_per_head;
           t.x = (n - t.y * p.n_tiles_per_head) | (uint32_t)p.nb << 16;
           t.z = step_entry(nullptr, 0);
         } else {
-          t = Small ? sh.word : __ldcg(&p.tiles[n]);
+          t = __ldcg(&p.tiles[n]);
         }
         e = t.z;
         nx.x = t.x & 0xffff;
         nx.y = t.x >> 16;
         nx.w = (int)t.y / p.hcount;
         nx.z = p.h0 + (int)t.y - nx.w * p.hcount;
-        if (Small && n_steps_of(nx.y) > 0) e = step_entry(steps_of(nx), 0);
       };
-      // The first tile of every CTA is fixed, the others are drawn (a small launch has no others).  Dense tiles are all
+      // The first tile of every CTA is fixed, the others are drawn.  Dense tiles are all
       // of one length: dealt in turn, so that dense calls share nothing and may overlap on one workspace.  (Drawn, the faster
       // SMs take the odd tiles: 12 x 33k 5604 us, dealt 5721.)
-      int mine = Small ? blockIdx.x / p.split : blockIdx.x;
-      fetch(mine);
-      auto draw = [&]() { fetch(Small ? p.n_tiles : p.dense ? mine += gridDim.x : gridDim.x + atomicAdd(p.counter, 1)); };
-      for (int t = 0;; ++t) {
+      int mine = blockIdx.x;
+      if (!Small) fetch(mine);
+      auto draw = [&]() { fetch(p.dense ? mine += gridDim.x : gridDim.x + atomicAdd(p.counter, 1)); };
+      for (int t = 0; !Small; ++t) {
         const int i = t % kTileRing;
         if (t >= kTileRing) ok = mbar_wait(&sh.tile_empty[i], (t / kTileRing - 1) & 1, abort);
         if (!ok) break;
@@ -472,13 +569,15 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
         if (!ok) break;
         if (n_steps == 0) draw();
       }
+      if (Small) settle(&sh.q_full[0], 0);  // (a CTA without a step has not waited for it)
       if (*abort) {
-        settle_pair(sh.q_full, nq);
+        if (!Small) settle_pair(sh.q_full, nq);
         settle_pair(sh.k_full, g);
       }
     }
   } else if (warp == kWarpV) {
     // ===== V producer
+    if (Small) pdl_wait();
     int g = 0;
     int4 ti;
     for (int t = 0; ok && next_tile(t, ti); ++t) {
@@ -507,6 +606,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     const uint64_t q_desc = smem_desc_sw128(smem_u32(smem + kOffQ), 16, 1024);
     const uint64_t k_desc = smem_desc_sw128(smem_u32(smem + kOffK), 16, 1024);
     const bool leader = elect_one();  // the same lane every time: commits track its MMAs
+    if (Small) pdl_wait();
     uint32_t g = 0, nq = 0;           // key steps and tiles with key steps so far
     int4 ti;
     for (int t = 0; ok && next_tile(t, ti); ++t) {
@@ -538,6 +638,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     // 2048 B per k-step.
     const uint64_t v_desc = smem_desc_sw128(smem_u32(smem + kOffV), kTileBytes / 2, 1024);
     const bool leader = elect_one();
+    if (Small) pdl_wait();
     uint32_t g = 0, nt = 0;  // key steps and tiles with key steps so far
     int4 ti;
     for (int t = 0; ok && next_tile(t, ti); ++t) {
@@ -574,6 +675,22 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
       __syncwarp();
       if (lane == 0) mbar_arrive(bar);
     };
+    if (Small) {
+      pdl_wait();
+      if (warp == 0) {
+        uint32_t U = p.nb;
+        if (!p.dense) {
+          const uint4 word = plan_tile<B>(plan, blockIdx.x / p.split, lane, sh.sets, [&](int) { return sh.steps; });
+          U = word.x >> 16;
+        }
+        __syncwarp();
+        if (lane == 0) {
+          sh.tile[0].y = U;
+          mbar_arrive(&sh.tile_full[0]);
+        }
+      }
+      named_barrier_sync(2, 256);
+    }
     uint32_t g0 = 0, nt = 0;  // key steps before the present tile, tiles with key steps before it
     int4 ti;
     for (int t = 0; ok && next_tile(t, ti); ++t) {
@@ -754,7 +871,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
 #pragma unroll
           for (int i = 0; i < 32; ++i)
             part[i ^ (row & 7)] = make_float4(__uint_as_float(v[4 * i]), __uint_as_float(v[4 * i + 1]), __uint_as_float(v[4 * i + 2]), __uint_as_float(v[4 * i + 3]));
-          sh.l[0][row] = make_float2(l_run, m_ref);
+          sh.part_l[row] = make_float2(l_run, m_ref);
           break;
         }
         const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
@@ -794,64 +911,41 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
       nt += n_steps > 0 ? 1 : 0;
     }
     if (shared_tile) {
-      // ===== the parts of a tile, one in every CTA of the cluster: each CTA puts together 128 / split rows
-      const int n = blockIdx.x / p.split, rows = 128 / p.split;
-      uint4 word;
-      if (p.dense) {
-        word.y = n / p.n_tiles_per_head;
-        word.x = n - word.y * p.n_tiles_per_head;
-      } else {
-        word = sh.word;
-      }
-      const int b = (int)word.y / p.hcount, hd = p.h0 + (int)word.y - b * p.hcount, tok0 = (word.x & 0xffff) * 128;
-      const uint32_t off_l = smem_u32(&sh.l[0][0]) - smem_u32(smem), off_abort = smem_u32(const_cast<int *>(&sh.abort)) - smem_u32(smem);
-      uint32_t base[kMaxSplit], gave_up = 0u;
-      cluster_sync();
-#pragma unroll
-      for (int i = 0; i < kMaxSplit; ++i) {
-        base[i] = cluster_address(smem_u32(smem), i < p.split ? i : 0);
-        gave_up |= cluster_ld1(base[i] + off_abort);
-      }
-#pragma unroll 2
-      for (int row = rank * rows + warp; row < (rank + 1) * rows; row += 8) {
-        float l[kMaxSplit], m[kMaxSplit], m_all = kNoReference, l_all = 0.f;
-        float4 x[kMaxSplit], o = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-        for (int i = 0; i < kMaxSplit; ++i) {
-          if (i >= p.split) break;
-          const float2 lm = cluster_ld2(base[i] + off_l + row * 8);
-          x[i] = cluster_ld4(base[i] + kOffK + row * 512 + ((lane ^ (row & 7)) << 4));
-          l[i] = lm.x;
-          m[i] = lm.x != 0.f ? lm.y : kNoReference;
-          m_all = fmaxf(m_all, m[i]);
+      // ===== the parts of a tile: each CTA puts together 128 / split rows, its own part of them with those that the other
+      // CTAs copy here: a bulk copy each as soon as a CTA has its part, into Q's second buffer and the output's place, which a
+      // launch of one tile per CTA does not use.
+      const int rows = 128 / p.split;
+      async_proxy_fence();
+      named_barrier_sync(1, 256);
+      const bool aborted = *abort != 0;
+      if (tid == 0) mbar_expect_tx(&sh.parts_full, (p.split - 1) * rows * (512 + (int)sizeof(float2)));
+      if (lane == 0 && warp < p.split - 1) {
+        // to CTA `to`, which holds the parts of the CTAs behind it in order
+        const int at = p.split - 2 - warp, to = (rank + 1 + warp) & (p.split - 1);
+        if (aborted) {
+          for (int i = 0; i < rows; ++i) sh.part_l[to * rows + i] = make_float2(-1.f, 0.f);
+          async_proxy_fence();
         }
-#pragma unroll
-        for (int i = 0; i < kMaxSplit; ++i) {
-          if (i >= p.split) break;
-          if (l[i] != 0.f) {  // (a part without keys has zeros; a sum that is not a number goes into the row's result)
-            const float f = ex2(m[i] - m_all);
-            l_all = fmaf(l[i], f, l_all);
-            o.x = fmaf(x[i].x, f, o.x);
-            o.y = fmaf(x[i].y, f, o.y);
-            o.z = fmaf(x[i].z, f, o.z);
-            o.w = fmaf(x[i].w, f, o.w);
-          }
-        }
-        const float inv = l_all > 0.f ? 1.f / l_all : 0.f;
-        const int tok = tok0 + row;
-        if (tok < p.N && gave_up == 0u) {  // (a tile of which a part gave up is not written)
-          const uint2 y = make_uint2(pack_bf16x2(o.x * inv, o.y * inv), pack_bf16x2(o.z * inv, o.w * inv));
-          *reinterpret_cast<uint2 *>(p.O + (long long)b * p.sb + (long long)hd * p.sh + (long long)tok * p.sn + lane * 4) = y;
-          if (lane == 0 && p.lse != nullptr)
-            p.lse[(size_t)(b * p.H + hd) * p.N + tok] = l_all > 0.f ? (m_all + log2f(l_all)) * 0.6931471805599453f : -INFINITY;
+        const uint32_t bar = cluster_address(smem_u32(&sh.parts_full), to);
+        bulk_copy_to_cluster(cluster_address(at < 2 ? parts.slot + at * (kTileBytes / 2) : parts.slot2, to), smem + kOffK + to * rows * 512, rows * 512, bar);
+        bulk_copy_to_cluster(cluster_address(smem_u32(&sh.in_l[at][0]), to), &sh.part_l[to * rows], rows * (int)sizeof(float2), bar);
+      }
+      {  // (not cut short by an abort: nobody leaves with copies on their way)
+        const long long t0 = clock64();
+        while (!mbar_try_wait(&sh.parts_full, 0) && clock64() - t0 < 2 * kWaitLimitCycles) {
         }
       }
-      cluster_sync();  // shared memory stays until everyone has read it
+      cluster_arrive();
+      at_barrier = true;
+      const int4 ti = sh.tile[0];
+      merge_parts(parts, rank, p.split, p.N - ti.x * 128, mbar_test_wait(&sh.parts_full, 0) && !aborted,
+                  p.O + (long long)ti.w * p.sb + (long long)ti.z * p.sh + (long long)ti.x * 128 * p.sn, p.sn,
+                  p.lse != nullptr ? p.lse + (size_t)(ti.w * p.H + ti.z) * p.N + ti.x * 128 : nullptr);
     }
   }
-  if (shared_tile && warp >= kWarpQK) {
-    cluster_sync();
-    cluster_sync();
+  if (Small && p.split > 1) {  // the copies from this CTA's memory are complete: their receivers have them
+    if (!at_barrier) cluster_arrive();
+    cluster_wait();
   }
 
   // ------------------------------------------------------------------ tear-down
