@@ -10,7 +10,7 @@
 //
 // Each axis is a contraction with the fp64 matrix instruction.  Folding x_j +- x_{n-j} halves it: cosines see the
 // even part, sines the odd one.  For 16 x 21 x 60 x 104 that is 1.9e8 fma (10 us at 18.5 T fma/s).  Two ways through it:
-// planes that a CTA holds are transformed along y and x in one kernel, another goes over t (40 us); any other shape goes
+// planes that a CTA holds are transformed along y and x in one kernel, another goes over t (39 us); any other shape goes
 // axis by axis through the workspace, in five launches (55 us for that one).
 #include <math.h>
 
@@ -276,9 +276,10 @@ __global__ void __launch_bounds__(1024) band_final_kernel(const double *__restri
 // The usual latent: a [y, x] plane of one channel and time is transformed along both of its axes by two CTAs, one for
 // the part that is even along y and one for the odd one, without a trip to the workspace in between; a second kernel
 // goes over t, and its last CTA puts the result together.  Two launches instead of five, 34 MB of traffic in the L2 less:
-// 16 x 21 x 60 x 104 takes 40.5 us instead of 55.3.  Neither kernel is near a rate (fp64 matrix pipe 33 and 13 % busy,
-// issue slots 44 and 47 %): 672 CTAs, three an SM, fold, wait and multiply in turn.  (With 64-bit remainders and the
-// cosine and sine of an entry side by side, so that a warp's entries collide in twice as many banks: 50.2 us.)
+// 16 x 21 x 60 x 104 takes 39.1 us instead of 55.3.  The products run at the rate of the fp64 matrix pipe, but the 672 CTAs,
+// three an SM, fold and multiply at about the same time; a third of the first kernel is the fold.  (Each CTA of a pair folding
+// the whole plane for its own half: 40.6 us.  64-bit remainders and the cosine and sine of an entry side by side, so that
+// a warp's entries collide in twice as many banks: 50.2.)
 
 constexpr int kPlaneThreads = 256, kPlaneWarps = kPlaneThreads / 32;
 constexpr int kPlaneMaxShared = 200 * 1024;  // of a CTA, in bytes
@@ -345,6 +346,10 @@ __device__ __forceinline__ void contract(double (&acc)[TILES][2], const double *
   }
 }
 
+__device__ __forceinline__ void cluster_store(uint32_t addr, double v) {
+  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(addr), "d"(v) : "memory");
+}
+
 // CTA 2 * plane + parity along y.
 __global__ void __launch_bounds__(kPlaneThreads, 3) plane_kernel(const float *__restrict__ ys, const float *__restrict__ yd, int ny, int nx,
                                                                  double *__restrict__ dst, double *__restrict__ dense_out,
@@ -361,26 +366,28 @@ __global__ void __launch_bounds__(kPlaneThreads, 3) plane_kernel(const float *__
   const int rows = odd ? my : hy + 1;  // samples along y of this parity: odd ones start at 1
   fill_trig_table(tab_x, nx);
   fill_trig_table(tab_y, ny, nx < kPlaneThreads ? nx : 0);  // (by the threads that have no entry of x)
+  tc::cluster_sync();  // (the other CTA has started: its memory is there)
   pdl_wait();
   pdl_launch_dependents();
   if (blockIdx.x == 0 && threadIdx.x == 0) *ticket = 0;
 
-  // folded along both axes, a warp per row; the loads of four rows at a time
+  // Folded along both axes, a warp per row.  The pair of CTAs shares the rows: a CTA takes every other row, with its mirror,
+  // and puts the even sums into the even CTA's memory and the odd ones into the other's.
   double dense = 0.0;
   const int row_tiles = (rows + 7) / 8, odd_cols = round_up(mx, 4);
   const float *s0 = ys + plane, *d0 = yd + plane;
+  const uint32_t even_a = tc::cluster_address(tc::smem_u32(A), 0), odd_a = tc::cluster_address(tc::smem_u32(A), 1);
   for (int j = lane; j < f.even_cols; j += 32) {
     const bool in = j <= hx, xpair = j >= 1 && j <= mx;
 #pragma unroll 2
-    for (int i = warp; i < row_tiles * 8; i += kPlaneWarps) {
-      const int jy = i + odd;
-      const bool real = in && i < rows, pair = real && jy >= 1 && jy <= my;
+    for (int jy = 2 * warp + odd; jy <= hy; jy += 2 * kPlaneWarps) {
+      const bool pair = jy >= 1 && jy <= my;
       const int at = jy * nx, mirror = (ny - jy) * nx;
       float s1[4], d1[4];
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const int off = (q < 2 ? at : mirror) + ((q & 1) ? nx - j : j);
-        const bool load = (q < 2 ? real : pair) && ((q & 1) == 0 || xpair);
+        const bool load = in && (q < 2 || pair) && ((q & 1) == 0 || xpair);
         s1[q] = load ? __ldg(&s0[off]) : 0.f;
         d1[q] = load ? __ldg(&d0[off]) : 0.f;
       }
@@ -391,25 +398,33 @@ __global__ void __launch_bounds__(kPlaneThreads, 3) plane_kernel(const float *__
         e[q] = (double)s1[q] - d;
         dense = fma(d, d, dense);
       }
-      const double u = odd ? e[0] - e[2] : e[0] + e[2], v = odd ? e[1] - e[3] : e[1] + e[3];
-      double *row = A + i * f.pitch_a;
-      row[j] = u + v;
-      if (xpair) row[f.even_cols + j - 1] = u - v;  // (zeros in the rows that fill the last tile)
+      const double u = e[0] + e[2], v = e[1] + e[3];
+      const uint32_t to_even = even_a + (jy * f.pitch_a + j) * 8;
+      cluster_store(to_even, u + v);
+      if (xpair) cluster_store(to_even + (f.even_cols - 1) * 8, u - v);
+      if (pair) {
+        const double x = e[0] - e[2], y = e[1] - e[3];
+        const uint32_t to_odd = odd_a + ((jy - 1) * f.pitch_a + j) * 8;
+        cluster_store(to_odd, x + y);
+        if (xpair) cluster_store(to_odd + (f.even_cols - 1) * 8, x - y);
+      }
     }
   }
-  for (int i = warp; i < row_tiles * 8; i += kPlaneWarps)
+  // zeros: the columns that fill the last step of four, the rows that fill the last tile
+  for (int i = warp; i < row_tiles * 8; i += kPlaneWarps) {
     for (int j = mx + lane; j < odd_cols; j += 32) A[i * f.pitch_a + f.even_cols + j] = 0.0;
-  if (!odd) {  // |y_dense|^2 of the plane
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) dense += __shfl_xor_sync(0xffffffffu, dense, o);
-    if (lane == 0) red[warp] = dense;
+    if (i >= rows)
+      for (int j = lane; j < f.even_cols + odd_cols; j += 32) A[i * f.pitch_a + j] = 0.0;
   }
-  __syncthreads();
-  if (!odd && threadIdx.x == 0) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) dense += __shfl_xor_sync(0xffffffffu, dense, o);
+  if (lane == 0) red[warp] = dense;
+  tc::cluster_sync();
+  if (threadIdx.x == 0) {  // |y_dense|^2 of the rows that this CTA read
     double sum = 0.0;
 #pragma unroll
     for (int i = 0; i < kPlaneWarps; ++i) sum += red[i];
-    dense_out[blockIdx.x >> 1] = sum;
+    dense_out[blockIdx.x] = sum;
   }
 
   // along x: lines are the rows; cosines of the even part, then sines of the odd one
@@ -457,7 +472,7 @@ __global__ void __launch_bounds__(kPlaneThreads, 3) plane_kernel(const float *__
 struct TimeArgs {
   const double *src;    // [C][n][inner]
   double *energies;     // [gridDim.x][4]
-  const double *dense;  // [planes]
+  const double *dense;  // [planes], two a plane
   int *ticket;
   double *out;
   int n, ny, nx, units_per_c, units, planes;
@@ -617,10 +632,10 @@ cudaError_t launch_planes(const float *ys, const float *yd, int C, int T, int H,
   p += align256(sizeof(double) * (size_t)C * T * H * W);
   a.energies = reinterpret_cast<double *>(p);
   p += align256(sizeof(double) * 4 * time_ctas(C, H, W));
-  double *dense = reinterpret_cast<double *>(p);
+  double *dense = reinterpret_cast<double *>(p);  // of the CTAs of the first kernel
   cudaError_t e = allow_shared_memory(plane_kernel, kPlaneMaxShared);
   if (e != cudaSuccess) return e;
-  e = launch_pdl(plane_kernel, dim3(2u * C * T), dim3(kPlaneThreads), plane_shared_bytes(H, W), s, ys, yd, H, W, coef, dense, a.ticket);
+  e = launch_pdl(plane_kernel, dim3(2u * C * T), dim3(kPlaneThreads), plane_shared_bytes(H, W), s, Cluster{2}, ys, yd, H, W, coef, dense, a.ticket);
   if (e != cudaSuccess) return e;
   ++*launches;
   a.src = coef;
@@ -631,7 +646,7 @@ cudaError_t launch_planes(const float *ys, const float *yd, int C, int T, int H,
   a.nx = W;
   a.units_per_c = time_units(1, H, W);
   a.units = time_units(C, H, W);
-  a.planes = C * T;
+  a.planes = 2 * C * T;
   a.n_freq = (double)T * H * W;
   a.w0 = weights[0];
   a.w1 = weights[1];
@@ -671,7 +686,7 @@ cudaError_t launch_axis(const AxisArgs &a, cudaStream_t s) {
 size_t band_error_workspace_bytes(int C, int T, int H, int W) {
   const size_t n = (size_t)C * T * H * W;
   if (planes_fit(T, H, W))
-    return 256 + align256(sizeof(double) * n) + align256(sizeof(double) * 4 * time_ctas(C, H, W)) + align256(sizeof(double) * (size_t)C * T);
+    return 256 + align256(sizeof(double) * n) + align256(sizeof(double) * 4 * time_ctas(C, H, W)) + align256(sizeof(double) * 2 * (size_t)C * T);
   return align256(sizeof(double2) * ((size_t)T + H + W)) + 2 * align256(sizeof(double) * n) +
          align256(sizeof(double) * 4 * n_energies(C, T, H, W)) + align256(sizeof(double) * n_ctas((long long)C * T * H, W));
 }
