@@ -2,9 +2,9 @@
 // importance, retain until the accumulated importance reaches the head's threshold; the minimal
 // cumulative-mass set of Observation I).  Importance = row softmax of the block-pooled Q.K^T scores.
 //
-// Two kernels.  pooled_scores_kernel contracts the pooled means with the fp64 matrix instruction
-// (mma.m8n8k4.f64), the 128 dims in ascending order for every score; the means arrive by cp.async in
-// shared-memory tiles.  The scores go to the workspace (they stay in L2).
+// Two kernels, or one for the rows of a small layer-step (mask_rows_kernel, below).  pooled_scores_kernel contracts the
+// pooled means with the fp64 matrix instruction (mma.m8n8k4.f64), the 128 dims in ascending order for every score; the
+// means arrive by cp.async in shared-memory tiles.  The scores go to the workspace (they stay in L2).
 // top_p_kernel gives each warp one row and finds the kept set WITHOUT a sort and without dividing by the
 // row sum z: the blocks above a threshold plus the lowest-index ties at it, where the threshold is the
 // largest element whose ">=" mass still reaches tau * z.  It decides in fp32 first: weights
