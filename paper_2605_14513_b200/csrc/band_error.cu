@@ -683,10 +683,10 @@ cudaError_t launch_axis(const AxisArgs &a, cudaStream_t s) {
 
 }  // namespace
 
+// What the way axis by axis takes, also where the other one does with half of it: a buffer made for some tensor goes on
+// serving every smaller one, whichever way that takes.
 size_t band_error_workspace_bytes(int C, int T, int H, int W) {
   const size_t n = (size_t)C * T * H * W;
-  if (planes_fit(T, H, W))
-    return 256 + align256(sizeof(double) * n) + align256(sizeof(double) * 4 * time_ctas(C, H, W)) + align256(sizeof(double) * 2 * (size_t)C * T);
   return align256(sizeof(double2) * ((size_t)T + H + W)) + 2 * align256(sizeof(double) * n) +
          align256(sizeof(double) * 4 * n_energies(C, T, H, W)) + align256(sizeof(double) * n_ctas((long long)C * T * H, W));
 }

@@ -74,3 +74,14 @@ def test_bad_arguments_are_rejected_on_the_host(heart):
     assert lib.heart_predict_mask(C.byref(bad), fake, fake, fake, null, C.byref(st2), fake, null) == heart.ERR_INVALID
     assert b"invalid" in lib.heart_strerror(heart.ERR_INVALID)
     assert b"unsupported" in lib.heart_strerror(heart.ERR_UNSUPPORTED)
+
+
+def test_band_error_workspace_serves_smaller_tensors(heart):
+    """Two fp64 copies of the tensor and a little more for every shape, whichever kernels it takes, so that a buffer made
+    for one tensor holds what any smaller one needs."""
+    size = heart.lib().heart_band_error_workspace_bytes
+    for shape in [(16, 21, 60, 104), (16, 21, 16, 32), (1, 96, 23, 23), (16, 33, 90, 160), (1, 1, 2, 3), (4, 97, 60, 104)]:
+        n = 16 * shape[0] * shape[1] * shape[2] * shape[3]
+        assert n <= size(*shape) <= 1.6 * n + 4096, shape
+    # 4 x 96 x 23 x 23 and the next smaller plane, which goes axis by axis
+    assert size(4, 96, 23, 23) >= size(4, 96, 22, 23) >= size(4, 96, 22, 22)
