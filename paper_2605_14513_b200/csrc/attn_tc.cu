@@ -116,7 +116,8 @@ struct AttnParams {
   int h0, hcount;  // this launch covers heads [h0, h0 + hcount) of every batch entry
   float scale_log2;
   int split;        // small launches: CTAs (one cluster) that share the key steps of a tile
-  int test_skip_v;  // test-hook builds only: CTA 0 leaves out the V copy of its second key step
+  int test_skip_v;      // test-hook builds only: CTA 0 leaves out the V copy of its second key step,
+  int test_skip_parts;  // CTA 1 does not send its part of a shared tile
 };
 
 __device__ __forceinline__ float fmax3(float a, float b, float c) {
@@ -924,14 +925,19 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     }
     if (shared_tile) {
       // ===== the parts of a tile: each CTA puts together 128 / split rows, its own part of them with those that the other
-      // CTAs copy here: a bulk copy each as soon as a CTA has its part, into Q's second buffer and the output's place, which a
-      // launch of one tile per CTA does not use.
+      // CTAs copy here: a bulk copy each as soon as a CTA has its part, into Q's second buffer, which a launch of one tile per CTA
+      // does not use, and the output's place, which a shared tile does not.
       const int rows = 128 / p.split;
       async_proxy_fence();
       named_barrier_sync(1, 256);
       const bool aborted = *abort != 0;
       if (tid == 0) mbar_expect_tx(&sh.parts_full, (p.split - 1) * rows * (512 + (int)sizeof(float2)));
-      if (lane == 0 && warp < p.split - 1) {
+#ifdef HEART_TEST_HOOKS
+      const bool send = !(p.test_skip_parts && blockIdx.x == 1);  // test-only library: one CTA's part never leaves
+#else
+      constexpr bool send = true;
+#endif
+      if (send && lane == 0 && warp < p.split - 1) {
         // to CTA `to`, which holds the parts of the CTAs behind it in order
         const int at = p.split - 2 - warp, to = (rank + 1 + warp) & (p.split - 1);
         if (aborted) {
@@ -942,15 +948,18 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
         bulk_copy_to_cluster(cluster_address(at < 2 ? parts.slot + at * (kTileBytes / 2) : parts.slot2, to), smem + kOffK + to * rows * 512, rows * 512, bar);
         bulk_copy_to_cluster(cluster_address(smem_u32(&sh.in_l[at][0]), to), &sh.part_l[to * rows], rows * (int)sizeof(float2), bar);
       }
-      {  // (not cut short by an abort: nobody leaves with copies on their way)
+      {  // (not cut short by an abort: nobody leaves with copies on their way.  A CTA that gives up sends its part all the
+         // same, within the limit of one wait: only one that is later still makes this wait run out)
         const long long t0 = clock64();
-        while (!mbar_try_wait(&sh.parts_full, 0) && clock64() - t0 < 2 * kWaitLimitCycles) {
-        }
+        bool there = mbar_try_wait(&sh.parts_full, 0);
+        while (!there && clock64() - t0 < 2 * kWaitLimitCycles) there = mbar_try_wait(&sh.parts_full, 0);
+        if (!there) *abort = 1;
       }
       cluster_arrive();
       at_barrier = true;
+      named_barrier_sync(1, 256);  // one answer for all warps
       const int4 ti = sh.tile[0];
-      merge_parts(parts, rank, p.split, p.N - ti.x * 128, mbar_test_wait(&sh.parts_full, 0) && !aborted,
+      merge_parts(parts, rank, p.split, p.N - ti.x * 128, *abort == 0,
                   p.O + (long long)ti.w * p.sb + (long long)ti.z * p.sh + (long long)ti.x * 128 * p.sn, p.sn,
                   p.lse != nullptr ? p.lse + (size_t)(ti.w * p.H + ti.z) * p.N + ti.x * 128 : nullptr);
     }
@@ -1143,6 +1152,7 @@ cudaError_t launch_attention(const Geom &g, const Workspace &w, const void *Q, c
   prm.scale_log2 = (float)(g.scale * 1.4426950408889634);
 #ifdef HEART_TEST_HOOKS
   prm.test_skip_v = (g.flags & 0x80000000u) ? 1 : 0;
+  prm.test_skip_parts = (g.flags & 0x40000000u) ? 1 : 0;
 #endif
   return g.block == 64 ? launch_bk<64>(g, w, mq, mk, mv, prm, kv_idx, kv_cnt, s, launches)
                        : launch_bk<128>(g, w, mq, mk, mv, prm, kv_idx, kv_cnt, s, launches);

@@ -6,7 +6,7 @@ released, the CTA exits and the workspace's status word reports HEART_ERR_DEVICE
 test-hook build of the library (same sources, HEART_TEST_HOOKS, a wait limit of 2e6 clocks) has one
 reserved flag bit that makes the V producer of CTA 0 leave out one copy -- neither the byte count is
 announced nor the copy issued -- so the waits that depend on that tile run out after about a
-millisecond.  Nothing traps and nothing waits without a bound.
+millisecond; another bit keeps a CTA's part of a shared tile from the other CTAs of its cluster.  Nothing traps and nothing waits without a bound.
 """
 import time
 
@@ -20,6 +20,7 @@ from paper_2605_14513_b200 import inputs
 pytestmark = pytest.mark.gpu
 
 TEST_SKIP_V = 0x80000000
+TEST_SKIP_PARTS = 0x40000000
 
 
 def dense_attention(h, flags, Q, K, V, wl):
@@ -78,7 +79,7 @@ def hooks():
 
 
 @pytest.mark.parametrize("block", [64, 128])
-@pytest.mark.parametrize("H,N", [(2, 420), (80, 257)])  # tiles shared by a cluster; 240 tiles of 2 or 3 steps for 148 CTAs
+@pytest.mark.parametrize("H,N", [(2, 420), (2, 2045), (80, 257)])  # tiles shared by two CTAs and by four; 240 tiles of 2 or 3 steps for 148 CTAs
 def test_other_tiles_are_complete_after_an_abort(hooks, block, H, N):
     h = hooks
     g = torch.Generator("cuda").manual_seed(N)
@@ -111,6 +112,37 @@ def test_other_tiles_are_complete_after_an_abort(hooks, block, H, N):
         h.heart_block_sparse_attn(cfg, Q, K, V, *use, again, ws)
         assert h.heart_get_status(ws) == 0
         assert torch.equal(again.view(torch.int16), ref.view(torch.int16))
+
+
+@pytest.mark.parametrize("block", [64, 128])
+@pytest.mark.parametrize("N,split", [(420, 2), (2045, 4)])
+def test_a_part_that_never_arrives(hooks, block, N, split):
+    """The CTAs that wait for it report it and leave all of their rows of the tile alone; its own rows, for which it has the
+    other parts, and the other tiles are complete."""
+    h, H = hooks, 2
+    g = torch.Generator("cuda").manual_seed(N + block)
+    Q, K, V = (torch.randn((1, H, N, 128), generator=g, device="cuda").to(torch.bfloat16) for _ in range(3))
+    cfg = h.make_config(1, H, N, block, flags=h.FORCE_DENSE)
+    ws = h.new_workspace(cfg)
+    ref, bad, again = (torch.full_like(Q, float("nan")) for _ in range(3))
+    h.heart_block_sparse_attn(cfg, Q, K, V, None, None, ref, ws)
+    assert h.heart_get_status(ws) == 0
+    cfg.flags |= TEST_SKIP_PARTS
+    t0 = time.perf_counter()
+    h.heart_block_sparse_attn(cfg, Q, K, V, None, None, bad, ws)
+    assert h.heart_get_status(ws) == h.ERR_DEVICE_CHECK
+    assert time.perf_counter() - t0 < 5.0
+    rows = 128 // split
+    for r in range(split):
+        part = bad[0, 0, r * rows : (r + 1) * rows]
+        if r != 1:
+            assert part.isnan().all()
+            part.copy_(ref[0, 0, r * rows : (r + 1) * rows])
+    assert torch.equal(bad.view(torch.int16), ref.view(torch.int16))
+    cfg.flags &= ~TEST_SKIP_PARTS
+    h.heart_block_sparse_attn(cfg, Q, K, V, None, None, again, ws)
+    assert h.heart_get_status(ws) == 0
+    assert torch.equal(again.view(torch.int16), ref.view(torch.int16))
 
 
 @pytest.mark.parametrize("block", [64, 128])
