@@ -10,8 +10,8 @@
 //
 // Each axis is a contraction with the fp64 matrix instruction.  Folding x_j +- x_{n-j} halves it: cosines see the
 // even part, sines the odd one.  For 16 x 21 x 60 x 104 that is 1.9e8 fma (10 us at 18.5 T fma/s).  Two ways through it:
-// planes that a CTA holds are transformed along y and x in one kernel, another goes over t (39 us); any other shape goes
-// axis by axis through the workspace, in five launches (55 us for that one).
+// planes that a CTA holds are transformed along y and x in one kernel, another goes over t (39 us); where that is not the
+// faster way (planes_pay), axis by axis through the workspace, in five launches (53 us for that one).
 #include <math.h>
 
 #include "common.cuh"
@@ -283,6 +283,7 @@ __global__ void __launch_bounds__(1024) band_final_kernel(const double *__restri
 
 constexpr int kPlaneThreads = 256, kPlaneWarps = kPlaneThreads / 32;
 constexpr int kPlaneMaxShared = 200 * 1024;  // of a CTA, in bytes
+constexpr int kTilesX = 4, kTilesY = 7;      // tiles of 8 lines that share the table entries of a warp, along x and y
 constexpr int kTimeThreads = 128, kTimeLines = 64, kTimePitch = kTimeLines + 4, kTimeMax = 96, kTimeCtas = 148 * 4;
 
 __host__ __device__ inline int round_up(int v, int m) { return (v + m - 1) / m * m; }
@@ -428,7 +429,7 @@ __global__ void __launch_bounds__(kPlaneThreads, 3) plane_kernel(const float *__
   }
 
   // along x: lines are the rows; cosines of the even part, then sines of the odd one
-  constexpr int TX = 4, TY = 7;  // tiles of 8 lines that share the table entries of a warp
+  constexpr int TX = kTilesX, TY = kTilesY;
   const int cos_x = (hx + 8) / 8, sin_x = (mx + 7) / 8;
   for (int t0 = 0; t0 < row_tiles; t0 += TX) {
     for (int kt = warp; kt < cos_x + sin_x; kt += kPlaneWarps) {
@@ -614,10 +615,41 @@ __global__ void __launch_bounds__(kTimeThreads, 4) time_kernel(const TimeArgs a)
   }
 }
 
-// Planes of 512 points and more that a CTA holds, and time axes whose samples of 64 lines it holds.  (Smaller planes do
-// not fill a CTA's warps, longer time axes go through the general pass in parts.)
+// Planes of 512 points and more that a CTA holds, and time axes whose samples of 64 lines it holds.
 bool planes_fit(int T, int H, int W) {
   return (long long)H * W >= 512 && (long long)H * W <= kPlaneMaxShared / 8 && plane_shared_bytes(H, W) <= kPlaneMaxShared && T <= kTimeMax;
+}
+
+// Products that a warp of plane_kernel takes one after the other: along x, then along y.
+int plane_steps(int ny, int nx) {
+  const int row_tiles = (ny / 2 + 8) / 8, col_tiles = (nx + 7) / 8;
+  const int rounds_x = (row_tiles + kTilesX - 1) / kTilesX * ((nx / 2 + 8) / 8 + ((nx - 1) / 2 + 7) / 8);
+  const int rounds_y = (ny / 2 + 8) / 8 * ((col_tiles + kTilesY - 1) / kTilesY);
+  const int each_x = round_up(nx / 2 + 1, 4) / 4 * (row_tiles < kTilesX ? row_tiles : kTilesX);
+  const int each_y = round_up(ny / 2 + 1, 4) / 4 * (col_tiles < kTilesY ? col_tiles : kTilesY);
+  return (rounds_x + kPlaneWarps - 1) / kPlaneWarps * each_x + (rounds_y + kPlaneWarps - 1) / kPlaneWarps * each_y;
+}
+
+// Whether plane by plane is the faster way, by 15 000 shapes measured both ways (C 1-32, T 1-96, 8 x 64 to 96 x 200 and 300 x 24
+// points).  Taken always, it was 2.5 % slower in the mean than the faster way of each shape and up to 2.2 times; by these lines
+// 0.4 % and up to 1.5 times, and 98 % of usual latents (C 4 or 16, T 5-33, 30-96 x 40-170) are within 5 %.  The CTAs of
+// plane_kernel hide each other's folds and chains while an SM has two or three.  Times in us, axis by axis / plane by plane:
+//  - a plane that fills an SM pays only while the planes make about one wave (16 x 21 x 90 x 160 134 / 140, one plane of it
+//    18 / 26, 4 x 17 x 88 x 160 40 / 32);
+//  - fewer CTAs than SMs run alone: the chain of a warp has to be short (4 x 7 x 72 x 144 24 / 33, 520 steps; 4 x 7 x 60 x 104
+//    18 / 14, 168), and while only some SMs have a second one (4 x 21 x 68 x 104 26 / 32);
+//  - a CTA costs some 3 us however small its plane, and tiles of eight lines of a narrow plane are padding in part: few of them
+//    are welcome, many are not (1 x 5 x 23 x 23 13.7 / 7.9, 16 x 96 x 23 x 23 32 / 52; 16 x 21 x 8 x 200 32 / 48,
+//    3 x 57 x 5 x 178 20 / 30, 3 x 2048 x 1 68 / 583).
+bool planes_pay(int C, int T, int H, int W) {
+  if (!planes_fit(T, H, W)) return false;
+  const long long ctas = 2LL * C * T;
+  const int steps = plane_steps(H, W), per_sm = (int)(226 * 1024 / (plane_shared_bytes(H, W) + 1100));  // (three, by registers)
+  if (per_sm == 1) return ctas > 60 && ctas <= 148;
+  if (H < 24 || W < 24) return ctas <= 148 ? steps <= 150 : ctas <= 592 && steps <= 100 && H >= 8;
+  if (steps <= 50) return ctas <= 888;
+  if (ctas <= 148) return steps <= 400;
+  return steps <= 340 || ctas > 222 || per_sm == 2;
 }
 int time_units(int C, int H, int W) { return C * ((H * W + kTimeLines - 1) / kTimeLines); }
 int time_ctas(int C, int H, int W) { return time_units(C, H, W) < kTimeCtas ? time_units(C, H, W) : kTimeCtas; }
@@ -695,7 +727,7 @@ cudaError_t launch_band_error(const float *ys, const float *yd, int C, int T, in
                               double eps, double *out, void *workspace, cudaStream_t s, int *launches) {
   const long long n = (long long)C * T * H * W;
   char *p = static_cast<char *>(workspace);
-  if (planes_fit(T, H, W)) return launch_planes(ys, yd, C, T, H, W, weights, eps, out, p, s, launches);
+  if (planes_pay(C, T, H, W)) return launch_planes(ys, yd, C, T, H, W, weights, eps, out, p, s, launches);
   double2 *tables = reinterpret_cast<double2 *>(p);  // of x, y, t
   p += align256(sizeof(double2) * ((size_t)T + H + W));
   double *A = reinterpret_cast<double *>(p);
