@@ -165,21 +165,20 @@ __device__ __forceinline__ double sum_range(const double *__restrict__ src, int 
   }
   return s;
 }
-// All n of them in four ascending ranges, s[q] that of range q, the ranges side by side.
+// All n <= 4 * kRangeLoads of them in four ascending ranges, s[q] that of range q, with all loads in flight together.
+constexpr int kRangeLoads = 10;
 __device__ __forceinline__ void sum_chunks(double (&s)[4], const double *__restrict__ src, int n) {
   const int per = (n + 3) / 4;
+  double v[4][kRangeLoads];
 #pragma unroll
-  for (int q = 0; q < 4; ++q) s[q] = 0.0;
-  for (int i = 0; i < per; i += 8) {
-    double v[4][8];
+  for (int q = 0; q < 4; ++q)
 #pragma unroll
-    for (int q = 0; q < 4; ++q)
+    for (int u = 0; u < kRangeLoads; ++u) v[q][u] = __ldcg(&src[(size_t)min(q * per + u, n - 1) * kD]);
 #pragma unroll
-      for (int u = 0; u < 8; ++u) v[q][u] = __ldcg(&src[(size_t)min(q * per + i + u, n - 1) * kD]);
+  for (int q = 0; q < 4; ++q) {
+    s[q] = 0.0;
 #pragma unroll
-    for (int q = 0; q < 4; ++q)
-#pragma unroll
-      for (int u = 0; u < 8; ++u) s[q] = i + u < per && q * per + i + u < n ? s[q] + v[q][u] : s[q];
+    for (int u = 0; u < kRangeLoads; ++u) s[q] = u < per && q * per + u < n ? s[q] + v[q][u] : s[q];
   }
 }
 

@@ -690,6 +690,16 @@ bool rows_kernel_fits(const Geom &g) {
   return (long long)g.R * ((g.nb + 7) / 8) <= 148 * per_sm;
 }
 
+// Whether the row kernel decides too.  Every CTA of a head adds up all of the head's partial sums then: that pays while there are
+// few CTAs, the sums take one trip to memory (a chunk is one block in such a step) and the attention behind them is a small launch,
+// which starts a launch earlier.  Steps in which every head refreshes (reuses) its mask, us, so and with mean_drift_kernel:
+// 8 heads x 20 blocks 20.1 (16.8), 19.6 (17.9); 2 x 40 23.3 (20.3), 22.8 (22.4); beyond the line 24 x 24 31.4 (27.3), 28.8 (25.7);
+// 16 x 64 52.2 (48.6), 47.4 (43.1).
+static bool rows_kernel_decides(const Geom &g) {
+  const bool gate_on = g.gate_lo > 0.0 || g.gate_hi < 1.0;
+  return !gate_on && g.R * ((g.nb + 7) / 8) <= kStatusHeadTickets && g.nb <= 4 * kRangeLoads && g.R * ((g.N + 127) / 128) <= 148;
+}
+
 template <int NJ, bool DECIDE>
 static cudaError_t launch_rows(const Geom &g, const RowArgs &a, cudaStream_t s) {
   const int smem = (int)sizeof(double) * rows_kernel_doubles(NJ, g.nb);
@@ -717,9 +727,8 @@ static RowArgs row_args(const Geom &g, const Workspace &w, const double *tau, he
 cudaError_t launch_decide_and_predict(const Geom &g, const Workspace &w, const DecideArgs &decide, const double *tau, heart_state st,
                                       cudaStream_t s, int *launches) {
   RowArgs a = row_args(g, w, tau, st);
-  const bool gate_on = g.gate_lo > 0.0 || g.gate_hi < 1.0;
   ++*launches;
-  if (gate_on || g.R > kStatusHeadTickets) {
+  if (!rows_kernel_decides(g)) {
     cudaError_t e = launch_decide(g, w, decide, s);
     if (e != cudaSuccess) return e;
     ++*launches;
@@ -731,7 +740,7 @@ cudaError_t launch_decide_and_predict(const Geom &g, const Workspace &w, const D
   a.nchunks = g.nchunks;
   a.decide = decide;
   a.decide.ticket = w.status + kStatusHeadTicketWord;
-  return g.nb <= 64 ? launch_rows<2, true>(g, a, s) : launch_rows<4, true>(g, a, s);
+  return launch_rows<2, true>(g, a, s);
 }
 
 cudaError_t launch_predict_mask(const Geom &g, const Workspace &w, const double *tau,
