@@ -391,8 +391,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
                                smem_u32(sh.in_l)};
   if (Small) {  // the barriers are initialised: for the Q copy below, and for the other CTAs' parts
     if (p.split > 1) {
-      // (a dense launch has next to nothing to wait for)
-      if (warp < 8 && !p.dense) merge_parts(parts, rank, p.split, 0, false, nullptr, 0, nullptr);
+      if (warp < 8) merge_parts(parts, rank, p.split, 0, false, nullptr, 0, nullptr);
       cluster_sync();
     } else {
       __syncthreads();
@@ -866,56 +865,53 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
           const float2 other = sh.l[nt & 1][row];
           l_run += other.x * ex2(other.y - m_ref);
         }
-        // 64 dims at a time, in a loop: half the instructions beside the other warpgroup's (40 x 33k 2821 us with all 128 unrolled,
-        // 2806 so, 2851 with 32 at a time, when O is handed back later; dense 12 x 33k 5650, 5557, 5608).  A row per thread would
-        // touch 32 lines with every store (2700-5000 clocks for a tile, during which the partner runs out of work): 32 dims
-        // at a time go through shared memory, so that four lanes write 64 bytes of a row.
+        uint32_t v[128];
+        if (n_steps > 0) {
+#pragma unroll
+          for (int ch = 0; ch < 4; ++ch) tmem_ld32(o_addr + ch * 32, *reinterpret_cast<uint32_t(*)[32]>(&v[ch * 32]));
+          tmem_wait_ld();
+          arrive(&sh.o_free);
+        } else {
+#pragma unroll
+          for (int i = 0; i < 128; ++i) v[i] = 0u;
+        }
+        if (shared_tile) {  // O as it is, where the keys were, with its row sums: the parts are put together below
+          float4 *part = reinterpret_cast<float4 *>(smem + kOffK + row * 512);
+#pragma unroll
+          for (int i = 0; i < 32; ++i)
+            part[i ^ (row & 7)] = make_float4(__uint_as_float(v[4 * i]), __uint_as_float(v[4 * i + 1]), __uint_as_float(v[4 * i + 2]), __uint_as_float(v[4 * i + 3]));
+          sh.part_l[row] = make_float2(l_run, m_ref);
+          break;
+        }
         const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
+        // A row per thread would touch 32 lines with every store (2700-5000 clocks for a tile, during which the
+        // partner runs out of work): 32 dims at a time go through shared memory, so that four lanes write 64
+        // bytes of a row.
         unsigned char *out = smem + kOffOut + warp * kOutBytes;
         uint16_t *tile_out = p.O + (long long)ti.w * p.sb + (long long)ti.z * p.sh + (long long)(ti.x * 128 + quarter * 32) * p.sn;
         const int rows = p.N - (ti.x * 128 + (int)quarter * 32);  // of this warp that exist
-        float4 *part = reinterpret_cast<float4 *>(smem + kOffK + row * 512);
-#pragma unroll 1
-        for (int ch = 0; ch < 2; ++ch) {
-          uint32_t v[64];
-          if (n_steps > 0) {
-            tmem_ld32(o_addr + ch * 64 + 0, *reinterpret_cast<uint32_t(*)[32]>(&v[0]));
-            tmem_ld32(o_addr + ch * 64 + 32, *reinterpret_cast<uint32_t(*)[32]>(&v[32]));
-            tmem_wait_ld();
-            if (ch == 1) arrive(&sh.o_free);
-          } else {
 #pragma unroll
-            for (int i = 0; i < 64; ++i) v[i] = 0u;
+        for (int ch = 0; ch < 4; ++ch) {
+#pragma unroll
+          for (int g4 = 0; g4 < 4; ++g4) {
+            float o[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) o[i] = __uint_as_float(v[ch * 32 + g4 * 8 + i]) * inv;
+            uint4 x;
+            x.x = pack_bf16x2(o[0], o[1]);
+            x.y = pack_bf16x2(o[2], o[3]);
+            x.z = pack_bf16x2(o[4], o[5]);
+            x.w = pack_bf16x2(o[6], o[7]);
+            *reinterpret_cast<uint4 *>(out + lane * 64 + ((g4 ^ (lane >> 1)) & 3) * 16) = x;
           }
-          if (shared_tile) {  // O as it is, where the keys were, with its row sums: the parts are put together below
+          __syncwarp();
 #pragma unroll
-            for (int i = 0; i < 16; ++i)
-              part[(ch * 16 + i) ^ (row & 7)] = make_float4(__uint_as_float(v[4 * i]), __uint_as_float(v[4 * i + 1]), __uint_as_float(v[4 * i + 2]), __uint_as_float(v[4 * i + 3]));
-            continue;
+          for (int i = 0; i < 4; ++i) {
+            const int rr = i * 8 + (lane >> 2), g4 = lane & 3;
+            const uint4 x = *reinterpret_cast<const uint4 *>(out + rr * 64 + ((g4 ^ (rr >> 1)) & 3) * 16);
+            if (rr < rows) *reinterpret_cast<uint4 *>(tile_out + (long long)rr * p.sn + ch * 32 + g4 * 8) = x;
           }
-#pragma unroll
-          for (int c = 0; c < 2; ++c) {
-#pragma unroll
-            for (int g4 = 0; g4 < 4; ++g4) {
-              float f[8];
-#pragma unroll
-              for (int i = 0; i < 8; ++i) f[i] = __uint_as_float(v[c * 32 + g4 * 8 + i]) * inv;
-              *reinterpret_cast<uint4 *>(out + lane * 64 + ((g4 ^ (lane >> 1)) & 3) * 16) =
-                  make_uint4(pack_bf16x2(f[0], f[1]), pack_bf16x2(f[2], f[3]), pack_bf16x2(f[4], f[5]), pack_bf16x2(f[6], f[7]));
-            }
-            __syncwarp();
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              const int rr = i * 8 + (lane >> 2), g4 = lane & 3;
-              const uint4 x = *reinterpret_cast<const uint4 *>(out + rr * 64 + ((g4 ^ (rr >> 1)) & 3) * 16);
-              if (rr < rows) *reinterpret_cast<uint4 *>(tile_out + (long long)rr * p.sn + (ch * 2 + c) * 32 + g4 * 8) = x;
-            }
-            __syncwarp();
-          }
-        }
-        if (shared_tile) {
-          sh.part_l[row] = make_float2(l_run, m_ref);
-          break;
+          __syncwarp();
         }
         if (valid_row && p.lse != nullptr)
           p.lse[(size_t)(ti.w * p.H + ti.z) * p.N + tok] = l_run > 0.f ? (m_ref + log2f(l_run)) * 0.6931471805599453f : -INFINITY;
