@@ -40,9 +40,9 @@
 //
 // Small launches (a tile per CTA at most) have an instance of their own, which plans its tile itself while Q comes in and, while
 // tiles are few, shares its key steps among a cluster of 2 or 4 CTAs: each CTA copies the others their share of the rows of its
-// part of O as soon as it has it, and puts its own share together.  2 heads x 2k, 32 tiles of up to 13 steps, from the end
-// of the kernel before: 23.0 k clocks when the CTAs read one another's parts behind a barrier, with the roles' first
-// instructions and Q fetched behind the plan, 18.9 k now; 2.3 k of them are the plan, 4 k the exchange of 48 KB each way.
+// part of O as soon as it has it, and puts its own share together.  2 heads x 2045 tokens, half of the blocks listed: 14.4 us when
+// the CTAs read one another's parts behind a barrier, with the roles' first instructions and Q fetched behind the plan,
+// 12.6 now.  (A first call of the merge code ahead of the wait, writing nothing, to have its instructions there: 12.9.)
 //
 // Every wait is bounded; a wait that runs out raises the CTA's abort flag and the status word, its roles
 // drain and stop.  The tile it worked on and those it had drawn already, or was dealt, stay unwritten (as does a tile that a
@@ -287,17 +287,16 @@ __global__ void __launch_bounds__(32 * kPlanWarps)
 }
 
 // Small launches: rows [rank * rows, (rank + 1) * rows) of a shared tile from the parts of the cluster's CTAs, by the
-// softmax warps.  A function that a kernel calls twice, the first time while it waits for the kernel before it, without
-// writing (`real` false): every CTA runs this code once, and from cold instructions it took 3 us.
+// softmax warps.
 struct PartAddresses {
   uint32_t own, own_l, slot, slot2, in_l;  // in shared memory
 };
-__device__ __noinline__ void merge_parts(const PartAddresses at, int rank, int split, int valid_rows, bool real, uint16_t *out, long long sn,
-                                         float *lse) {
+__device__ __forceinline__ void merge_parts(const PartAddresses at, int rank, int split, int valid_rows, uint16_t *out, long long sn,
+                                            float *lse) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, rows = 128 / split;
   // a warp: four rows at a time, eight lanes each, lane q of them pieces q, q + 8, q + 16 and q + 24 of four dims
 #pragma unroll 1
-  for (int i0 = warp * 4 + (lane >> 3); i0 < (real ? rows : 32); i0 += 32) {
+  for (int i0 = warp * 4 + (lane >> 3); i0 < rows; i0 += 32) {
     const int row = rank * rows + i0, q = lane & 7;
     float l[kMaxSplit], m[kMaxSplit], m_all = kNoReference, l_all = 0.f;
     uint32_t src[kMaxSplit];
@@ -332,7 +331,7 @@ __device__ __noinline__ void merge_parts(const PartAddresses at, int rank, int s
       }
     }
     const float inv = l_all > 0.f ? 1.f / l_all : 0.f;
-    if (real && row < valid_rows && !gave_up) {  // (a tile of which a part gave up is not written)
+    if (row < valid_rows && !gave_up) {  // (a tile of which a part gave up is not written)
 #pragma unroll
       for (int k = 0; k < 4; ++k)
         *reinterpret_cast<uint2 *>(out + row * sn + (q + 8 * k) * 4) = make_uint2(pack_bf16x2(o[k].x * inv, o[k].y * inv), pack_bf16x2(o[k].z * inv, o[k].w * inv));
@@ -390,12 +389,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
   const PartAddresses parts = {smem_u32(smem + kOffK), smem_u32(sh.part_l), smem_u32(smem + kOffQ + kTileBytes), smem_u32(smem + kOffOut),
                                smem_u32(sh.in_l)};
   if (Small) {  // the barriers are initialised: for the Q copy below, and for the other CTAs' parts
-    if (p.split > 1) {
-      if (warp < 8) merge_parts(parts, rank, p.split, 0, false, nullptr, 0, nullptr);
-      cluster_sync();
-    } else {
-      __syncthreads();
-    }
+    if (p.split > 1) cluster_sync();
+    else __syncthreads();
   }
   // Launched with programmatic stream serialisation: everything above overlaps the end of the kernels
   // before it.  A kernel that follows (the next layer-step's block-sum pass) may be scheduled once every
@@ -955,9 +950,10 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
       at_barrier = true;
       named_barrier_sync(1, 256);  // one answer for all warps
       const int4 ti = sh.tile[0];
-      merge_parts(parts, rank, p.split, p.N - ti.x * 128, *abort == 0,
-                  p.O + (long long)ti.w * p.sb + (long long)ti.z * p.sh + (long long)ti.x * 128 * p.sn, p.sn,
-                  p.lse != nullptr ? p.lse + (size_t)(ti.w * p.H + ti.z) * p.N + ti.x * 128 : nullptr);
+      if (*abort == 0)
+        merge_parts(parts, rank, p.split, p.N - ti.x * 128,
+                    p.O + (long long)ti.w * p.sb + (long long)ti.z * p.sh + (long long)ti.x * 128 * p.sn, p.sn,
+                    p.lse != nullptr ? p.lse + (size_t)(ti.w * p.H + ti.z) * p.N + ti.x * 128 : nullptr);
     }
   }
   if (Small && p.split > 1) {  // the copies from this CTA's memory are complete: their receivers have them
