@@ -32,8 +32,11 @@ constexpr int kSmallScoreTiles = 148;  // 64 x 64 score tiles of a launch up to 
 // 161 against 167); short rows gain nothing and pay for the CTAs.
 template <int NJ>
 constexpr int kRowsPerCta = NJ >= 24 ? 2 : 8;
+// CTAs that an SM has to hold, which leaves 96 registers a thread for 24 words and more, 80 for 16, 64 for 8, 48 for 2.  At 32
+// words that spills a little and pays with many rows (24 heads x 929 blocks 280 us, 285 with 128 registers; one head 37 and 35).
+// At 24 and 16 words another CTA would not pay for its spills (24 heads x 700 blocks 164 us with 12, 161 with 10).
 template <int NJ>
-constexpr int kCtasPerSm = NJ >= 32 ? 10 : NJ >= 24 ? 12 : NJ >= 8 ? 4 : 5;  // (the registers that leaves: 96, 80, 64, 48)
+constexpr int kCtasPerSm = NJ >= 24 ? 10 : NJ >= 16 ? 3 : NJ >= 8 ? 4 : 5;
 constexpr int kMaxCand = 64;    // candidates the direct threshold evaluation takes
 constexpr float kMassBand = 1.5e-5f;  // of z: cuts whose mass is closer to tau * z are decided in fp64
 // Blocks are ranked by their weight, lowest index first among equals.  Weights exp(s - max) round to the same double
