@@ -460,7 +460,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     }
   };
   // V: [block][dim half][64 keys][64 dims] for blocks of 64.  A product takes 16 keys, so blocks may lie apart, and a copy
-  // brings whole rows: two copies a step instead of four (12 x 33k 1149 us instead of 1160, 40 x 33k 2735 instead of 2766).
+  // brings whole rows: two copies a step instead of four (whole steps of 40 x 33k 2839 us instead of 2882, 12 x 33k 1185 instead of
+  // 1196, 8 x 33k 433 instead of 445; dense 12 x 33k 5744 instead of 5788).
   auto load_v = [&](unsigned char *dst, uint64_t *bar, uint32_t e, int hidx, int bidx) {
     mbar_expect_tx(bar, kTileBytes);
 #pragma unroll

@@ -66,7 +66,6 @@ bool state_ok(const heart_state *st) {
   return st && st->anchor_q && st->anchor_k && st->has_anchor && st->mask_bits && st->kv_idx && st->kv_cnt;
 }
 
-// Mask prediction inside a layer-step (the refresh flags are the ones the decision kernel just wrote).
 // The steps between the block sums and the attention: drift, decision, masks of the refreshed heads.
 cudaError_t decide_for_step(const Geom &g, const Workspace &w, const void *Q, const void *K, const double *delta, const double *tau,
                             heart_state st, double *drift_out, uint8_t *refresh_out, cudaStream_t s) {

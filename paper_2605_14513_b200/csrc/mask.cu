@@ -529,9 +529,9 @@ __global__ void __launch_bounds__(32 * kRowsPerCta<NJ>, kCtasPerSm<NJ>) top_p_ke
 }
 
 // Small layer-steps: a CTA takes eight query blocks of a head from the pooled means to the lists, a warp per row, so that one
-// launch does the work of two or three (whole steps: 2 x 2048 tokens 26.7 us with three, 24.5 with one; 2 x 12 x 2465 with the
-// gate 71.4 and 68.6).  Bound by latency.  DECIDE (no layer gate, a ticket for every head): every CTA of a head adds up the head's token means and decides for itself, bit for bit like mean_drift_kernel; the CTA that took the
-// last of the head's tickets, when all of them have read the old anchor, moves it.
+// launch does the work of two or three.  Bound by latency.  DECIDE (the smallest steps without the layer gate, a ticket for every
+// head): every CTA of a head adds up the head's token means and decides for itself, bit for bit like mean_drift_kernel; the
+// CTA that took the last of the head's tickets, when all of them have read the old anchor, moves it.
 struct RowArgs {
   const double *bmean, *tau;
   int R, nb;
@@ -683,8 +683,11 @@ cudaError_t launch_top_p(const Geom &g, const Workspace &w, const double *tau, c
   return launch_nj<32>(g, w, tau, refresh, st, pitch, s, expect_sig);
 }
 
-// One wave of CTAs (by their shared memory: five an SM at 32 blocks, two at 64, one at 128): a second wave would read every
-// head's key means once more for each eight rows, which the tiles of pooled_scores_kernel do not.
+// About one wave of CTAs, by their shared memory: three an SM at 32 blocks, two at 64, one at 128 (up to six at 16 and fewer, of which
+// the registers hold five).  A second wave would read every head's key means once more for each eight rows, which the tiles
+// of pooled_scores_kernel do not.  Steps that refresh every head, us, with separate kernels / with this one: 37 heads x 64 blocks
+// 95.5 / 92.5, 9 x 128 82.5 / 80.6, 111 x 32 120.2 / 119.9; beyond the line 45 x 64 111.9 / 111.4, 12 x 128 88.1 / 89.3, 16 x 96
+// 74.3 / 77.0.
 bool rows_kernel_fits(const Geom &g) {
   const int nj = (g.nb + 31) / 32;
   if (nj > 4 || (g.flags & HEART_ESTIMATOR_ANTIDIAG)) return false;
