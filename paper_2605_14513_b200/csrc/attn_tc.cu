@@ -10,7 +10,7 @@
 // 1280 (operands of the products and the TMA writes, 128 bytes a clock).  The chain softmax -> products
 // -> softmax of one step is about 3000 clocks long, hand-overs included, so it has to be off the critical
 // path: one persistent CTA per SM works on one query tile at a time and two softmax warpgroups take its
-// key steps in turn.  Scores are double-buffered in tensor memory, and because P has columns of its own,
+// key steps (nearly) in turn.  Scores are double-buffered in tensor memory, and because P has columns of its own,
 // S_{h+2} is computed as soon as the scores of step h sit in registers: a warpgroup finds its next
 // scores ready when it ends a step.  (Two streams on different tiles with P over the scores, one
 // warpgroup each, ran at 1870-2100 clocks per tile and step: each stream waited 1200-1500 of ~3900 clocks for
@@ -19,10 +19,14 @@
 //
 // Warp roles (registers are moved from the helper warps to the softmax warps at start); g counts the key
 // steps of a CTA over all its tiles, buffers and barriers go by g & 1:
-//   warps 0-3, 4-7  softmax of the even / odd steps: one thread per query row (lane quarter = warp & 3).  A
+//   warps 0-3, 4-7  softmax of a step: one thread per query row (lane quarter = warp & 3).  A
 //               thread loads its row of S_g (128 columns), hands the buffer back, takes the max, agrees on the
 //               row's reference with its partner in the other warpgroup, writes P_g = 2^(s*scale*log2e - m)
-//               as bf16 and adds the row sum.  The warpgroup that has a tile's last step writes O / l (and lse).
+//               as bf16 and adds the row sum.  The warpgroup that does not have a tile's last step takes the first one of the
+//               next tile and then writes O / l (and lse) of the tile, by a bulk copy from the place of its Q; meanwhile the
+//               other one takes the second and the third.  (The warpgroup of the last step waited 1300 clocks for the last
+//               products and wrote for 3300 more, with its partner waiting for its step of the next tile: 40 x 33k, 69 tiles a
+//               CTA, 2860 us, now 2745; 2 x 12 x 2465 72.5, now 69.5.)
 //   warp 8      issues S_g = Q K_g^T once step g - 2 has emptied the buffer, warp 11 O += P_g V_g.
 //   warp 9      V producer, warp 10 K and Q producer (draws the tiles and announces them): TMA loads
 //               (cp.async.bulk.tensor, 128-byte swizzle, completion on mbarriers), two 32 KB buffers each.
@@ -31,6 +35,12 @@
 // before; a row whose reference moved gets its part of O rescaled by the warp that moved it, once the
 // products of the steps before are complete, and both partners rescale their own row sums.
 // Tensor memory: O (128 columns) | S[2] (2 x 128) | P[2] (2 x 64).
+//
+// Instructions: an SM keeps 32 KB of them (a loop of 24 KB runs at full rate, one of 48 KB at a third), the kernel has 60, and
+// twelve warps are in different places of it.  So the loop over a softmax warp's steps holds only what every step needs, in one
+// piece; what a step rarely needs (a wait that takes long, a ragged block, a reference that moves) stands outside and the loop is left
+// for it.  With those in the loop 12 x 33k fetched 1.7 times as often and 2 x 12 x 2465 1.4 times, in 4 and 10 % more clocks.
+// (A small launch goes through all of them once: there they stand where they are needed, 0.1 to 0.4 us of 13 to 24.)
 //
 // The step lists come from attn_plan_kernel (one warp per tile), which runs just before; the tiles are
 // taken in the order of tile_order_kernel: head-major (the K/V of one or two heads stay in L2), within a
@@ -68,11 +78,12 @@ constexpr float kNoReference = -3.0e38f;  // below every logit: the first step m
 // below 1: weights are at most 2^8, so n keys with values up to 2^120 / n cannot overflow O (all of it above 1, with
 // weights up to 2^64, left 2^64 / n), and a weight of 2^-110 of the largest is still a normal number.
 constexpr float kHeadroom = 16.f, kMaxGrowth = 8.f;
+constexpr uint32_t kShortWait = 20;  // ns that a softmax warp waits for its scores before it leaves the loop over its steps
 constexpr int kMaxSplit = 4;  // CTAs that share a tile in a small launch
 
 // Shared-memory plan (the dynamic allocation itself is 1024-byte aligned).
-constexpr int kOutBytes = 2048;  // per softmax warp: 32 rows x 32 dims of the output
-constexpr int kOffQ = 0, kOffK = 2 * kTileBytes, kOffV = 4 * kTileBytes, kOffOut = 6 * kTileBytes, kOffBar = kOffOut + 8 * kOutBytes;
+constexpr int kOffQ = 0, kOffK = 2 * kTileBytes, kOffV = 4 * kTileBytes;
+constexpr int kOffPart = 6 * kTileBytes, kOffBar = kOffPart + kTileBytes / 2;  // small launches: the third part of a shared tile
 
 struct AttnShared {
   uint64_t q_full[2], k_full[2], v_full[2];  // TMA -> issuer
@@ -81,14 +92,19 @@ struct AttnShared {
   uint64_t p_full[2];      // P_g written (one arrival per softmax warp)
   uint64_t pv_done[2];     // P_g V_g complete (V_g and P_g are free)
   uint64_t m_ready[2][4];  // references after step g, per lane quarter
+  uint64_t o_full[2];      // the products of a tile are complete, per tile & 1 (a barrier of its own: the warpgroup that waits for it
+                           // may be two phases of pv_done behind)
   uint64_t o_free;         // O of a tile has been read
+  uint64_t out_done[2];    // a tile's output has left the place of its Q
   uint64_t tile_full[kTileRing], tile_empty[kTileRing];
   uint64_t drain[2];       // abort path: the issuers' products in flight have landed
   int4 tile[kTileRing];    // query tile of its head, listed key blocks, head, batch entry (-1: no tile left)
   uint32_t entry[4];       // the key steps in flight, for the softmax warps: entry[g & 3] is written before K_g is asked
                            // for and read before the scores of step g are handed back, which K_{g+4} waits for
   float m[2][128];         // references after step g
-  float2 l[2][128];        // row sum and its reference of the warpgroup without the last step, per tile & 1
+  float2 l[2][128];        // row sum and its reference of the warpgroup with a tile's last step, per tile & 1
+  float2 own[2][128];      // the same of the other one, per warpgroup, until it writes the tile
+  int4 written[2][8];      // that tile, per softmax warp
   uint32_t tmem_base;
   int abort;
   // small launches: the parts of a tile that this CTA puts together, the tile's plan
@@ -116,6 +132,7 @@ struct AttnParams {
   int h0, hcount;  // this launch covers heads [h0, h0 + hcount) of every batch entry
   float scale_log2;
   int split;        // small launches: CTAs (one cluster) that share the key steps of a tile
+  int late;         // the warpgroup with a tile's first step takes its next one a step later: CTAs have several tiles
   int test_skip_v;      // test-hook builds only: CTA 0 leaves out the V copy of its second key step,
   int test_skip_parts;  // CTA 1 does not send its part of a shared tile
 };
@@ -343,7 +360,8 @@ __device__ __forceinline__ void merge_parts(const PartAddresses at, int rank, in
 template <int B, bool Small>
 __global__ void __launch_bounds__(kAttnThreads, 1)
     attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
-                   const __grid_constant__ CUtensorMap map_v, const AttnParams p, const PlanParams plan) {
+                   const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_o, const AttnParams p,
+                   const PlanParams plan) {
   extern __shared__ __align__(1024) unsigned char smem[];
   AttnShared &sh = *reinterpret_cast<AttnShared *>(smem + kOffBar);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -365,7 +383,11 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
       mbar_init(&sh.tile_full[i], 1);
       mbar_init(&sh.tile_empty[i], kTileReaders);
     }
+    mbar_init(&sh.o_full[0], 1);
+    mbar_init(&sh.o_full[1], 1);
     mbar_init(&sh.o_free, 4);
+    mbar_init(&sh.out_done[0], 4);
+    mbar_init(&sh.out_done[1], 4);
     mbar_init(&sh.drain[0], 1);
     mbar_init(&sh.drain[1], 1);
     mbar_init(&sh.parts_full, 1);
@@ -384,9 +406,10 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     tma_prefetch_desc(&map_q);
     tma_prefetch_desc(&map_k);
     tma_prefetch_desc(&map_v);
+    tma_prefetch_desc(&map_o);
   }
   const int rank = Small ? (int)cluster_ctarank() : 0;
-  const PartAddresses parts = {smem_u32(smem + kOffK), smem_u32(sh.part_l), smem_u32(smem + kOffQ + kTileBytes), smem_u32(smem + kOffOut),
+  const PartAddresses parts = {smem_u32(smem + kOffK), smem_u32(sh.part_l), smem_u32(smem + kOffQ + kTileBytes), smem_u32(smem + kOffPart),
                                smem_u32(sh.in_l)};
   if (Small) {  // the barriers are initialised: for the Q copy below, and for the other CTAs' parts
     if (p.split > 1) cluster_sync();
@@ -424,9 +447,25 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
   // Waits of a whole warp; ok turns false when one runs out or the CTA aborts.  The usual case is a barrier
   // that is complete already.
   bool ok = true;
-  auto complete = [](uint64_t *bar, uint32_t parity) { return __all_sync(0xffffffffu, mbar_test_wait(bar, parity)) != 0; };
+  auto out_of_time = [&](uint32_t &since) -> bool {  // since: 0 at a wait's first call
+    const uint32_t now = clock() | 1u;
+    if (since == 0) since = now;
+    if (*abort == 0 && now - since <= (uint32_t)kWaitLimitCycles) return false;
+    *abort = 1;
+    return true;
+  };
   auto wait = [&](uint64_t *bar, uint32_t parity) {
-    if (__builtin_expect(!complete(bar, parity), 0)) ok = __all_sync(0xffffffffu, mbar_wait(bar, parity, abort)) && ok;
+    uint32_t since = 0;
+#pragma unroll 1
+    while (__builtin_expect(!__all_sync(0xffffffffu, mbar_try_wait(bar, parity)), 0))
+      if (__any_sync(0xffffffffu, out_of_time(since))) return ok = false;
+    return ok;
+  };
+  auto wait1 = [&](uint64_t *bar, uint32_t parity) {  // by one thread
+    uint32_t since = 0;
+#pragma unroll 1
+    while (__builtin_expect(!mbar_try_wait(bar, parity), 0))
+      if (out_of_time(since)) return ok = false;
     return ok;
   };
   auto small_tile = [&](int U) {
@@ -471,11 +510,12 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
   // Shared memory must not be released under a copy in flight: a producer that stops early (abort)
   // waits, bounded, for the copies it has issued.
   auto settle = [&](uint64_t *bar, uint32_t parity) {
-    const long long t0 = clock64();
-    while (!mbar_try_wait(bar, parity) && clock64() - t0 < 40000000LL) {
+    const uint32_t t0 = clock();
+    while (!mbar_try_wait(bar, parity) && (uint32_t)clock() - t0 < 40000000u) {
     }
   };
   auto settle_pair = [&](uint64_t *bar, int issued) {  // the last two of `issued` copies on a pair of barriers
+#pragma unroll 1
     for (int i = issued > 2 ? issued - 2 : 0; i < issued; ++i) settle(&bar[i & 1], (i >> 1) & 1);
   };
 
@@ -504,75 +544,72 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
         int4 ti = sh.tile[0];
         mbar_expect_tx(&sh.q_full[0], kTileBytes);
         tma_load_5d(smem + kOffQ, &map_q, &sh.q_full[0], 0, ti.x * 128, 0, ti.z, ti.w);
-        ok = mbar_wait(&sh.tile_full[0], 0, abort);
+        wait1(&sh.tile_full[0], 0);
         ti = sh.tile[0];
         small_tile(ti.y);
         const int n_steps = ok && rank < parts_of_tile ? n_steps_of(ti.y) : 0;
         const uint32_t *steps = steps_of(ti);
 #pragma unroll 1
         for (; g < n_steps; ++g) {
-          if (g >= 2) ok = mbar_wait(&sh.s_full[g & 1], ((g - 2) >> 1) & 1, abort);
+          if (g >= 2) wait1(&sh.s_full[g & 1], ((g - 2) >> 1) & 1);
           if (!ok) break;
           const uint32_t e = step_entry(steps, g);
           sh.entry[g & 3] = e;
           load_k(smem + kOffK + (g & 1) * kTileBytes, &sh.k_full[g & 1], e, ti.z, ti.w);
         }
       }
-      int4 nx;               // the tile that is announced next and its first key step, fetched ahead of time
-      uint32_t e = 0;
-      auto fetch = [&](int n) {
-        nx.w = -1;
-        if (n >= p.n_tiles) return;
-        uint4 t;
-        if (p.dense) {
-          t.y = n / p.n_tiles_per_head;
-          t.x = (n - t.y * p.n_tiles_per_head) | (uint32_t)p.nb << 16;
-          t.z = step_entry(nullptr, 0);
-        } else {
-          t = __ldcg(&p.tiles[n]);
-        }
-        e = t.z;
-        nx.x = t.x & 0xffff;
-        nx.y = t.x >> 16;
-        nx.w = (int)t.y / p.hcount;
-        nx.z = p.h0 + (int)t.y - nx.w * p.hcount;
-      };
       // The first tile of every CTA is fixed, the others are drawn.  Dense tiles are all
       // of one length: dealt in turn, so that dense calls share nothing and may overlap on one workspace.  (Drawn, the faster
       // SMs take the odd tiles: 12 x 33k 5604 us, dealt 5721.)
-      int mine = blockIdx.x;
-      if (!Small) fetch(mine);
-      auto draw = [&]() { fetch(p.dense ? mine += gridDim.x : gridDim.x + atomicAdd(p.counter, 1)); };
+      int n = blockIdx.x;
+#pragma unroll 1
       for (int t = 0; !Small; ++t) {
+        int4 ti = make_int4(0, 0, 0, -1);
+        uint32_t e = 0;  // its next key step, fetched ahead of time
+        if (n < p.n_tiles) {
+          uint4 word;
+          if (p.dense) {
+            word.y = n / p.n_tiles_per_head;
+            word.x = (n - word.y * p.n_tiles_per_head) | (uint32_t)p.nb << 16;
+            word.z = step_entry(nullptr, 0);
+          } else {
+            word = __ldcg(&p.tiles[n]);
+          }
+          e = word.z;
+          ti.x = word.x & 0xffff;
+          ti.y = word.x >> 16;
+          ti.w = (int)word.y / p.hcount;
+          ti.z = p.h0 + (int)word.y - ti.w * p.hcount;
+        }
         const int i = t % kTileRing;
-        if (t >= kTileRing) ok = mbar_wait(&sh.tile_empty[i], (t / kTileRing - 1) & 1, abort);
-        if (!ok) break;
-        const int4 ti = nx;
+        if (t >= kTileRing && !wait1(&sh.tile_empty[i], (t / kTileRing - 1) & 1)) break;
         sh.tile[i] = ti;
         mbar_arrive(&sh.tile_full[i]);
         if (ti.w < 0) break;
         const int n_steps = n_steps_of(ti.y);
         const uint32_t *steps = steps_of(ti);
-        uint32_t e_now = e;
+        int n_next = p.dense ? n + gridDim.x : 0;
+        if (n_steps == 0 && !p.dense) n_next = gridDim.x + atomicAdd(p.counter, 1);
+#pragma unroll 1
         for (int h = 0; h < n_steps; ++h, ++g) {
           const uint32_t e_next = h + 1 < n_steps ? step_entry(steps, h + 1) : 0u;
-          if (g >= 2) ok = mbar_wait(&sh.s_full[g & 1], ((g - 2) >> 1) & 1, abort);
-          if (!ok) break;
-          sh.entry[g & 3] = e_now;
-          load_k(smem + kOffK + (g & 1) * kTileBytes, &sh.k_full[g & 1], e_now, ti.z, ti.w);
+          if (g >= 2 && !wait1(&sh.s_full[g & 1], ((g - 2) >> 1) & 1)) break;
+          sh.entry[g & 3] = e;
+          load_k(smem + kOffK + (g & 1) * kTileBytes, &sh.k_full[g & 1], e, ti.z, ti.w);
           if (h == 0) {
-            // its buffer is free: the last step of the tile before the previous one is complete
+            // its buffer is free: the last step of the tile before the previous one is complete, its output gone
+            if (nq >= 2 && !wait1(&sh.out_done[nq & 1], ((nq - 2) >> 1) & 1)) break;
             mbar_expect_tx(&sh.q_full[nq & 1], kTileBytes);
             tma_load_5d(smem + kOffQ + (nq & 1) * kTileBytes, &map_q, &sh.q_full[nq & 1], 0, ti.x * 128, 0, ti.z, ti.w);
             ++nq;
           }
           // The next tile is drawn at the last moment that hides the trip to memory: drawn with the first step, a
           // CTA on a long tile already owned another one while others ran out (2 x 12 x 2465: 56.9 us against 55.2).
-          if (h == n_steps - 1) draw();
-          e_now = e_next;
+          if (h == n_steps - 1 && !p.dense) n_next = gridDim.x + atomicAdd(p.counter, 1);
+          e = e_next;
         }
         if (!ok) break;
-        if (n_steps == 0) draw();
+        n = n_next;
       }
       if (Small) settle(&sh.q_full[0], 0);  // (a CTA without a step has not waited for it)
       if (*abort) {
@@ -585,10 +622,12 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     if (Small) pdl_wait();
     int g = 0;
     int4 ti;
+#pragma unroll 1
     for (int t = 0; ok && next_tile(t, ti); ++t) {
       const int n_steps = n_steps_of(ti.y);
       const uint32_t *steps = steps_of(ti);
       uint32_t e_next = n_steps > 0 ? step_entry(steps, 0) : 0u;
+#pragma unroll 1
       for (int h = 0; h < n_steps; ++h, ++g) {
         const uint32_t e = e_next;
         if (h + 1 < n_steps) e_next = step_entry(steps, h + 1);
@@ -614,12 +653,14 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     if (Small) pdl_wait();
     uint32_t g = 0, nq = 0;           // key steps and tiles with key steps so far
     int4 ti;
+#pragma unroll 1
     for (int t = 0; ok && next_tile(t, ti); ++t) {
       const int n_steps = n_steps_of(ti.y);
       if (n_steps == 0) continue;
       wait(&sh.q_full[nq & 1], (nq >> 1) & 1);
       const uint64_t qd = desc_at(q_desc, (nq & 1) * (kTileBytes >> 4));
       ++nq;
+#pragma unroll 1
       for (int h = 0; h < n_steps; ++h, ++g) {  // S_g = Q K_g^T
         const uint32_t b = g & 1;
         if (g >= 2) wait(&sh.s_free[b], ((g - 2) >> 1) & 1);
@@ -646,11 +687,13 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     if (Small) pdl_wait();
     uint32_t g = 0, nt = 0;  // key steps and tiles with key steps so far
     int4 ti;
+#pragma unroll 1
     for (int t = 0; ok && next_tile(t, ti); ++t) {
       const int n_steps = n_steps_of(ti.y);
       if (n_steps == 0) continue;
       if (nt > 0) wait(&sh.o_free, (nt - 1) & 1);
       ++nt;
+#pragma unroll 1
       for (int h = 0; h < n_steps; ++h, ++g) {  // O (+)= P_g V_g
         const uint32_t b = g & 1;
         wait(&sh.v_full[b], (g >> 1) & 1);
@@ -661,6 +704,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
 #pragma unroll
           for (int ks = 0; ks < 8; ++ks)
             mma_ts(tmem, tmem + 384 + b * 64 + ks * 8, desc_at(vd, B == 128 ? ks * 128 : (ks >> 2) * (kTileBytes >> 5) + (ks & 3) * 128), idesc, (h > 0 || ks > 0) ? 1u : 0u);
+          if (h == n_steps - 1) tc_commit(&sh.o_full[(nt - 1) & 1]);
           tc_commit(&sh.pv_done[b]);
         }
         __syncwarp();
@@ -668,11 +712,11 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     }
     drain_products(leader, &sh.drain[1]);
   } else if (warp < 8) {
-    // ===== softmax / correction / epilogue: thread = one query row, steps g with g & 1 == w
+    // ===== softmax / correction / epilogue: thread = one query row
     setmaxnreg_inc<kRegsSoftmax>();
     const uint32_t w = warp >> 2, quarter = warp & 3;
     const int row = quarter * 32 + lane;  // row inside the 128-row query tile
-    const uint32_t o_addr = tmem + (quarter << 21), s_addr = o_addr + 128 + w * 128, p_addr = o_addr + 384 + w * 64;
+    const uint32_t o_addr = tmem + (quarter << 21), s_addr = o_addr + 128, p_addr = o_addr + 384;
     const float c = p.scale_log2;
     const uint64_t c2 = pack_f32x2(c, c);
     auto arrive = [&](uint64_t *bar) {  // this warp's tensor-memory accesses so far are ordered before it
@@ -697,103 +741,151 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
       named_barrier_sync(2, 256);
     }
     uint32_t g0 = 0, nt = 0;  // key steps before the present tile, tiles with key steps before it
-    int4 ti;
-    for (int t = 0; ok && next_tile(t, ti); ++t) {
-      const int n_steps = n_steps_of(ti.y);
-      float m_ref = kNoReference, l_run = 0.f;  // (rows without a key keep the reference)
-      const uint32_t h0 = (w ^ g0) & 1;         // this warpgroup's first step of the tile
-      for (int h = h0; h < n_steps; h += 2) {
-        const uint32_t g = g0 + h;
+    int n_steps = 0, h = 0;   // of the present tile; this warpgroup's next step of it
+    bool leads = w == 0;      // takes the tile's first step
+    bool pending = false;     // the tile before is this warpgroup's to write
+    bool live = true;
+    float m_ref = kNoReference, l_run = 0.f;
+    // Why the loop over the steps was left: what a step rarely needs stands outside of it.
+    enum { kNothing, kNotThere, kMask, kRescale } why = kNothing;
+    bool masked = false;      // the keys of the step that do not count have been taken out
+    float alpha = 1.f;        // O and the sums change scale by it
+    auto advance = [&]() -> bool {  // to this warpgroup's next step; true if the output of the tile before comes first
+      // Steps are taken in turn, but that the second and third go to one warpgroup: the other one writes the output of
+      // the tile before meanwhile.  (In a CTA's first tile too: the order of a row's sum goes by the shape alone.)
+      const bool first = h < 2;
+      h += first && p.late ? 3 - 2 * h : 2;
+      return first && pending;
+    };
+    auto mask_keys = [&](uint32_t b, uint32_t e) {
+      // Keys that do not count get a score of -inf in tensor memory, where a loop over columns is a loop;
+      // the step is then like any other.  (As 128 selects between the loads and the weights it slowed all
+      // steps by 7 %; a branch of its own, 32 columns at a time, took 5000-9000 clocks instead of 2600.)
+      const uint32_t flags = (e >> (10 + (quarter >> 1))) & 0x10001u, s_at = s_addr + b * 128;
+      int n0, n1;  // keys of each half that count
+      if (B == 128) {
+        n0 = p.N - (int)e * 128;
+        n1 = n0 - 64;
+      } else {
+        n0 = (flags & 1u) ? p.N - (int)(e & 0x3ff) * 64 : 0;
+        n1 = (flags >> 16) ? p.N - (int)((e >> 16) & 0x3ff) * 64 : 0;
+      }
+      tc_fence_after();
+#pragma unroll 1
+      for (int col = 0; col < 128; col += 8) {
+        const int n = (col < 64 ? n0 : n1 + 64) - col;  // columns of these eight that count
+        if (n <= 0) {
+          tmem_st8_fill(s_at + col, 0xff800000u);
+        } else {
+#pragma unroll 1
+          for (int i = n; i < 8; ++i) tmem_st1(s_at + col + i, 0xff800000u);
+        }
+      }
+      tmem_wait_st();
+    };
+    auto end_tile = [&]() {
+      if (n_steps == 0) return;
+      const int last = n_steps - 1;
+      const bool mine = leads == (p.late ? last == 0 || (last > 2 && (last & 1)) : !(last & 1));  // had the last step
+      leads = !mine;
+      if (!mine) {
+        pending = true;
+        sh.own[w][row] = make_float2(l_run, m_ref);
+      }
+      g0 += n_steps;
+      ++nt;
+    };
+    int t = 0;
+    auto next = [&]() {  // tile
+      int4 ti;
+      live = next_tile(t++, ti);
+      if (!live) return;
+      if (lane == 0) sh.written[nt & 1][warp] = ti;
+      n_steps = n_steps_of(ti.y);
+      h = leads ? 0 : 1;
+      m_ref = kNoReference;  // (rows without a key keep it)
+      l_run = 0.f;
+      if (n_steps == 0 && leads) {  // rows without any key
+        const int tok = ti.x * 128 + row;
+        if (shared_tile) {
+          sh.part_l[row] = make_float2(0.f, kNoReference);  // (nothing else of this part is read)
+        } else if (tok < p.N) {
+          uint4 *out = reinterpret_cast<uint4 *>(p.O + (long long)ti.w * p.sb + (long long)ti.z * p.sh + (long long)tok * p.sn);
+#pragma unroll 1
+          for (int i = 0; i < 16; ++i) out[i] = make_uint4(0u, 0u, 0u, 0u);
+          if (p.lse != nullptr) p.lse[(size_t)(ti.w * p.H + ti.z) * p.N + tok] = -INFINITY;
+        }
+      }
+    };
+    if (Small) next();  // (the only one)
+    for (;;) {
+#pragma unroll 1
+      while (h < n_steps) {
+        const uint32_t g = g0 + h, b = g & 1, s_at = s_addr + b * 128, p_at = p_addr + b * 64;
         // The scores, and the references after the step before (half a step old by now, as a rule), are asked for
         // together: a barrier that is complete costs ~170 clocks to ask, one after the other as many again.  (With the
-        // same for P below, 24 x 119k: 15.95 to 15.3 M clocks.)
-        const bool there = mbar_test_wait(&sh.s_full[w], (g >> 1) & 1) &
-                           (g == 0 || mbar_test_wait(&sh.m_ready[w ^ 1][quarter], ((g - 1) >> 1) & 1));
+        // same for P below, 24 x 119k: 15.95 to 15.3 M clocks.)  A parity tells two phases in a row apart: behind a step that
+        // the other warpgroup took on this buffer, the answer for the scores holds once that step's partner has its reference.
+        auto ask = [&](uint64_t *bar, uint32_t parity) { return Small ? mbar_test_wait(bar, parity) : mbar_try_wait(bar, parity, kShortWait); };
+        const bool m_there = ask(&sh.m_ready[b ^ 1][quarter], ((g - 1) >> 1) & 1) || g == 0;
+        const bool there = ask(&sh.s_full[b], (g >> 1) & 1) && m_there;
         if (__builtin_expect(!__all_sync(0xffffffffu, there), 0)) {
-          wait(&sh.s_full[w], (g >> 1) & 1);
-          if (g > 0) wait(&sh.m_ready[w ^ 1][quarter], ((g - 1) >> 1) & 1);
+          if (!Small) {
+            why = kNotThere;
+            break;
+          }
+          // (a small launch waits for most of its few steps, and comes by all instructions for the first time)
+          if (g > 0) wait(&sh.m_ready[b ^ 1][quarter], ((g - 1) >> 1) & 1);
+          wait(&sh.s_full[b], (g >> 1) & 1);
         }
         const uint32_t e = sh.entry[g & 3];
         // which halves of the step this row's query block lists, whether the step holds the ragged last block
         const uint32_t flags = (e >> (10 + (quarter >> 1))) & 0x10001u;  // (64-token blocks)
         const bool ragged = B == 128 ? (int)(e + 1) * 128 > p.N : (e & 0x10001000u) != 0u;
         tc_fence_after();
-        const float m_prev = h > 0 ? sh.m[w ^ 1][row] : kNoReference;
+        const float m_prev = h > 0 ? sh.m[b ^ 1][row] : kNoReference;  // the reference as the step before left it
+        auto take_reference = [&]() {
+          l_run *= ex2(m_ref - m_prev);
+          m_ref = m_prev;
+        };
         Sums sums = {0.f, 0.f, 0.f, 0.f};
-        // Agrees on the reference of step g given the row's maximum; true if it is not the one this warp has
-        // used so far (some row).
+        // Agrees on the reference of step g given the row's maximum; true if it moves (some row).
+        bool moved = false;
         auto new_reference = [&](float x_max) -> bool {
-          const bool grow = x_max > m_prev + kMaxGrowth;
-          const float m_new = grow ? x_max + kHeadroom : m_prev;
-          sh.m[w][row] = m_new;
+          const bool grow = x_max > m_ref + kMaxGrowth;
+          const float m_new = grow ? x_max + kHeadroom : m_ref;
+          sh.m[b][row] = m_new;
           __syncwarp();
-          if (lane == 0) mbar_arrive(&sh.m_ready[w][quarter]);
-          if (__builtin_expect(!__any_sync(0xffffffffu, m_new != m_ref), 1)) return false;
-          l_run *= ex2(m_ref - m_new);
+          if (lane == 0) mbar_arrive(&sh.m_ready[b][quarter]);
+          if (__builtin_expect(!__any_sync(0xffffffffu, grow), 1)) return false;
+          moved = true;
+          alpha = ex2(m_ref - m_new);
+          l_run *= alpha;
           m_ref = m_new;
-          if (h > 0 && __any_sync(0xffffffffu, grow)) {
-            // O changes scale: the products of the steps before have to be complete
-            if (g >= 2) wait(&sh.pv_done[w], ((g - 2) >> 1) & 1);
-            if (wait(&sh.pv_done[w ^ 1], ((g - 1) >> 1) & 1)) {
-              tc_fence_after();
-              const float alpha = ex2(m_prev - m_new);
-              const uint64_t alpha2 = pack_f32x2(alpha, alpha);
-#pragma unroll 1
-              for (int ch = 0; ch < 8; ++ch) {
-                uint32_t v[16];
-                tmem_ld16(o_addr + ch * 16, v);
-                tmem_wait_ld();
-#pragma unroll
-                for (int i = 0; i < 16; i += 2) {
-                  float lo, hi;
-                  unpack_f32x2(mul_f32x2(pack_f32x2(__uint_as_float(v[i]), __uint_as_float(v[i + 1])), alpha2), lo, hi);
-                  v[i] = __float_as_uint(lo);
-                  v[i + 1] = __float_as_uint(hi);
-                }
-                tmem_st16(o_addr + ch * 16, v);
-              }
-            }
-          }
           return true;
         };
-        // the product that read this warpgroup's P two steps ago is complete
+        if (__builtin_expect(ragged && !masked, 0)) {
+          if (!Small) {
+            why = kMask;
+            break;
+          }
+          mask_keys(b, e);
+        }
+        // the product that read this P two steps ago is complete
         auto p_free = [&]() {
-          if (g >= 2) wait(&sh.pv_done[w], ((g - 2) >> 1) & 1);
+          if (g >= 2) wait(&sh.pv_done[b], ((g - 2) >> 1) & 1);
           tc_fence_after();
         };
-        if (__builtin_expect(ragged, 0)) {
-          // Keys that do not count get a score of -inf in tensor memory, where a loop over columns is a loop;
-          // the step is then like any other.  (As 128 selects between the loads and the weights it slowed all
-          // steps by 7 %; a branch of its own, 32 columns at a time, took 5000-9000 clocks instead of 2600.)
-          int n0, n1;  // keys of each half that count
-          if (B == 128) {
-            n0 = p.N - (int)e * 128;
-            n1 = n0 - 64;
-          } else {
-            n0 = (flags & 1u) ? p.N - (int)(e & 0x3ff) * 64 : 0;
-            n1 = (flags >> 16) ? p.N - (int)((e >> 16) & 0x3ff) * 64 : 0;
-          }
-#pragma unroll 1
-          for (int col = 0; col < 128; col += 8) {
-            const int n = (col < 64 ? n0 : n1 + 64) - col;  // columns of these eight that count
-            if (n <= 0) {
-              tmem_st8_fill(s_addr + col, 0xff800000u);
-            } else {
-#pragma unroll 1
-              for (int i = n; i < 8; ++i) tmem_st1(s_addr + col + i, 0xff800000u);
-            }
-          }
-          tmem_wait_st();
-        }
         if (__builtin_expect(B == 128 || flags == 0x10001u || ragged, 1)) {
           // The exponentials of the first 32 keys are taken with the reference as it was while the row maximum is
           // found, and once more, by the same instructions, in the rare step that moves it (a tile's first ones:
           // a copy of its own for them cost 2 % of the clocks of a tile with 10-20 steps, from cold instructions).
           uint32_t s[128], pk[32];
 #pragma unroll
-          for (int q = 0; q < 4; ++q) tmem_ld32(s_addr + q * 32, *reinterpret_cast<uint32_t(*)[32]>(&s[q * 32]));
+          for (int q = 0; q < 4; ++q) tmem_ld32(s_at + q * 32, *reinterpret_cast<uint32_t(*)[32]>(&s[q * 32]));
+          take_reference();
           tmem_wait_ld();
-          arrive(&sh.s_free[w]);
+          arrive(&sh.s_free[b]);
           uint64_t neg_m2;
           bool again = false;
 #pragma unroll 1
@@ -805,120 +897,155 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
             again = !again && new_reference(x_max);
           } while (__builtin_expect(again, 0));
           // p_free, asked for ahead of these exponentials
-          const bool p_done = g < 2 || mbar_test_wait(&sh.pv_done[w], ((g - 2) >> 1) & 1);
+          const bool p_done = g < 2 || mbar_test_wait(&sh.pv_done[b], ((g - 2) >> 1) & 1);
           exp32(&s[32], c2, neg_m2, &pk[16], sums);
-          if (__builtin_expect(!__all_sync(0xffffffffu, p_done), 0)) wait(&sh.pv_done[w], ((g - 2) >> 1) & 1);
+          if (__builtin_expect(!__all_sync(0xffffffffu, p_done), 0)) wait(&sh.pv_done[b], ((g - 2) >> 1) & 1);
           tc_fence_after();
-          tmem_st32(p_addr, pk);
+          tmem_st32(p_at, pk);
           exp32(&s[64], c2, neg_m2, &pk[0], sums);
           exp32(&s[96], c2, neg_m2, &pk[16], sums);
-          tmem_st32(p_addr + 32, pk);
-        } else if (flags != 0u) {
-          // This row's query block lists one of the step's two blocks.  The product reads all 128 keys of
-          // the step: zeros for the other one.
-          const uint32_t v = flags >> 16;
-          uint32_t s[64], pk[32];
-          tmem_ld32(s_addr + v * 64, *reinterpret_cast<uint32_t(*)[32]>(&s[0]));
-          tmem_ld32(s_addr + v * 64 + 32, *reinterpret_cast<uint32_t(*)[32]>(&s[32]));
-#pragma unroll
-          for (int i = 0; i < 32; ++i) pk[i] = 0u;
-          tmem_wait_ld();
-          arrive(&sh.s_free[w]);
-          new_reference(max64(s) * c);
-          p_free();
-          tmem_st32(p_addr + (32 - v * 32), pk);
-          const uint64_t neg_m2 = pack_f32x2(-m_ref, -m_ref);
-          exp32(&s[0], c2, neg_m2, &pk[0], sums);
-          exp32(&s[32], c2, neg_m2, &pk[16], sums);
-          tmem_st32(p_addr + v * 32, pk);
+          tmem_st32(p_at + 32, pk);
         } else {
-          // none of the step's blocks is listed by this row's query block
-          uint32_t pk[32];
-#pragma unroll
-          for (int i = 0; i < 32; ++i) pk[i] = 0u;
-          arrive(&sh.s_free[w]);
-          new_reference(-INFINITY);
+          // This row's query block lists one of the step's two blocks or none.  The product reads all 128 keys of the
+          // step: zeros for the others.  (Short code rather than fast code: the step is bound by its products.)
+          const uint32_t v = flags >> 16;
+          uint32_t s[64], pk[16];
+          tmem_ld32(s_at + v * 64, *reinterpret_cast<uint32_t(*)[32]>(&s[0]));
+          tmem_ld32(s_at + v * 64 + 32, *reinterpret_cast<uint32_t(*)[32]>(&s[32]));
+          take_reference();
+          tmem_wait_ld();
+          arrive(&sh.s_free[b]);
+          const float x_max = max64(s) * c;
+          new_reference(flags != 0u ? x_max : -INFINITY);
           p_free();
-          tmem_st32(p_addr, pk);
-          tmem_st32(p_addr + 32, pk);
+          const uint64_t neg_m2 = pack_f32x2(-m_ref, -m_ref);
+          const uint32_t n_exp = flags != 0u ? 4 : 0;
+#pragma unroll 1
+          for (uint32_t i = n_exp; i < 8; ++i) tmem_st8_fill(p_at + ((v * 32 + i * 8) & 63), 0u);
+#pragma unroll 1
+          for (uint32_t i = 0; i < n_exp; i += 2) {
+            exp32(&s[0], c2, neg_m2, &pk[0], sums);
+            tmem_st16(p_at + v * 32 + i * 8, pk);
+#pragma unroll
+            for (int k = 0; k < 32; ++k) s[k] = s[32 + k];
+          }
         }
         l_run += (sums.a + sums.b) + (sums.c + sums.d);
-        if (h == n_steps - 2) sh.l[nt & 1][row] = make_float2(l_run, m_ref);  // the partner finishes the tile
-        tmem_wait_st();
+        if (h == n_steps - 1) sh.l[nt & 1][row] = make_float2(l_run, m_ref);  // the other warpgroup finishes the tile
         if (!ok) break;
-        arrive(&sh.p_full[w]);
-      }
-      if (!ok) break;
-      // epilogue: O / l, one row per thread, by the warpgroup that had the last step (a tile without key
-      // steps: by the one whose turn it is)
-      const uint32_t g_last = g0 + n_steps - 1;
-      if (n_steps > 0 ? (g_last & 1) == w : (t & 1) == (int)w) {
-        const int tok = ti.x * 128 + row;
-        const bool valid_row = tok < p.N;
-        if (n_steps > 0 && !wait(&sh.pv_done[w], (g_last >> 1) & 1)) break;
-        tc_fence_after();
-        if (n_steps > 1) {
-          const float2 other = sh.l[nt & 1][row];
-          l_run += other.x * ex2(other.y - m_ref);
-        }
-        uint32_t v[128];
-        if (n_steps > 0) {
-#pragma unroll
-          for (int ch = 0; ch < 4; ++ch) tmem_ld32(o_addr + ch * 32, *reinterpret_cast<uint32_t(*)[32]>(&v[ch * 32]));
-          tmem_wait_ld();
-          arrive(&sh.o_free);
-        } else {
-#pragma unroll
-          for (int i = 0; i < 128; ++i) v[i] = 0u;
-        }
-        if (shared_tile) {  // O as it is, where the keys were, with its row sums: the parts are put together below
-          float4 *part = reinterpret_cast<float4 *>(smem + kOffK + row * 512);
-#pragma unroll
-          for (int i = 0; i < 32; ++i)
-            part[i ^ (row & 7)] = make_float4(__uint_as_float(v[4 * i]), __uint_as_float(v[4 * i + 1]), __uint_as_float(v[4 * i + 2]), __uint_as_float(v[4 * i + 3]));
-          sh.part_l[row] = make_float2(l_run, m_ref);
+        if (__builtin_expect(moved && h > 0, 0)) {
+          why = kRescale;
           break;
         }
-        const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
-        // A row per thread would touch 32 lines with every store (2700-5000 clocks for a tile, during which the
-        // partner runs out of work): 32 dims at a time go through shared memory, so that four lanes write 64
-        // bytes of a row.
-        unsigned char *out = smem + kOffOut + warp * kOutBytes;
-        uint16_t *tile_out = p.O + (long long)ti.w * p.sb + (long long)ti.z * p.sh + (long long)(ti.x * 128 + quarter * 32) * p.sn;
-        const int rows = p.N - (ti.x * 128 + (int)quarter * 32);  // of this warp that exist
+        tmem_wait_st();
+        arrive(&sh.p_full[b]);
+        masked = false;
+        if (__builtin_expect(advance(), 0)) break;
+      }
+      if (why != kNothing && ok) {
+        const uint32_t g = g0 + h, b = g & 1;
+        if (why == kNotThere) {
+          if (g > 0) wait(&sh.m_ready[b ^ 1][quarter], ((g - 1) >> 1) & 1);
+          wait(&sh.s_full[b], (g >> 1) & 1);
+        } else if (why == kMask) {
+          mask_keys(b, sh.entry[g & 3]);
+          masked = true;
+        } else {
+          // O changes scale: the products of the steps before have to be complete
+          if (wait(&sh.pv_done[b ^ 1], ((g - 1) >> 1) & 1)) {
+            tc_fence_after();
+            const uint64_t alpha2 = pack_f32x2(alpha, alpha);
+#pragma unroll 1
+            for (int ch = 0; ch < 8; ++ch) {
+              uint32_t v[16];
+              tmem_ld16(o_addr + ch * 16, v);
+              tmem_wait_ld();
 #pragma unroll
-        for (int ch = 0; ch < 4; ++ch) {
-#pragma unroll
-          for (int g4 = 0; g4 < 4; ++g4) {
-            float o[8];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) o[i] = __uint_as_float(v[ch * 32 + g4 * 8 + i]) * inv;
-            uint4 x;
-            x.x = pack_bf16x2(o[0], o[1]);
-            x.y = pack_bf16x2(o[2], o[3]);
-            x.z = pack_bf16x2(o[4], o[5]);
-            x.w = pack_bf16x2(o[6], o[7]);
-            *reinterpret_cast<uint4 *>(out + lane * 64 + ((g4 ^ (lane >> 1)) & 3) * 16) = x;
+              for (int i = 0; i < 16; i += 2) {
+                float lo, hi;
+                unpack_f32x2(mul_f32x2(pack_f32x2(__uint_as_float(v[i]), __uint_as_float(v[i + 1])), alpha2), lo, hi);
+                v[i] = __float_as_uint(lo);
+                v[i + 1] = __float_as_uint(hi);
+              }
+              tmem_st16(o_addr + ch * 16, v);
+            }
+            tmem_wait_st();
+            arrive(&sh.p_full[b]);
+            masked = false;
+            advance();
           }
-          __syncwarp();
+        }
+        const bool whole_step = why == kRescale;
+        why = kNothing;
+        if (!ok) break;
+        if (!whole_step) continue;
+      }
+      if (!ok) break;
+      if (Small && h >= n_steps) end_tile();
+      if (pending) {
+        // ===== the output of the tile before, O / l, one row per thread
+        pending = false;
+        const uint32_t q_buf = (nt - 1) & 1;
+        const int4 to = sh.written[q_buf][warp];
+        if (!wait(&sh.o_full[q_buf], ((nt - 1) >> 1) & 1)) break;
+        tc_fence_after();
+        const float2 own = sh.own[w][row], other = sh.l[q_buf][row];
+        const float l = other.x + own.x * ex2(own.y - other.y), m = other.y;
+        const float inv = l > 0.f ? 1.f / l : 0.f;
+        const uint64_t inv2 = pack_f32x2(inv, inv);
+        // Through the place of the tile's Q, a copy of 32 rows a warp; rows behind the last token are not written.
+        unsigned char *out = smem + kOffQ + q_buf * kTileBytes + quarter * (kTileBytes / 4);
+#pragma unroll 1
+        for (int half = 0; half < 2; ++half) {  // of the dims (short code: it is fetched anew for every tile)
+          uint32_t v[64];
+          tmem_ld32(o_addr + half * 64, *reinterpret_cast<uint32_t(*)[32]>(&v[0]));
+          tmem_ld32(o_addr + half * 64 + 32, *reinterpret_cast<uint32_t(*)[32]>(&v[32]));
+          tmem_wait_ld();
+          if (half == 1) arrive(&sh.o_free);
+          if (shared_tile) {  // O as it is, where the keys were, with its row sums: the parts are put together below
+            float4 *part = reinterpret_cast<float4 *>(smem + kOffK + row * 512) + half * 16;
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const int rr = i * 8 + (lane >> 2), g4 = lane & 3;
-            const uint4 x = *reinterpret_cast<const uint4 *>(out + rr * 64 + ((g4 ^ (rr >> 1)) & 3) * 16);
-            if (rr < rows) *reinterpret_cast<uint4 *>(tile_out + (long long)rr * p.sn + ch * 32 + g4 * 8) = x;
+            for (int i = 0; i < 16; ++i)
+              part[i ^ (row & 7)] = make_float4(__uint_as_float(v[4 * i]), __uint_as_float(v[4 * i + 1]), __uint_as_float(v[4 * i + 2]), __uint_as_float(v[4 * i + 3]));
+          } else {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {  // eight dims: 16 bytes of a row of 64 dims, swizzled as the copy expects them
+              uint32_t x[4];
+#pragma unroll
+              for (int k = 0; k < 4; ++k) {
+                float lo, hi;
+                unpack_f32x2(mul_f32x2(pack_f32x2(__uint_as_float(v[i * 8 + 2 * k]), __uint_as_float(v[i * 8 + 2 * k + 1])), inv2), lo, hi);
+                x[k] = pack_bf16x2(lo, hi);
+              }
+              *reinterpret_cast<uint4 *>(out + half * (kTileBytes / 8) + lane * 128 + ((i ^ (lane & 7)) << 4)) = make_uint4(x[0], x[1], x[2], x[3]);
+            }
+          }
+        }
+        if (shared_tile) {
+          sh.part_l[row] = make_float2(l, m);
+        } else {
+          async_proxy_fence();
+          __syncwarp();
+          const int tok = to.x * 128 + row;
+          if (lane == 0 && tok < p.N) tma_store_5d(&map_o, out, 0, tok, 0, to.z, to.w);
+          if (p.lse != nullptr && tok < p.N)
+            p.lse[(size_t)(to.w * p.H + to.z) * p.N + tok] = l > 0.f ? (m + log2f(l)) * 0.6931471805599453f : -INFINITY;
+          if (lane == 0) {
+            bulk_wait_read();
+            mbar_arrive(&sh.out_done[q_buf]);
           }
           __syncwarp();
         }
-        if (valid_row && p.lse != nullptr)
-          p.lse[(size_t)(ti.w * p.H + ti.z) * p.N + tok] = l_run > 0.f ? (m_ref + log2f(l_run)) * 0.6931471805599453f : -INFINITY;
       }
-      g0 += n_steps;
-      nt += n_steps > 0 ? 1 : 0;
+      if (h < n_steps) continue;
+      if (Small || !live) break;
+      end_tile();
+      next();
     }
     if (shared_tile) {
       // ===== the parts of a tile: each CTA puts together 128 / split rows, its own part of them with those that the other
       // CTAs copy here: a bulk copy each as soon as a CTA has its part, into Q's second buffer, which a launch of one tile per CTA
-      // does not use, and the output's place, which a shared tile does not.
+      // does not use, and a place for the third one.
       const int rows = 128 / p.split;
       async_proxy_fence();
       named_barrier_sync(1, 256);
@@ -1061,7 +1188,7 @@ bool make_map(CUtensorMap *m, const void *base, const Geom &g, int rows, int hal
 }
 
 template <int B>
-cudaError_t launch_bk(const Geom &g, const Workspace &w, const CUtensorMap &mq, const CUtensorMap &mk, const CUtensorMap &mv,
+cudaError_t launch_bk(const Geom &g, const Workspace &w, const CUtensorMap &mq, const CUtensorMap &mk, const CUtensorMap &mv, const CUtensorMap &mo,
                       AttnParams prm, const int32_t *kv_idx, const int32_t *kv_cnt, cudaStream_t s, int *launches) {
   cudaError_t e;
   const int n_heads = g.B * prm.hcount;
@@ -1083,9 +1210,10 @@ cudaError_t launch_bk(const Geom &g, const Workspace &w, const CUtensorMap &mq, 
   plan.hcount = prm.hcount;
   plan.ragged = (int)(g.N % g.block != 0);
   plan.status = prm.status;
+  prm.late = all_tiles > (size_t)kSms;  // by the tiles of all heads, not of this launch: a call that runs its heads in groups gives the same bits
   if (prm.n_tiles <= kSms) {
-    // Shared among CTAs as far as there are SMs, with at least two key steps each if all are listed.  By the tiles of all
-    // heads, not of this launch: a call that runs its heads in groups gives the same bits.
+    // Shared among CTAs as far as there are SMs, with at least two key steps each if all are listed (by the tiles of all
+    // heads as well).
     prm.split = 1;
     for (int n = kMaxSplit; n >= 2 && prm.split == 1; n /= 2)
       if (all_tiles * n <= kSplitCtas && prm.step_pitch >= 2 * n) prm.split = n;
@@ -1093,7 +1221,7 @@ cudaError_t launch_bk(const Geom &g, const Workspace &w, const CUtensorMap &mq, 
     if (e != cudaSuccess) return e;
     ++*launches;
     return launch_pdl(attn_tc_kernel<B, true>, dim3(prm.n_tiles * prm.split), dim3(kAttnThreads), kAttnSmem, s, Cluster{prm.split}, mq, mk,
-                      mv, prm, plan);
+                      mv, mo, prm, plan);
   }
   if (!prm.dense) {
     e = launch_pdl(attn_plan_kernel<B>, dim3((prm.n_tiles + kPlanWarps - 1) / kPlanWarps), dim3(32 * kPlanWarps), 0, s, plan, prm.n_tiles,
@@ -1112,7 +1240,7 @@ cudaError_t launch_bk(const Geom &g, const Workspace &w, const CUtensorMap &mq, 
   e = allow_shared_memory(attn_tc_kernel<B, false>, kAttnSmem);
   if (e != cudaSuccess) return e;
   ++*launches;
-  return launch_pdl(attn_tc_kernel<B, false>, dim3(kSms), dim3(kAttnThreads), kAttnSmem, s, mq, mk, mv, prm, plan);
+  return launch_pdl(attn_tc_kernel<B, false>, dim3(kSms), dim3(kAttnThreads), kAttnSmem, s, mq, mk, mv, mo, prm, plan);
 }
 
 }  // namespace
@@ -1124,8 +1252,8 @@ cudaError_t launch_attention(const Geom &g, const Workspace &w, const void *Q, c
     h0 = 0;
     hcount = g.H;
   }
-  CUtensorMap mq, mk, mv;
-  if (!make_map(&mq, Q, g, 128, 2) || !make_map(&mk, K, g, g.block, g.block == 128 ? 2 : 1) || !make_map(&mv, V, g, g.block, 2))
+  CUtensorMap mq, mk, mv, mo;
+  if (!make_map(&mq, Q, g, 128, 2) || !make_map(&mo, O, g, 32, 2) || !make_map(&mk, K, g, g.block, g.block == 128 ? 2 : 1) || !make_map(&mv, V, g, g.block, 2))
     return cudaErrorInvalidValue;
   AttnParams prm = {};
   prm.O = static_cast<uint16_t *>(O);
@@ -1147,8 +1275,8 @@ cudaError_t launch_attention(const Geom &g, const Workspace &w, const void *Q, c
   prm.test_skip_v = (g.flags & 0x80000000u) ? 1 : 0;
   prm.test_skip_parts = (g.flags & 0x40000000u) ? 1 : 0;
 #endif
-  return g.block == 64 ? launch_bk<64>(g, w, mq, mk, mv, prm, kv_idx, kv_cnt, s, launches)
-                       : launch_bk<128>(g, w, mq, mk, mv, prm, kv_idx, kv_cnt, s, launches);
+  return g.block == 64 ? launch_bk<64>(g, w, mq, mk, mv, mo, prm, kv_idx, kv_cnt, s, launches)
+                       : launch_bk<128>(g, w, mq, mk, mv, mo, prm, kv_idx, kv_cnt, s, launches);
 }
 
 }  // namespace heart

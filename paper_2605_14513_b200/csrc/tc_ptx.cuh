@@ -78,12 +78,13 @@ __device__ __forceinline__ bool mbar_test_wait(uint64_t *bar, uint32_t parity) {
   return ok != 0;
 }
 __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, volatile int *abort) {
-  if (mbar_test_wait(bar, parity)) return true;  // the usual case on the softmax side: already complete
-  const long long t0 = clock64();
+  // (the low word of the clock: a try returns long before it has gone round from the limit to zero)
+  static_assert(kWaitLimitCycles <= 4000000000LL, "the limit is compared in 32 bits");
+  const uint32_t t0 = clock();
   while (true) {
     if (mbar_try_wait(bar, parity)) return true;
     if (*abort) return false;
-    if (clock64() - t0 > kWaitLimitCycles) {
+    if ((uint32_t)clock() - t0 > (uint32_t)kWaitLimitCycles) {
       *abort = 1;
       return false;
     }
@@ -110,6 +111,16 @@ __device__ __forceinline__ void tma_load_5d(void *smem_dst, const CUtensorMap *m
       "r"(c3), "r"(c4)
       : "memory");
 }
+// A box from shared memory (the fence of its writers is behind them), as a group of its own; rows outside the tensor are left out.
+__device__ __forceinline__ void tma_store_5d(const CUtensorMap *map, const void *smem_src, int c0, int c1, int c2, int c3, int c4) {
+  asm volatile("cp.async.bulk.tensor.5d.global.shared::cta.bulk_group [%0, {%2, %3, %4, %5, %6}], [%1];" ::"l"(
+                   reinterpret_cast<uint64_t>(map)),
+               "r"(smem_u32(smem_src)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4)
+               : "memory");
+  asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+}
+// This thread's stores have read their shared memory.
+__device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 __device__ __forceinline__ void tma_prefetch_desc(const CUtensorMap *map) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
 }

@@ -1,0 +1,53 @@
+"""How the two softmax warpgroups share the steps of one tile after the other: tiles of 0 to 7 key steps in every order, so that either
+warpgroup has a tile's last step and writes the tile before, in layouts whose rows lie between rows of something else (the output
+leaves by bulk copies of 32 rows), and the same bits on every run and for every order of the tiles."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2605_14513_b200 import inputs
+
+from parity import check_attention, to_np
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("block", [64, 128])
+@pytest.mark.parametrize("H,N,most", [
+    (90, 128 * 7 - 31, 7),  # 630 tiles: four or five a CTA; the last rows of a head fill no copy
+    (400, 128 + 33, 2),     # tiles of one and two steps only: the roles change with every tile
+    (149, 120, 1),          # one tile more than CTAs
+])
+def test_turns(oracle, block, H, N, most):
+    from paper_2605_14513_b200 import heart
+
+    rs = np.random.RandomState(block + H + N)
+    g = torch.Generator("cuda").manual_seed(H * N)
+    Q, K, V = (torch.randn((1, N, H, 128), generator=g, device="cuda").to(torch.bfloat16).permute(0, 2, 1, 3) for _ in range(3))
+    nb = heart.n_blocks(N, block)
+    idx, cnt = np.full((H, nb, nb), -1, np.int32), np.zeros((H, nb), np.int32)
+    for r in range(H):
+        for I in range(nb):
+            sel = rs.permutation(nb)[: rs.randint(0, min(nb, most * 128 // block) + 1)]
+            cnt[r, I] = len(sel)
+            idx[r, I, : len(sel)] = sel
+    lists = torch.from_numpy(idx).cuda(), torch.from_numpy(cnt).cuda()
+    cfg = heart.config_for(Q, block)
+    ws = heart.new_workspace(cfg)
+    ref, lse_ref = oracle.block_sparse_attn(*(inputs.bits(t) for t in (Q, K, V)), block, idx, cnt, want_lse=True)
+    first = None
+    for _ in range(3):
+        whole = torch.full((1, N + 2, H, 128), 7.0, device="cuda", dtype=torch.bfloat16)  # a row of something else on both sides
+        O = whole[:, 1:-1].permute(0, 2, 1, 3)
+        lse = torch.full((H, N), float("nan"), device="cuda")
+        heart.heart_block_sparse_attn(cfg, Q, K, V, *lists, O, ws, lse=lse)
+        assert heart.heart_get_status(ws) == 0
+        assert (whole[:, 0] == 7.0).all() and (whole[:, -1] == 7.0).all()
+        if first is None:
+            first = O.clone(), lse
+            check_attention(to_np(O.float()).astype(np.float64).reshape(H, N, 128), ref)
+            got, fin = to_np(lse), np.isfinite(lse_ref)
+            assert np.array_equal(np.isneginf(got), np.isneginf(lse_ref))
+            # fp32 accumulation of bf16-rounded weights (2^-9 relative each) in the sum behind the logarithm
+            assert np.allclose(got[fin], lse_ref[fin], rtol=0, atol=2.0 ** -8)
+        assert torch.equal(O.contiguous().view(torch.int16), first[0].contiguous().view(torch.int16)) and torch.equal(lse, first[1])
