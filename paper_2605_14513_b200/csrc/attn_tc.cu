@@ -365,6 +365,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
   extern __shared__ __align__(1024) unsigned char smem[];
   AttnShared &sh = *reinterpret_cast<AttnShared *>(smem + kOffBar);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const bool dense = B == 128 && p.dense;  // (dense calls come with blocks of 128)
   volatile int *abort = &sh.abort;
 
   // ------------------------------------------------------------------ set-up
@@ -438,11 +439,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     return p.steps + ((size_t)(ti.w * p.H + ti.z) * p.n_tiles_per_head + ti.x) * p.step_pitch;
   };
   auto step_entry = [&](const uint32_t *steps, int h) -> uint32_t {
-    if (!p.dense) return Small ? steps[h] : __ldcg(&steps[h]);
-    if (Small) h += first_step(p.nb, rank);
-    if (B == 128) return h;
-    const uint32_t ragged = (p.N & 63) ? p.nb - 1 : 0x3ff + 1, a = 2 * h, b = 2 * h + 1;
-    return (a | 3u << 10 | (a == ragged ? 1u << 12 : 0u)) | (b < (uint32_t)p.nb ? b | 3u << 10 | (b == ragged ? 1u << 12 : 0u) : a) << 16;
+    if (!dense) return Small ? steps[h] : __ldcg(&steps[h]);
+    return Small ? h + first_step(p.nb, rank) : h;
   };
   // Waits of a whole warp; ok turns false when one runs out or the CTA aborts.  The usual case is a barrier
   // that is complete already.
@@ -568,7 +566,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
         uint32_t e = 0;  // its next key step, fetched ahead of time
         if (n < p.n_tiles) {
           uint4 word;
-          if (p.dense) {
+          if (dense) {
             word.y = n / p.n_tiles_per_head;
             word.x = (n - word.y * p.n_tiles_per_head) | (uint32_t)p.nb << 16;
             word.z = step_entry(nullptr, 0);
@@ -588,8 +586,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
         if (ti.w < 0) break;
         const int n_steps = n_steps_of(ti.y);
         const uint32_t *steps = steps_of(ti);
-        int n_next = p.dense ? n + gridDim.x : 0;
-        if (n_steps == 0 && !p.dense) n_next = gridDim.x + atomicAdd(p.counter, 1);
+        int n_next = dense ? n + gridDim.x : 0;
+        if (n_steps == 0 && !dense) n_next = gridDim.x + atomicAdd(p.counter, 1);
 #pragma unroll 1
         for (int h = 0; h < n_steps; ++h, ++g) {
           const uint32_t e_next = h + 1 < n_steps ? step_entry(steps, h + 1) : 0u;
@@ -605,7 +603,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
           }
           // The next tile is drawn at the last moment that hides the trip to memory: drawn with the first step, a
           // CTA on a long tile already owned another one while others ran out (2 x 12 x 2465: 56.9 us against 55.2).
-          if (h == n_steps - 1 && !p.dense) n_next = gridDim.x + atomicAdd(p.counter, 1);
+          if (h == n_steps - 1 && !dense) n_next = gridDim.x + atomicAdd(p.counter, 1);
           e = e_next;
         }
         if (!ok) break;
@@ -728,7 +726,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
       pdl_wait();
       if (warp == 0) {
         uint32_t U = p.nb;
-        if (!p.dense) {
+        if (!dense) {
           const uint4 word = plan_tile<B>(plan, blockIdx.x / p.split, lane, sh.sets, [&](int) { return sh.steps; });
           U = word.x >> 16;
         }
@@ -1245,12 +1243,19 @@ cudaError_t launch_bk(const Geom &g, const Workspace &w, const CUtensorMap &mq, 
 
 }  // namespace
 
-cudaError_t launch_attention(const Geom &g, const Workspace &w, const void *Q, const void *K, const void *V,
+cudaError_t launch_attention(const Geom &given, const Workspace &w, const void *Q, const void *K, const void *V,
                              const int32_t *kv_idx, const int32_t *kv_cnt, bool dense, void *O, float *lse,
                              cudaStream_t s, int *launches, int h0, int hcount) {
   if (hcount <= 0) {
     h0 = 0;
-    hcount = g.H;
+    hcount = given.H;
+  }
+  // A key step is 128 tokens either way: dense calls take blocks of 128, with a box where those of 64 take two, and half the
+  // tests in a step (12 x 33k 5757 us with those of 64, 5665 so; the same bits).
+  Geom g = given;
+  if (dense) {
+    g.block = 128;
+    g.nb = (g.N + 127) / 128;
   }
   CUtensorMap mq, mk, mv, mo;
   if (!make_map(&mq, Q, g, 128, 2) || !make_map(&mo, O, g, 32, 2) || !make_map(&mk, K, g, g.block, g.block == 128 ? 2 : 1) || !make_map(&mv, V, g, g.block, 2))

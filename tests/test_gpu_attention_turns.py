@@ -51,3 +51,21 @@ def test_turns(oracle, block, H, N, most):
             # fp32 accumulation of bf16-rounded weights (2^-9 relative each) in the sum behind the logarithm
             assert np.allclose(got[fin], lse_ref[fin], rtol=0, atol=2.0 ** -8)
         assert torch.equal(O.contiguous().view(torch.int16), first[0].contiguous().view(torch.int16)) and torch.equal(lse, first[1])
+
+
+@pytest.mark.parametrize("H,N", [(2, 1), (1, 130), (2, 2045), (60, 700)])  # shared tiles, one a CTA, several; ragged blocks of either size
+def test_dense_calls_do_not_depend_on_the_block(H, N):
+    from paper_2605_14513_b200 import heart
+
+    g = torch.Generator("cuda").manual_seed(H * N)
+    Q, K, V = (torch.randn((1, H, N, 128), generator=g, device="cuda").to(torch.bfloat16) for _ in range(3))
+    outs = []
+    for block in (64, 128):
+        cfg = heart.make_config(1, H, N, block, flags=heart.FORCE_DENSE)
+        ws, O, lse = heart.new_workspace(cfg), torch.full_like(Q, float("nan")), torch.full((H, N), float("nan"), device="cuda")
+        heart.heart_block_sparse_attn(cfg, Q, K, V, None, None, O, ws, lse=lse)
+        assert heart.heart_get_status(ws) == 0
+        outs.append((O, lse))
+    assert torch.equal(outs[0][0].view(torch.int16), outs[1][0].view(torch.int16)) and torch.equal(outs[0][1], outs[1][1])
+    ref = torch.nn.functional.scaled_dot_product_attention(Q.double(), K.double(), V.double())
+    check_attention(to_np(outs[0][0].float()).astype(np.float64).reshape(H, N, 128), to_np(ref).reshape(H, N, 128))
