@@ -48,7 +48,7 @@ struct Workspace {
   double *bmean;      // [2][R][nb][D]  per-block (pooled) means of Q (0) and K (1)
   double *psum;       // [2][R][nchunks][D]  per-CTA partial token sums
   double *mean;       // [2][R][D]      token means of the current step
-  uint8_t *pre;       // [R]            head-wise decision before the gate
+  uint8_t *pre;       // [R]            head-wise decision before the gate (bit 1: the head had an anchor)
   uint8_t *refresh;   // [R]            final decision of the current step
   double *drift;      // [R]
   void *plan;         // of an attention call, which besides it touches the status words only (a mask prediction for
@@ -107,6 +107,7 @@ struct DecideArgs {
   double *drift_out;
   uint8_t *refresh_out;
   int *ticket;  // zero between launches (the layer gate's counter, or one a head)
+  bool gate_later;  // the kernel behind the drift applies the layer gate: pre_ws gets the head-wise decision | had an anchor << 1
 };
 
 #ifdef __CUDACC__

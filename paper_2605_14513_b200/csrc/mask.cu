@@ -537,7 +537,8 @@ struct RowArgs {
   int R, nb;
   double scale;
   unsigned flags;
-  const uint8_t *refresh;  // without DECIDE
+  const uint8_t *refresh;  // kBefore
+  const double *mean;      // kGateHere
   uint32_t *mask_bits;
   int32_t *kv_idx, *kv_cnt;
   int idx_stride, W;
@@ -548,8 +549,11 @@ struct RowArgs {
 constexpr int kRowsKernelThreads = 256, kRowsKernelPitch = kD + 4;
 __host__ __device__ inline int rows_kernel_doubles(int nj, int nb) { return (8 + (nb + 7) / 8 * 8) * kRowsKernelPitch + 2 * 8 * nj * 32; }
 
-template <int NJ, bool DECIDE>
+// Where the decisions come from: mean_drift_kernel, this kernel, mean_drift_kernel with the layer gate applied here.
+enum Decided { kBefore, kHere, kGateHere };
+template <int NJ, Decided HOW>
 __global__ void __launch_bounds__(kRowsKernelThreads) mask_rows_kernel(const RowArgs a) {
+  constexpr bool DECIDE = HOW == kHere;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int nb = a.nb, keys = (nb + 7) / 8 * 8, r = blockIdx.y, I0 = blockIdx.x * 8;
   double *tile = reinterpret_cast<double *>(smem_raw);  // 8 query rows, then the key rows
@@ -569,7 +573,31 @@ __global__ void __launch_bounds__(kRowsKernelThreads) mask_rows_kernel(const Row
   }
   pdl_wait();
   pdl_launch_dependents();
-  if (!DECIDE && a.refresh[r] == 0) return;  // (decided by mean_drift_kernel, which has the layer gate)
+  if (!DECIDE) {
+    // Decided by mean_drift_kernel.  With the layer gate on, every CTA applies it to its head, from the head-wise decisions of the
+    // batch entry, and the first one of a head moves the anchor: by the last CTA of mean_drift_kernel that was a chain of four
+    // trips to memory in front of this kernel (2 x 12 heads x 2465 tokens: that kernel 8.1 us, 4.2 without; the step 67.2 and 64.5).
+    bool rf = HOW == kBefore && a.refresh[r] != 0;
+    if (HOW == kGateHere) {
+      const int H = a.decide.H, b0 = r / H * H;
+      int n = 0;
+      for (int i = tid; i - tid < H; i += kRowsKernelThreads) n += __syncthreads_count(i < H && (__ldcg(&a.decide.pre_ws[b0 + i]) & 1));
+      const int pre = __ldcg(&a.decide.pre_ws[r]);
+      const double f = (double)n / (double)H;
+      rf = (pre & 1) != 0;
+      if (f < a.decide.gate_lo) rf = rf && !(pre & 2);
+      else if (f > a.decide.gate_hi) rf = true;
+      if (blockIdx.x == 0) {
+        if (tid == 0) {
+          a.decide.refresh_ws[r] = rf;
+          if (a.decide.refresh_out) a.decide.refresh_out[r] = rf;
+          if (rf) a.decide.has_anchor[r] = 1;
+        }
+        if (rf) ((tid >> 7) ? a.decide.anchor_k : a.decide.anchor_q)[(size_t)r * kD + (tid & (kD - 1))] = __ldcg(&a.mean[((size_t)(tid >> 7) * a.R + r) * kD + (tid & (kD - 1))]);
+      }
+    }
+    if (!rf) return;
+  }
   const double *bq = a.bmean + (size_t)r * nb * kD, *bk = a.bmean + ((size_t)a.R + r) * nb * kD;
 #pragma unroll 8
   for (int e = tid; e < (8 + keys) * (kD / 2); e += kRowsKernelThreads) {
@@ -706,12 +734,12 @@ static bool rows_kernel_decides(const Geom &g) {
   return !gate_on && g.R * ((g.nb + 7) / 8) <= kStatusHeadTickets && g.nb <= 4 * kRangeLoads && g.R * ((g.N + 127) / 128) <= 148;
 }
 
-template <int NJ, bool DECIDE>
+template <int NJ, Decided HOW>
 static cudaError_t launch_rows(const Geom &g, const RowArgs &a, cudaStream_t s) {
   const int smem = (int)sizeof(double) * rows_kernel_doubles(NJ, g.nb);
-  cudaError_t e = allow_shared_memory(mask_rows_kernel<NJ, DECIDE>, (int)sizeof(double) * rows_kernel_doubles(NJ, NJ * 32));
+  cudaError_t e = allow_shared_memory(mask_rows_kernel<NJ, HOW>, (int)sizeof(double) * rows_kernel_doubles(NJ, NJ * 32));
   if (e != cudaSuccess) return e;
-  return launch_pdl(mask_rows_kernel<NJ, DECIDE>, dim3((g.nb + 7) / 8, g.R), dim3(kRowsKernelThreads), (size_t)smem, s, a);
+  return launch_pdl(mask_rows_kernel<NJ, HOW>, dim3((g.nb + 7) / 8, g.R), dim3(kRowsKernelThreads), (size_t)smem, s, a);
 }
 
 static RowArgs row_args(const Geom &g, const Workspace &w, const double *tau, heart_state st) {
@@ -735,18 +763,22 @@ cudaError_t launch_decide_and_predict(const Geom &g, const Workspace &w, const D
   RowArgs a = row_args(g, w, tau, st);
   ++*launches;
   if (!rows_kernel_decides(g)) {
-    cudaError_t e = launch_decide(g, w, decide, s);
+    a.decide = decide;
+    a.decide.gate_later = g.gate_lo > 0.0 || g.gate_hi < 1.0;
+    a.mean = w.mean;
+    a.refresh = w.refresh;
+    cudaError_t e = launch_decide(g, w, a.decide, s);
     if (e != cudaSuccess) return e;
     ++*launches;
-    a.refresh = w.refresh;
-    return g.nb <= 64 ? launch_rows<2, false>(g, a, s) : launch_rows<4, false>(g, a, s);
+    if (a.decide.gate_later) return g.nb <= 64 ? launch_rows<2, kGateHere>(g, a, s) : launch_rows<4, kGateHere>(g, a, s);
+    return g.nb <= 64 ? launch_rows<2, kBefore>(g, a, s) : launch_rows<4, kBefore>(g, a, s);
   }
   a.psum = w.psum;
   a.N = g.N;
   a.nchunks = g.nchunks;
   a.decide = decide;
   a.decide.ticket = w.status + kStatusHeadTicketWord;
-  return launch_rows<2, true>(g, a, s);
+  return launch_rows<2, kHere>(g, a, s);
 }
 
 cudaError_t launch_predict_mask(const Geom &g, const Workspace &w, const double *tau,

@@ -158,7 +158,7 @@ __device__ void apply_gate(int R, const double *mean, const DecideArgs &a, int *
 //   drift[r]      = sum_d |anchor_q - mean_q| + sum_d |anchor_k - mean_k|   (fixed-shape reductions)
 // and the head-wise rule of Algorithm 1.  With the layer gate off (the usual case) that is the final
 // decision and the CTA moves its own anchor; with the gate on, the CTA that finishes last (a ticket
-// counter) applies the gate for every batch entry.
+// counter) applies the gate for every batch entry, or the row kernel behind this one does (gate_later).
 __global__ void __launch_bounds__(1024) mean_drift_kernel(const double *__restrict__ psum, int R, int N,
                                                           int nchunks, double *__restrict__ mean,
                                                           const DecideArgs a) {
@@ -206,6 +206,9 @@ __global__ void __launch_bounds__(1024) mean_drift_kernel(const double *__restri
       if (a.refresh_out) a.refresh_out[r] = rf;
       if (rf) a.has_anchor[r] = 1;
       sh_rf = rf;
+    } else if (a.gate_later) {
+      a.pre_ws[r] = (rf ? 1 : 0) | (had ? 2 : 0);
+      last = 0;
     } else {
       a.pre_ws[r] = rf;
       __threadfence();
@@ -272,6 +275,7 @@ DecideArgs decide_args(const Geom &g, const Workspace &w, const double *delta, h
   a.drift_out = drift_out;
   a.refresh_out = refresh_out;
   a.ticket = w.status + kStatusTicketWord;
+  a.gate_later = false;
   return a;
 }
 
@@ -282,7 +286,7 @@ cudaError_t launch_decide(const Geom &g, const Workspace &w, const double *delta
 }
 cudaError_t launch_decide(const Geom &g, const Workspace &w, const DecideArgs &a, cudaStream_t s) {
   const bool gate_on = g.gate_lo > 0.0 || g.gate_hi < 1.0;
-  return launch_pdl(mean_drift_kernel, dim3(g.R), dim3(1024), gate_on ? gate_shared_bytes(g.B, g.H) : 0, s, (const double *)w.psum, g.R, g.N,
+  return launch_pdl(mean_drift_kernel, dim3(g.R), dim3(1024), gate_on && !a.gate_later ? gate_shared_bytes(g.B, g.H) : 0, s, (const double *)w.psum, g.R, g.N,
                     g.nchunks, w.mean, a);
 }
 
