@@ -234,31 +234,31 @@ __global__ void __launch_bounds__(kThreadsAd, 1)
 // One CTA per (query block I, head r), fp64: the (max, sum) pairs of the block's groups become
 // scores[r][I][J] = ln(importance(I, J)) (-inf for importance 0), which the top-p kernel reads like
 // pooled scores.  A query block without a full group gets equal scores (uniform importance).
-// One warp per group of the block (at most 8): row maximum and row sum by shuffles, the weights of
+// One warp per group of the block (8, or 4 of a 64-token block): row maximum and row sum by shuffles, the weights of
 // the lane's key blocks stay in registers in between; they meet in shared memory, where a thread adds up
 // the groups of a key block one after the other.  Every reduction has a fixed shape: bit-reproducible.
-template <int NJ>  // NJ * 32 >= n_b
-__global__ void __launch_bounds__(256, 2) antidiag_reduce_kernel(const float2 *__restrict__ pairs, int Ns, int nb,
-                                                                 int g, int pitch, const uint8_t *__restrict__ refresh,
+template <int NJ, int G>  // NJ * 32 >= n_b, G groups per block
+__global__ void __launch_bounds__(32 * G, 16 / G) antidiag_reduce_kernel(const float2 *__restrict__ pairs, int Ns, int nb,
+                                                                 int pitch, const uint8_t *__restrict__ refresh,
                                                                  double *__restrict__ scores) {
   const int I = blockIdx.x, r = blockIdx.y;
   pdl_wait();
   pdl_launch_dependents();
   if (refresh != nullptr && refresh[r] == 0) return;
-  extern __shared__ __align__(16) double wgt[];  // [g][NJ * 32]
+  extern __shared__ __align__(16) double wgt[];  // [G][NJ * 32]
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int a0 = I * g, a1 = min(a0 + g, Ns);
-  const int nJ = (Ns + g - 1) / g;  // key blocks that hold at least one full group
+  const int a0 = I * G, a1 = min(a0 + G, Ns);
+  const int nJ = (Ns + G - 1) / G;  // key blocks that hold at least one full group
   double *srow = scores + ((size_t)r * nb + I) * pitch;
   if (a1 <= a0) {
-    for (int J = tid; J < pitch; J += 256) srow[J] = 0.0;
+    for (int J = tid; J < pitch; J += 32 * G) srow[J] = 0.0;
     return;
   }
   constexpr int kPerLane = NJ;
   const double ln2 = 0.6931471805599453;
   double e[kPerLane];
-  const int a = a0 + warp;  // this warp's group (g <= 8 warps have one)
-  if (warp < g && a < a1) {
+  const int a = a0 + warp;  // this warp's group
+  if (a < a1) {
     const float2 *prow = pairs + ((size_t)r * Ns + a) * nb;
     float mxf = -INFINITY;
 #pragma unroll
@@ -285,7 +285,7 @@ __global__ void __launch_bounds__(256, 2) antidiag_reduce_kernel(const float2 *_
   }
   __syncthreads();
   const double inv = 1.0 / (double)(a1 - a0);
-  for (int J = tid; J < pitch; J += 256) {
+  for (int J = tid; J < pitch; J += 32 * G) {
     double w = 0.0;
     for (int n = 0; n < a1 - a0; ++n) w += wgt[n * kPerLane * 32 + J];  // groups in ascending order: a fixed summation order
     w = (J < nJ) ? w * inv : 0.0;
@@ -315,14 +315,21 @@ cudaError_t launch_scores(const CUtensorMap &mq, const CUtensorMap &mk, const Ad
   return launch_pdl(antidiag_scores_kernel<G>, dim3(2 * pairs), dim3(kThreadsAd), smem, s, Cluster{2}, mq, mk, prm);
 }
 
-template <int NJ>
-cudaError_t launch_reduce(const Geom &g, const float2 *pairs, int Ns, int grp, int pitch, const uint8_t *refresh, double *scores,
-                          cudaStream_t s) {
-  const int smem = grp * NJ * 32 * (int)sizeof(double);
-  cudaError_t e = allow_shared_memory(antidiag_reduce_kernel<NJ>, 8 * NJ * 32 * (int)sizeof(double));
+template <int NJ, int G>
+cudaError_t launch_reduce(const Geom &g, const float2 *pairs, int Ns, int pitch, const uint8_t *refresh, double *scores, cudaStream_t s) {
+  constexpr int smem = G * NJ * 32 * (int)sizeof(double);
+  cudaError_t e = allow_shared_memory(antidiag_reduce_kernel<NJ, G>, smem);
   if (e != cudaSuccess) return e;
-  return launch_pdl(antidiag_reduce_kernel<NJ>, dim3(g.nb, g.R), dim3(256), (size_t)smem, s, pairs, Ns, g.nb, grp, pitch, refresh,
-                    scores);
+  return launch_pdl(antidiag_reduce_kernel<NJ, G>, dim3(g.nb, g.R), dim3(32 * G), (size_t)smem, s, pairs, Ns, g.nb, pitch, refresh, scores);
+}
+// The instance for the words of a row, an even number of them.  (With one for up to 8, 16, 24 or 32, and eight warps for the four groups
+// of a 64-token block, whole calls, us, then / now: 12 heads x 512 blocks of 64 257.6 / 232.2, 40 x 200 174.7 / 165.7, 4 x 591 of 128
+// 337.5 / 313.6.)
+template <int G, int NJ = 2>
+cudaError_t launch_reduce_of(int nj, const Geom &g, const float2 *pairs, int Ns, int pitch, const uint8_t *refresh, double *scores, cudaStream_t s) {
+  if constexpr (NJ < HEART_MAX_BLOCKS / 32)
+    if (nj > NJ) return launch_reduce_of<G, NJ + 2>(nj, g, pairs, Ns, pitch, refresh, scores, s);
+  return launch_reduce<NJ, G>(g, pairs, Ns, pitch, refresh, scores, s);
 }
 
 }  // namespace
@@ -354,10 +361,8 @@ cudaError_t launch_antidiag_scores(const Geom &g, const Workspace &w, const void
   }
   const float2 *pairs = reinterpret_cast<const float2 *>(w.pairs);
   const int nj = (g.nb + 31) / 32;
-  cudaError_t e = nj <= 8    ? launch_reduce<8>(g, pairs, Ns, grp, pitch, refresh, w.scores, s)
-                  : nj <= 16 ? launch_reduce<16>(g, pairs, Ns, grp, pitch, refresh, w.scores, s)
-                  : nj <= 24 ? launch_reduce<24>(g, pairs, Ns, grp, pitch, refresh, w.scores, s)
-                             : launch_reduce<32>(g, pairs, Ns, grp, pitch, refresh, w.scores, s);
+  cudaError_t e = grp == 4 ? launch_reduce_of<4>(nj, g, pairs, Ns, pitch, refresh, w.scores, s)
+                           : launch_reduce_of<8>(nj, g, pairs, Ns, pitch, refresh, w.scores, s);
   ++*launches;
   return e;
 }

@@ -31,12 +31,12 @@ constexpr int kSmallScoreTiles = 148;  // 64 x 64 score tiles of a launch up to 
 // 108 with two; from 513 blocks on two are no slower anywhere (whole call, tau 0.97: 40 x 591 blocks 268 against 274 us, 16 x 735
 // 161 against 167); short rows gain nothing and pay for the CTAs.
 template <int NJ>
-constexpr int kRowsPerCta = NJ >= 24 ? 2 : 8;
-// CTAs that an SM has to hold, which leaves 96 registers a thread for 24 words and more, 80 for 16, 64 for 8, 48 for 2.  At 32
+constexpr int kRowsPerCta = NJ > 16 ? 2 : 8;
+// CTAs that an SM has to hold, which leaves 96 registers a thread for more than 16 words, 80 for 12 and more, 64 for 4, 48 for 2.  At 32
 // words that spills a little and pays with many rows (24 heads x 929 blocks 280 us, 285 with 128 registers; one head 37 and 35).
 // At 24 and 16 words another CTA would not pay for its spills (24 heads x 700 blocks 164 us with 12, 161 with 10).
 template <int NJ>
-constexpr int kCtasPerSm = NJ >= 24 ? 10 : NJ >= 16 ? 3 : NJ >= 8 ? 4 : 5;
+constexpr int kCtasPerSm = NJ > 16 ? 10 : NJ >= 12 ? 3 : NJ >= 4 ? 4 : 5;
 constexpr int kMaxCand = 64;    // candidates the direct threshold evaluation takes
 constexpr float kMassBand = 1.5e-5f;  // of z: cuts whose mass is closer to tau * z are decided in fp64
 // Blocks are ranked by their weight, lowest index first among equals.  Weights exp(s - max) round to the same double
@@ -680,6 +680,16 @@ static cudaError_t launch_nj(const Geom &g, const Workspace &w, const double *ta
                     expect_sig);
 }
 
+// The instance for the words of a row, an even number of them.  (With one for up to 2, 8, 16, 24 or 32, whole calls, us, then / now:
+// 9 heads x 100 blocks 11.1 / 9.4, 12 x 300 34.8 / 32.6, 24 x 520 123.0 / 113.2, 24 x 820 267.2 / 248.4, 24 x 929 335.4 / 327.1.)
+template <int NJ = 2>
+static cudaError_t launch_top_p_of(int nj, const Geom &g, const Workspace &w, const double *tau, const uint8_t *refresh, heart_state st,
+                                   int pitch, cudaStream_t s, unsigned long long expect_sig) {
+  if constexpr (NJ < HEART_MAX_BLOCKS / 32)
+    if (nj > NJ) return launch_top_p_of<NJ + 2>(nj, g, w, tau, refresh, st, pitch, s, expect_sig);
+  return launch_nj<NJ>(g, w, tau, refresh, st, pitch, s, expect_sig);
+}
+
 template <int WT, int TD, int STAGES>
 static cudaError_t launch_scores(const Geom &g, const Workspace &w, const uint8_t *refresh, cudaStream_t s,
                                  unsigned long long expect_sig) {
@@ -704,11 +714,7 @@ cudaError_t launch_top_p(const Geom &g, const Workspace &w, const double *tau, c
                          heart_state st, cudaStream_t s, int *launches, unsigned long long expect_sig) {
   ++*launches;
   const int nj = (g.nb + 31) / 32, pitch = nj * 32;
-  if (nj <= 2) return launch_nj<2>(g, w, tau, refresh, st, pitch, s, expect_sig);
-  if (nj <= 8) return launch_nj<8>(g, w, tau, refresh, st, pitch, s, expect_sig);
-  if (nj <= 16) return launch_nj<16>(g, w, tau, refresh, st, pitch, s, expect_sig);
-  if (nj <= 24) return launch_nj<24>(g, w, tau, refresh, st, pitch, s, expect_sig);
-  return launch_nj<32>(g, w, tau, refresh, st, pitch, s, expect_sig);
+  return launch_top_p_of(nj, g, w, tau, refresh, st, pitch, s, expect_sig);
 }
 
 // About one wave of CTAs, by their shared memory: three an SM at 32 blocks, two at 64, one at 128 (up to six at 16 and fewer, of which
