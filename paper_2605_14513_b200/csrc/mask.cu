@@ -25,7 +25,6 @@ namespace heart {
 using tc::ex2;
 using tc::mma_f64;
 
-constexpr int kSmallScoreTiles = 148;  // 64 x 64 score tiles of a launch up to which 32 x 32 ones are used
 // Rows (warps) per CTA of the top-p kernel.  A row that needs the fp64 search takes many times longer than the
 // others and holds its CTA: 22296 rows of 929 take 121 us with eight rows a CTA,
 // 108 with two; from 513 blocks on two are no slower anywhere (whole call, tau 0.97: 40 x 591 blocks 268 against 274 us, 16 x 735
@@ -704,9 +703,15 @@ static cudaError_t launch_scores(const Geom &g, const Workspace &w, const uint8_
 cudaError_t launch_pooled_scores(const Geom &g, const Workspace &w, const uint8_t *refresh, cudaStream_t s,
                                  int *launches, unsigned long long expect_sig) {
   ++*launches;
-  // Few tiles: small ones with all dims loaded at once, so that the work spreads over the SMs.
-  const long long tiles64 = (long long)((g.nb + 63) / 64) * ((g.nb + 63) / 64) * g.R;
-  if (tiles64 <= kSmallScoreTiles) return launch_scores<16, 128, 1>(g, w, refresh, s, expect_sig);
+  // Tiles of 64 x 64 scores read their operands half as often as tiles of 32 x 32, which leave less of the chip idle: up to half a wave
+  // of large ones (a tile an SM) small ones with all dims loaded at once, up to a whole one small ones in three stages,
+  // beyond that these where their waves, at 0.35 of a large one's time, are shorter: few waves, or much padding.  Whole calls timed
+  // both ways on 354 shapes (129 to 1000 blocks, 1 to 40 heads), against the first kind up to a wave and large ones beyond: 0.978 in
+  // the mean, largest 1.037 (520 x 1 head); us, before / now: 24 heads x 130 blocks 21.6 / 17.4, 30 x 200 36.4 / 32.3, 3 x 600 39.1 / 36.2.
+  const long long n64 = (g.nb + 63) / 64, n32 = (g.nb + 31) / 32, tiles64 = n64 * n64 * g.R, tiles32 = n32 * n32 * g.R;
+  auto waves = [](long long tiles) { return (tiles + 147) / 148; };
+  if (tiles64 <= 74) return launch_scores<16, 128, 1>(g, w, refresh, s, expect_sig);
+  if (tiles64 <= 148 || 35 * waves(tiles32) < 100 * waves(tiles64)) return launch_scores<16, 32, 3>(g, w, refresh, s, expect_sig);
   return launch_scores<32, 16, 3>(g, w, refresh, s, expect_sig);
 }
 
