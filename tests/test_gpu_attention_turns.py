@@ -17,6 +17,8 @@ pytestmark = pytest.mark.gpu
     (90, 128 * 7 - 31, 7),  # 630 tiles: four or five a CTA; the last rows of a head fill no copy
     (400, 128 + 33, 2),     # tiles of one and two steps only: the roles change with every tile
     (149, 120, 1),          # one tile more than CTAs
+    (2, 4500, 36),          # 72 tiles, a pair of CTAs each
+    (24, 340, 3),           # 72 tiles of few steps: a CTA each
 ])
 def test_turns(oracle, block, H, N, most):
     from paper_2605_14513_b200 import heart
@@ -53,7 +55,7 @@ def test_turns(oracle, block, H, N, most):
         assert torch.equal(O.contiguous().view(torch.int16), first[0].contiguous().view(torch.int16)) and torch.equal(lse, first[1])
 
 
-@pytest.mark.parametrize("H,N", [(2, 1), (1, 130), (2, 2045), (60, 700)])  # shared tiles, one a CTA, several; ragged blocks of either size
+@pytest.mark.parametrize("H,N", [(2, 1), (1, 130), (2, 2045), (60, 700), (1, 9000), (1, 9473)])  # shared tiles (71: pairs; 75: a CTA each), several; ragged blocks
 def test_dense_calls_do_not_depend_on_the_block(H, N):
     from paper_2605_14513_b200 import heart
 
