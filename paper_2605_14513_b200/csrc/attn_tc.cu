@@ -1216,12 +1216,12 @@ cudaError_t launch_bk(const Geom &g, const Workspace &w, const CUtensorMap &mq, 
     // and the wait for the others': it pays from eight key steps a tile on, and lists have half of all or less.  us with a
     // CTA a tile and with two: 48 tiles of at most six steps, of which lists name 2 to 4, 9.7 and 10.9; 72 tiles, 36 steps,
     // whole steps of 2 x 4500 tokens 36.1 and 29.9, 24 steps dense 27.3 and 21.4; 1 head x 9000 tokens 29.5 and 21.0, dense 61.1 and 38.6.
-    // (72 tiles whose lists name one or two of 48 blocks: 8.0 and 9.9.)
+    // (With a third of the blocks listed, 22 steps are 23.9 and 24.3; 72 tiles whose lists name one or two of 72 blocks 8.0 and 9.9.)
     const int steps = prm.step_pitch;  // of a tile whose blocks list all
     prm.split = 1;
     if (all_tiles * 4 <= kSplitCtas && steps >= 8) prm.split = 4;
     else if (all_tiles * 2 <= kSplitCtas && steps >= (prm.dense ? 4 : 8)) prm.split = 2;
-    else if (all_tiles * 2 <= kSms && steps >= (prm.dense ? 8 : 20)) prm.split = 2;
+    else if (all_tiles * 2 <= kSms && steps >= (prm.dense ? 8 : 28)) prm.split = 2;
     e = allow_shared_memory(attn_tc_kernel<B, true>, kAttnSmem);
     if (e != cudaSuccess) return e;
     ++*launches;
