@@ -801,6 +801,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
       live = next_tile(t++, ti);
       if (!live) return;
       if (lane == 0) sh.written[nt & 1][warp] = ti;
+      __syncwarp();  // all lanes read it when they write the tile, in a small launch maybe with no step in between
       n_steps = n_steps_of(ti.y);
       h = leads ? 0 : 1;
       m_ref = kNoReference;  // (rows without a key keep it)

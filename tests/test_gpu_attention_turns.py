@@ -55,6 +55,28 @@ def test_turns(oracle, block, H, N, most):
         assert torch.equal(O.contiguous().view(torch.int16), first[0].contiguous().view(torch.int16)) and torch.equal(lse, first[1])
 
 
+@pytest.mark.parametrize("block", [64, 128])
+@pytest.mark.parametrize("H,N", [(3, 128), (5, 77), (20, 500), (60, 300), (2, 2045)])  # clusters of four for the last; whole and ragged tiles
+def test_one_step_and_no_other(oracle, block, H, N):
+    """Small launches whose tiles have exactly one key step: the warpgroup without a step writes the tile and its log-sum-exps straight
+    away, by what it has just noted of the tile."""
+    from paper_2605_14513_b200 import heart
+
+    g = torch.Generator("cuda").manual_seed(H * N + block)
+    Q, K, V = (torch.randn((1, H, N, 128), generator=g, device="cuda").to(torch.bfloat16) for _ in range(3))
+    nb = heart.n_blocks(N, block)
+    idx, cnt = np.full((H, nb, nb), -1, np.int32), np.ones((H, nb), np.int32)
+    idx[:, :, 0] = (np.arange(H)[:, None] + np.arange(nb) * block // 128) % nb
+    cfg = heart.config_for(Q, block)
+    ws, O, lse = heart.new_workspace(cfg), torch.full_like(Q, float("nan")), torch.full((H, N), float("nan"), device="cuda")
+    heart.heart_block_sparse_attn(cfg, Q, K, V, torch.from_numpy(idx).cuda(), torch.from_numpy(cnt).cuda(), O, ws, lse=lse)
+    assert heart.heart_get_status(ws) == 0
+    ref, lse_ref = oracle.block_sparse_attn(*(inputs.bits(t) for t in (Q, K, V)), block, idx, cnt, want_lse=True)
+    check_attention(to_np(O.float()).astype(np.float64).reshape(H, N, 128), ref)
+    # fp32 accumulation of bf16-rounded weights (2^-9 relative each) in the sum behind the logarithm
+    assert np.allclose(to_np(lse), lse_ref, rtol=0, atol=2.0 ** -8)
+
+
 @pytest.mark.parametrize("H,N", [(2, 1), (1, 130), (2, 2045), (60, 700), (1, 9000), (1, 9473)])  # shared tiles (71: pairs; 75: a CTA each), several; ragged blocks
 def test_dense_calls_do_not_depend_on_the_block(H, N):
     from paper_2605_14513_b200 import heart
