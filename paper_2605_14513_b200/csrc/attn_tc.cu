@@ -55,8 +55,8 @@
 // 12.6 now.  (A first call of the merge code ahead of the wait, writing nothing, to have its instructions there: 12.9.)
 //
 // Every wait is bounded; a wait that runs out raises the CTA's abort flag and the status word, its roles
-// drain and stop.  The tile it worked on and those it had drawn already, or was dealt, stay unwritten (as does a tile that a
-// cluster shares); the other CTAs take the rest.
+// drain and stop.  A tile whose products are complete is still written; the tile that the wait was for and those the CTA had drawn
+// already, or was dealt, stay unwritten (as does a tile that a cluster shares); the other CTAs take the rest.
 #include <cuda.h>
 
 #include "common.cuh"
@@ -136,7 +136,8 @@ struct AttnParams {
   int split;        // small launches: CTAs (one cluster) that share the key steps of a tile
   int late;         // the warpgroup with a tile's first step takes its next one a step later: CTAs have several tiles
   int test_skip_v;      // test-hook builds only: CTA 0 leaves out the V copy of its second key step,
-  int test_skip_parts;  // CTA 1 does not send its part of a shared tile
+  int test_skip_parts;  // CTA 1 does not send its part of a shared tile,
+  int test_skip_k;      // CTA 0 leaves out the K copy of its second tile's first key step
 };
 
 __device__ __forceinline__ float fmax3(float a, float b, float c) {
@@ -595,6 +596,9 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
           const uint32_t e_next = h + 1 < n_steps ? step_entry(steps, h + 1) : 0u;
           if (g >= 2 && !wait1(&sh.s_full[g & 1], ((g - 2) >> 1) & 1)) break;
           sh.entry[g & 3] = e;
+#ifdef HEART_TEST_HOOKS
+          if (!(p.test_skip_k && blockIdx.x == 0 && t == 1 && h == 0))
+#endif
           load_k(smem + kOffK + (g & 1) * kTileBytes, &sh.k_full[g & 1], e, ti.z, ti.w);
           if (h == 0) {
             // its buffer is free: the last step of the tile before the previous one is complete, its output gone
@@ -978,17 +982,16 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
         }
         const bool whole_step = why == kRescale;
         why = kNothing;
-        if (!ok) break;
-        if (!whole_step) continue;
+        if (ok && !whole_step) continue;
       }
-      if (!ok) break;
-      if (Small && h >= n_steps) end_tile();
+      if (Small && ok && h >= n_steps) end_tile();
       if (pending) {
-        // ===== the output of the tile before, O / l, one row per thread
+        // ===== the output of the tile before, O / l, one row per thread (when this CTA gives up, too, if the tile's products are
+        // complete: it lacks nothing of what did not come)
         pending = false;
         const uint32_t q_buf = (nt - 1) & 1;
         const int4 to = sh.written[q_buf][warp];
-        if (!wait(&sh.o_full[q_buf], ((nt - 1) >> 1) & 1)) break;
+        if (ok ? !wait(&sh.o_full[q_buf], ((nt - 1) >> 1) & 1) : !__all_sync(0xffffffffu, mbar_test_wait(&sh.o_full[q_buf], ((nt - 1) >> 1) & 1))) break;
         tc_fence_after();
         const float2 own = sh.own[w][row], other = sh.l[q_buf][row];
         const float l = other.x + own.x * ex2(own.y - other.y), m = other.y;
@@ -1038,6 +1041,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
           __syncwarp();
         }
       }
+      if (!ok) break;
       if (h < n_steps) continue;
       if (Small || !live) break;
       end_tile();
@@ -1287,6 +1291,7 @@ cudaError_t launch_attention(const Geom &given, const Workspace &w, const void *
 #ifdef HEART_TEST_HOOKS
   prm.test_skip_v = (g.flags & 0x80000000u) ? 1 : 0;
   prm.test_skip_parts = (g.flags & 0x40000000u) ? 1 : 0;
+  prm.test_skip_k = (g.flags & 0x20000000u) ? 1 : 0;
 #endif
   return g.block == 64 ? launch_bk<64>(g, w, mq, mk, mv, mo, prm, kv_idx, kv_cnt, s, launches)
                        : launch_bk<128>(g, w, mq, mk, mv, mo, prm, kv_idx, kv_cnt, s, launches);

@@ -6,7 +6,8 @@ released, the CTA exits and the workspace's status word reports HEART_ERR_DEVICE
 test-hook build of the library (same sources, HEART_TEST_HOOKS, a wait limit of 2e6 clocks) has one
 reserved flag bit that makes the V producer of CTA 0 leave out one copy -- neither the byte count is
 announced nor the copy issued -- so the waits that depend on that tile run out after about a
-millisecond; another bit keeps a CTA's part of a shared tile from the other CTAs of its cluster.  Nothing traps and nothing waits without a bound.
+millisecond; another bit keeps a CTA's part of a shared tile from the other CTAs of its cluster, a third leaves out the K copy of the
+first key step of CTA 0's second tile.  Nothing traps and nothing waits without a bound.
 """
 import time
 
@@ -21,6 +22,7 @@ pytestmark = pytest.mark.gpu
 
 TEST_SKIP_V = 0x80000000
 TEST_SKIP_PARTS = 0x40000000
+TEST_SKIP_K = 0x20000000
 
 
 def dense_attention(h, flags, Q, K, V, wl):
@@ -109,6 +111,47 @@ def test_other_tiles_are_complete_after_an_abort(hooks, block, H, N):
             bad[0, head, 128 * t : 128 * t + 128] = ref[0, head, 128 * t : 128 * t + 128]
         assert torch.equal(bad.view(torch.int16), ref.view(torch.int16))
         cfg.flags &= ~TEST_SKIP_V
+        h.heart_block_sparse_attn(cfg, Q, K, V, *use, again, ws)
+        assert h.heart_get_status(ws) == 0
+        assert torch.equal(again.view(torch.int16), ref.view(torch.int16))
+
+
+@pytest.mark.parametrize("block", [64, 128])
+@pytest.mark.parametrize("H,N", [(200, 257), (80, 1000), (600, 128), (300, 256)])  # four tiles a CTA, of 3, 8, 1 and 2 steps
+def test_a_finished_tile_survives_the_abort_of_the_next(hooks, block, H, N):
+    """The products of CTA 0's first tile are complete when the wait for its second tile's first scores runs out: the first
+    tile's output and log-sum-exps are there, the second tile is the one that is lost."""
+    h = hooks
+    g = torch.Generator("cuda").manual_seed(N + block)
+    Q, K, V = (torch.randn((1, H, N, 128), generator=g, device="cuda").to(torch.bfloat16) for _ in range(3))
+    nb, tiles = h.n_blocks(N, block), (N + 127) // 128
+    idx = torch.arange(nb, dtype=torch.int32, device="cuda").expand(H, nb, nb).contiguous()
+    cnt = torch.full((H, nb), nb, dtype=torch.int32, device="cuda")
+    for dense in (True, False):
+        cfg = h.make_config(1, H, N, block, flags=h.FORCE_DENSE if dense else 0)
+        use = (None, None) if dense else (idx, cnt)
+        ws = h.new_workspace(cfg)
+        ref, bad = (torch.full_like(Q, float("nan")) for _ in range(2))
+        lse_ref, lse_bad = (torch.full((H, N), float("nan"), device="cuda") for _ in range(2))
+        h.heart_block_sparse_attn(cfg, Q, K, V, *use, ref, ws, lse=lse_ref)
+        assert h.heart_get_status(ws) == 0 and not ref.isnan().any()
+        cfg.flags |= TEST_SKIP_K
+        t0 = time.perf_counter()
+        h.heart_block_sparse_attn(cfg, Q, K, V, *use, bad, ws, lse=lse_bad)
+        assert h.heart_get_status(ws) == h.ERR_DEVICE_CHECK
+        assert time.perf_counter() - t0 < 5.0
+        lost = [(head, t) for head in range(H) for t in range(tiles) if bad[0, head, 128 * t].isnan().any()]
+        if dense:  # dealt in turn
+            assert lost == [divmod(n, tiles) for n in range(148, H * tiles, 148)]
+        else:  # its second tile, and those drawn behind it already
+            assert 1 <= len(lost) <= 3
+        for head, t in lost:
+            rows = slice(128 * t, 128 * t + 128)
+            assert bad[0, head, rows].isnan().all() and lse_bad[head, rows].isnan().all()
+            bad[0, head, rows], lse_bad[head, rows] = ref[0, head, rows], lse_ref[head, rows]
+        assert torch.equal(bad.view(torch.int16), ref.view(torch.int16)) and torch.equal(lse_bad, lse_ref)
+        again = torch.full_like(Q, float("nan"))
+        cfg.flags &= ~TEST_SKIP_K
         h.heart_block_sparse_attn(cfg, Q, K, V, *use, again, ws)
         assert h.heart_get_status(ws) == 0
         assert torch.equal(again.view(torch.int16), ref.view(torch.int16))
