@@ -135,9 +135,9 @@ struct AttnParams {
   float scale_log2;
   int split;        // small launches: CTAs (one cluster) that share the key steps of a tile
   int late;         // the warpgroup with a tile's first step takes its next one a step later: CTAs have several tiles
-  int test_skip_v;      // test-hook builds only: CTA 0 leaves out the V copy of its second key step,
-  int test_skip_parts;  // CTA 1 does not send its part of a shared tile,
-  int test_skip_k;      // CTA 0 leaves out the K copy of its second tile's first key step
+  // test-hook builds only: CTA 0 leaves out the V copy of its second key step (1) or the K copy of its second tile's first
+  // step (2), CTA 1 does not send its part of a shared tile (4)
+  int test_skip;
 };
 
 __device__ __forceinline__ float fmax3(float a, float b, float c) {
@@ -597,7 +597,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
           if (g >= 2 && !wait1(&sh.s_full[g & 1], ((g - 2) >> 1) & 1)) break;
           sh.entry[g & 3] = e;
 #ifdef HEART_TEST_HOOKS
-          if (!(p.test_skip_k && blockIdx.x == 0 && t == 1 && h == 0))
+          if (!((p.test_skip & 2) && blockIdx.x == 0 && t == 1 && h == 0))
 #endif
           load_k(smem + kOffK + (g & 1) * kTileBytes, &sh.k_full[g & 1], e, ti.z, ti.w);
           if (h == 0) {
@@ -639,7 +639,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
 #ifdef HEART_TEST_HOOKS
         // Test-only library: one V tile is never requested (neither the byte count nor the copy), so the
         // waits that depend on it run out and the abort path is taken.
-        if (p.test_skip_v && blockIdx.x == 0 && g == 1) continue;
+        if ((p.test_skip & 1) && blockIdx.x == 0 && g == 1) continue;
 #endif
         if (lane == 0) load_v(smem + kOffV + (g & 1) * kTileBytes, &sh.v_full[g & 1], e, ti.z, ti.w);
       }
@@ -984,14 +984,15 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
         why = kNothing;
         if (ok && !whole_step) continue;
       }
-      if (Small && ok && h >= n_steps) end_tile();
+      if (Small && !ok) break;
+      if (Small && h >= n_steps) end_tile();
       if (pending) {
         // ===== the output of the tile before, O / l, one row per thread (when this CTA gives up, too, if the tile's products are
         // complete: it lacks nothing of what did not come)
         pending = false;
         const uint32_t q_buf = (nt - 1) & 1;
         const int4 to = sh.written[q_buf][warp];
-        if (ok ? !wait(&sh.o_full[q_buf], ((nt - 1) >> 1) & 1) : !__all_sync(0xffffffffu, mbar_test_wait(&sh.o_full[q_buf], ((nt - 1) >> 1) & 1))) break;
+        if (Small || ok ? !wait(&sh.o_full[q_buf], ((nt - 1) >> 1) & 1) : !__all_sync(0xffffffffu, mbar_test_wait(&sh.o_full[q_buf], ((nt - 1) >> 1) & 1))) break;
         tc_fence_after();
         const float2 own = sh.own[w][row], other = sh.l[q_buf][row];
         const float l = other.x + own.x * ex2(own.y - other.y), m = other.y;
@@ -1057,7 +1058,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
       const bool aborted = *abort != 0;
       if (tid == 0) mbar_expect_tx(&sh.parts_full, (p.split - 1) * rows * (512 + (int)sizeof(float2)));
 #ifdef HEART_TEST_HOOKS
-      const bool send = !(p.test_skip_parts && blockIdx.x == 1);  // test-only library: one CTA's part never leaves
+      const bool send = !((p.test_skip & 4) && blockIdx.x == 1);  // test-only library: one CTA's part never leaves
 #else
       constexpr bool send = true;
 #endif
@@ -1289,9 +1290,7 @@ cudaError_t launch_attention(const Geom &given, const Workspace &w, const void *
   prm.hcount = hcount;
   prm.scale_log2 = (float)(g.scale * 1.4426950408889634);
 #ifdef HEART_TEST_HOOKS
-  prm.test_skip_v = (g.flags & 0x80000000u) ? 1 : 0;
-  prm.test_skip_parts = (g.flags & 0x40000000u) ? 1 : 0;
-  prm.test_skip_k = (g.flags & 0x20000000u) ? 1 : 0;
+  prm.test_skip = (g.flags & 0x80000000u ? 1 : 0) | (g.flags & 0x20000000u ? 2 : 0) | (g.flags & 0x40000000u ? 4 : 0);
 #endif
   return g.block == 64 ? launch_bk<64>(g, w, mq, mk, mv, mo, prm, kv_idx, kv_cnt, s, launches)
                        : launch_bk<128>(g, w, mq, mk, mv, mo, prm, kv_idx, kv_cnt, s, launches);
