@@ -912,9 +912,11 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
           tmem_st32(p_at + 32, pk);
         } else {
           // This row's query block lists one of the step's two blocks or none.  The product reads all 128 keys of the
-          // step: zeros for the others.  (Short code rather than fast code: the step is bound by its products.)
+          // step: zeros for the others, in one store (eight keys at a time: 12 x 33k, 30 % of the blocks at random, 2658 us instead of
+          // 2538, whole steps of 40 x 33k 0.4 % more).  The exponentials in a loop: unrolled, the random lists take 2 % less, short
+          // ones, 24 x 2465, 0.6 % more.
           const uint32_t v = flags >> 16;
-          uint32_t s[64], pk[16];
+          uint32_t s[64], pk[16], zeros[32];
           tmem_ld32(s_at + v * 64, *reinterpret_cast<uint32_t(*)[32]>(&s[0]));
           tmem_ld32(s_at + v * 64 + 32, *reinterpret_cast<uint32_t(*)[32]>(&s[32]));
           take_reference();
@@ -925,8 +927,10 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
           p_free();
           const uint64_t neg_m2 = pack_f32x2(-m_ref, -m_ref);
           const uint32_t n_exp = flags != 0u ? 4 : 0;
-#pragma unroll 1
-          for (uint32_t i = n_exp; i < 8; ++i) tmem_st8_fill(p_at + ((v * 32 + i * 8) & 63), 0u);
+#pragma unroll
+          for (int i = 0; i < 32; ++i) zeros[i] = 0u;
+          tmem_st32(p_at + (32 - v * 32), zeros);
+          if (n_exp == 0) tmem_st32(p_at + v * 32, zeros);
 #pragma unroll 1
           for (uint32_t i = 0; i < n_exp; i += 2) {
             exp32(&s[0], c2, neg_m2, &pk[0], sums);
