@@ -810,15 +810,19 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
       h = leads ? 0 : 1;
       m_ref = kNoReference;  // (rows without a key keep it)
       l_run = 0.f;
-      if (n_steps == 0 && leads) {  // rows without any key
-        const int tok = ti.x * 128 + row;
+      if (n_steps == 0) {  // rows without any key: 16 a warp, two at a time (a row a thread, by one warpgroup, took 42.8 us
+                           // instead of 33.4 for 12 x 33k of such tiles)
         if (shared_tile) {
-          sh.part_l[row] = make_float2(0.f, kNoReference);  // (nothing else of this part is read)
-        } else if (tok < p.N) {
-          uint4 *out = reinterpret_cast<uint4 *>(p.O + (long long)ti.w * p.sb + (long long)ti.z * p.sh + (long long)tok * p.sn);
+          if (leads) sh.part_l[row] = make_float2(0.f, kNoReference);  // (nothing else of this part is read)
+        } else {
+          int tok = ti.x * 128 + (int)warp * 16 + (lane >> 4);
+          uint16_t *out = p.O + (long long)ti.w * p.sb + (long long)ti.z * p.sh + tok * p.sn + (lane & 15) * 8;
+          float *lse = p.lse == nullptr ? nullptr : p.lse + (size_t)(ti.w * p.H + ti.z) * p.N;
 #pragma unroll 1
-          for (int i = 0; i < 16; ++i) out[i] = make_uint4(0u, 0u, 0u, 0u);
-          if (p.lse != nullptr) p.lse[(size_t)(ti.w * p.H + ti.z) * p.N + tok] = -INFINITY;
+          for (int i = 0; i < 8 && tok < p.N; ++i, tok += 2, out += 2 * p.sn) {
+            *reinterpret_cast<uint4 *>(out) = make_uint4(0u, 0u, 0u, 0u);
+            if (lse != nullptr && (lane & 15) == 0) lse[tok] = -INFINITY;
+          }
         }
       }
     };
