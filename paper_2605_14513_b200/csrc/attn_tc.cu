@@ -26,7 +26,8 @@
 //               next tile and then writes O / l (and lse) of the tile, by a bulk copy from the place of its Q; meanwhile the
 //               other one takes the second and the third.  (The warpgroup of the last step waited 1300 clocks for the last
 //               products and wrote for 3300 more, with its partner waiting for its step of the next tile: 40 x 33k, 69 tiles a
-//               CTA, 2860 us, now 2745; 2 x 12 x 2465 72.5, now 69.5.)
+//               CTA, 2860 us, now 2745; 2 x 12 x 2465 72.5, now 69.5.)  A tile of one step, with many tiles of two, is still written
+//               by the warpgroup of its last step, before that one goes on.
 //   warp 8      issues S_g = Q K_g^T once step g - 2 has emptied the buffer, warp 11 O += P_g V_g.
 //   warp 9      V producer, warp 10 K and Q producer (draws the tiles and announces them): TMA loads
 //               (cp.async.bulk.tensor, 128-byte swizzle, completion on mbarriers), two 32 KB buffers each.
@@ -104,8 +105,8 @@ struct AttnShared {
   uint32_t entry[4];       // the key steps in flight, for the softmax warps: entry[g & 3] is written before K_g is asked
                            // for and read before the scores of step g are handed back, which K_{g+4} waits for
   float m[2][128];         // references after step g
-  float2 l[2][128];        // row sum and its reference of the warpgroup with a tile's last step, per tile & 1
-  float2 own[2][128];      // the same of the other one, per warpgroup, until it writes the tile
+  float2 l[2][2][128];     // row sums and their references for the warpgroup that writes a tile: per tile & 1 and warpgroup; in a small
+                           // launch the ones of the tile's last step, and those of the writer
   int4 written[2][8];      // that tile, per softmax warp
   uint32_t tmem_base;
   int abort;
@@ -134,7 +135,8 @@ struct AttnParams {
   int h0, hcount;  // this launch covers heads [h0, h0 + hcount) of every batch entry
   float scale_log2;
   int split;        // small launches: CTAs (one cluster) that share the key steps of a tile
-  int late;         // the warpgroup with a tile's first step takes its next one a step later: CTAs have several tiles
+  short at_once;    // a tile of at most so many steps is written by the warpgroup of its last step, before that one goes on
+  short late;       // the warpgroup with a tile's first step takes its next one a step later: CTAs have several tiles
   // test-hook builds only: CTA 0 leaves out the V copy of its second key step (1) or the K copy of its second tile's first
   // step (2), CTA 1 does not send its part of a shared tile (4)
   int test_skip;
@@ -747,7 +749,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     uint32_t g0 = 0, nt = 0;  // key steps before the present tile, tiles with key steps before it
     int n_steps = 0, h = 0;   // of the present tile; this warpgroup's next step of it
     bool leads = w == 0;      // takes the tile's first step
-    bool pending = false;     // the tile before is this warpgroup's to write
+    uint32_t pending = 0;     // the tile before is this warpgroup's to write: 1 behind its first step of the next one, 2 before
     bool live = true;
     float m_ref = kNoReference, l_run = 0.f;
     // Why the loop over the steps was left: what a step rarely needs stands outside of it.
@@ -759,7 +761,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
       // the tile before meanwhile.  (In a CTA's first tile too: the order of a row's sum goes by the shape alone.)
       const bool first = h < 2;
       h += first && p.late ? 3 - 2 * h : 2;
-      return first && pending;
+      return first && pending != 0;
     };
     auto mask_keys = [&](uint32_t b, uint32_t e) {
       // Keys that do not count get a score of -inf in tensor memory, where a loop over columns is a loop;
@@ -788,13 +790,15 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
       tmem_wait_st();
     };
     auto end_tile = [&]() {
-      if (n_steps == 0) return;
+      if (n_steps == 0) return;  // (a tile without keys)
       const int last = n_steps - 1;
       const bool mine = leads == (p.late ? last == 0 || (last > 2 && (last & 1)) : !(last & 1));  // had the last step
       leads = !mine;
-      if (!mine) {
-        pending = true;
-        sh.own[w][row] = make_float2(l_run, m_ref);
+      const bool at_once = !Small && n_steps <= p.at_once;
+      if (mine == at_once) {
+        pending = at_once ? 2 : 1;
+        if (Small) sh.l[1][w][row] = make_float2(l_run, m_ref);
+        if (at_once && n_steps == 1) sh.l[nt & 1][w ^ 1][row] = make_float2(0.f, kNoReference);  // (the other one had no step)
       }
       g0 += n_steps;
       ++nt;
@@ -828,6 +832,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     };
     if (Small) next();  // (the only one)
     for (;;) {
+      if (Small || pending != 2)  // (a tile that is written at once comes before the steps of the next one)
 #pragma unroll 1
       while (h < n_steps) {
         const uint32_t g = g0 + h, b = g & 1, s_at = s_addr + b * 128, p_at = p_addr + b * 64;
@@ -944,7 +949,12 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
           }
         }
         l_run += (sums.a + sums.b) + (sums.c + sums.d);
-        if (h == n_steps - 1) sh.l[nt & 1][row] = make_float2(l_run, m_ref);  // the other warpgroup finishes the tile
+        // for the warpgroup that writes the tile (each one's last step is among the tile's last three)
+        if (Small) {
+          if (h == n_steps - 1) sh.l[0][nt & 1][row] = make_float2(l_run, m_ref);
+        } else {
+          if (h >= n_steps - 3) sh.l[nt & 1][w][row] = make_float2(l_run, m_ref);
+        }
         if (!ok) break;
         if (__builtin_expect(moved && h > 0, 0)) {
           why = kRescale;
@@ -997,13 +1007,16 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
       if (pending) {
         // ===== the output of the tile before, O / l, one row per thread (when this CTA gives up, too, if the tile's products are
         // complete: it lacks nothing of what did not come)
-        pending = false;
+        const uint32_t w_last = pending == 2 ? w : w ^ 1;
+        pending = 0;
         const uint32_t q_buf = (nt - 1) & 1;
         const int4 to = sh.written[q_buf][warp];
         if (Small || ok ? !wait(&sh.o_full[q_buf], ((nt - 1) >> 1) & 1) : !__all_sync(0xffffffffu, mbar_test_wait(&sh.o_full[q_buf], ((nt - 1) >> 1) & 1))) break;
         tc_fence_after();
-        const float2 own = sh.own[w][row], other = sh.l[q_buf][row];
-        const float l = other.x + own.x * ex2(own.y - other.y), m = other.y;
+        // the sums of the warpgroup with the tile's last step, whose reference O has, and of the other one
+        const float2 last = Small ? sh.l[0][q_buf][row] : sh.l[q_buf][w_last][row];
+        const float2 other = Small ? sh.l[1][w][row] : sh.l[q_buf][w_last ^ 1][row];
+        const float l = last.x + other.x * ex2(other.y - last.y), m = last.y;
         const float inv = l > 0.f ? 1.f / l : 0.f;
         const uint64_t inv2 = pack_f32x2(inv, inv);
         // Through the place of the tile's Q, a copy of 32 rows a warp; rows behind the last token are not written.
@@ -1224,6 +1237,11 @@ cudaError_t launch_bk(const Geom &g, const Workspace &w, const CUtensorMap &mq, 
   plan.hcount = prm.hcount;
   plan.ragged = (int)(g.N % g.block != 0);
   plan.status = prm.status;
+  // The other warpgroup has a step of a short tile or none, so most of the next tile would wait for the output behind its first step: us
+  // at once, and behind a step of the next tile, for tiles of one step, 12 x 33k 71.5 and 98.9, 24 x 2465 20.8 and 23.1, 40 x 1000 19.8 and
+  // 20.8; of two, 12 x 33k 91 and 110, 8 x 16000 39.1 and 44.0, 1200 tiles of 5000 tokens a head 44.8 and 50.3, but 520 tiles 26.4 and 26.0,
+  // 320 tiles of 1000 24.0 and 22.1: with few tiles a CTA the way to the first output counts.
+  prm.at_once = prm.n_tiles >= 5 * kSms ? 2 : 1;
   prm.late = all_tiles > (size_t)kSms;  // by the tiles of all heads, not of this launch: a call that runs its heads in groups gives the same bits
   if (prm.n_tiles <= kSms) {
     // Shared among CTAs as far as there are SMs (by the tiles of all heads as well).  Sharing costs 1.2 us for the copies of the parts

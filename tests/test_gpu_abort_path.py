@@ -117,7 +117,7 @@ def test_other_tiles_are_complete_after_an_abort(hooks, block, H, N):
 
 
 @pytest.mark.parametrize("block", [64, 128])
-@pytest.mark.parametrize("H,N", [(200, 257), (80, 1000), (600, 128), (300, 256)])  # four tiles a CTA, of 3, 8, 1 and 2 steps
+@pytest.mark.parametrize("H,N", [(200, 257), (80, 1000), (600, 128), (300, 256), (400, 256)])  # four tiles a CTA and more, of 3, 8, 1, 2 and 2 steps
 def test_a_finished_tile_survives_the_abort_of_the_next(hooks, block, H, N):
     """The products of CTA 0's first tile are complete when the wait for its second tile's first scores runs out: the first
     tile's output and log-sum-exps are there, the second tile is the one that is lost."""

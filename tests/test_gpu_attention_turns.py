@@ -15,6 +15,7 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("block", [64, 128])
 @pytest.mark.parametrize("H,N,most", [
     (90, 128 * 7 - 31, 7),  # 630 tiles: four or five a CTA; the last rows of a head fill no copy
+    (110, 128 * 7 - 31, 7), # 770: short tiles are written at once, the others behind a step of the next one
     (400, 128 + 33, 2),     # tiles of one and two steps only: the roles change with every tile
     (149, 120, 1),          # one tile more than CTAs
     (2, 4500, 36),          # 72 tiles, a pair of CTAs each
