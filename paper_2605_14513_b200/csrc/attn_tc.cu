@@ -432,9 +432,9 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
   tc_fence_after();
   const uint32_t tmem = sh.tmem_base;
 
-  // Key steps of a tile with U listed key blocks that this CTA takes, and the first one of them.  (A tile of one step is not
-  // shared: its cluster's first CTA takes it and the others leave.  2 x 2048 tokens: 8.6 us against 12.4 with one key block
-  // listed, 5.9 against 9.5 with none.)
+  // Key steps of a tile with U listed key blocks that this CTA takes, and the first one of them.  (A tile of fewer than four steps is
+  // not shared: its cluster's first CTA takes it and the others leave.  64 tiles, us with two CTAs on each tile and with one: two steps
+  // 10.0 and 9.2, three 10.6 and 10.2, four 10.7 and 10.9; 32 tiles with four CTAs 10.7 and 9.0, 10.6 and 10.1, 10.8 and 10.8.)
   bool shared_tile = false, at_barrier = false;
   int parts_of_tile = 1;
   auto first_step = [&](int U, int part) -> int { return Small ? (B == 128 ? U : (U + 1) / 2) * part / parts_of_tile : 0; };
@@ -472,7 +472,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     return ok;
   };
   auto small_tile = [&](int U) {
-    shared_tile = p.split > 1 && U > (B == 128 ? 1 : 2);
+    shared_tile = p.split > 1 && (B == 128 ? U : (U + 1) / 2) >= 4;
     parts_of_tile = shared_tile ? p.split : 1;
   };
   // The announced tile t; false: none left (or abort).  Every lane of the warp gets the same answer.
@@ -1244,11 +1244,13 @@ cudaError_t launch_bk(const Geom &g, const Workspace &w, const CUtensorMap &mq, 
   prm.at_once = prm.n_tiles >= 5 * kSms ? 2 : 1;
   prm.late = all_tiles > (size_t)kSms;  // by the tiles of all heads, not of this launch: a call that runs its heads in groups gives the same bits
   if (prm.n_tiles <= kSms) {
-    // Shared among CTAs as far as there are SMs (by the tiles of all heads as well).  Sharing costs 1.2 us for the copies of the parts
-    // and the wait for the others': it pays from eight key steps a tile on, and lists have half of all or less.  us with a
-    // CTA a tile and with two: 48 tiles of at most six steps, of which lists name 2 to 4, 9.7 and 10.9; 72 tiles, 36 steps,
-    // whole steps of 2 x 4500 tokens 36.1 and 29.9, 24 steps dense 27.3 and 21.4; 1 head x 9000 tokens 29.5 and 21.0, dense 61.1 and 38.6.
-    // (With a third of the blocks listed, 22 steps are 23.9 and 24.3; 72 tiles whose lists name one or two of 72 blocks 8.0 and 9.9.)
+    // Shared among CTAs as far as there are SMs (by the tiles of all heads as well).  The kernel shares tiles of four steps and more, as
+    // planned; the launch goes by the steps a tile could have, because one as clusters costs by itself, 0.6 us with 28 CTAs to 1.3 with
+    // 148 (launches back to back: the next one finds no room while it runs).  Dense calls have all their steps: pairs from four on, to all
+    // SMs from eight on.  Lists, us with a CTA a tile and with two: up to 64 tiles, seven steps possible and all listed 11.9 and 11.4
+    // (14 tiles) or 12.7 and 12.7 (63), two listed 7.5 and 7.9 or 8.0 and 9.2; 65 to 74 tiles, 36 possible: all 34.0 and 24.3, 70 % at
+    // random 31.5 and 22.7, ten 14.5 and 13.9, eight 13.0 and 13.0, six 11.5 and 12.3, two 8.1 and 9.4; 22 possible, a third listed, 23.9
+    // and 24.3.
     const int steps = prm.step_pitch;  // of a tile whose blocks list all
     prm.split = 1;
     if (all_tiles * 4 <= kSplitCtas && steps >= 8) prm.split = 4;

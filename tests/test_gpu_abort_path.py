@@ -81,7 +81,8 @@ def hooks():
 
 
 @pytest.mark.parametrize("block", [64, 128])
-@pytest.mark.parametrize("H,N", [(2, 420), (2, 2045), (80, 257)])  # tiles shared by two CTAs and by four; 240 tiles of 2 or 3 steps for 148 CTAs
+# tiles shared by two CTAs if dense, by four, by two (lists too, 9 and 36 steps); 240 tiles of 2 or 3 steps for 148 CTAs
+@pytest.mark.parametrize("H,N", [(2, 420), (2, 2045), (4, 1029), (2, 4500), (80, 257)])
 def test_other_tiles_are_complete_after_an_abort(hooks, block, H, N):
     h = hooks
     g = torch.Generator("cuda").manual_seed(N)

@@ -16,7 +16,7 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("B,H,N", [
     (1, 1, 1),       # one row
     (1, 2, 130),     # one key step a part is too few: not shared
-    (2, 1, 512),     # two CTAs a tile
+    (2, 1, 512),     # dense: two CTAs a tile
     (1, 2, 2045),    # 32 tiles: four CTAs
     (1, 4, 1029),    # 36 tiles: two
     (1, 65, 255),    # 130 tiles: not shared

@@ -57,17 +57,24 @@ def test_turns(oracle, block, H, N, most):
 
 
 @pytest.mark.parametrize("block", [64, 128])
-@pytest.mark.parametrize("H,N", [(3, 128), (5, 77), (20, 500), (60, 300), (2, 2045)])  # clusters of four for the last; whole and ragged tiles
-def test_one_step_and_no_other(oracle, block, H, N):
-    """Small launches whose tiles have exactly one key step: the warpgroup without a step writes the tile and its log-sum-exps straight
-    away, by what it has just noted of the tile."""
+@pytest.mark.parametrize("H,N,steps", [
+    (3, 128, 1), (5, 77, 1), (20, 500, 1), (60, 300, 1),
+    (2, 2045, 1), (2, 2045, 3), (2, 2045, 4),  # launched as clusters of four; shared from four steps on
+    (4, 1029, 2), (4, 1029, 3), (4, 1029, 4),  # of two
+    (2, 4500, 3), (2, 4500, 5),                # 72 tiles, pairs
+])
+def test_tiles_of_a_few_steps_in_small_launches(oracle, block, H, N, steps):
+    """With one step, the warpgroup without it writes the tile and its log-sum-exps straight away, by what it has just noted of the
+    tile; up to three, one CTA of a cluster takes all of them."""
     from paper_2605_14513_b200 import heart
 
     g = torch.Generator("cuda").manual_seed(H * N + block)
     Q, K, V = (torch.randn((1, H, N, 128), generator=g, device="cuda").to(torch.bfloat16) for _ in range(3))
-    nb = heart.n_blocks(N, block)
-    idx, cnt = np.full((H, nb, nb), -1, np.int32), np.ones((H, nb), np.int32)
-    idx[:, :, 0] = (np.arange(H)[:, None] + np.arange(nb) * block // 128) % nb
+    nb, per = heart.n_blocks(N, block), 128 // block
+    idx, cnt = np.full((H, nb, nb), -1, np.int32), np.full((H, nb), min(nb, steps * per), np.int32)
+    first = per * (np.arange(H)[:, None] + np.arange(nb) // per)  # the query blocks of a tile list the same key blocks
+    for k in range(cnt[0, 0]):
+        idx[:, :, k] = (first + k) % nb
     cfg = heart.config_for(Q, block)
     ws, O, lse = heart.new_workspace(cfg), torch.full_like(Q, float("nan")), torch.full((H, N), float("nan"), device="cuda")
     heart.heart_block_sparse_attn(cfg, Q, K, V, torch.from_numpy(idx).cuda(), torch.from_numpy(cnt).cuda(), O, ws, lse=lse)
