@@ -101,3 +101,27 @@ def test_dense_calls_do_not_depend_on_the_block(H, N):
     assert torch.equal(outs[0][0].view(torch.int16), outs[1][0].view(torch.int16)) and torch.equal(outs[0][1], outs[1][1])
     ref = torch.nn.functional.scaled_dot_product_attention(Q.double(), K.double(), V.double())
     check_attention(to_np(outs[0][0].float()).astype(np.float64).reshape(H, N, 128), to_np(ref).reshape(H, N, 128))
+
+
+@pytest.mark.parametrize("block", [64, 128])
+@pytest.mark.parametrize("dense", [False, True])
+@pytest.mark.parametrize("H,N", [(40, 420), (16, 1300)])  # 160 and 176 tiles in all, 8 to 12 in a group of heads
+def test_head_groups_give_the_bits_of_the_whole(block, dense, H, N):
+    """heart_step_host runs its heads in groups, of a tile per CTA here, heart_step all of them with several tiles per CTA: the order
+    of a row's sums goes by the tiles of all heads, so the outputs are equal bit for bit."""
+    from paper_2605_14513_b200 import heart
+
+    g = torch.Generator("cuda").manual_seed(H * N + block)
+    Q, K, V = (torch.randn((1, H, N, 128), generator=g, device="cuda").to(torch.bfloat16) for _ in range(3))
+    cfg = heart.make_config(1, H, N, block, flags=heart.FORCE_DENSE if dense else 0)
+    delta = torch.full((H,), -1.0, dtype=torch.float64, device="cuda")
+    tau = torch.linspace(0.3, 0.95, H, dtype=torch.float64, device="cuda")
+    whole, groups, ws, ws_host = heart.State(cfg), heart.State(cfg), heart.new_workspace(cfg), heart.new_workspace(cfg)
+    O = torch.full_like(Q, float("nan"))
+    heart.heart_step(cfg, Q, K, V, delta, tau, whole, O, ws)
+    host = [x.cpu().pin_memory() for x in (Q, K, V)]
+    O_host = torch.full(Q.shape, float("nan"), dtype=torch.bfloat16).pin_memory()
+    heart.heart_step_host(cfg, *host, delta, tau, groups, O_host, tuple(torch.empty_like(Q) for _ in range(4)), ws_host)
+    assert heart.heart_get_status(ws) == 0 and heart.heart_get_status(ws_host) == 0
+    assert not O.isnan().any()
+    assert torch.equal(O.cpu().view(torch.int16), O_host.view(torch.int16))
