@@ -704,14 +704,16 @@ cudaError_t launch_pooled_scores(const Geom &g, const Workspace &w, const uint8_
                                  int *launches, unsigned long long expect_sig) {
   ++*launches;
   // Tiles of 64 x 64 scores read their operands half as often as tiles of 32 x 32, which leave less of the chip idle: up to half a wave
-  // of large ones (a tile an SM) small ones with all dims loaded at once, up to a whole one small ones in three stages,
+  // of large ones (a tile an SM) small ones with all dims loaded at once, up to three waves of small ones these in three stages,
   // beyond that these where their waves, at 0.35 of a large one's time, are shorter: few waves, or much padding.  Whole calls timed
   // both ways on 354 shapes (129 to 1000 blocks, 1 to 40 heads), against the first kind up to a wave and large ones beyond: 0.978 in
-  // the mean, largest 1.037 (520 x 1 head); us, before / now: 24 heads x 130 blocks 21.6 / 17.4, 30 x 200 36.4 / 32.3, 3 x 600 39.1 / 36.2.
+  // the mean, us, before / now: 24 heads x 130 blocks 21.6 / 17.4, 30 x 200 36.4 / 32.3, 3 x 600 39.1 / 36.2.  One wave of large ones
+  // against four of small ones, 31 shapes: 0.96 in the mean, 768 blocks 14.3 / 16.8, 8 x 256 12.7 / 14.3, largest 14.4 / 13.9 (5 x 289);
+  // against three, 56 shapes: 1.17, 12 x 192 12.5 / 10.6.
   const long long n64 = (g.nb + 63) / 64, n32 = (g.nb + 31) / 32, tiles64 = n64 * n64 * g.R, tiles32 = n32 * n32 * g.R;
   auto waves = [](long long tiles) { return (tiles + 147) / 148; };
   if (tiles64 <= 74) return launch_scores<16, 128, 1>(g, w, refresh, s, expect_sig);
-  if (tiles64 <= 148 || 35 * waves(tiles32) < 100 * waves(tiles64)) return launch_scores<16, 32, 3>(g, w, refresh, s, expect_sig);
+  if (tiles32 <= 3 * 148 || 35 * waves(tiles32) < 100 * waves(tiles64)) return launch_scores<16, 32, 3>(g, w, refresh, s, expect_sig);
   return launch_scores<32, 16, 3>(g, w, refresh, s, expect_sig);
 }
 
