@@ -2,9 +2,9 @@
 
 `build()` makes the product library.  `build_test_hooks()` makes a second, test-only library
 (libheart_testhooks.so) from the same sources with HEART_TEST_HOOKS defined and a short bounded-wait
-limit: in it a reserved flag bit makes the attention kernel's V producer, or the antidiagonal kernel's
-producer, leave out one copy, so that the kernels' time-out / abort / drain paths can be exercised by a test
-without faulting or hanging anything.  The product library does not contain that hook.
+limit: in it reserved flag bits make the attention kernel's V or K producer, or the antidiagonal kernel's
+producer, leave out one copy, or keep a CTA's part of a shared tile from the others, so that the kernels' time-out / abort / drain
+paths can be exercised by a test without faulting or hanging anything.  The product library does not contain those hooks.
 """
 from __future__ import annotations
 

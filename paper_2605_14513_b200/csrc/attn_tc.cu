@@ -79,8 +79,9 @@ constexpr float kNoReference = -3.0e38f;  // below every logit: the first step m
 // below 1: weights are at most 2^8, so n keys with values up to 2^120 / n cannot overflow O (all of it above 1, with
 // weights up to 2^64, left 2^64 / n), and a weight of 2^-110 of the largest is still a normal number.
 constexpr float kHeadroom = 16.f, kMaxGrowth = 8.f;
-// ns that a softmax warp waits for its scores before it leaves the loop over its steps (20 instead of 500: 24 x 119k, at the power limit,
-// 11210 us instead of 11014, 40 x 76k 13554 instead of 13376, 16 x 8k 142.2 instead of 141.5)
+// ns that a softmax warp waits for its scores before it leaves the loop over its steps for a bounded wait.  (Nothing hangs on it: us with
+// 20 and with 500, 24 x 119k 10941 and 10959, 40 x 76k 13146 and 13165, 16 x 8k 141.7 and 142.0, antidiagonal 12 x 33k 1073 and 1071, where
+// two runs differ by as much.)
 constexpr uint32_t kShortWait = 500;
 constexpr int kMaxSplit = 4;  // CTAs that share a tile in a small launch
 
